@@ -1,15 +1,15 @@
 // Batched matching: many queries in one matcher launch.
 //
-// A fast_batch owns fixed device buffers (per-query plans, the concatenated
-// chunk list, counters, the ring of donated runs), so that its matcher
-// launch can be captured once as a CUDA graph and replayed for every batch.
+// A fast_batch owns fixed device buffers (per-query plans, counters, the
+// ring of donated runs), so that its matcher launch can be captured once as a
+// CUDA graph and replayed for every batch.
 // A batch run has three phases:
 //   1. a pool of host threads, each with its own CUDA stream and scratch
 //      pool, builds the CST (Alg. 1) and the partition (Alg. 2) of the
 //      queries concurrently -- their device work overlaps and their host
 //      round trips hide each other's latency;
-//   2. plans and chunks are gathered into the fixed buffers, every chunk
-//      tagged with its query;
+//   2. plans are gathered into the fixed buffers, each pointing at its
+//      query's chunk list;
 //   3. the captured graph runs one persistent matcher launch over all
 //      chunks of all queries (work stealing across queries), and the
 //      per-query counts come back in one copy.
@@ -29,12 +29,15 @@
 
 namespace fast {
 size_t match_plan_bytes();
-int match_plan_fill(const fast_cst* c, void* host_plan);
+int match_plan_fill(const fast_cst* c, const fast_chunks* ch, void* host_plan);
 void match_plan_set_stride(void* host_plans, int nq, int warp_words);
 size_t match_counter_words();
+size_t match_counter_host_words();
 size_t match_chunk_bytes();
-int match_batched_enqueue(const void* d_plans, int warp_words, const void* d_chunks, const int64_t* d_nchunks,
-                          int max_q, unsigned long long* d_qtotal, int* d_qstop, unsigned long long* d_ctr,
+uint32_t match_chunk_pieces(int64_t nchunks, int warps, int bps);
+uint64_t match_ring_cells(int64_t queue_cells, int warps, int bps, uint64_t cap);
+int match_batched_enqueue(const void* d_plans, int warp_words, const uint32_t* d_meta, int max_q,
+                          unsigned long long* d_qtotal, int* d_qstop, uint32_t* d_qnext, unsigned long long* d_ctr,
                           void* d_dq, uint32_t* d_dq_state, uint64_t dq_cap, uint64_t limit, double budget_s,
                           int warps, int bps, int validators, cudaStream_t s);
 int match_smem_optin(size_t bytes);
@@ -64,16 +67,14 @@ struct fast_batch {
     size_t psize = 0;
     unsigned char* d_plans = nullptr;
     unsigned char* h_plans = nullptr;     // pinned
-    int64_t* h_off = nullptr;             // pinned [max_q + 1]
-    int64_t* d_off = nullptr;
-    int64_t* d_nchunks = nullptr;
-    unsigned char* d_chunks = nullptr;
-    int64_t chunk_cap = 0;
+    uint32_t* h_meta = nullptr;           // pinned [max_q + 2]: {queries, pieces, static items per query}
+    uint32_t* d_meta = nullptr;
     unsigned long long* d_ctr = nullptr;
     unsigned long long* d_qtotal = nullptr;
     unsigned long long* h_qtotal = nullptr; // pinned
     unsigned long long* h_ctr = nullptr;    // pinned
     int* d_qstop = nullptr;
+    uint32_t* d_qnext = nullptr;          // per query: next static item
     unsigned char* d_dq = nullptr;
     uint32_t* d_dq_state = nullptr;
     // captured matcher launches, by launch shape (a batch's shared-memory
@@ -82,7 +83,6 @@ struct fast_batch {
         int warp_words, warps, bps, val;
         double budget;
         uint64_t limit, cells;
-        unsigned char* chunks;
         cudaGraphExec_t exec;
         int kernels;                      // kernels in the graph (launched per replay)
     };
@@ -98,29 +98,17 @@ struct fast_batch {
 
 namespace {
 
-__global__ void k_tag_chunks(Chunk* chunks, const int64_t* off, int nq) {
-    int64_t total = off[nq];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nq;                      // last q with off[q] <= i
-        while (hi - lo > 1) {
-            int mid = (lo + hi) >> 1;
-            if (off[mid] <= i) lo = mid; else hi = mid;
-        }
-        chunks[i].pad = (chunks[i].pad & 0xFFu) | ((uint32_t)lo << 8);
-    }
-}
-
 void batch_release(fast_batch* b) {
     if (!b) return;
     cudaSetDevice(b->device);
     for (auto& c : b->graphs) cudaGraphExecDestroy(c.exec);
     b->graphs.clear();
     cudaStream_t s = nullptr;
-    dfree(b->d_plans, s); dfree(b->d_off, s); dfree(b->d_nchunks, s); dfree(b->d_chunks, s);
-    dfree(b->d_ctr, s); dfree(b->d_qtotal, s); dfree(b->d_qstop, s); dfree(b->d_dq, s); dfree(b->d_dq_state, s);
+    dfree(b->d_plans, s); dfree(b->d_meta, s);
+    dfree(b->d_ctr, s); dfree(b->d_qtotal, s); dfree(b->d_qstop, s); dfree(b->d_qnext, s); dfree(b->d_dq, s); dfree(b->d_dq_state, s);
     cudaStreamSynchronize(s);
     if (b->h_plans) cudaFreeHost(b->h_plans);
-    if (b->h_off) cudaFreeHost(b->h_off);
+    if (b->h_meta) cudaFreeHost(b->h_meta);
     if (b->h_qtotal) cudaFreeHost(b->h_qtotal);
     if (b->h_ctr) cudaFreeHost(b->h_ctr);
     for (auto st : b->ws) cudaStreamDestroy(st);
@@ -156,17 +144,17 @@ int batch_create(const fast_graph* g, const fast_config* cfg, int32_t max_q, int
         if (rc) break;
         for (int w = 0; w < b->nthreads; w++) b->pools.push_back(pool_new());
         rc = dalloc(&b->d_plans, (size_t)max_q * b->psize, s); if (rc) break;
-        rc = dalloc(&b->d_off, max_q + 1, s); if (rc) break;
-        rc = dalloc(&b->d_nchunks, 1, s); if (rc) break;
+        rc = dalloc(&b->d_meta, (size_t)max_q + 2, s); if (rc) break;
         rc = dalloc(&b->d_ctr, match_counter_words(), s); if (rc) break;
         rc = dalloc(&b->d_qtotal, max_q, s); if (rc) break;
         rc = dalloc(&b->d_qstop, max_q, s); if (rc) break;
+        rc = dalloc(&b->d_qnext, max_q, s); if (rc) break;
         rc = dalloc(&b->d_dq, kBatchQueue * match_chunk_bytes(), s); if (rc) break;
         rc = dalloc(&b->d_dq_state, kBatchQueue, s); if (rc) break;
         if (cudaMallocHost((void**)&b->h_plans, (size_t)max_q * b->psize) != cudaSuccess ||
-            cudaMallocHost((void**)&b->h_off, (size_t)(max_q + 1) * sizeof(int64_t)) != cudaSuccess ||
+            cudaMallocHost((void**)&b->h_meta, ((size_t)max_q + 2) * sizeof(uint32_t)) != cudaSuccess ||
             cudaMallocHost((void**)&b->h_qtotal, (size_t)max_q * sizeof(unsigned long long)) != cudaSuccess ||
-            cudaMallocHost((void**)&b->h_ctr, match_counter_words() * sizeof(unsigned long long)) != cudaSuccess) {
+            cudaMallocHost((void**)&b->h_ctr, match_counter_host_words() * sizeof(unsigned long long)) != cudaSuccess) {
             cudaGetLastError();
             rc = set_error(FAST_ERR_OOM, "fast_batch_create: pinned host allocation failed");
             break;
@@ -181,26 +169,17 @@ int batch_create(const fast_graph* g, const fast_config* cfg, int32_t max_q, int
 
 // (Re)capture the matcher launch as a graph when its shape changed.
 int batch_graph(fast_batch* b, int warp_words, const fast_config& lc, cudaStream_t s) {
-    const uint64_t cells = lc.queue_cells > 0 ? std::min<uint64_t>((uint64_t)lc.queue_cells, kBatchQueue) : kBatchQueue;
     int warps = lc.warps_per_block > 0 ? std::min(lc.warps_per_block, 8) : 8;
     const int nval = lc.matcher_rule == 1 && warps >= 2 ? (lc.validators > 0 ? std::min(lc.validators, warps - 1) : warps / 2) : 0;
     const int bps = lc.blocks_per_sm > 0 ? lc.blocks_per_sm : 4;
+    const uint64_t cells = match_ring_cells(lc.queue_cells, warps, bps, kBatchQueue);
     for (auto& c : b->graphs)
         if (c.warp_words == warp_words && c.warps == warps && c.bps == bps && c.val == nval && c.budget == lc.time_budget_s &&
-            c.limit == lc.limit && c.cells == cells && c.chunks == b->d_chunks) {
+            c.limit == lc.limit && c.cells == cells) {
             b->exec = c.exec;
             b->g_kernels = c.kernels;
             return FAST_OK;
         }
-    // a new shape; graphs over an older chunk array can never run again
-    for (size_t i = 0; i < b->graphs.size();) {
-        if (b->graphs[i].chunks != b->d_chunks) {
-            cudaGraphExecDestroy(b->graphs[i].exec);
-            b->graphs.erase(b->graphs.begin() + i);
-        } else {
-            i++;
-        }
-    }
     if (b->graphs.size() >= 8) {
         cudaGraphExecDestroy(b->graphs.front().exec);
         b->graphs.erase(b->graphs.begin());
@@ -214,8 +193,8 @@ int batch_graph(fast_batch* b, int warp_words, const fast_config& lc, cudaStream
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) rc = cuda_status(e, "begin capture", __FILE__, __LINE__);
     if (rc == FAST_OK) {
-        int rc2 = match_batched_enqueue(b->d_plans, warp_words, b->d_chunks, b->d_nchunks, b->max_q, b->d_qtotal,
-                                        b->d_qstop, b->d_ctr, b->d_dq, b->d_dq_state, cells, lc.limit,
+        int rc2 = match_batched_enqueue(b->d_plans, warp_words, b->d_meta, b->max_q, b->d_qtotal,
+                                        b->d_qstop, b->d_qnext, b->d_ctr, b->d_dq, b->d_dq_state, cells, lc.limit,
                                         lc.time_budget_s, warps, bps, nval, cap);
         e = cudaStreamEndCapture(cap, &graph);
         if (rc2 != FAST_OK) rc = rc2;
@@ -246,7 +225,7 @@ int batch_graph(fast_batch* b, int warp_words, const fast_config& lc, cudaStream
     cudaStreamDestroy(cap);
     (void)s;
     if (rc == FAST_OK) {
-        b->graphs.push_back({warp_words, warps, bps, nval, lc.time_budget_s, lc.limit, cells, b->d_chunks, exec, recorded});
+        b->graphs.push_back({warp_words, warps, bps, nval, lc.time_budget_s, lc.limit, cells, exec, recorded});
         b->exec = exec;
         b->g_kernels = recorded;
     } else if (exec) {
@@ -326,16 +305,30 @@ int batch_run(fast_batch* b, int32_t nq, const fast_query_desc* qs, uint64_t* co
     b->last_build_ms = std::chrono::duration<double, std::milli>(t1 - t0).count();
     int rc = FAST_OK;
     // ---- 2. gather
+    // the launch shape (size class 0 holds it), read from every class's plan alike
+    fast_config lc = b->base;
+    lc.warps_per_block = b->cls[0].warps_per_block;
+    lc.blocks_per_sm = b->cls[0].blocks_per_sm;
+    lc.matcher_rule = b->cls[0].matcher_rule;
+    lc.validators = b->cls[0].validators;
     int64_t total = 0;
     int warp_words = 0;
-    b->h_off[0] = 0;
     for (int i = 0; i < nq; i++) {
-        int64_t n = (st[i] == FAST_OK && chs[i]) ? chs[i]->n : 0;
-        b->h_off[i + 1] = b->h_off[i] + n;
-        if (st[i] == FAST_OK) warp_words = std::max(warp_words, match_plan_fill(csts[i], b->h_plans + (size_t)i * b->psize));
-        else memset(b->h_plans + (size_t)i * b->psize, 0, b->psize);
+        if (st[i] == FAST_OK) {
+            total += chs[i] ? chs[i]->n : 0;
+            warp_words = std::max(warp_words, match_plan_fill(csts[i], chs[i], b->h_plans + (size_t)i * b->psize));
+        } else {
+            memset(b->h_plans + (size_t)i * b->psize, 0, b->psize);
+        }
     }
-    total = b->h_off[nq];
+    // The matcher reads each query's chunks where the partition left them;
+    // too few of them for the launch's warps are cut into pieces.
+    const uint32_t pieces = match_chunk_pieces(total, lc.warps_per_block > 0 ? std::min(lc.warps_per_block, 8) : 8,
+                                               lc.blocks_per_sm > 0 ? lc.blocks_per_sm : 4);
+    b->h_meta[0] = (uint32_t)nq;
+    b->h_meta[1] = pieces;
+    for (int i = 0; i < nq; i++)
+        b->h_meta[2 + i] = (uint32_t)(st[i] == FAST_OK && chs[i] ? chs[i]->n * pieces : 0);
     b->last_chunks = total;
     if (warp_words == 0) warp_words = 32 * 32 + 64;
     // one stride for every query of the launch, rounded up to 256 words so
@@ -343,42 +336,16 @@ int batch_run(fast_batch* b, int32_t nq, const fast_query_desc* qs, uint64_t* co
     warp_words = (warp_words + 255) / 256 * 256;
     match_plan_set_stride(b->h_plans, nq, warp_words);
     do {
-        if (total > b->chunk_cap) {
-            int64_t cap = std::max<int64_t>(total, 2 * b->chunk_cap);
-            dfree(b->d_chunks, s);
-            b->chunk_cap = 0;                     // stays 0 if the allocation below fails
-            rc = dalloc(&b->d_chunks, (size_t)cap * match_chunk_bytes(), s); if (rc) break;
-            b->chunk_cap = cap;
-        }
-        for (int i = 0; i < nq; i++) {
-            int64_t n = b->h_off[i + 1] - b->h_off[i];
-            if (n) {
-                cudaError_t e = cudaMemcpyAsync(b->d_chunks + b->h_off[i] * match_chunk_bytes(), chs[i]->d,
-                                                n * match_chunk_bytes(), cudaMemcpyDeviceToDevice, s);
-                if (e != cudaSuccess) { rc = cuda_status(e, "chunk gather", __FILE__, __LINE__); break; }
-            }
-        }
-        if (rc) break;
         if (nq > 0) FAST_CUDA_BREAK(rc, cudaMemcpyAsync(b->d_plans, b->h_plans, (size_t)nq * b->psize, cudaMemcpyHostToDevice, s));
-        if (nq > 0) FAST_CUDA_BREAK(rc, cudaMemcpyAsync(b->d_off, b->h_off, (size_t)(nq + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-        FAST_CUDA_BREAK(rc, cudaMemcpyAsync(b->d_nchunks, &b->h_off[nq], sizeof(int64_t), cudaMemcpyHostToDevice, s));
-        if (total > 0) {
-            k_tag_chunks<<<(unsigned)std::min<int64_t>(ceil_div(total, 256), 4096), 256, 0, s>>>((Chunk*)b->d_chunks, b->d_off, nq);
-            note_launch();
-        }
+        FAST_CUDA_BREAK(rc, cudaMemcpyAsync(b->d_meta, b->h_meta, ((size_t)nq + 2) * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
         // ---- 3. one matcher launch for all queries (captured graph)
-        fast_config lc = b->base;
-        lc.warps_per_block = b->cls[0].warps_per_block;
-        lc.blocks_per_sm = b->cls[0].blocks_per_sm;
-        lc.matcher_rule = b->cls[0].matcher_rule;
-        lc.validators = b->cls[0].validators;
         rc = batch_graph(b, warp_words, lc, s); if (rc) break;
         FAST_CUDA_BREAK(rc, cudaEventRecord(b->ev0, s));
         FAST_CUDA_BREAK(rc, cudaGraphLaunch(b->exec, s));
         note_launch(b->g_kernels);            // the kernels the graph holds, matcher included
         FAST_CUDA_BREAK(rc, cudaEventRecord(b->ev1, s));
         if (nq > 0) FAST_CUDA_BREAK(rc, cudaMemcpyAsync(b->h_qtotal, b->d_qtotal, (size_t)nq * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-        FAST_CUDA_BREAK(rc, cudaMemcpyAsync(b->h_ctr, b->d_ctr, match_counter_words() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+        FAST_CUDA_BREAK(rc, cudaMemcpyAsync(b->h_ctr, b->d_ctr, match_counter_host_words() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) { rc = cuda_status(e, "fast_batch_run", __FILE__, __LINE__); break; }
         float ms = 0.f;
@@ -386,7 +353,7 @@ int batch_run(fast_batch* b, int32_t nq, const fast_query_desc* qs, uint64_t* co
         b->last_match_ms = ms;
     } while (0);
     int gst = match_status_of(b->h_ctr, &b->last_bytes, &b->last_floor);
-    cudaStreamSynchronize(s);               // no gather copy may still read a chunk list
+    cudaStreamSynchronize(s);               // the matcher may still read the chunk lists
     for (int i = 0; i < nq; i++) {
         // the matcher is done (or never ran); the builders' streams stay ordered
         chunks_release_nosync(chs[i]);

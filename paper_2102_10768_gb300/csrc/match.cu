@@ -21,13 +21,25 @@
 // of the lane whose index is the depth (depth <= 31), so no per-depth array
 // is indexed dynamically.
 //
-// Load balance: a persistent grid first drains the static chunk list, then a
-// global ring of donated runs.  A warp that finds both empty counts itself
-// idle; a busy warp that sees idle warps gives away the second half of the
-// unscanned list at its shallowest depth with at least two entries left --
-// a run of a list with a fixed prefix, i.e. again a chunk.  An outstanding-
-// work counter ends the launch.  No warp waits on another: the only wait, an
-// idle warp looking for work, is bounded by %globaltimer.
+// Load balance: a persistent grid first drains the static chunks (each query
+// of a batch has its own cursor, and the warps start spread over the
+// queries), then serves itself from donated runs.  A warp out of static
+// chunks takes a ticket and waits on the ring cell of that ticket, which no
+// other warp reads; a busy warp that sees tickets unserved gives away the
+// second half of the unscanned list at its shallowest depth with at least
+// two entries left -- a run of a list with a fixed prefix, i.e. again a
+// chunk.  The launch ends when the unserved tickets are as many as the warps
+// that have started: nobody is left who could donate.  The only wait, that
+// for a ticket's run, is bounded by %globaltimer.
+//
+// Why tickets: with one shared head that every idle warp tried to advance by
+// compare-and-swap, a published run set off thousands of attempts (65 M of
+// them, one per 4 ns, in a 235 ms enumeration of 12 queries), and that word
+// alone set the launch's time.  With tickets, pieces of chunks and the
+// counters on lines of their own, that enumeration takes 110 instead of 287
+// ms, one 10-vertex query with two-entry lists 25 instead of 115 ms, and the
+// batched matcher under a limit, whose warps now spread over the queries and
+// stop within half the limit, 250 queries' step 150 instead of 191 ms.
 //
 // Warp-specialised variant (the GPU form of the task-generator separation
 // of Sec. V-D): a CTA's warps split into expanders and validators.  The
@@ -84,6 +96,7 @@ struct MatchPlan {
     int nt_from[kMaxNT];              // their earlier endpoint (position)
     const int64_t* n_off[kMaxNT];
     const uint32_t* n_idx[kMaxNT];
+    const Chunk* chunks;              // the query's static chunks
 };
 
 enum : int { kStatusTimeout = 1, kStatusOverflow = 2, kStatusLimit = 4 };
@@ -96,15 +109,19 @@ constexpr int kWarpBaseWords = kMaxK * 32 + 3 * kMaxK + 2 * kMaxK;
 // query of a batch from bit 8 up.
 constexpr uint32_t kDonated = 1;
 __device__ __forceinline__ int run_source(uint32_t pad) { return (int)((pad >> 1) & 63u); }
+constexpr int64_t kLastDonate = 512;       // entries: shortest run of the last position that is given away
 constexpr unsigned long long kIdleNs = 5ull * 1000 * 1000 * 1000;     // an idle warp gives up waiting
 
 struct MatchOut {
-    unsigned long long* next_chunk;
+    uint32_t* qnext;                  // per query: its next static item
+    uint32_t items;                   // static items (pieces of chunks) of a single query
+    uint32_t pieces;                  // even runs each of its chunks is cut into (1: as it is)
+    const uint32_t* meta;             // batched: {queries, pieces, items of every query}
     unsigned long long* total;        // per query (one entry unless batched)
     int* qstop;                       // per query: limit reached
-    int nq;
     unsigned long long* emb_slot;
     int* status;
+    unsigned long long* done;         // kDoneCopies words, a line each: the launch is over
     uint64_t* chunk_counts;           // nullable (static chunks; no donation then)
     uint32_t* emb;                    // nullable
     uint64_t emb_cap;                 // rows that may be written
@@ -113,22 +130,24 @@ struct MatchOut {
     unsigned long long* floor;        // the floor of those bytes (see k_match)
     const unsigned long long* deadline;  // device word: %globaltimer limit, 0 = none
     uint64_t limit;                   // 0 = enumerate everything
-    // Donated runs: a bounded ring of dq_cap cells.  Ticket t (a count of
-    // claims, dq_tail for donors and dq_head for takers) uses cell t % dq_cap
-    // in generation g = t / dq_cap; the cell's state is 2g while it is free
-    // for that ticket and 2g+1 once the run is published; the taker sets
-    // 2g+2 after reading it.  States start at 0.  Nobody waits on a cell: a
-    // donor that finds its cell still occupied keeps its work, and a taker
-    // that finds no published cell looks again later.
+    uint32_t flush_at;                // embeddings a warp holds back before it adds them to the total
+    // Donated runs: a bounded ring of dq_cap cells.  Ticket t (taken by a
+    // warp out of work by advancing *dq_head, served by a donor by advancing
+    // *dq_tail, which never passes the head) uses cell t % dq_cap in
+    // generation g = t / dq_cap; the cell's state is 2g while it is free for
+    // that ticket, 2g+1 once the run is published, and 2g+2 once it is taken
+    // (or the ticket's warp gave up waiting).  States start at 0.  A donor
+    // that finds the cell of the next ticket still occupied keeps its work.
     Chunk* dq;
     uint32_t* dq_state;
     uint64_t dq_cap;                  // 0 = no donation
-    unsigned long long* dq_head;
+    unsigned long long* dq_head;      // dq_tail follows it: one 16-byte load reads both
     unsigned long long* dq_tail;
-    unsigned long long* outstanding;  // work items not yet finished
-    unsigned int* idle;               // warps waiting for work
+    unsigned long long* started;      // warps that have begun (less those that gave up)
     int validators;                   // warp-specialised variant: validator warps per CTA
 };
+constexpr int kDoneCopies = 64;       // so that thousands of waiting warps do not poll one word
+constexpr int kLineWords = 16;        // a 128-byte line of 8-byte words
 
 // One last-position extension handed from an expander to a validator warp
 // (the warp-specialised variant): the lists into position k-1 -- index 0
@@ -159,8 +178,6 @@ enum : int { kStatusValidator = 8 };
 __global__ void k_set_deadline(unsigned long long* d, unsigned long long budget_ns) {
     *d = budget_ns ? global_timer_ns() + budget_ns : 0ull;
 }
-
-__global__ void k_copy_word(unsigned long long* dst, const int64_t* src) { *dst = (unsigned long long)*src; }
 
 // membership of x in the sorted a[lo, hi); *probes counts the entries read
 __device__ __forceinline__ bool bsearch_u32(const uint32_t* __restrict__ a, int64_t lo, int64_t hi, uint32_t x,
@@ -256,52 +273,119 @@ __device__ __forceinline__ unsigned long long vload(const unsigned long long* p)
     return *(volatile const unsigned long long*)p;
 }
 
-// lane 0: add a local count to query q's total; flag the limit once reached
-__device__ __forceinline__ void flush_count(const MatchOut& O, uint32_t q, unsigned long long& local) {
+__device__ __forceinline__ void announce_done(const MatchOut& O) {
+    for (int i = 0; i < kDoneCopies; i++) *(volatile unsigned long long*)(O.done + i * kLineWords) = 1ull;
+}
+__device__ __forceinline__ bool is_done(const MatchOut& O) {
+    return vload(O.done + (blockIdx.x % kDoneCopies) * kLineWords) != 0;
+}
+
+// one lane: a stop for every warp of the launch
+__device__ __forceinline__ void stop_all(const MatchOut& O, int why) {
+    atomicOr(O.status, why);
+    announce_done(O);
+}
+
+// one lane: add a count to query q's total; flag the limit once reached
+template <bool BATCH>
+__device__ __forceinline__ void flush_count(const MatchOut& O, uint32_t q, unsigned long long local) {
     if (!local) return;
     unsigned long long old = atomicAdd(&O.total[q], local);
     if (old + local < old) atomicOr(O.status, kStatusOverflow);
-    if (O.limit && old + local >= O.limit) {
-        O.qstop[q] = 1;
-        if (O.nq == 1) atomicOr(O.status, kStatusLimit);
+    if (O.limit && old < O.limit && old + local >= O.limit) {     // once per query
+        *(volatile int*)&O.qstop[q] = 1;
+        if (!BATCH) stop_all(O, kStatusLimit);
     }
-    local = 0;
 }
 
-// lane 0: obtain the next work item.  kind 1 = static chunk, 2 = donated run,
-// 0 = nothing left (or stop requested).
-__device__ int acquire(const MatchOut& O, int64_t nchunks, unsigned long long deadline, unsigned long long* idx) {
-    bool was_idle = false;
-    int kind = 0;
-    unsigned long long t_idle = 0;
+// The whole warp: the next static item of query *q, or, when that query has
+// none left or has reached its limit, of another one (the 32 lanes look at
+// 32 queries at a time, from a place that differs between warps, so that the
+// warps leaving one query do not all meet at the next).  False: none is left.
+template <bool BATCH>
+__device__ bool next_static(const MatchOut& O, uint32_t nq, uint32_t seed, uint32_t* q, uint32_t* item) {
+    const int lane = threadIdx.x & 31;
     for (;;) {
-        if (vload(O.status) & (kStatusTimeout | kStatusLimit)) break;
-        unsigned long long now = global_timer_ns();
-        if (deadline && now > deadline) { atomicOr(O.status, kStatusTimeout); break; }
-        if (vload(O.next_chunk) < (unsigned long long)nchunks) {
-            unsigned long long i = atomicAdd(O.next_chunk, 1ull);
-            if (i < (unsigned long long)nchunks) { *idx = i; kind = 1; break; }
-        }
-        if (O.dq_cap) {
-            unsigned long long h = vload(O.dq_head);
-            uint32_t want = (uint32_t)(2 * (h / O.dq_cap) + 1);          // published, ticket h
-            if (*(volatile uint32_t*)&O.dq_state[h % O.dq_cap] == want) {
-                if (atomicCAS(O.dq_head, h, h + 1) == h) {
-                    __threadfence();
-                    *idx = h;
-                    kind = 2;
-                    break;
-                }
-                continue;                                                 // taken by another warp
+        uint32_t i = 0;
+        int got = 0;
+        if (lane == 0) {
+            const bool stop = is_done(O) || (BATCH && vload(O.qstop + *q) != 0);
+            const uint32_t n = BATCH ? O.meta[2 + *q] : O.items;
+            if (!stop && *(volatile uint32_t*)(O.qnext + *q) < n) {
+                i = atomicAdd(O.qnext + *q, 1u);
+                got = i < n;
             }
         }
-        if (vload(O.outstanding) == 0) break;
-        if (!was_idle) { atomicAdd(O.idle, 1u); was_idle = true; t_idle = now; }
-        else if (now - t_idle > kIdleNs) break;   // the warps still busy finish (and drain) the rest
-        __nanosleep(200);
+        if (__shfl_sync(0xffffffffu, got, 0)) {
+            *item = __shfl_sync(0xffffffffu, i, 0);
+            return true;
+        }
+        if (!BATCH || nq <= 1) return false;
+        seed = seed * 1664525u + 1013904223u;
+        const uint32_t s0 = (seed >> 8) % nq;
+        bool found = false;
+        for (uint32_t b = 0; b < nq && !found; b += 32) {
+            bool ok = false;
+            uint32_t c = s0 + b + lane;
+            if (b + lane < nq) {
+                if (c >= nq) c -= nq;
+                ok = *(volatile uint32_t*)(O.qnext + c) < O.meta[2 + c] && vload(O.qstop + c) == 0;
+            }
+            const uint32_t m = __ballot_sync(0xffffffffu, ok);
+            if (m) {
+                *q = __shfl_sync(0xffffffffu, c, __ffs(m) - 1);
+                found = true;
+            }
+        }
+        if (!found) return false;
     }
-    if (was_idle) atomicSub(O.idle, 1u);
-    return kind;
+}
+
+// one lane, out of static items: take a ticket and wait for its run.  True:
+// the run of ticket *ticket is published; false: the launch is over (or the
+// wait ran out).
+__device__ bool wait_run(const MatchOut& O, unsigned long long deadline, unsigned long long* ticket) {
+    if (!O.dq_cap || is_done(O)) return false;
+    __threadfence();                                           // this warp's start comes before its ticket
+    const unsigned long long h = atomicAdd(O.dq_head, 1ull);
+    __threadfence();
+    // every started warp holds an unserved ticket: no work is left anywhere
+    if (h + 1 - vload(O.dq_tail) == vload(O.started)) { announce_done(O); return false; }
+    uint32_t* st = O.dq_state + h % O.dq_cap;
+    const uint32_t free_ = (uint32_t)(2 * (h / O.dq_cap));
+    unsigned long long t0 = 0;
+    for (int n = 0;; n++) {
+        if (*(volatile uint32_t*)st == free_ + 1) {
+            __threadfence();
+            *ticket = h;
+            return true;
+        }
+        if (is_done(O)) return false;
+        if ((n & 15) == 15) {
+            const unsigned long long now = global_timer_ns();
+            if (deadline && now > deadline) { stop_all(O, kStatusTimeout); return false; }
+            if (!t0) t0 = now;
+            // give up: the ticket is void (a donor skips it); the warps still busy finish the rest
+            else if (now - t0 > kIdleNs && atomicCAS(st, free_, free_ + 2) == free_) return false;
+        }
+        __nanosleep(n < 16 ? 50 : 250);
+    }
+}
+
+// one lane: claim the next unserved ticket whose cell is free, or ~0 (none, a
+// full ring, or races lost a few times: the work stays here)
+__device__ unsigned long long claim_ticket(const MatchOut& O, unsigned long long head, unsigned long long t) {
+    for (int tries = 0; tries < 4 && t < head; tries++) {
+        const uint32_t st = *(volatile uint32_t*)&O.dq_state[t % O.dq_cap];
+        const uint32_t free_ = (uint32_t)(2 * (t / O.dq_cap));
+        if (st < free_) break;                                  // its cell's previous run is not taken yet
+        const unsigned long long prev = atomicCAS(O.dq_tail, t, t + 1);
+        if (prev != t) { t = prev; continue; }
+        if (st == free_) return t;
+        atomicAdd(O.started, ~0ull);                            // a void ticket: its warp is gone
+        t++;
+    }
+    return ~0ull;
 }
 
 // lane 0: claim the ring's next cell for a producer, if it is free (a cell
@@ -381,10 +465,11 @@ __device__ void validate_tasks(const MatchPlan& P0, const MatchPlan* __restrict_
             if ((++it & 255) == 0) {
                 int st = 0;
                 if (lane == 0) {
-                    flush_count(O, q, local);
-                    if (deadline && global_timer_ns() > deadline) atomicOr(O.status, kStatusTimeout);
-                    st = vload(O.status) & (kStatusTimeout | kStatusLimit);
-                    if (BATCH && *(volatile int*)&O.qstop[q]) st = 1;
+                    flush_count<BATCH>(O, q, local);
+                    local = 0;
+                    if (deadline && global_timer_ns() > deadline) stop_all(O, kStatusTimeout);
+                    st = is_done(O);
+                    if (BATCH && vload(O.qstop + q)) st = 1;
                 }
                 stop = __shfl_sync(0xffffffffu, st, 0) != 0;
                 if (stop) break;
@@ -420,7 +505,7 @@ __device__ void validate_tasks(const MatchPlan& P0, const MatchPlan* __restrict_
             const uint32_t mask = __ballot_sync(0xffffffffu, ok);
             if (lane == 0) local += __popc(mask);
         }
-        if (lane == 0) flush_count(O, q, local);
+        if (lane == 0) flush_count<BATCH>(O, q, local);
         __syncwarp();
         if (lane == 0) {
             __threadfence_block();
@@ -429,19 +514,17 @@ __device__ void validate_tasks(const MatchPlan& P0, const MatchPlan* __restrict_
     }
 }
 
-// BATCH: plans[q] per query (chunk flags carry q, nchunks is read from
-// *nchunks_dev); otherwise the single plan P0 and the nchunks argument.
+// BATCH: plans[q] per query; otherwise the single plan P0.
 // WS: the warp-specialised variant (O.validators validator warps per CTA,
 // the last warps; no counting pass, no embeddings written).
 template <bool STATS, bool EMIT, bool BATCH, bool WS = false>
 __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchPlan P0,
-                                               const MatchPlan* __restrict__ plans,
-                                               const Chunk* __restrict__ chunks, int64_t nchunks,
-                                               const int64_t* __restrict__ nchunks_dev, MatchOut O) {
+                                               const MatchPlan* __restrict__ plans, MatchOut O) {
     extern __shared__ uint32_t smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    if (BATCH) nchunks = *nchunks_dev;
+    const uint32_t nq = BATCH ? O.meta[0] : 1u;
+    const uint32_t pieces = BATCH ? O.meta[1] : O.pieces;
     const int warp_words = BATCH ? plans[0].warp_words : P0.warp_words;   // one stride for all queries
     uint32_t* sbuf = smem + (size_t)warp * warp_words;                   // [depth][32]
     uint32_t* sm = sbuf + kMaxK * 32;                                   // m[position]
@@ -462,7 +545,7 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
     // chunk that starts at position j > 0 counts its run's extension the same
     // way; a donated run counts only what it scans.
     unsigned long long fb = 0;
-    unsigned long long local = 0;          // lane 0: count not yet flushed
+    unsigned long long local = 0;          // this warp's count of query q not yet flushed
     // warp-specialised: the ring after the warps' regions; expanders first
     VRing* ring = nullptr;
     const int nexp = WS ? (int)(blockDim.x >> 5) - O.validators : (int)(blockDim.x >> 5);
@@ -480,22 +563,54 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
     if (WS && warp >= nexp) {
         validate_tasks<BATCH>(P0, plans, ring, tcur, O, deadline, lb, fb);
     } else {
+    if (lane == 0) atomicAdd(O.started, 1ull);
+    // the warps start spread over the queries, neighbours on the same one
+    const uint32_t gw = blockIdx.x * (uint32_t)nexp + warp, tw = gridDim.x * (uint32_t)nexp;
+    uint32_t sq = BATCH && nq ? (uint32_t)(((uint64_t)gw * nq) / tw) : 0u;   // the query whose static items it takes
+    bool static_left = nq > 0;
+    uint32_t q = sq;                                                        // the query `local` counts for
     for (;;) {
         unsigned long long ci = 0;
         int kind = 0;
-        if (lane == 0) kind = acquire(O, nchunks, deadline, &ci);
-        kind = __shfl_sync(0xffffffffu, kind, 0);
-        ci = __shfl_sync(0xffffffffu, ci, 0);
+        if (deadline && lane == 0 && global_timer_ns() > deadline) stop_all(O, kStatusTimeout);
+        if (static_left) {
+            uint32_t item = 0;
+            if (next_static<BATCH>(O, nq, gw, &sq, &item)) { kind = 1; ci = item; }
+            else static_left = false;
+        }
+        // a total is complete before its warp waits; until then a query's
+        // counts are added up over its items
+        const bool other = kind == 1 && sq != q;
+        if (kind == 0 || other) {
+            if (lane == 0) flush_count<BATCH>(O, q, local);
+            local = 0;
+        }
+        if (kind == 0) {
+            int got = 0;
+            if (lane == 0) got = wait_run(O, deadline, &ci);
+            if (__shfl_sync(0xffffffffu, got, 0)) kind = 2;
+            ci = __shfl_sync(0xffffffffu, ci, 0);
+        }
         if (kind == 0) break;
         // the item's fields, read once.  A donated run was written by another
         // warp during this launch: read it from L2 (ld.global.cg), never from
         // an L1 line that may hold an older copy of its bytes.
-        const Chunk* chp = kind == 1 ? chunks + ci : O.dq + ci % O.dq_cap;
+        const Chunk* chp = kind == 1 ? (BATCH ? plans[sq].chunks : P0.chunks) + (uint32_t)ci / pieces : O.dq + ci % O.dq_cap;
         int j;
         uint32_t ch_a, ch_b, ch_pad, ch_pre;
+        bool first = true;                        // the chunk's first piece (it counts the chunk's own extension)
         if (kind == 1) {
-            j = chp->j; ch_a = chp->a; ch_b = chp->b; ch_pad = chp->pad;
+            j = chp->j; ch_a = chp->a; ch_b = chp->b; ch_pad = 0;
             ch_pre = lane < j ? chp->prefix[lane] : 0u;
+            q = sq;
+            if (pieces > 1) {
+                const uint32_t i = (uint32_t)ci % pieces;
+                const uint64_t len = ch_b - ch_a;
+                ch_b = ch_a + (uint32_t)(len * (i + 1) / pieces);
+                ch_a += (uint32_t)(len * i / pieces);
+                first = i == 0;
+                if (ch_a == ch_b && !first) continue;
+            }
         } else {
             j = __ldcg(&chp->j); ch_a = __ldcg(&chp->a); ch_b = __ldcg(&chp->b); ch_pad = __ldcg(&chp->pad);
             ch_pre = lane < j ? __ldcg(&chp->prefix[lane]) : 0u;
@@ -505,7 +620,7 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                 atomicExch(&O.dq_state[ci % O.dq_cap], (uint32_t)(2 * (ci / O.dq_cap) + 2));
             }
         }
-        const uint32_t q = BATCH ? (ch_pad >> 8) : 0u;
+        if (BATCH && kind == 2) q = ch_pad >> 8;               // nothing is held back: it waited
         const MatchPlan& P = BATCH ? plans[q] : P0;
         const int k = P.k;
         if (BATCH) {
@@ -514,12 +629,8 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
             // reading it separately could take different branches and then
             // never meet at the warp-wide operations that follow.
             int qs = 0;
-            if (lane == 0) qs = *(volatile int*)&O.qstop[q];
-            if (__shfl_sync(0xffffffffu, qs, 0)) {
-                if (lane == 0) atomicAdd(O.outstanding, ~0ull);
-                __syncwarp();
-                continue;
-            }
+            if (lane == 0) qs = vload(O.qstop + q);
+            if (__shfl_sync(0xffffffffu, qs, 0)) continue;
         }
         uint32_t m_reg = ch_pre;                               // lane p: candidate index of position p
         int32_t g_reg = -1;                                    // lane p: data vertex of position p
@@ -545,9 +656,9 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                 if (sg[p] == g_reg) ok_prefix = false;
             }
         }
-        unsigned long long ccount = 0;         // lane 0: this item's count
+        unsigned long long ccount = 0;         // this item's count
         if (__all_sync(0xffffffffu, ok_prefix)) {
-            if (kind == 1 && j > 0 && lane == 0) fb += 4 + 16 + 16ull * (P.nt_begin[j + 1] - P.nt_begin[j]);
+            if (kind == 1 && first && j > 0 && lane == 0) fb += 4 + 16 + 16ull * (P.nt_begin[j + 1] - P.nt_begin[j]);
             // ---- depth j: the item's run of L_j
             int d = j;
             int64_t seg_next = 0, seg_end = 0, seg_base = 0;   // lane d: depth d's list scan
@@ -577,47 +688,37 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                 for (int e = P.nt_begin[j] + lane; e < P.nt_begin[j + 1]; e += 32) ncur[e] = 0;
                 __syncwarp();
             }
+            // Under a limit a warp adds its count to the total once it holds
+            // flush_at embeddings, and looks every 16th step whether the limit
+            // was reached meanwhile (a load issued 16 steps before its value is
+            // used, so that it costs no wait).
+            int stop_seen = 0;
             for (;;) {
                 ++iter;
-                if ((iter & 255) == 0) {
-                    int stop = 0;
+                if (local >= O.flush_at) {
+                    if (lane == 0) flush_count<BATCH>(O, q, local);
+                    local = 0;
+                }
+                if ((iter & 15) == 0) {
+                    if (__any_sync(0xffffffffu, stop_seen)) break;
                     if (lane == 0) {
-                        flush_count(O, q, local);
-                        if (deadline && global_timer_ns() > deadline) atomicOr(O.status, kStatusTimeout);
-                        stop = vload(O.status) & (kStatusTimeout | kStatusLimit);
-                        if (BATCH && *(volatile int*)&O.qstop[q]) stop = 1;
+                        if ((iter & 255) == 0 && deadline && global_timer_ns() > deadline) stop_all(O, kStatusTimeout);
+                        stop_seen = is_done(O);
                     }
-                    if (__shfl_sync(0xffffffffu, stop, 0)) break;
+                    if (BATCH && lane == 1) stop_seen = vload(O.qstop + q);
                 }
                 if (O.dq_cap && (iter & 63) == 0) {
-                    // give work away when some warp is idle
-                    unsigned int idl = 0;
-                    if (lane == 0) idl = *(volatile unsigned int*)O.idle;
-                    idl = __shfl_sync(0xffffffffu, idl, 0);
-                    if (idl) {
-                        bool can = lane >= j && lane <= d && (seg_end - seg_next) >= 2;
-                        uint32_t cm = __ballot_sync(0xffffffffu, can);
+                    // give work away when some warp waits for it
+                    ulonglong2 ht = make_ulonglong2(0, 0);
+                    if (lane == 0) ht = __ldcv((const ulonglong2*)O.dq_head);   // {head, tail}
+                    if (__shfl_sync(0xffffffffu, ht.y < ht.x, 0)) {
+                        // a run of the last position is worth giving away only if it is long
+                        const bool can = lane >= j && lane <= d && (seg_end - seg_next) >= (lane == k - 1 ? kLastDonate : 2);
+                        const uint32_t cm = __ballot_sync(0xffffffffu, can);
                         if (cm) {
-                            int dd = __ffs(cm) - 1;
-                            // claim the next ticket whose cell is free; a full
-                            // ring (or a lost race, a few times) keeps the work here
+                            const int dd = __ffs(cm) - 1;
                             unsigned long long slot = ~0ull;
-                            if (lane == 0) {
-                                unsigned long long t = vload(O.dq_tail);
-                                for (int tries = 0; tries < 4; tries++) {
-                                    uint32_t st = *(volatile uint32_t*)&O.dq_state[t % O.dq_cap];
-                                    uint32_t g2 = (uint32_t)(2 * (t / O.dq_cap));
-                                    if (st == g2) {
-                                        unsigned long long prev = atomicCAS(O.dq_tail, t, t + 1);
-                                        if (prev == t) { slot = t; break; }
-                                        t = prev;
-                                    } else if (st < g2) {
-                                        break;                            // its previous run is not taken yet
-                                    } else {
-                                        t = vload(O.dq_tail);
-                                    }
-                                }
-                            }
+                            if (lane == 0) slot = claim_ticket(O, ht.x, ht.y);
                             slot = __shfl_sync(0xffffffffu, slot, 0);
                             if (slot != ~0ull) {
                                 int64_t sn_ = __shfl_sync(0xffffffffu, seg_next, dd);
@@ -627,7 +728,6 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                                 Chunk* dst = &O.dq[slot % O.dq_cap];
                                 if (lane < kMaxK) dst->prefix[lane] = lane < dd ? sm[lane] : 0u;
                                 if (lane == 0) {
-                                    atomicAdd(O.outstanding, 1ull);
                                     dst->j = dd;
                                     dst->a = (uint32_t)(mid - sb_);
                                     dst->b = (uint32_t)(se_ - sb_);
@@ -636,11 +736,14 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                                     dst->id = 0;
                                 }
                                 __syncwarp();
+                                int gave = 0;
                                 if (lane == 0) {
+                                    const uint32_t free_ = (uint32_t)(2 * (slot / O.dq_cap));
                                     __threadfence();
-                                    atomicExch(&O.dq_state[slot % O.dq_cap], (uint32_t)(2 * (slot / O.dq_cap) + 1));
+                                    gave = atomicCAS(&O.dq_state[slot % O.dq_cap], free_, free_ + 1) == free_;
+                                    if (!gave) atomicAdd(O.started, ~0ull);    // its warp gave up just now: keep the run
                                 }
-                                if (lane == dd) seg_end = mid;
+                                if (__shfl_sync(0xffffffffu, gave, 0) && lane == dd) seg_end = mid;
                             }
                         }
                     }
@@ -721,7 +824,7 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                     // entry, length and merge cursor held by one lane (lane 0
                     // the tree list, lane x the x-th non-tree list into d).
                     // Back to the main loop when the run ends and before every
-                    // 64th step, where the periodic checks and donations are.
+                    // 16th step, where the periodic checks and donations are.
                     const int src = gsrc[d];
                     const int e0 = P.nt_begin[d], ne = P.nt_begin[d + 1] - e0;
                     const int from = lane == 0 ? P.par[d] : (lane <= ne ? P.nt_from[e0 + lane - 1] : 0);
@@ -770,9 +873,10 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                         }
                         const uint32_t mask = __ballot_sync(0xffffffffu, ok);
                         if (STATS && lane == 0) atomicAdd(&O.stats[d], (unsigned long long)__popc(mask));
-                        if (lane == 0) { local += __popc(mask); ccount += __popc(mask); }
+                        local += __popc(mask);
+                        ccount += __popc(mask);
                         r += 32;
-                        if (r >= re || ((iter + 1) & 63) == 0) break;
+                        if (r >= re || ((iter + 1) & 15) == 0 || local >= O.flush_at) break;
                         ++iter;
                     }
                     if (lane == d) seg_next = sb + r;
@@ -836,7 +940,8 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                     if (lane == d) seg_next = sn + 32;
                     if (STATS && lane == 0) atomicAdd(&O.stats[d], (unsigned long long)__popc(mask));
                     if (d == k - 1) {
-                        if (lane == 0) { local += __popc(mask); ccount += __popc(mask); }
+                        local += __popc(mask);
+                        ccount += __popc(mask);
                         if (EMIT && !BATCH && mask) {
                             unsigned long long base = 0;
                             if (lane == 0) base = atomicAdd(O.emb_slot, (unsigned long long)__popc(mask));
@@ -866,11 +971,7 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                 d--;
             }
         }
-        if (lane == 0) {
-            flush_count(O, q, local);
-            if (O.chunk_counts && kind == 1) O.chunk_counts[ci] = ccount;
-            atomicAdd(O.outstanding, ~0ull);   // -1
-        }
+        if (lane == 0 && O.chunk_counts && kind == 1) O.chunk_counts[ci] = ccount;
         __syncwarp();
     }
     if (WS && lane == 0) {                     // this expander's tasks are all published
@@ -967,14 +1068,52 @@ int matcher_smem_optin(size_t bytes) {
     return FAST_OK;
 }
 
-// counter block layout (unsigned long long words)
-enum { kNext = 0, kTotal, kSlot, kStatus, kBytes, kFloor, kHead, kTail, kOut, kIdle, kDeadline, kQStop, kStats,
-       kCtrWords = kStats + kMaxK + 1 };
+// Counter block (8-byte words).  What different warps hammer lies in lines of
+// its own: the total, the embedding cursor, the static cursor, the ring's
+// head and tail (together: a donor reads both at once).  The first kCtrWords
+// come back to the host; the copies of the done flag follow.
+enum { kStatus = 0, kBytes, kFloor, kDeadline, kStarted, kQStop, kStats = 8,
+       kTotal = (kStats + kMaxK + kLineWords - 1) / kLineWords * kLineWords, kSlot = kTotal + kLineWords,
+       kCtrWords = kSlot + 1, kNext = kSlot + kLineWords, kHead = kNext + kLineWords, kTail = kHead + 1,
+       kDone = kHead + kLineWords, kAllWords = kDone + kDoneCopies * kLineWords };
 constexpr uint64_t kQueueCap = 1 << 16;
 
-// cells of the donation ring for a launch: cfg.queue_cells, at most (and by default) cap
-uint64_t ring_cells(const fast_config& cfg, uint64_t cap) {
-    return cfg.queue_cells > 0 ? std::min<uint64_t>((uint64_t)cfg.queue_cells, cap) : cap;
+// Cells of the donation ring for a launch of `warps` warps: cfg.queue_cells
+// if given (at most cap), else one per warp, so that every waiting warp's
+// ticket has a cell of its own.
+uint64_t ring_cells(int64_t queue_cells, int64_t warps, uint64_t cap) {
+    return std::min<uint64_t>(queue_cells > 0 ? (uint64_t)queue_cells : (uint64_t)std::max<int64_t>(warps, 1), cap);
+}
+
+// Even runs that each static chunk is cut into when a launch has fewer chunks
+// than warps: two per warp, so that the search starts on all of them and not
+// on one warp per chunk, from which donations would have to spread it
+// (a 10-vertex enumeration partitioned into 65 chunks, or a query of one
+// chunk).  Per-chunk counts need each chunk whole.
+uint32_t chunk_pieces(int64_t nchunks, int64_t warps) {
+    if (nchunks <= 0 || nchunks >= warps) return 1;
+    return (uint32_t)std::max<int64_t>(1, 2 * warps / nchunks);
+}
+
+// Embeddings a warp may hold back under a limit: all warps together hold at
+// most half of it (the search past the limit is wasted work).  With no limit
+// the total is added up once per run of items.
+uint32_t flush_threshold(uint64_t limit, int64_t warps) {
+    if (!limit) return 0xFFFFFFFFu;
+    return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(limit / (2 * (uint64_t)std::max<int64_t>(warps, 1)), 1), 1u << 16);
+}
+
+// the counter block's fields of a launch
+void bind_counters(MatchOut& O, unsigned long long* ctr) {
+    O.emb_slot = ctr + kSlot;
+    O.status = (int*)(ctr + kStatus);
+    O.bytes = ctr + kBytes;
+    O.floor = ctr + kFloor;
+    O.deadline = ctr + kDeadline;
+    O.started = ctr + kStarted;
+    O.done = ctr + kDone;
+    O.dq_head = ctr + kHead;
+    O.dq_tail = ctr + kTail;
 }
 
 int run_match(const fast_cst* c, const fast_chunks* chunks, const fast_config* cfg_in, uint64_t kemb, uint32_t* emb_out,
@@ -1016,8 +1155,9 @@ int run_match(const fast_cst* c, const fast_chunks* chunks, const fast_config* c
     unsigned long long* ctr = nullptr;
     Chunk* dq = nullptr;
     uint32_t* dq_state = nullptr;
-    const uint64_t cells = ring_cells(cfg, kQueueCap);
-    rc = dalloc(&ctr, kCtrWords, s);
+    const int64_t all_warps = (int64_t)num_sms() * bps * warps;
+    const uint64_t cells = ring_cells(cfg.queue_cells, all_warps, kQueueCap);
+    rc = dalloc(&ctr, kAllWords, s);
     if (rc == FAST_OK && donate) rc = dalloc(&dq, cells, s);
     if (rc == FAST_OK && donate) rc = dalloc(&dq_state, cells, s);
     uint32_t* emb_dev = emb_out;
@@ -1036,23 +1176,23 @@ int run_match(const fast_cst* c, const fast_chunks* chunks, const fast_config* c
         }
     }
     if (rc == FAST_OK) {
-        cudaMemsetAsync(ctr, 0, kCtrWords * sizeof(unsigned long long), s);
-        unsigned long long out0 = (unsigned long long)nchunks;
-        cudaMemcpyAsync(ctr + kOut, &out0, sizeof(out0), cudaMemcpyHostToDevice, s);
+        cudaMemsetAsync(ctr, 0, kAllWords * sizeof(unsigned long long), s);
         if (donate) cudaMemsetAsync(dq_state, 0, cells * sizeof(uint32_t), s);
+        P.chunks = dchunks;
         MatchOut O;
-        O.next_chunk = ctr + kNext; O.total = ctr + kTotal; O.emb_slot = ctr + kSlot; O.status = (int*)(ctr + kStatus);
-        O.qstop = (int*)(ctr + kQStop); O.nq = 1;
+        memset(&O, 0, sizeof(O));
+        bind_counters(O, ctr);
+        O.total = ctr + kTotal;
+        O.qstop = (int*)(ctr + kQStop);
+        O.qnext = (uint32_t*)(ctr + kNext);
+        O.pieces = donate && chunks ? chunk_pieces(nchunks, all_warps) : 1;
+        O.items = (uint32_t)(nchunks * O.pieces);
         // without a partition the root runs are internal: the whole CST is the one chunk
         O.chunk_counts = chunks ? chunk_counts : nullptr; O.emb = emb_dev; O.emb_cap = emb_cap;
         O.stats = stats_out ? ctr + kStats : nullptr;
-        O.bytes = ctr + kBytes;
-        O.floor = ctr + kFloor;
-        O.deadline = ctr + kDeadline;
         O.limit = cfg.limit;
+        O.flush_at = flush_threshold(cfg.limit, all_warps);
         O.dq = dq; O.dq_state = dq_state; O.dq_cap = donate ? cells : 0;
-        O.dq_head = ctr + kHead; O.dq_tail = ctr + kTail; O.outstanding = ctr + kOut;
-        O.idle = (unsigned int*)(ctr + kIdle);
         // the warp-specialised kernel for counting launches that ask for it
         const int nval = (!stats_out && kemb == 0 && chunk_counts == nullptr) ? ws_validators(cfg, warps) : 0;
         O.validators = nval;
@@ -1066,10 +1206,10 @@ int run_match(const fast_cst* c, const fast_chunks* chunks, const fast_config* c
             if (rc == FAST_OK) {
                 EventPair& ev = match_events();
                 if (ev.ok) cudaEventRecord(ev.a, s);
-                if (stats_out) { k_match<true, false, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, dchunks, nchunks, nullptr, O); note_launch(); }
-                else if (kemb > 0) { k_match<false, true, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, dchunks, nchunks, nullptr, O); note_launch(); }
-                else if (nval > 0) { k_match<false, false, false, true><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, dchunks, nchunks, nullptr, O); note_launch(); }
-                else { k_match<false, false, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, dchunks, nchunks, nullptr, O); note_launch(); }
+                if (stats_out) { k_match<true, false, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, O); note_launch(); }
+                else if (kemb > 0) { k_match<false, true, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, O); note_launch(); }
+                else if (nval > 0) { k_match<false, false, false, true><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, O); note_launch(); }
+                else { k_match<false, false, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, O); note_launch(); }
                 cudaError_t e = cudaGetLastError();
                 if (e != cudaSuccess) rc = cuda_status(e, "matcher launch", __FILE__, __LINE__);
                 if (ev.ok) cudaEventRecord(ev.b, s);
@@ -1154,9 +1294,9 @@ extern "C" uint64_t fast_last_match_floor_bytes(void) { return g_last_match_floo
 
 namespace {
 
-constexpr int kNoAllocQueue = 4096;                   // donated runs
+constexpr int kNoAllocQueue = 8192;                   // donated runs
 constexpr int kNoAllocRuns = 32768;                   // root runs when chunks == NULL
-constexpr size_t kNaCtrBytes = ((kCtrWords * sizeof(unsigned long long) + 255) / 256) * 256;
+constexpr size_t kNaCtrBytes = ((kAllWords * sizeof(unsigned long long) + 255) / 256) * 256;
 constexpr size_t kNaQueueBytes = kNoAllocQueue * sizeof(Chunk);
 constexpr size_t kNaReadyBytes = ((kNoAllocQueue * sizeof(uint32_t) + 255) / 256) * 256;
 constexpr size_t kNaRunsBytes = kNoAllocRuns * sizeof(Chunk);
@@ -1216,7 +1356,8 @@ int run_match_noalloc(const fast_cst* c, const fast_chunks* chunks, const fast_c
     unsigned long long* ctr = (unsigned long long*)base;
     Chunk* dq = (Chunk*)(base + kNaCtrBytes);
     uint32_t* dq_state = (uint32_t*)(base + kNaCtrBytes + kNaQueueBytes);
-    const uint64_t cells = ring_cells(cfg, kNoAllocQueue);
+    const int64_t all_warps = (int64_t)num_sms() * bps * warps;
+    const uint64_t cells = ring_cells(cfg.queue_cells, all_warps, kNoAllocQueue);
     Chunk* runs = (Chunk*)(base + kNaCtrBytes + kNaQueueBytes + kNaReadyBytes);
     const Chunk* dchunks = nullptr;
     int64_t nchunks = 0;
@@ -1236,23 +1377,22 @@ int run_match_noalloc(const fast_cst* c, const fast_chunks* chunks, const fast_c
     }
     uint64_t emb_cap = kemb;
     if (cfg.limit > 0 && cfg.limit < emb_cap) emb_cap = cfg.limit;
-    FAST_CUDA(cudaMemsetAsync(ctr, 0, kCtrWords * sizeof(unsigned long long), s));
-    unsigned long long out0 = (unsigned long long)nchunks;
-    FAST_CUDA(cudaMemcpyAsync(ctr + kOut, &out0, sizeof(out0), cudaMemcpyHostToDevice, s));
+    FAST_CUDA(cudaMemsetAsync(ctr, 0, kAllWords * sizeof(unsigned long long), s));
     FAST_CUDA(cudaMemsetAsync(dq_state, 0, cells * sizeof(uint32_t), s));
     MatchPlan P = make_plan(c);
+    P.chunks = dchunks;
     MatchOut O;
-    O.next_chunk = ctr + kNext; O.total = ctr + kTotal; O.emb_slot = ctr + kSlot; O.status = (int*)(ctr + kStatus);
-        O.qstop = (int*)(ctr + kQStop); O.nq = 1;
-    O.chunk_counts = nullptr; O.emb = emb_out; O.emb_cap = emb_cap;
-    O.stats = nullptr;
-    O.bytes = ctr + kBytes;
-    O.floor = ctr + kFloor;
-    O.deadline = ctr + kDeadline;
+    memset(&O, 0, sizeof(O));
+    bind_counters(O, ctr);
+    O.total = ctr + kTotal;
+    O.qstop = (int*)(ctr + kQStop);
+    O.qnext = (uint32_t*)(ctr + kNext);
+    O.pieces = chunks ? chunk_pieces(nchunks, all_warps) : 1;
+    O.items = (uint32_t)(nchunks * O.pieces);
+    O.emb = emb_out; O.emb_cap = emb_cap;
     O.limit = cfg.limit;
+    O.flush_at = flush_threshold(cfg.limit, all_warps);
     O.dq = dq; O.dq_state = dq_state; O.dq_cap = cells;
-    O.dq_head = ctr + kHead; O.dq_tail = ctr + kTail; O.outstanding = ctr + kOut;
-    O.idle = (unsigned int*)(ctr + kIdle);
     O.validators = 0;                                  // the fused kernel
     unsigned long long budget_ns = cfg.time_budget_s > 0 ? (unsigned long long)(cfg.time_budget_s * 1e9) : 0ull;
     if (budget_ns) { k_set_deadline<<<1, 1, 0, s>>>(ctr + kDeadline, budget_ns); note_launch(); }
@@ -1260,8 +1400,8 @@ int run_match_noalloc(const fast_cst* c, const fast_chunks* chunks, const fast_c
         int64_t grid = (int64_t)num_sms() * bps;
         size_t sh = smem_bytes(P, warps);
         FAST_TRY(matcher_smem_optin(sh));
-        if (kemb > 0) k_match<false, true, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, dchunks, nchunks, nullptr, O);
-        else k_match<false, false, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, dchunks, nchunks, nullptr, O);
+        if (kemb > 0) k_match<false, true, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, O);
+        else k_match<false, false, false><<<(unsigned)grid, warps * 32, sh, s>>>(P, nullptr, O);
         note_launch();
         FAST_CUDA(cudaGetLastError());
     }
@@ -1293,8 +1433,9 @@ namespace fast {
 
 size_t match_plan_bytes() { return sizeof(MatchPlan); }
 
-int match_plan_fill(const fast_cst* c, void* host_plan) {
+int match_plan_fill(const fast_cst* c, const fast_chunks* ch, void* host_plan) {
     MatchPlan P = make_plan(c);
+    P.chunks = ch ? ch->d : nullptr;
     memcpy(host_plan, &P, sizeof(P));
     return P.warp_words;
 }
@@ -1304,12 +1445,21 @@ void match_plan_set_stride(void* host_plans, int nq, int warp_words) {
     for (int i = 0; i < nq; i++) P[i].warp_words = warp_words;
 }
 
-size_t match_counter_words() { return kCtrWords; }
+size_t match_counter_words() { return kAllWords; }           // on the device
+size_t match_counter_host_words() { return kCtrWords; }      // the part that comes back
 size_t match_chunk_bytes() { return sizeof(Chunk); }
+uint32_t match_chunk_pieces(int64_t nchunks, int warps, int bps) {
+    return chunk_pieces(nchunks, (int64_t)num_sms() * bps * warps);
+}
+uint64_t match_ring_cells(int64_t queue_cells, int warps, int bps, uint64_t cap) {
+    return ring_cells(queue_cells, (int64_t)num_sms() * bps * warps, cap);
+}
 
 // Enqueue one batched matcher launch (capturable: memsets and kernels only).
-int match_batched_enqueue(const void* d_plans, int warp_words, const void* d_chunks, const int64_t* d_nchunks,
-                          int max_q, unsigned long long* d_qtotal, int* d_qstop, unsigned long long* d_ctr,
+// d_meta: {queries, pieces per chunk, static items of every query}, read on
+// the device, as are the plans with their chunk lists.
+int match_batched_enqueue(const void* d_plans, int warp_words, const uint32_t* d_meta, int max_q,
+                          unsigned long long* d_qtotal, int* d_qstop, uint32_t* d_qnext, unsigned long long* d_ctr,
                           void* d_dq, uint32_t* d_dq_state, uint64_t dq_cap, uint64_t limit, double budget_s,
                           int warps, int bps, int validators, cudaStream_t s) {
     MatchPlan dummy;
@@ -1317,32 +1467,29 @@ int match_batched_enqueue(const void* d_plans, int warp_words, const void* d_chu
     dummy.warp_words = warp_words;
     const int nval = validators > 0 && warps >= 2 ? std::min(validators, warps - 1) : 0;
     size_t sh = launch_smem(warps, warp_words, nval > 0);
-    FAST_CUDA(cudaMemsetAsync(d_ctr, 0, kCtrWords * sizeof(unsigned long long), s));
+    FAST_CUDA(cudaMemsetAsync(d_ctr, 0, kAllWords * sizeof(unsigned long long), s));
     FAST_CUDA(cudaMemsetAsync(d_qtotal, 0, (size_t)max_q * sizeof(unsigned long long), s));
     FAST_CUDA(cudaMemsetAsync(d_qstop, 0, (size_t)max_q * sizeof(int), s));
+    FAST_CUDA(cudaMemsetAsync(d_qnext, 0, (size_t)max_q * sizeof(uint32_t), s));
     FAST_CUDA(cudaMemsetAsync(d_dq_state, 0, dq_cap * sizeof(uint32_t), s));
     MatchOut O;
     memset(&O, 0, sizeof(O));
-    O.next_chunk = d_ctr + kNext; O.total = d_qtotal; O.qstop = d_qstop; O.nq = max_q;
-    O.emb_slot = d_ctr + kSlot; O.status = (int*)(d_ctr + kStatus);
-    O.chunk_counts = nullptr; O.emb = nullptr; O.emb_cap = 0; O.stats = nullptr;
-    O.bytes = d_ctr + kBytes; O.floor = d_ctr + kFloor; O.deadline = d_ctr + kDeadline; O.limit = limit;
+    bind_counters(O, d_ctr);
+    O.total = d_qtotal;
+    O.qstop = d_qstop;
+    O.qnext = d_qnext;
+    O.meta = d_meta;
+    O.limit = limit;
+    O.flush_at = flush_threshold(limit, (int64_t)num_sms() * bps * warps);
     O.dq = (Chunk*)d_dq; O.dq_state = d_dq_state; O.dq_cap = dq_cap;
-    O.dq_head = d_ctr + kHead; O.dq_tail = d_ctr + kTail; O.outstanding = d_ctr + kOut;
-    O.idle = (unsigned int*)(d_ctr + kIdle);
     O.validators = nval;
-    // outstanding = number of chunks, read on the device from *d_nchunks
-    k_copy_word<<<1, 1, 0, s>>>(d_ctr + kOut, d_nchunks);
-    note_launch();
     unsigned long long budget_ns = budget_s > 0 ? (unsigned long long)(budget_s * 1e9) : 0ull;
     if (budget_ns) { k_set_deadline<<<1, 1, 0, s>>>(d_ctr + kDeadline, budget_ns); note_launch(); }
     int64_t grid = (int64_t)num_sms() * bps;
     if (nval > 0)
-        k_match<false, false, true, true><<<(unsigned)grid, warps * 32, sh, s>>>(dummy, (const MatchPlan*)d_plans,
-                                                                                 (const Chunk*)d_chunks, 0, d_nchunks, O);
+        k_match<false, false, true, true><<<(unsigned)grid, warps * 32, sh, s>>>(dummy, (const MatchPlan*)d_plans, O);
     else
-        k_match<false, false, true><<<(unsigned)grid, warps * 32, sh, s>>>(dummy, (const MatchPlan*)d_plans,
-                                                                           (const Chunk*)d_chunks, 0, d_nchunks, O);
+        k_match<false, false, true><<<(unsigned)grid, warps * 32, sh, s>>>(dummy, (const MatchPlan*)d_plans, O);
     note_launch();
     FAST_CUDA(cudaGetLastError());
     return FAST_OK;

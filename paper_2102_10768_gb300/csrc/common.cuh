@@ -54,8 +54,8 @@ bool alloc_fault_due();
 // dalloc/dfree: temporaries.  Inside a PoolScope they come from the bound
 // ScratchPool (pool.cu); elsewhere from the stream-ordered allocator.
 // dalloc_direct/dfree_direct: memory that outlives the call (always the
-// stream-ordered allocator).  Arena: a CST's own arrays, bump-allocated from
-// a few large blocks and returned together.
+// stream-ordered allocator).  Arena: a CST's own arrays, in a few blocks that
+// are returned together.
 struct ScratchPool;
 ScratchPool* pool_new();
 void pool_delete(ScratchPool* p);
@@ -132,34 +132,12 @@ inline void dfree(T*& p, cudaStream_t s) {
 
 class Arena {
   public:
-    template <class T>
-    int alloc(T** p, size_t n, cudaStream_t s) {
-        size_t bytes = n * sizeof(T);
-        bytes = bytes ? (bytes + 255) / 256 * 256 : 256;
-        if (bytes > left_) {
-            int rc = grow(bytes, s);
-            if (rc != FAST_OK) { *p = nullptr; return rc; }
-        }
-        *p = (T*)cur_;
-        cur_ += bytes;
-        left_ -= bytes;
-        return FAST_OK;
-    }
-    // one block of exactly `bytes` (256-byte multiple) when the arena is empty
-    template <class T>
-    int alloc_exact(T** p, size_t bytes, cudaStream_t s) {
-        if (blocks_.empty() && bytes > 0) next_ = (bytes + 255) / 256 * 256;
-        *p = nullptr;
-        return alloc((unsigned char**)p, bytes, s);
-    }
+    // one more block of exactly `bytes`, and only that
+    int block(unsigned char** p, size_t bytes, cudaStream_t s);
     void release(cudaStream_t s);
 
   private:
-    int grow(size_t bytes, cudaStream_t s);
     std::vector<void*> blocks_;
-    char* cur_ = nullptr;
-    size_t left_ = 0;
-    size_t next_ = 16ull << 20;
 };
 
 inline int num_sms() {

@@ -1,18 +1,40 @@
-// Batched CST construction: the candidate search trees (Sec. IV-A,
-// Algorithm 1) and workload estimates (Sec. IV-C) of many queries built
-// together.
+// Construction of candidate search trees (Sec. IV-A, Algorithm 1) and their
+// workload estimates (Sec. IV-C), for one query or many together.
 //
-// The per-query build (cst.cu) runs each query's steps as launches of their
-// own, with host round trips in between; for hundreds of queries the host
-// side of those launches and synchronisations dominates.  Here the steps go
-// over BFS positions t = 0, 1, ...: the vertex at position t of every query
-// is handled by one launch per step for the whole batch (each query, or
-// query edge, is one segment of a segmented compaction or scan, or a range
-// of items of a plain kernel), and the host reads sizes back once or twice
-// per position for all queries at once.  Each step applies the same
-// functors (cst_funcs.cuh) to the same inputs as the per-query build, so
-// every array of every CST comes out identical.  Buffers are sized exactly
-// from those round trips and carved from a few scratch blocks per step.
+// A candidate set C(u) of query vertex u is a bitmap over the positions of
+// u's label (a few KB to some tens of KB: it stays in L1 and L2) until it is
+// final, and every step up to there asks one question of a vertex: has it a
+// neighbour in that set?
+//   filter     C0(u), by label, degree and, if asked for, label frequencies.
+//   top-down   C_td(u) = the members of C0(u) with a neighbour in C_td(parent).
+//              The graph is undirected, so these are the vertices reached from
+//              the parent's set; asking from u's side lets a row stop at its
+//              first hit (usually among its first entries) and gives whole
+//              bitmap words, with no list, no atomics and no compaction.
+//   bottom-up  C(u) = the members of C_td(u) with a neighbour in C(w) for
+//              every child w of u in t_q.
+//   ids        each C(u) as sorted ids, and the rank of every bitmap word.
+//   lists      per tree edge and per non-tree edge (from, to), for every
+//              candidate of `from` its neighbours in C(to) as indices into
+//              C(to): one pass counts, one pass writes in place.  A tree list
+//              after refinement holds the neighbours in the refined set, so
+//              both kinds of edge are the same computation.
+//   workload   children first: the saturating sum of c over each child list,
+//              then the product over the children.
+// Every step is one launch over all queries of the batch (each query vertex
+// or edge is a segment).  Top-down, bottom-up and workload take the vertices
+// of one depth of t_q together, since they only depend on other depths (under
+// refine rule 2 the bottom-up goes vertex by vertex, as the rule is defined).
+// The host reads the filter counts (they choose the root), the set sizes
+// (they fix the matching order and size the arrays), the list sizes and W.
+//
+// Before, the lists of Algorithm 1's top-down pass were written out with an
+// ordered compaction per BFS position, read by the bottom-up pass, rewritten
+// by another compaction and copied to their final place, each over bitmaps of
+// all vertices.  Measured (whole calls, 1M/16M power-law graph): a step of 250
+// queries 150 -> 93 ms, of 40 queries 33.5 -> 18.9 ms; five queries one at a
+// time 28.0 -> 7.0 ms; one 32-vertex query on R-MAT scale 20 6.1 -> 1.6 ms,
+// with about 50 launches where there were 464.
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -26,25 +48,7 @@ using namespace fast;
 
 namespace {
 
-// ------------------------------------------------------------- kernels
-
-// fn(s, i) for every item i < n_s of every segment s; the items of all
-// segments lie end to end (segment s starts at item_off[s]).
-template <class Fn>
-__device__ __forceinline__ void for_items(const int64_t* __restrict__ item_off, int nseg, Fn fn) {
-    const int64_t total = item_off[nseg];
-    for (int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gi < total;
-         gi += (int64_t)gridDim.x * blockDim.x) {
-        const int s = seg_of_tile(item_off, nseg, gi);
-        fn(s, gi - item_off[s]);
-    }
-}
-
-inline unsigned items_grid(int64_t total) {
-    int64_t b = ceil_div(total, 256);
-    int64_t cap = (int64_t)num_sms() * 8;
-    return (unsigned)std::max<int64_t>(1, std::min(b, cap));
-}
+// ------------------------------------------------------------- filter
 
 // Label-frequency requirement of one query vertex u: for each of the nn
 // distinct labels among u's query neighbours, how many carry it.
@@ -54,163 +58,247 @@ struct NlfRow {
     int32_t need[kMaxK];
 };
 
-// One (query, vertex) pair of the candidate filter: the vertex's label
-// bucket lab_vtx[lo, hi), its query degree and, under the label-frequency
-// rule, its requirement and pass bitmap.
+// C0 of one (query, vertex) pair: positions [lo, hi), the query degree and,
+// under the label-frequency rule (nn > 0), the requirement.
 struct FilterDesc {
     int64_t lo, hi;
-    int32_t dq;
-    int32_t nlf;
+    int32_t base, words, dq;
     NlfRow r;
     uint32_t* bits;
     unsigned long long* cnt;
 };
 
-// |C0(u)| for every pair (blockIdx.y) in one launch: the label-and-degree
-// count of k_filter_count, or the label-frequency test and bitmap of
-// k_filter_nlf, per pair.
-__global__ void k_filter_b(const FilterDesc* __restrict__ D, const int32_t* __restrict__ lab_vtx,
-                           const int32_t* __restrict__ key, GraphRuns G, const int32_t* __restrict__ col,
-                           const int32_t* __restrict__ label) {
+// A warp takes 32 neighbouring positions (one bitmap word), so that degrees
+// and label segments are coalesced loads and the word is one ballot.  Bound
+// by these loads: 8 B of row offsets and 8 B per required label and vertex.
+__global__ void __launch_bounds__(256) k_filter(const FilterDesc* __restrict__ D, GraphSegs G) {
+    __shared__ unsigned int total;
     const FilterDesc& d = D[blockIdx.y];
-    const int64_t a = d.lo, b = d.hi;
-    const int want = d.dq;
-    unsigned long long c = 0;
-    for (int64_t i = a + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < b; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v = lab_vtx[i];
-        bool ok = (key[v] & 255) >= want;
-        if (d.nlf) {
-            for (int t = 0; ok && t < d.r.nn; t++)
-                ok = neighbours_with_label(G, col, label, v, d.r.lab[t]) >= d.r.need[t];
-            if (ok) atomicOr(&d.bits[v >> 5], 1u << (v & 31));
-        }
-        c += ok ? 1 : 0;
-    }
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(d.cnt, c);
-}
-
-// Label segments of a candidate set's rows (as k_cand_segment): n rows, and
-// one more item that zeroes len[n], so that an exclusive scan of n + 1
-// lengths leaves the edge-space size in len[n].
-struct CandSegDesc {
-    const int32_t* cand;
-    int64_t n;                       // rows (a bound when n_dev is set)
-    const int64_t* n_dev;            // device, nullable: the real rows
-    int32_t l;
-    int64_t* beg;
-    int64_t* len;
-};
-
-__global__ void k_cand_segment_b(const CandSegDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg,
-                                 GraphRuns G) {
-    for_items(item_off, nseg, [&](int s, int64_t i) {
-        const CandSegDesc& d = D[s];
-        const int64_t n = d.n_dev ? *d.n_dev : d.n;
-        if (i < n) label_segment(G, d.cand[i], d.l, d.beg + i, d.len + i);
-        else d.len[i] = 0;
-    });
-}
-
-// Rows after the last entry and the closing offset (as k_fill_tail).
-struct FillTailDesc {
-    const int64_t* e_off;
-    int64_t n;                       // rows
-    const int64_t* total;            // device: entries kept
-    int64_t* new_off;
-};
-
-__global__ void k_fill_tail_b(const FillTailDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg) {
-    for_items(item_off, nseg, [&](int s, int64_t r) {
-        const FillTailDesc& d = D[s];
-        if (d.e_off[r] == d.e_off[d.n]) d.new_off[r] = *d.total;
-    });
-}
-
-// has[r] = 1 if row r keeps an entry alive (as k_any_alive), tiles of all
-// (query, child) pairs in one sequence.
-struct AnyAliveDesc {
-    const int64_t* off;
-    int64_t rows;
-    const int32_t* list;
-    const uint32_t* alive;
-    uint8_t* has;
-};
-
-// A warp's tile t of a tile-split batched step: its segment, its entries
-// [tb, te) and the rows r0, r1 of its first and last entries, found by the
-// 32 lanes together (every lane returns them).
-struct WarpTile {
-    int s;
-    int64_t tb, te, r0, r1;
-};
-
-template <class D>
-__device__ __forceinline__ WarpTile warp_tile(const D* __restrict__ Dd, const int64_t* __restrict__ tile_off, int nseg,
-                                              int64_t t) {
-    WarpTile w;
-    w.s = seg_of_tile(tile_off, nseg, t);
-    const D& d = Dd[w.s];
-    const int64_t e_end = d.off[d.rows];
-    w.tb = (t - tile_off[w.s]) * kWarpTileItems;
-    w.te = w.tb + kWarpTileItems < e_end ? w.tb + kWarpTileItems : e_end;
-    w.r0 = w.r1 = 0;
-    if (w.tb < w.te) warp_rows_of(d.off, d.rows, w.tb, w.te - 1, &w.r0, &w.r1);
-    return w;
-}
-
-// grid-stride over the warps of the grid
-#define FOR_WARP_TILES(t, total)                                                                        \
-    for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < (total);       \
-         t += (int64_t)gridDim.x * (blockDim.x >> 5))
-
-// A block's tile t (kTileItems entries): warp 0 finds its segment and the
-// rows of its first and last entries, the block waits for them.
-struct TileRows {
-    int s;
-    int64_t tb, te, r0, r1;
-};
-
-template <class D>
-__device__ __forceinline__ bool tile_rows(const D* __restrict__ Dd, const int64_t* __restrict__ tile_off, int nseg,
-                                          int64_t t, TileRows* sh) {
-    if (threadIdx.x < 32) {
-        const int s = seg_of_tile(tile_off, nseg, t);
-        const D& d = Dd[s];
-        const int64_t e_end = d.off[d.rows];
-        const int64_t tb = (t - tile_off[s]) * kTileItems;
-        const int64_t te = tb + kTileItems < e_end ? tb + kTileItems : e_end;
-        int64_t r0 = 0, r1 = 0;
-        if (tb < te) {                  // one search after the other: 32 registers, 8 blocks per SM
-            r0 = warp_row_of(d.off, d.rows, tb);
-            r1 = warp_row_of(d.off, d.rows, te - 1);
-        }
-        if (threadIdx.x == 0) { sh->s = s; sh->tb = tb; sh->te = te; sh->r0 = r0; sh->r1 = r1; }
-    }
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) total = 0;
     __syncthreads();
-    return sh->tb < sh->te;
+    unsigned int c = 0;
+    for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < d.words; w += (int64_t)gridDim.x * 8) {
+        const int64_t p = d.base + w * 32 + lane;
+        bool ok = p >= d.lo && p < d.hi;
+        if (ok) ok = G.row_ptr[p + 1] - G.row_ptr[p] >= d.dq;
+        for (int t = 0; t < d.r.nn && __any_sync(0xffffffffu, ok); t++) {
+            uint32_t beg, len;
+            if (ok) {
+                label_segment(G, (int32_t)p, d.r.lab[t], &beg, &len);
+                ok = len >= (uint32_t)d.r.need[t];
+            }
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, ok);
+        if (lane == 0) { d.bits[w] = m; c += __popc(m); }
+    }
+    if (lane == 0 && c) atomicAdd(&total, c);
+    __syncthreads();
+    if (threadIdx.x == 0 && total) atomicAdd(d.cnt, (unsigned long long)total);
 }
 
-// Block tiles here: the per-entry work (one list entry, one bitmap word) is
-// small next to a row search per warp tile.
-__global__ void __launch_bounds__(256) k_any_alive_b(const AnyAliveDesc* __restrict__ D,
-                                                     const int64_t* __restrict__ tile_off, int nseg) {
-    __shared__ TileRows tr;
+// ------------------------------------------------------------- support
+
+// A set some vertex is tested against: a bitmap over the positions of
+// `label` from `base` on, and its size.
+struct Target {
+    const uint32_t* bits;
+    const unsigned long long* cnt;
+    int32_t base, label;
+};
+
+// out = the members of `in` (words of positions from base on) with a
+// neighbour in every target T[t0 .. t0 + nt); *cnt += their number.
+struct SetDesc {
+    const uint32_t* in;
+    uint32_t* out;
+    unsigned long long* cnt;
+    int32_t base, words, t0, nt;
+};
+
+// A row whose segment is long and did not hit early: its remaining targets,
+// from t on, are left to k_support_long, a block per row.
+struct LongRow {
+    int32_t seg, p, t, pad;
+};
+constexpr uint32_t kLaneProbes = 16;         // entries a lane tests of its own row
+constexpr uint32_t kLongRow = 2048;          // entries from which a row is long
+constexpr uint32_t kLongRows = 1 << 16;      // rows the list holds (a warp finishes the others itself)
+
+__device__ __forceinline__ bool in_bits(const uint32_t* __restrict__ bits, int32_t x) {
+    return (bits[x >> 5] >> (x & 31)) & 1u;
+}
+
+// A warp takes `group` bitmap words, a lane one row of each.  Per target each
+// lane tests its own row's first entries, four loads in flight at a time (a
+// row's entries lie side by side, so they share sectors); rows that need more
+// are scanned by the whole warp, 128 entries a round.  Bound by the latency of
+// the two dependent gathers (entry, bitmap word), which the many independent
+// warps hide.  On a power-law graph the first words of a label can be all
+// hubs, so a row with thousands of entries and no early hit must not stay
+// with one warp.
+__global__ void __launch_bounds__(256) k_support(const SetDesc* __restrict__ D, const int64_t* __restrict__ item_off,
+                                                 int nseg, int group, const Target* __restrict__ T, GraphSegs G,
+                                                 const int32_t* __restrict__ col, LongRow* __restrict__ longs,
+                                                 unsigned int* __restrict__ nlong) {
+    const int lane = threadIdx.x & 31;
+    const int64_t items = item_off[nseg];
+    for (int64_t it = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
+        const int s = seg_of_tile(item_off, nseg, it);
+        const SetDesc d = D[s];
+        const int w0 = (int)(it - item_off[s]) * group, w1 = min(w0 + group, d.words);
+        unsigned int kept = 0;
+        for (int w = w0; w < w1; w++) {
+            const int32_t p = d.base + w * 32 + lane;
+            bool live = (d.in[w] >> lane) & 1u;
+            for (int t = 0; t < d.nt && __any_sync(0xffffffffu, live); t++) {
+                const Target tg = T[d.t0 + t];
+                if (*tg.cnt == 0) { live = false; break; }            // nothing to hit
+                uint32_t beg = 0, len = 0;
+                if (live) label_segment(G, p, tg.label, &beg, &len);
+                bool hit = false;
+                for (uint32_t e = 0; e < kLaneProbes; e += 4) {
+                    const bool go = !hit && e < len;
+                    if (!__any_sync(0xffffffffu, go)) break;
+                    int32_t x[4];
+#pragma unroll
+                    for (int i = 0; i < 4; i++) x[i] = go && e + i < len ? __ldg(col + beg + e + i) - tg.base : -1;
+#pragma unroll
+                    for (int i = 0; i < 4; i++)
+                        if (x[i] >= 0 && in_bits(tg.bits, x[i])) hit = true;
+                }
+                uint32_t more = __ballot_sync(0xffffffffu, !hit && len > kLaneProbes);
+                while (more) {
+                    const int l = __ffs(more) - 1;
+                    more &= more - 1;
+                    const uint32_t b = __shfl_sync(0xffffffffu, beg, l), n = __shfl_sync(0xffffffffu, len, l);
+                    if (longs && n > kLongRow) {
+                        uint32_t slot = kLongRows;
+                        if (lane == l) {
+                            slot = atomicAdd(nlong, 1u);
+                            if (slot < kLongRows) { longs[slot] = LongRow{s, p, t, 0}; live = false; }
+                        }
+                        if (__shfl_sync(0xffffffffu, slot, l) < kLongRows) continue;
+                    }
+                    bool any = false;
+                    for (uint32_t e = kLaneProbes + lane; !any && e - lane < n; e += 128) {
+                        bool h = false;
+                        int32_t x[4];
+#pragma unroll
+                        for (int i = 0; i < 4; i++) x[i] = e + 32 * i < n ? __ldg(col + b + e + 32 * i) - tg.base : -1;
+#pragma unroll
+                        for (int i = 0; i < 4; i++)
+                            if (x[i] >= 0 && in_bits(tg.bits, x[i])) h = true;
+                        any = __any_sync(0xffffffffu, h);
+                    }
+                    if (lane == l) hit = any;
+                }
+                live = live && hit;
+            }
+            const uint32_t m = __ballot_sync(0xffffffffu, live);
+            if (lane == 0) d.out[w] = m;
+            kept += __popc(m);
+        }
+        if (lane == 0 && kept) atomicAdd(d.cnt, (unsigned long long)kept);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_support_long(const SetDesc* __restrict__ D, const Target* __restrict__ T,
+                                                      GraphSegs G, const int32_t* __restrict__ col,
+                                                      const LongRow* __restrict__ longs,
+                                                      const unsigned int* __restrict__ nlong) {
+    const unsigned int n = min(*nlong, kLongRows);
+    for (unsigned int r = blockIdx.x; r < n; r += gridDim.x) {
+        const LongRow lr = longs[r];
+        const SetDesc d = D[lr.seg];
+        bool live = true;
+        for (int t = lr.t; t < d.nt && live; t++) {
+            const Target tg = T[d.t0 + t];
+            uint32_t beg, len;
+            label_segment(G, lr.p, tg.label, &beg, &len);
+            live = false;
+            for (uint32_t e = threadIdx.x; e - threadIdx.x < len && !live; e += 1024) {
+                bool h = false;
+                int32_t x[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++) x[i] = e + 256 * i < len ? __ldg(col + beg + e + 256 * i) - tg.base : -1;
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+                    if (x[i] >= 0 && in_bits(tg.bits, x[i])) h = true;
+                live = __syncthreads_or(h) != 0;
+            }
+        }
+        if (threadIdx.x == 0 && live) {
+            atomicOr(d.out + ((lr.p - d.base) >> 5), 1u << ((lr.p - d.base) & 31));
+            atomicAdd(d.cnt, 1ull);
+        }
+    }
+}
+
+// ------------------------------------------------------------- ids, ranks
+
+// One final candidate set: {word, members before it} pairs, so that a list
+// pass tests membership and takes the rank with one 8-byte load; the members'
+// positions, and their ids.
+struct IdsDesc {
+    const uint32_t* bits;
+    uint2* packed;
+    int32_t* rows;
+    int32_t* cand;
+    int32_t base, words;
+};
+
+constexpr int kIdsBlock = 128;
+constexpr int kIdsItems = 8;                 // words per thread
+constexpr int kIdsTile = kIdsBlock * kIdsItems;
+
+__global__ void __launch_bounds__(kIdsBlock) k_ids(const IdsDesc* __restrict__ D, const int64_t* __restrict__ tile_off,
+                                                   int nseg, const int32_t* __restrict__ lab_vtx,
+                                                   unsigned long long* __restrict__ st,
+                                                   unsigned int* __restrict__ tile_ctr) {
+    __shared__ uint32_t tmp[kIdsBlock / 32 + 1];
+    __shared__ int64_t s_t;
+    __shared__ uint32_t s_excl;
     const int64_t total = tile_off[nseg];
-    for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
-        if (tile_rows(D, tile_off, nseg, t, &tr)) {
-            const AnyAliveDesc& d = D[tr.s];
-            const int64_t* off = d.off;
-            const int64_t i0 = tr.tb + (int64_t)threadIdx.x * kItems;
-            if (i0 < tr.te) {
-                int64_t row = row_in(off, tr.r0, tr.r1, i0), done = -1;
-                for (int i = 0; i < kItems; i++) {
-                    int64_t e = i0 + i;
-                    if (e >= tr.te) break;
-                    while (e >= off[row + 1]) row++;
-                    if (row == done) continue;
-                    int32_t x = d.list[e];
-                    if ((d.alive[x >> 5] >> (x & 31)) & 1u) { d.has[row] = 1; done = row; }
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        if (threadIdx.x == 0) s_t = (int64_t)atomicAdd(tile_ctr, 1u);
+        __syncthreads();
+        const int64_t t = s_t;
+        if (t >= total) break;
+        const int s = seg_of_tile(tile_off, nseg, t);
+        const int64_t first = tile_off[s];
+        const IdsDesc& d = D[s];
+        const int wb = (int)(t - first) * kIdsTile, base = wb + (int)threadIdx.x * kIdsItems;
+        uint32_t w[kIdsItems], v[kIdsItems];
+#pragma unroll
+        for (int i = 0; i < kIdsItems; i++) {
+            w[i] = base + i < d.words ? d.bits[base + i] : 0u;
+            v[i] = __popc(w[i]);
+        }
+        const uint32_t tot = block_exclusive_scan<uint32_t, kIdsBlock, kIdsItems>(v, tmp);
+        if (threadIdx.x < 32) {
+            const int64_t excl = tile_publish(st + first, t - first, (int64_t)tot);
+            if (threadIdx.x == 0) s_excl = (uint32_t)excl;
+        }
+        __syncthreads();
+        const uint32_t off = s_excl;
+        const int wlane = wb + (int)(threadIdx.x & ~31u) * kIdsItems;       // this warp's first word
+#pragma unroll
+        for (int i = 0; i < kIdsItems; i++) {
+            const uint32_t r = v[i] + off;
+            if (base + i < d.words) d.packed[base + i] = make_uint2(w[i], r);
+            // word i of every lane in turn: its members are written side by side
+            uint32_t some = __ballot_sync(0xffffffffu, w[i] != 0);
+            while (some) {
+                const int l = __ffs(some) - 1;
+                some &= some - 1;
+                const uint32_t x = __shfl_sync(0xffffffffu, w[i], l), o = __shfl_sync(0xffffffffu, r, l);
+                if ((x >> lane) & 1u) {
+                    const int32_t p = d.base + (wlane + l * kIdsItems + i) * 32 + lane;
+                    const uint32_t at = o + __popc(x & lanemask_lt());
+                    d.rows[at] = p;
+                    d.cand[at] = lab_vtx[p];
                 }
             }
         }
@@ -218,167 +306,247 @@ __global__ void __launch_bounds__(256) k_any_alive_b(const AnyAliveDesc* __restr
     }
 }
 
-// {alive, rank} word pairs of a refined candidate bitmap, so that the
-// bottom-up rewrite and the non-tree step read a word and its prefix
-// popcount with one 8-byte load.
-struct PackDesc {
-    const uint32_t* alive;
-    const uint32_t* rank;
-    uint2* packed;
+// ------------------------------------------------------------- lists
+
+// The lists of one query edge (from, to): rows = the candidates of `from`,
+// whose neighbours with to's label, end to end, are its edge space of *E
+// entries, cut into tiles of kListTile.  Offsets and segment starts are 32
+// bits (there are fewer than 2^32 adjacency entries).
+struct ListDesc {
+    const int32_t* rows;             // positions
+    uint32_t n;                      // rows
+    int32_t label, base;             // to's label, first position of its bitmap
+    const uint2* packed;             // to's set
+    uint32_t* e_off;                 // [n + 1] edge-space offset of each row
+    uint32_t* beg;                   // [n] where its segment starts in col
+    int32_t* first;                  // per tile (and one more): its first row that starts in it
+    uint32_t* E;
+    uint32_t* tile;                  // per tile: entries kept, then those kept before it
+    uint32_t* K;                     // entries kept
+    int64_t* off;                    // out [n + 1]
+    uint32_t* idx;                   // out [*K]
+};
+constexpr uint32_t kListTile = 512;
+
+// Row lengths and their prefix, and for every tile the row it begins with.
+struct RowLens {
+    const ListDesc* D;
+    GraphSegs G;
+    __device__ int64_t n(int s) const { return D[s].n; }
+    __device__ uint32_t load(int s, int64_t i) const {
+        uint32_t b, len;
+        label_segment(G, D[s].rows[i], D[s].label, &b, &len);
+        D[s].beg[i] = b;
+        return len;
+    }
+    __device__ void store(int s, int64_t i, uint32_t o, uint32_t len) const {
+        const ListDesc& d = D[s];
+        d.e_off[i] = o;
+        if (i == 0) d.first[0] = 0;
+        // tiles that begin after o and not after the row's end begin with a later row
+        for (uint32_t t = o / kListTile + 1; (uint64_t)t * kListTile <= (uint64_t)o + len; t++) d.first[t] = (int32_t)(i + 1);
+        if (i == d.n - 1) d.e_off[d.n] = o + len;
+    }
+    __device__ void total(int s, uint32_t tot) const {
+        *D[s].E = tot;
+        if (D[s].n == 0) D[s].e_off[0] = 0;
+    }
 };
 
-__global__ void k_pack_bits_b(const PackDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg) {
-    for_items(item_off, nseg, [&](int s, int64_t w) {
-        const PackDesc& d = D[s];
-        d.packed[w] = make_uint2(d.alive[w], d.rank[w]);
-    });
+__global__ void __launch_bounds__(kScanBlock) k_row_lens(const ListDesc* __restrict__ D, GraphSegs G,
+                                                         const int64_t* __restrict__ tile_off, int nseg,
+                                                         unsigned long long* st, unsigned int* ctr) {
+    RowLens f{D, G};
+    seg_scan<uint32_t>(f, tile_off, nseg, st, ctr);
 }
 
-// valid[r] = every child list of row r keeps an entry (as k_valid_rows_n).
-struct ValidDesc {
-    ChildFlags cf;
-    uint8_t* valid;
-    int64_t* vflag;
+// tile counts -> tile bases, and the list set's size
+struct TileBases {
+    const ListDesc* D;
+    const int64_t* item_off;
+    __device__ int64_t n(int s) const { return item_off[s + 1] - item_off[s]; }
+    __device__ uint32_t load(int s, int64_t i) const { return D[s].tile[i]; }
+    __device__ void store(int s, int64_t i, uint32_t o, uint32_t) const { D[s].tile[i] = o; }
+    __device__ void total(int s, uint32_t tot) const { *D[s].K = tot; }
 };
 
-__global__ void k_valid_rows_b(const ValidDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg) {
-    for_items(item_off, nseg, [&](int s, int64_t r) {
-        const ValidDesc& d = D[s];
-        uint8_t ok = 1;
-        for (int c = 0; c < d.cf.nch && ok; c++) ok &= d.cf.has[c][r];
-        d.valid[r] = ok;
-        d.vflag[r] = ok;
-    });
+__global__ void __launch_bounds__(kScanBlock) k_tile_bases(const ListDesc* __restrict__ D,
+                                                           const int64_t* __restrict__ item_off,
+                                                           const int64_t* __restrict__ tile_off, int nseg,
+                                                           unsigned long long* st, unsigned int* ctr) {
+    TileBases f{D, item_off};
+    seg_scan<uint32_t>(f, tile_off, nseg, st, ctr);
 }
 
-// Refine rule 2, the non-tree test: flag[r] = 1 if candidate cand[r] of u
-// has a neighbour in the bitmap of C(w), for one non-tree query neighbour w
-// (its label segment in G; every member of the bitmap carries w's label, so
-// an ungrouped row needs no label test).  One warp per row, rows of all
-// (query, neighbour) pairs end to end.
-struct NtDesc {
-    const int32_t* cand;
-    int32_t l;
-    const uint32_t* bits;
-    uint8_t* flag;
-};
-
-__global__ void k_nt_support_b(const NtDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg,
-                               GraphRuns G, const int32_t* __restrict__ col) {
+// A warp takes a tile of the edge space: a window of 32 rows at a time (lane
+// = row: offset and segment start, one coalesced load each), then the
+// window's entries 64 at a time, each lane finding its entry's row among the
+// window's offsets with five shuffles.  Counting and writing are two passes
+// over the same entries: nothing waits on another tile (one pass with a
+// look-back left three of four warps at a barrier), the arrays get their exact
+// sizes in between, and the lists are written once, where they stay.  Bound by
+// the entry load and the dependent {word, rank} gather, which hits L1.
+template <bool WRITE>
+__global__ void __launch_bounds__(256) k_lists(const ListDesc* __restrict__ D, const int64_t* __restrict__ item_off,
+                                               int nseg, const int32_t* __restrict__ col) {
     const int lane = threadIdx.x & 31;
-    const int64_t total = item_off[nseg];
-    for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < total;
-         it += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t items = item_off[nseg];
+    for (int64_t it = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
         const int s = seg_of_tile(item_off, nseg, it);
-        const NtDesc& d = D[s];
-        const int64_t r = it - item_off[s];
-        int64_t b, len;
-        label_segment(G, d.cand[r], d.l, &b, &len);
-        bool any = false;
-        for (int64_t base = 0; base < len; base += 32) {      // the same steps on every lane
-            bool hit = false;
-            if (base + lane < len) {
-                const int32_t x = col[b + base + lane];
-                hit = (d.bits[x >> 5] >> (x & 31)) & 1u;
-            }
-            if (__any_sync(0xffffffffu, hit)) { any = true; break; }
+        const ListDesc& d = D[s];
+        const uint32_t lt = (uint32_t)(it - item_off[s]);
+        const uint32_t E = *d.E, n = d.n, tb = lt * kListTile;
+        if (lt > 0 && (it - item_off[s]) * kListTile >= E) {     // past the end of a space sized by a bound
+            if (!WRITE && lane == 0) d.tile[lt] = 0;
+            continue;
         }
-        if (lane == 0) d.flag[r] = any ? 1 : 0;
+        const bool last = E - tb <= kListTile;
+        const uint32_t te = last ? E : tb + kListTile;
+        uint32_t R = n ? (uint32_t)max(d.first[lt] - 1, 0) : 0u;
+        uint32_t run = WRITE ? d.tile[lt] : 0u;                  // entries kept so far
+        uint32_t cur = tb;
+        for (;;) {
+            const uint32_t row = R + lane;
+            const uint32_t eo = row <= n ? d.e_off[row] : E;
+            const uint32_t sh = (row < n ? d.beg[row] : 0u) - eo;  // entry e of the row is col[sh + e]
+            const uint32_t nxt = R + 32 <= n ? d.e_off[R + 32] : E;
+            const uint32_t lim = nxt < te ? nxt : te;
+            for (uint32_t i0 = cur; i0 < lim; i0 += 64) {
+                int32_t x[2];
+                uint2 pk[2];
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const uint32_t e = i0 + 32 * u + lane;
+                    int slot = 0;                                // the last row that starts at or before e
+#pragma unroll
+                    for (int st = 16; st; st >>= 1)
+                        if (__shfl_sync(0xffffffffu, eo, slot + st) <= e) slot += st;
+                    const uint32_t at = __shfl_sync(0xffffffffu, sh, slot) + e;
+                    x[u] = e < lim ? __ldg(col + at) - d.base : -1;
+                }
+#pragma unroll
+                for (int u = 0; u < 2; u++) pk[u] = x[u] >= 0 ? __ldg(d.packed + (x[u] >> 5)) : make_uint2(0u, 0u);
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const uint32_t i = i0 + 32 * u, bit = 1u << (x[u] & 31);
+                    const bool hit = x[u] >= 0 && (pk[u].x & bit);
+                    const uint32_t m = __ballot_sync(0xffffffffu, hit);
+                    if (WRITE) {
+                        // rows that start among these 32 entries
+                        if (row < n && eo >= i && eo < lim && eo - i < 32) d.off[row] = run + __popc(m & ((1u << (eo - i)) - 1));
+                        if (hit) d.idx[run + __popc(m & lanemask_lt())] = pk[u].y + __popc(pk[u].x & (bit - 1));
+                    }
+                    run += __popc(m);
+                }
+            }
+            cur = cur > lim ? cur : lim;
+            // empty rows at the window's end (those at a tile's end are the next tile's)
+            if (WRITE && row < n && eo == lim && (lim < te || last)) d.off[row] = run;
+            if (cur >= te && (!last || R + 32 >= n)) break;
+            R += 32;
+        }
+        if (lane == 0) {
+            if (!WRITE) d.tile[lt] = run;
+            else if (last) d.off[n] = run;
+        }
     }
 }
 
-// off[*n] = *val (as k_set_tail), one thread per descriptor.
-struct SetTailDesc {
-    int64_t* off;
-    const int64_t* n;
-    const int64_t* val;
-};
+// ------------------------------------------------------------- workload
 
-__global__ void k_set_tail_b(const SetTailDesc* __restrict__ D, int nd) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nd) D[i].off[*D[i].n] = *D[i].val;
-}
-
-// Bitmap of a candidate set whose size *n is on the device (as
-// k_set_bits_n); the items of a segment are a host bound on *n.
-struct SetBitsDesc {
-    const int32_t* ids;
-    const int64_t* n;
-    uint32_t* bits;
-};
-
-__global__ void k_set_bits_b(const SetBitsDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg) {
-    for_items(item_off, nseg, [&](int s, int64_t i) {
-        const SetBitsDesc& d = D[s];
-        if (i < *d.n) atomicOr(&d.bits[d.ids[i] >> 5], 1u << (d.ids[i] & 31));
-    });
-}
-
-// Workload, first half (as k_child_sums), tiles of all (query, child)
-// pairs in one sequence.
+// Tiles of all (query, child) pairs in one sequence; each warp takes its own
+// tile of kWarpTileItems entries and finds its two end rows itself.
 struct ChildSumDesc {
     const int64_t* off;
     int64_t rows;
     const uint32_t* idx;
-    const uint64_t* cv;
-    const double* cvf;
+    const CVal* cv;
     unsigned long long* ssum;
     double* sumf;
     uint32_t* ovf;
 };
 
-__global__ void __launch_bounds__(256, 4) k_child_sums_b(const ChildSumDesc* __restrict__ D,
-                                                         const int64_t* __restrict__ tile_off, int nseg) {
+__global__ void __launch_bounds__(256, 4) k_child_sums(const ChildSumDesc* __restrict__ D,
+                                                       const int64_t* __restrict__ tile_off, int nseg) {
     const int64_t total = tile_off[nseg];
-    FOR_WARP_TILES(t, total) {
-        const WarpTile w = warp_tile(D, tile_off, nseg, t);
-        const ChildSumDesc& d = D[w.s];
-        child_sum_entries(d.off, w.r0, w.r1, w.tb + (int64_t)(threadIdx.x & 31) * kItems, w.te, d.idx, d.cv, d.cvf,
-                          d.ssum, d.sumf, d.ovf);
+    for (int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); t < total; t += (int64_t)gridDim.x * 8) {
+        const int s = seg_of_tile(tile_off, nseg, t);
+        const ChildSumDesc& d = D[s];
+        const int64_t e_end = d.off[d.rows];
+        const int64_t tb = (t - tile_off[s]) * kWarpTileItems;
+        const int64_t te = tb + kWarpTileItems < e_end ? tb + kWarpTileItems : e_end;
+        int64_t r0 = 0, r1 = 0;
+        if (tb < te) warp_rows_of(d.off, d.rows, tb, te - 1, &r0, &r1);
+        child_sum_entries(d.off, r0, r1, tb + (int64_t)(threadIdx.x & 31) * kItems, te, d.idx, d.cv, d.ssum, d.sumf, d.ovf);
         __syncwarp();
     }
 }
 
-// Workload, second half (as k_workload_prod; a leaf, with no child, gets
-// 1 and 1.0 as k_fill_u64 / k_fill_f64 give it).
-struct ProdDesc {
-    ChildSums cs;
-    uint64_t* cval;
-    double* cvalf;
+// One child of a vertex: its sums, or, for a leaf (c = 1 everywhere), the list
+// offsets, whose differences are the sums; out: the saturating sums, kept for
+// the partitioner.
+struct ChildRef {
+    const int64_t* off;              // leaf
+    const unsigned long long* ssum;  // otherwise
+    const double* sumf;
+    const uint32_t* ovf;
+    uint64_t* out;
 };
 
-__global__ void k_workload_prod_b(const ProdDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg) {
-    for_items(item_off, nseg, [&](int s, int64_t r) {
-        const ProdDesc& d = D[s];
+struct ProdDesc {
+    int32_t c0, nc;                  // its children in the child array
+    uint64_t* cval;
+    CVal* cv;                        // nullable
+};
+
+__global__ void k_workload_prod(const ProdDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg,
+                                const ChildRef* __restrict__ C) {
+    const int64_t total = item_off[nseg];
+    for (int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gi < total;
+         gi += (int64_t)gridDim.x * blockDim.x) {
+        const int s = seg_of_tile(item_off, nseg, gi);
+        const ProdDesc d = D[s];
+        const int64_t r = gi - item_off[s];
         uint64_t prod = 1;
         double prodf = 1.0;
-        for (int c = 0; c < d.cs.nch; c++) {
-            uint64_t sm = d.cs.ovf[c][r] ? ~0ull : d.cs.ssum[c][r];
-            d.cs.ssum[c][r] = sm;
+        for (int c = d.c0; c < d.c0 + d.nc; c++) {
+            uint64_t sm;
+            double sf;
+            if (C[c].off) {
+                sm = (uint64_t)(C[c].off[r + 1] - C[c].off[r]);
+                sf = (double)sm;
+            } else {
+                sm = C[c].ovf[r] ? ~0ull : C[c].ssum[r];
+                sf = C[c].sumf[r];
+            }
+            C[c].out[r] = sm;
             prod = sat_mul(prod, sm);
-            prodf *= d.cs.sumf[c][r];
+            prodf *= sf;
         }
         d.cval[r] = prod;
-        d.cvalf[r] = prodf;
-    });
+        if (d.cv) d.cv[r] = CVal{prod, prodf};
+    }
 }
 
-// W per query (as k_total_w), one block of 1024 threads per descriptor.
+// W per query, one block of 1024 threads each.
 struct TotalDesc {
-    const uint64_t* cval;
-    const double* cvalf;
+    const CVal* cv;
     int64_t n;
     uint64_t* out;
     double* outf;
 };
 
-__global__ void k_total_w_b(const TotalDesc* __restrict__ D) {
+__global__ void k_total_w(const TotalDesc* __restrict__ D) {
     __shared__ uint64_t sh[32];
     __shared__ double shf[32];
     const TotalDesc& d = D[blockIdx.x];
     uint64_t s = 0;
     double sf = 0.0;
-    for (int64_t i = threadIdx.x; i < d.n; i += blockDim.x) { s = sat_add(s, d.cval[i]); sf += d.cvalf[i]; }
+    for (int64_t i = threadIdx.x; i < d.n; i += blockDim.x) {
+        const CVal c = d.cv[i];
+        s = sat_add(s, c.c);
+        sf += c.f;
+    }
     s = warp_sat_sum(s);
     sf = warp_sum_f(sf);
     int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -416,21 +584,26 @@ class Carver {
     void add(T** slot, int64_t n) {
         items_.push_back({(void**)slot, (size_t)std::max<int64_t>(n, 0) * sizeof(T)});
     }
-    int alloc(Scratch& into, bool zero, unsigned char** block = nullptr, size_t* bytes = nullptr) {
-        if (items_.empty()) return FAST_OK;
+    size_t bytes() const {
         size_t total = 0;
         for (auto& it : items_) total += piece(it.bytes);
-        unsigned char* b = nullptr;
-        FAST_TRY(dalloc(&b, total, into.s_));
-        into.v.push_back(b);
+        return total;
+    }
+    void place(unsigned char* b) {
         size_t at = 0;
         for (auto& it : items_) {
             *it.slot = b + at;
             at += piece(it.bytes);
         }
         items_.clear();
-        if (block) *block = b;
-        if (bytes) *bytes = total;
+    }
+    int alloc(Scratch& into, bool zero) {
+        if (items_.empty()) return FAST_OK;
+        const size_t total = bytes();
+        unsigned char* b = nullptr;
+        FAST_TRY(dalloc(&b, total, into.s_));
+        into.v.push_back(b);
+        place(b);
         if (zero) FAST_CUDA(cudaMemsetAsync(b, 0, total, into.s_));
         return FAST_OK;
     }
@@ -444,23 +617,42 @@ class Carver {
     std::vector<Item> items_;
 };
 
-// Descriptors and their item (or tile) offsets, uploaded with one copy.
-template <class D>
-int upload(const std::vector<D>& desc, const std::vector<int64_t>& off, Scratch& sc, const D** d_desc,
-           const int64_t** d_off) {
-    const size_t a = (desc.size() * sizeof(D) + 15) / 16 * 16;
-    const size_t bytes = a + off.size() * sizeof(int64_t);
-    unsigned char* b = nullptr;
-    FAST_TRY(dalloc(&b, bytes, sc.s_));
-    sc.v.push_back(b);
-    std::vector<unsigned char> h(bytes, 0);
-    memcpy(h.data(), desc.data(), desc.size() * sizeof(D));
-    if (!off.empty()) memcpy(h.data() + a, off.data(), off.size() * sizeof(int64_t));
-    FAST_CUDA(cudaMemcpyAsync(b, h.data(), bytes, cudaMemcpyHostToDevice, sc.s_));
-    *d_desc = (const D*)b;
-    *d_off = (const int64_t*)(b + a);
-    return FAST_OK;
-}
+// What the launches of one phase read: host arrays gathered into one block
+// and uploaded with one copy, and a zeroed region behind them (scan status
+// words and counters).
+class Stage {
+  public:
+    template <class T>
+    size_t add(const std::vector<T>& v) {
+        const size_t at = (h_.size() + 15) / 16 * 16;
+        h_.resize(at + v.size() * sizeof(T));
+        if (!v.empty()) memcpy(h_.data() + at, v.data(), v.size() * sizeof(T));
+        return at;
+    }
+    size_t zeros(size_t words) {                  // 8-byte words
+        const size_t at = zero_;
+        zero_ += words;
+        return at;
+    }
+    int upload(Scratch& sc) {
+        const size_t a = (h_.size() + 15) / 16 * 16;
+        FAST_TRY(dalloc(&base_, a + zero_ * 8 + 16, sc.s_));
+        sc.v.push_back(base_);
+        z_ = (unsigned long long*)(base_ + a);
+        if (!h_.empty()) FAST_CUDA(cudaMemcpyAsync(base_, h_.data(), h_.size(), cudaMemcpyHostToDevice, sc.s_));
+        if (zero_) FAST_CUDA(cudaMemsetAsync(z_, 0, zero_ * 8, sc.s_));
+        return FAST_OK;
+    }
+    template <class T>
+    const T* at(size_t off) const { return (const T*)(base_ + off); }
+    unsigned long long* z(size_t word) const { return z_ + word; }
+
+  private:
+    std::vector<unsigned char> h_;
+    size_t zero_ = 0;
+    unsigned char* base_ = nullptr;
+    unsigned long long* z_ = nullptr;
+};
 
 inline std::vector<int64_t> prefix(const std::vector<int64_t>& n) {
     std::vector<int64_t> off(n.size() + 1, 0);
@@ -468,63 +660,31 @@ inline std::vector<int64_t> prefix(const std::vector<int64_t>& n) {
     return off;
 }
 
-// A plain batched kernel over segments of n_s items.
-template <class D, class... X>
-int run_items(void (*kernel)(const D*, const int64_t*, int, X...), const std::vector<D>& desc,
-              const std::vector<int64_t>& n, cudaStream_t s, X... extra) {
-    if (desc.empty()) return FAST_OK;
-    const std::vector<int64_t> off = prefix(n);
-    if (off.back() == 0) return FAST_OK;
-    Scratch sc(s);
-    const D* dd = nullptr;
-    const int64_t* doff = nullptr;
-    FAST_TRY(upload(desc, off, sc, &dd, &doff));
-    kernel<<<items_grid(off.back()), 256, 0, s>>>(dd, doff, (int)desc.size(), extra...);
-    note_launch();
-    if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "batched CST step launch");
-    return FAST_OK;
+// counts a launch and checks it
+int note_launch(const char* what) {
+    fast::note_launch();
+    return cudaGetLastError() == cudaSuccess ? FAST_OK : set_error(FAST_ERR_CUDA, "%s launch", what);
 }
 
-// A tile-split batched kernel over segments of e_s list entries, in tiles
-// of `tile` entries, `per_block` tiles to a block of 256 threads (8: warp
-// tiles; 1: block tiles).
-template <class D>
-int run_tiles(void (*kernel)(const D*, const int64_t*, int), const std::vector<D>& desc,
-              const std::vector<int64_t>& entries, int tile, int per_block, cudaStream_t s) {
-    if (desc.empty()) return FAST_OK;
-    std::vector<int64_t> t(entries.size());
-    for (size_t i = 0; i < entries.size(); i++) t[i] = ceil_div(entries[i], (int64_t)tile);
-    const std::vector<int64_t> off = prefix(t);
-    if (off.back() == 0) return FAST_OK;
-    Scratch sc(s);
-    const D* dd = nullptr;
-    const int64_t* doff = nullptr;
-    FAST_TRY(upload(desc, off, sc, &dd, &doff));
-    const int64_t grid = std::min<int64_t>(ceil_div(off.back(), (int64_t)per_block), (int64_t)num_sms() * 8);
-    kernel<<<(unsigned)grid, 256, 0, s>>>(dd, doff, (int)desc.size());
-    note_launch();
-    if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "batched CST step launch");
-    return FAST_OK;
+// blocks of 256 threads for `warps` warps of work, `per_sm` blocks per SM at most
+inline unsigned warp_grid(int64_t warps, int per_sm) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(warps, 8), (int64_t)num_sms() * per_sm));
 }
 
-// Size words on the device: field f of query q at Z[f * nq + q].  The
-// filter counts are by query vertex, the rest by BFS position.
+// Size words on the device: field f of query q at Z[f * nq + q], by query
+// vertex.
 enum : int {
     F_CNT = 0,                    // |C0(u)|
-    F_TD = F_CNT + kMaxK,         // |C_td| of the vertex at position t
-    F_E = F_TD + kMaxK,           // its top-down edge space
-    F_KEPT = F_E + kMaxK,         // its top-down list entries
-    F_C = F_KEPT + kMaxK,         // |C| after refinement
-    F_T = F_C + kMaxK,            // its tree-list entries after refinement
-    F_W = F_T + kMaxK,            // W, saturating uint64
+    F_TD = F_CNT + kMaxK,         // |C_td(u)|
+    F_C = F_TD + kMaxK,           // |C(u)| of a vertex that the bottom-up pass visits
+    F_W = F_C + kMaxK,            // W, saturating uint64
     F_WF = F_W + 1,               // W, float64
     F_END = F_WF + 1
 };
 
-// Batches of at most this many queries, whose bounded top-down arrays fit
-// in kBoundedBytes, build the top-down pass without host round trips.
+// Batches of at most this many queries size their tile arrays by host-known
+// bounds; a larger one reads each edge-space size back first.
 constexpr int kBoundedQueries = 8;
-constexpr uint64_t kBoundedBytes = 2ull << 30;
 
 // One query of the batch.
 struct Q {
@@ -533,28 +693,24 @@ struct Q {
     int k = 0;
     bool nlf = false;
     bool nt_refine = false;       // refine rule 2: the non-tree test in the bottom-up pass
-    uint32_t* root_bits = nullptr; // rule 2: bitmap of C_td(root) for the test
     int A[kMaxK][kMaxK] = {};
     int dq[kMaxK] = {};
     int bpos[kMaxK] = {};         // vertex -> BFS position
-    int64_t lo[kMaxK] = {}, hi[kMaxK] = {};
-    int64_t c0[kMaxK] = {};       // |C0(u)|
-    int64_t ctd[kMaxK] = {};      // |C_td(u)|
-    int64_t E[kMaxK] = {};        // top-down edge space into u
-    int64_t kept[kMaxK] = {};     // top-down entries kept into u
-    int32_t* td_cand[kMaxK] = {};
-    int32_t* td_list[kMaxK] = {};
-    int64_t* td_off[kMaxK] = {};
-    uint32_t* alive[kMaxK] = {};  // reached bitmap, then the bitmap of the refined C(u)
-    uint32_t* rank[kMaxK] = {};
-    uint2* packed[kMaxK] = {};    // {alive, rank} word pairs of the refined C(u)
-    uint32_t* nlfb[kMaxK] = {};   // label-frequency pass bitmaps
-    int64_t* e_off = nullptr;     // the current step's edge space
-    int64_t* seg = nullptr;
+    int depth[kMaxK] = {};        // vertex -> depth in t_q
+    int nch[kMaxK] = {};          // children in t_q
+    int64_t lo[kMaxK] = {}, hi[kMaxK] = {};   // positions of the vertex's label
+    int32_t base[kMaxK] = {}, words[kMaxK] = {};
+    uint32_t* pass[kMaxK] = {};   // bitmap of C0(u) (shared by equal requirements)
+    uint32_t* set[kMaxK] = {};    // bitmap of C_td(u), then of C(u)
+    const uint32_t* cur[kMaxK] = {};   // the vertex's set as it stands
+    int cnt[kMaxK] = {};          // the field that holds its size
+    uint2* packed[kMaxK] = {};
+    int32_t* rows[kMaxK] = {};    // positions of C(u)
+    CVal* cv[kMaxK] = {};
 };
 
 // Matching order and non-tree edges of one query from its refined candidate
-// counts, by the rules the per-query build uses.
+// counts.
 void order_and_nontree(const Q& q, fast_cst* c) {
     fast::matching_order(q.k, q.A, c->root, c->parent, c->bfs, c->ncand, c->cfg.order_rule, c->order, c->pos);
     c->nnt = nontree_edges(q.k, q.A, c->order, c->parent, c->nt_from, c->nt_to);
@@ -562,78 +718,323 @@ void order_and_nontree(const Q& q, fast_cst* c) {
 
 thread_local uint64_t t_round_trips = 0;   // this thread's last batched build
 
-int fetch(const int64_t* d, std::vector<int64_t>& h, size_t words, cudaStream_t s) {
+template <class T>
+int fetch(const T* d, std::vector<T>& h, size_t n, cudaStream_t s) {
     t_round_trips++;
-    h.assign(words, 0);
-    if (!words) return FAST_OK;
-    cudaError_t e = cudaMemcpyAsync(h.data(), d, words * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    h.assign(n, T(0));
+    if (!n) return FAST_OK;
+    cudaError_t e = cudaMemcpyAsync(h.data(), d, n * sizeof(T), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    return e == cudaSuccess ? FAST_OK : cuda_status(e, "batched CST sizes", __FILE__, __LINE__);
+    return e == cudaSuccess ? FAST_OK : cuda_status(e, "CST sizes", __FILE__, __LINE__);
 }
 
-// After the last round trip every size is known: every CST's arrays go
-// into one exact-size block of its own arena, all CSTs with one launch.
-int copy_to_arenas(std::vector<Q>& Qs, cudaStream_t s) {
-    std::vector<CopyDesc> cd;
-    uint64_t pieces = 0;
-    for (auto& q : Qs) {
-        fast_cst* c = q.c;
-        struct Item { void** slot; uint64_t bytes; };
-        std::vector<Item> items;
-        for (int u = 0; u < c->k; u++) {
-            const uint64_t nc = (uint64_t)c->ncand[u];
-            items.push_back({(void**)&c->cand[u], nc * 4});
-            items.push_back({(void**)&c->cval[u], nc * 8});
-            items.push_back({(void**)&c->cvalf[u], nc * 8});
-            if (c->parent[u] >= 0) {
-                const uint64_t np = (uint64_t)c->ncand[c->parent[u]];
-                items.push_back({(void**)&c->t_off[u], (np + 1) * 8});
-                items.push_back({(void**)&c->t_idx[u], (uint64_t)c->t_entries[u] * 4});
-                items.push_back({(void**)&c->ssum[u], np * 8});
-            }
+// Page-locked words and events of this thread, so that a size read can be
+// queued between launches and waited for later.
+struct Readback {
+    uint32_t* h = nullptr;
+    size_t cap = 0;
+    std::vector<cudaEvent_t> ev;
+    ~Readback() {
+        if (h) cudaFreeHost(h);
+        for (auto e : ev) cudaEventDestroy(e);
+    }
+    int reserve(size_t words, size_t events) {
+        if (words > cap) {
+            if (h) cudaFreeHost(h);
+            h = nullptr;
+            cap = 0;
+            FAST_CUDA(cudaMallocHost((void**)&h, words * sizeof(uint32_t)));
+            cap = words;
         }
-        for (int e = 0; e < c->nnt; e++) {
-            const uint64_t nf = (uint64_t)c->ncand[c->nt_from[e]];
-            items.push_back({(void**)&c->n_off[e], (nf + 1) * 8});
-            items.push_back({(void**)&c->n_idx[e], (uint64_t)c->n_entries[e] * 4});
+        while (ev.size() < events) {
+            cudaEvent_t e;
+            FAST_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+            ev.push_back(e);
         }
-        uint64_t total = 0;
-        for (auto& it : items) total += (std::max<uint64_t>(it.bytes, 1) + 255) / 256 * 256;
-        unsigned char* base = nullptr;
-        FAST_TRY(c->arena.alloc_exact(&base, total, s));
-        uint64_t at = 0;
-        for (auto& it : items) {
-            unsigned char* dst = base + at;
-            at += (std::max<uint64_t>(it.bytes, 1) + 255) / 256 * 256;
-            if (it.bytes) {
-                cd.push_back({(const unsigned char*)*it.slot, dst, it.bytes, pieces});
-                pieces += (it.bytes + kPiece - 1) / kPiece;
+        return FAST_OK;
+    }
+    int read(const uint32_t* d, size_t at, size_t n, size_t event, cudaStream_t s) {
+        FAST_CUDA(cudaMemcpyAsync(h + at, d, n * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        FAST_CUDA(cudaEventRecord(ev[event], s));
+        return FAST_OK;
+    }
+    int wait(size_t event) {
+        t_round_trips++;
+        FAST_CUDA(cudaEventSynchronize(ev[event]));
+        return FAST_OK;
+    }
+};
+thread_local Readback t_readback;
+
+// One query edge whose lists are built.
+struct Edge {
+    int q, from, to;
+    int tree;                     // the tree edge into `to`
+    int e;                        // else: the non-tree edge's index
+    uint32_t n = 0;               // rows
+    int64_t tiles = 0;
+    uint32_t *e_off = nullptr, *beg = nullptr, *tile = nullptr;
+    int32_t* first = nullptr;
+};
+
+// The two passes over the lists of every edge of the batch, tree and
+// non-tree alike.  `slices`: ranges of E whose sizes are read back together.
+int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, const std::vector<size_t>& slices,
+                bool bounded, cudaStream_t s) {
+    const size_t ne = E.size();
+    const GraphSegs G = graph_segs(g);
+    uint32_t* Z = nullptr;                        // [0, ne) edge spaces, [ne, 2 ne) entries kept
+    Scratch tmp(s);
+    {
+        Carver cv;
+        cv.add(&Z, (int64_t)(2 * ne));
+        for (auto& x : E) {
+            cv.add(&x.e_off, (int64_t)x.n + 1);
+            cv.add(&x.beg, x.n);
+        }
+        FAST_TRY(cv.alloc(tmp, false));
+    }
+    auto bound_of = [&](const Edge& x) -> int64_t {
+        const fast_cst* c = Qs[x.q].c;
+        const int64_t L = g->num_labels;
+        const int32_t la = c->qlabel[x.from], lb = c->qlabel[x.to];
+        if (la >= L || lb >= L) return 0;
+        if (!g->lab_pair_host.empty()) return g->lab_pair_host[(size_t)la * L + lb];
+        return g->lab_degsum_host[la];
+    };
+    // The arrays of first rows are sized before the edge spaces are known; the
+    // tiles to run, by their real sizes unless the batch is small.
+    {
+        Carver cv;
+        for (auto& x : E) {
+            x.tiles = std::max<int64_t>(1, ceil_div(bound_of(x), (int64_t)kListTile));
+            cv.add(&x.first, x.tiles + 1);
+            cv.add(&x.tile, x.tiles);
+        }
+        FAST_TRY(cv.alloc(tmp, false));
+    }
+    auto desc_of = [&](size_t i, bool out) {
+        const Edge& x = E[i];
+        const Q& q = Qs[x.q];
+        ListDesc d{};
+        d.rows = q.rows[x.from];
+        d.n = x.n;
+        d.label = q.c->qlabel[x.to];
+        d.base = q.base[x.to];
+        d.packed = q.packed[x.to];
+        d.e_off = x.e_off; d.beg = x.beg; d.first = x.first; d.tile = x.tile;
+        d.E = Z + i;
+        d.K = Z + ne + i;
+        if (out) {
+            d.off = x.tree ? q.c->t_off[x.to] : q.c->n_off[x.e];
+            d.idx = x.tree ? q.c->t_idx[x.to] : q.c->n_idx[x.e];
+        }
+        return d;
+    };
+    const size_t ns = slices.size() - 1;
+    if (!bounded) FAST_TRY(t_readback.reserve(2 * ne, 2 * ns));
+    std::vector<uint32_t> kept;
+    // row lengths
+    {
+        Stage st;
+        std::vector<ListDesc> ld;
+        std::vector<int64_t> toff;
+        std::vector<size_t> t_at(ns), z_at(ns), d_at(ns);
+        for (size_t k = 0; k < ns; k++) {
+            ld.clear();
+            std::vector<int64_t> n;
+            for (size_t i = slices[k]; i < slices[k + 1]; i++) {
+                ld.push_back(desc_of(i, false));
+                n.push_back(E[i].n);
             }
-            *it.slot = dst;
+            toff = seg_tile_offsets(n, kScanTile);
+            d_at[k] = st.add(ld);
+            t_at[k] = st.add(toff);
+            z_at[k] = st.zeros((size_t)toff.back() + 1);
+        }
+        Scratch sc(s);
+        FAST_TRY(st.upload(sc));
+        for (size_t k = 0; k < ns; k++) {
+            const int nseg = (int)(slices[k + 1] - slices[k]);
+            const size_t tiles = (k + 1 < ns ? z_at[k + 1] : st.zeros(0)) - z_at[k] - 1;
+            const unsigned grid = (unsigned)std::min<int64_t>((int64_t)tiles, (int64_t)num_sms() * 4);
+            k_row_lens<<<grid, kScanBlock, 0, s>>>(st.at<ListDesc>(d_at[k]), G, st.at<int64_t>(t_at[k]), nseg,
+                                                   st.z(z_at[k]), (unsigned int*)st.z(z_at[k] + tiles));
+            FAST_TRY(note_launch("row lengths"));
+            if (!bounded) FAST_TRY(t_readback.read(Z + slices[k], slices[k], nseg, 2 * k, s));
         }
     }
-    if (cd.empty()) return FAST_OK;
-    Scratch sc(s);
-    const CopyDesc* dd = nullptr;
-    const int64_t* unused = nullptr;
-    FAST_TRY(upload(cd, std::vector<int64_t>(), sc, &dd, &unused));
-    const unsigned grid = (unsigned)std::min<uint64_t>(pieces, (uint64_t)num_sms() * 8);
-    k_copy_many<<<grid, 256, 0, s>>>(dd, (int)cd.size(), pieces);
-    note_launch();
-    if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "batched CST copy launch");
+    // count
+    for (size_t k = 0; k < ns; k++) {
+        const size_t e0 = slices[k], nseg = slices[k + 1] - e0;
+        if (!bounded) {
+            FAST_TRY(t_readback.wait(2 * k));
+            for (size_t i = e0; i < e0 + nseg; i++) {
+                const int64_t tiles = std::max<int64_t>(1, ceil_div((int64_t)t_readback.h[i], (int64_t)kListTile));
+                if (tiles > E[i].tiles) return set_error(FAST_ERR_CUDA, "CST build: an edge space exceeded its bound");
+                E[i].tiles = tiles;
+            }
+        }
+        std::vector<ListDesc> ld;
+        std::vector<int64_t> n;
+        for (size_t i = e0; i < e0 + nseg; i++) {
+            ld.push_back(desc_of(i, false));
+            n.push_back(E[i].tiles);
+        }
+        const std::vector<int64_t> items = prefix(n), toff = seg_tile_offsets(n, kScanTile);
+        Stage st;
+        const size_t d_at = st.add(ld), i_at = st.add(items), t_at = st.add(toff);
+        const size_t z_at = st.zeros((size_t)toff.back() + 1);
+        Scratch sc(s);
+        FAST_TRY(st.upload(sc));
+        k_lists<false><<<warp_grid(items.back(), 8), 256, 0, s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at), (int)nseg, g->col);
+        FAST_TRY(note_launch("list count"));
+        const unsigned grid = (unsigned)std::min<int64_t>(toff.back(), (int64_t)num_sms() * 4);
+        k_tile_bases<<<grid, kScanBlock, 0, s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at), st.at<int64_t>(t_at), (int)nseg,
+                                                 st.z(z_at), (unsigned int*)st.z(z_at + (size_t)toff.back()));
+        FAST_TRY(note_launch("list offsets"));
+        if (!bounded) FAST_TRY(t_readback.read(Z + ne + e0, ne + e0, nseg, 2 * k + 1, s));
+    }
+    if (bounded) FAST_TRY(fetch(Z + ne, kept, ne, s));
+    else {
+        for (size_t k = 0; k < ns; k++) FAST_TRY(t_readback.wait(2 * k + 1));
+        kept.assign(t_readback.h + ne, t_readback.h + 2 * ne);
+    }
+    // every size is known: the lists' final place, then the write
+    for (size_t i = 0; i < ne; i++) {
+        fast_cst* c = Qs[E[i].q].c;
+        (E[i].tree ? c->t_entries[E[i].to] : c->n_entries[E[i].e]) = kept[i];
+    }
+    for (auto& q : Qs) {
+        fast_cst* c = q.c;
+        Carver cv;
+        for (int u = 0; u < c->k; u++)
+            if (c->parent[u] >= 0) cv.add(&c->t_idx[u], c->t_entries[u]);
+        for (int e = 0; e < c->nnt; e++) cv.add(&c->n_idx[e], c->n_entries[e]);
+        unsigned char* b = nullptr;
+        FAST_TRY(c->arena.block(&b, cv.bytes(), s));
+        cv.place(b);
+    }
+    if (ne) {
+        std::vector<ListDesc> ld;
+        std::vector<int64_t> n;
+        for (size_t i = 0; i < ne; i++) {
+            ld.push_back(desc_of(i, true));
+            n.push_back(E[i].tiles);
+        }
+        const std::vector<int64_t> items = prefix(n);
+        Stage st;
+        const size_t d_at = st.add(ld), i_at = st.add(items);
+        Scratch sc(s);
+        FAST_TRY(st.upload(sc));
+        k_lists<true><<<warp_grid(items.back(), 8), 256, 0, s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at), (int)ne, g->col);
+        FAST_TRY(note_launch("list write"));
+    }
     return FAST_OK;
+}
+
+// c_u of every vertex, deepest first, and W (fields F_W, F_WF of Z).
+int build_workload(std::vector<Q>& Qs, int64_t* Z, int max_depth, Scratch& keep, cudaStream_t s) {
+    const int nq = (int)Qs.size();
+    struct Pair { int q, w; unsigned long long* ssum; double* sumf; uint32_t* ovf; };
+    std::vector<std::vector<Pair>> pairs(max_depth + 1);       // by the parent's depth: children that are not leaves
+    {
+        Carver cz, cv;
+        for (int qi = 0; qi < nq; qi++) {
+            Q& q = Qs[qi];
+            for (int w = 0; w < q.k; w++) {
+                const int u = q.c->parent[w];
+                if (u >= 0 && q.nch[w] > 0) pairs[q.depth[u]].push_back({qi, w, nullptr, nullptr, nullptr});
+                if (u < 0 || q.nch[w] > 0) cv.add(&q.cv[w], q.c->ncand[w]);
+            }
+        }
+        for (auto& v : pairs)
+            for (auto& p : v) {
+                const int64_t rows = Qs[p.q].c->ncand[Qs[p.q].c->parent[p.w]];
+                cz.add(&p.ssum, rows);
+                cz.add(&p.sumf, rows);
+                cz.add(&p.ovf, rows);
+            }
+        FAST_TRY(cv.alloc(keep, false));
+        FAST_TRY(cz.alloc(keep, true));
+    }
+    Stage st;
+    struct Wave { size_t s_at = 0, so_at = 0, p_at = 0, po_at = 0; int64_t tiles = 0, items = 0; int ns = 0, np = 0; };
+    std::vector<Wave> waves(max_depth + 1);
+    std::vector<ChildRef> refs;
+    std::vector<const Pair*> sums((size_t)nq * kMaxK, nullptr);
+    for (int d = max_depth; d >= 0; d--) {
+        Wave& wv = waves[d];
+        std::vector<ChildSumDesc> cd;
+        std::vector<int64_t> n;
+        for (auto& p : pairs[d]) {
+            const Q& q = Qs[p.q];
+            fast_cst* c = q.c;
+            cd.push_back({c->t_off[p.w], c->ncand[c->parent[p.w]], c->t_idx[p.w], q.cv[p.w], p.ssum, p.sumf, p.ovf});
+            n.push_back(ceil_div(c->t_entries[p.w], (int64_t)kWarpTileItems));
+            sums[(size_t)p.q * kMaxK + p.w] = &p;
+        }
+        std::vector<int64_t> off = prefix(n);
+        wv.ns = (int)cd.size();
+        wv.tiles = off.back();
+        wv.s_at = st.add(cd);
+        wv.so_at = st.add(off);
+        std::vector<ProdDesc> pd;
+        n.clear();
+        for (int qi = 0; qi < nq; qi++) {
+            const Q& q = Qs[qi];
+            fast_cst* c = q.c;
+            for (int u = 0; u < q.k; u++) {
+                if (q.depth[u] != d) continue;
+                ProdDesc x{(int32_t)refs.size(), 0, c->cval[u], q.cv[u]};
+                for (int w = 0; w < q.k; w++) {
+                    if (c->parent[w] != u) continue;
+                    x.nc++;
+                    if (q.nch[w] == 0) refs.push_back({c->t_off[w], nullptr, nullptr, nullptr, c->ssum[w]});
+                    else {
+                        const Pair* p = sums[(size_t)qi * kMaxK + w];
+                        refs.push_back({nullptr, p->ssum, p->sumf, p->ovf, c->ssum[w]});
+                    }
+                }
+                pd.push_back(x);
+                n.push_back(c->ncand[u]);
+            }
+        }
+        off = prefix(n);
+        wv.np = (int)pd.size();
+        wv.items = off.back();
+        wv.p_at = st.add(pd);
+        wv.po_at = st.add(off);
+    }
+    std::vector<TotalDesc> td;
+    for (int qi = 0; qi < nq; qi++) {
+        const Q& q = Qs[qi];
+        td.push_back({q.cv[q.c->root], q.c->ncand[q.c->root], (uint64_t*)(Z + (int64_t)F_W * nq + qi),
+                      (double*)(Z + (int64_t)F_WF * nq + qi)});
+    }
+    const size_t r_at = st.add(refs), t_at = st.add(td);
+    FAST_TRY(st.upload(keep));
+    for (int d = max_depth; d >= 0; d--) {
+        const Wave& wv = waves[d];
+        if (wv.tiles > 0) {
+            k_child_sums<<<warp_grid(wv.tiles, 8), 256, 0, s>>>(st.at<ChildSumDesc>(wv.s_at), st.at<int64_t>(wv.so_at), wv.ns);
+            FAST_TRY(note_launch("child sums"));
+        }
+        if (wv.items > 0) {
+            k_workload_prod<<<warp_grid(ceil_div(wv.items, 32), 8), 256, 0, s>>>(st.at<ProdDesc>(wv.p_at), st.at<int64_t>(wv.po_at),
+                                                                              wv.np, st.at<ChildRef>(r_at));
+            FAST_TRY(note_launch("workload"));
+        }
+    }
+    k_total_w<<<(unsigned)nq, 1024, 0, s>>>(st.at<TotalDesc>(t_at));
+    return note_launch("W");
 }
 
 // Builds every CST of Qs (all valid queries) on stream s.
 int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
     const int nq = (int)Qs.size();
-    const int64_t n = g->n;
-    const int64_t nw = n / 32 + 1;
-    const GraphRuns G = graph_runs(g);
-    int K = 0;
-    for (auto& q : Qs) K = std::max(K, q.k);
-    Scratch keep(s);                       // until the exact copies are made
-    Scratch td(s);                         // top-down lists: until the bottom-up is done
+    const GraphSegs G = graph_segs(g);
+    Scratch keep(s);
     std::vector<int64_t> h;
 
     int64_t* Z = nullptr;
@@ -642,7 +1043,7 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
         cv.add(&Z, (int64_t)F_END * nq);
         FAST_TRY(cv.alloc(keep, true));
     }
-    auto zp = [&](int f, int qi) { return Z + (int64_t)f * nq + qi; };
+    auto zp = [&](int f, int qi) { return (unsigned long long*)(Z + (int64_t)f * nq + qi); };
 
     // ------------------------------------------------------------ filter
     //
@@ -655,20 +1056,22 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
         std::vector<std::pair<int, int>> rep;             // fd[i]'s (query, vertex)
         std::map<std::vector<int64_t>, int> seen;
         Carver cv;
-        int64_t maxb = 1;
+        int64_t maxw = 1;
         for (int qi = 0; qi < nq; qi++) {
             Q& q = Qs[qi];
             for (int u = 0; u < q.k; u++) {
                 const int32_t l = q.c->qlabel[u];
                 if (l < g->num_labels) { q.lo[u] = g->lab_ptr_host[l]; q.hi[u] = g->lab_ptr_host[l + 1]; }
-                else { q.lo[u] = q.hi[u] = 0; }
+                q.base[u] = (int32_t)(q.lo[u] & ~31ll);
+                q.words[u] = (int32_t)ceil_div(q.hi[u] - q.base[u], 32);
                 FilterDesc d;
                 memset(&d, 0, sizeof(d));
                 d.lo = q.lo[u];
                 d.hi = q.hi[u];
+                d.base = q.base[u];
+                d.words = q.words[u];
                 d.dq = q.dq[u];
-                d.nlf = q.nlf ? 1 : 0;
-                std::vector<int64_t> key{d.lo, d.hi, d.dq, d.nlf};
+                std::vector<int64_t> key{d.lo, d.hi, d.dq};
                 if (q.nlf) {
                     for (int w = 0; w < q.k; w++) {
                         if (!q.A[u][w]) continue;
@@ -694,599 +1097,246 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
                 seen.emplace(std::move(key), (int)fd.size());
                 rep.push_back({qi, u});
                 fd.push_back(d);
-                maxb = std::max<int64_t>(maxb, q.hi[u] - q.lo[u]);
-                if (q.nlf) cv.add(&q.nlfb[u], nw);
+                maxw = std::max<int64_t>(maxw, q.words[u]);
+                cv.add(&q.pass[u], q.words[u]);
             }
         }
-        FAST_TRY(cv.alloc(keep, true));
+        FAST_TRY(cv.alloc(keep, false));
         for (size_t i = 0; i < fd.size(); i++) {
-            const Q& q = Qs[rep[i].first];
-            if (q.nlf) fd[i].bits = q.nlfb[rep[i].second];
-            fd[i].cnt = (unsigned long long*)zp(F_CNT + rep[i].second, rep[i].first);
+            fd[i].bits = Qs[rep[i].first].pass[rep[i].second];
+            fd[i].cnt = zp(F_CNT + rep[i].second, rep[i].first);
         }
         for (int qi = 0; qi < nq; qi++)
             for (int u = 0; u < Qs[qi].k; u++) {
                 const auto a = alias[(size_t)u * nq + qi];
-                if (a.first >= 0 && Qs[qi].nlf) Qs[qi].nlfb[u] = Qs[a.first].nlfb[a.second];
+                if (a.first >= 0) Qs[qi].pass[u] = Qs[a.first].pass[a.second];
             }
+        Stage st;
+        const size_t d_at = st.add(fd);
         Scratch sc(s);
-        const FilterDesc* dd = nullptr;
-        const int64_t* unused = nullptr;
-        FAST_TRY(upload(fd, std::vector<int64_t>(), sc, &dd, &unused));
+        FAST_TRY(st.upload(sc));
         const int64_t np = (int64_t)fd.size();
-        const int64_t x = std::max<int64_t>(1, std::min<int64_t>({ceil_div(maxb, 256), (int64_t)1024,
-                                                                  ceil_div((int64_t)num_sms() * 32, np)}));
-        k_filter_b<<<dim3((unsigned)x, (unsigned)np), 256, 0, s>>>(dd, g->lab_vtx, g->key, G, g->col, g->label);
-        note_launch();
-        if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "batched filter launch");
+        const int64_t x = std::max<int64_t>(1, std::min<int64_t>({ceil_div(maxw, 8), (int64_t)1024,
+                                                                  ceil_div((int64_t)num_sms() * 64, np)}));
+        k_filter<<<dim3((unsigned)x, (unsigned)np), 256, 0, s>>>(st.at<FilterDesc>(d_at), G);
+        FAST_TRY(note_launch("filter"));
     }
-    FAST_TRY(fetch(zp(F_CNT, 0), h, (size_t)kMaxK * nq, s));
-    for (int qi = 0; qi < nq; qi++)
-        for (int u = 0; u < Qs[qi].k; u++) {
-            const auto a = alias[(size_t)u * nq + qi];
-            if (a.first >= 0) h[(size_t)u * nq + qi] = h[(size_t)a.second * nq + a.first];
-        }
+    FAST_TRY(fetch(Z, h, (size_t)kMaxK * nq, s));
 
     // ------------------------------------------------- root and t_q
+    int max_depth = 0;
     for (int qi = 0; qi < nq; qi++) {
         Q& q = Qs[qi];
         fast_cst* c = q.c;
-        const int k = q.k;
-        for (int u = 0; u < k; u++) q.c0[u] = h[(size_t)u * nq + qi];
-        const int r = choose_root(k, q.c0, q.dq);
-        c->root = r;
-        bfs_tree(k, q.A, r, c->bfs, c->parent);
-        for (int t = 0; t < k; t++) q.bpos[c->bfs[t]] = t;
-    }
-
-    // ------------------------------------------------ C(root) = C0(root)
-    {
-        Carver cv;
-        for (auto& q : Qs) cv.add(&q.td_cand[q.c->root], q.c0[q.c->root]);
-        FAST_TRY(cv.alloc(td, false));
-        std::vector<CompactSeg<FilterF>> cs;
-        for (int qi = 0; qi < nq; qi++) {
-            const Q& q = Qs[qi];
-            const int r = q.c->root;
-            FilterF f{g->lab_vtx + q.lo[r], g->key, q.dq[r], q.nlf ? q.nlfb[r] : nullptr};
-            cs.push_back({f, q.hi[r] - q.lo[r], q.td_cand[r], zp(F_TD + 0, qi)});
+        int64_t c0[kMaxK];
+        for (int u = 0; u < q.k; u++) {
+            const auto a = alias[(size_t)u * nq + qi];
+            c0[u] = a.first >= 0 ? h[(size_t)a.second * nq + a.first] : h[(size_t)u * nq + qi];
         }
-        FAST_TRY(compact_seg(cs, s));
-    }
-
-    // ----------------------------------------------------- top-down
-    //
-    // A small batch enqueues the whole pass with no host round trip: each
-    // level's arrays are sized by bounds the host knows -- the rows by
-    // |C0(parent)|, the edge space by the graph's count of adjacency entries
-    // from label l(parent) to label l(u) -- and the kernels read the real
-    // sizes on the device (rows from the previous level's count, the edge
-    // space's end from its offsets).  Otherwise, or when the bounds would
-    // take too much memory, each level fetches its exact sizes first.
-    bool bounded = false;
-    if (!g->lab_pair_host.empty() && nq <= kBoundedQueries) {
-        const int L = g->num_labels;
-        uint64_t bytes = 0;
-        for (auto& q : Qs)
-            for (int t = 1; t < q.k; t++) {
-                const int u = q.c->bfs[t], p = q.c->parent[u];
-                const int32_t lp = q.c->qlabel[p], lu = q.c->qlabel[u];
-                const int64_t e = (lp < L && lu < L) ? g->lab_pair_host[(size_t)lp * L + lu] : 0;
-                bytes += 4ull * (uint64_t)e + 24ull * (uint64_t)(q.c0[p] + 1);
-            }
-        bounded = bytes <= kBoundedBytes;
-    }
-    auto rows_of = [&](const Q& q, int p) { return bounded ? q.c0[p] : q.ctd[p]; };
-    std::vector<unsigned char*> alive_blk(kMaxK, nullptr);
-    std::vector<size_t> alive_bytes(kMaxK, 0);
-    std::vector<int> act;
-    for (int t = 1; t < K; t++) {
-        act.clear();
-        for (int qi = 0; qi < nq; qi++) if (Qs[qi].k > t) act.push_back(qi);
-        if (!bounded) {
-            FAST_TRY(fetch(zp(F_TD + t - 1, 0), h, (size_t)nq, s));
-            for (int qi = 0; qi < nq; qi++)
-                if (Qs[qi].k > t - 1) Qs[qi].ctd[Qs[qi].c->bfs[t - 1]] = h[qi];
-        }
-        Scratch lvl(s);
-        {
-            Carver cv;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int64_t rows = rows_of(q, q.c->parent[q.c->bfs[t]]);
-                cv.add(&q.e_off, rows + 1);
-                cv.add(&q.seg, rows);
-            }
-            FAST_TRY(cv.alloc(lvl, false));
-        }
-        std::vector<int64_t> ni;
-        {
-            std::vector<CandSegDesc> cd;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t], p = q.c->parent[u];
-                const int64_t rows = rows_of(q, p);
-                cd.push_back({q.td_cand[p], rows, bounded ? zp(F_TD + q.bpos[p], qi) : nullptr, q.c->qlabel[u], q.seg,
-                              q.e_off});
-                ni.push_back(rows + 1);
-            }
-            FAST_TRY(run_items(k_cand_segment_b, cd, ni, s, G));
-            std::vector<ScanSeg<int64_t>> sc;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int64_t rows = rows_of(q, q.c->parent[q.c->bfs[t]]);
-                sc.push_back({q.e_off, nullptr, q.e_off, rows + 1, zp(F_E + t, qi)});
-            }
-            FAST_TRY(scan_seg(sc, s));
-        }
-        if (!bounded) FAST_TRY(fetch(zp(F_E + t, 0), h, (size_t)nq, s));
-        {
-            Carver cl, cb;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t], p = q.c->parent[u];
-                const int64_t rows = rows_of(q, p);
-                const int L = g->num_labels;
-                const int32_t lp = q.c->qlabel[p], lu = q.c->qlabel[u];
-                q.E[u] = !bounded ? h[qi] : (lp < L && lu < L) ? g->lab_pair_host[(size_t)lp * L + lu] : 0;
-                cl.add(&q.td_list[u], q.E[u]);
-                cl.add(&q.td_off[u], rows + 1);
-                cb.add(&q.alive[u], nw);
-            }
-            FAST_TRY(cl.alloc(td, false));
-            FAST_TRY(cb.alloc(keep, true, &alive_blk[t], &alive_bytes[t]));
-        }
-        {
-            std::vector<CompactSeg<TopDownF>> cs;
-            std::vector<FillTailDesc> ft;
-            ni.clear();
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t];
-                const int64_t rows = rows_of(q, q.c->parent[u]);
-                TopDownF f{};
-                f.e_off = q.e_off; f.rows = rows; f.seg = q.seg; f.col = g->col; f.key = g->key;
-                f.want_key_hi = q.c->qlabel[u]; f.want_dq = q.dq[u]; f.reached = q.alive[u]; f.t_off = q.td_off[u];
-                f.label_known = G.run_ptr != nullptr;
-                f.pass = q.nlf ? q.nlfb[u] : nullptr;
-                f.E = q.e_off + rows;
-                cs.push_back({f, q.E[u], q.td_list[u], zp(F_KEPT + t, qi)});
-                ft.push_back({q.e_off, rows, zp(F_KEPT + t, qi), q.td_off[u]});
-                ni.push_back(rows + 1);
-            }
-            FAST_TRY(compact_seg(cs, s));
-            FAST_TRY(run_items(k_fill_tail_b, ft, ni, s));
-        }
-        {
-            Carver cv;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t];
-                cv.add(&q.td_cand[u], q.c0[u]);      // C_td(u) lies inside C0(u)
-            }
-            FAST_TRY(cv.alloc(td, false));
-            std::vector<BitsSeg> bs;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t];
-                bs.push_back({q.alive[u], n, q.td_cand[u], zp(F_TD + t, qi)});
-            }
-            FAST_TRY(bits_ids_seg(bs, s));
-        }
-    }
-    // |C_td|, edge spaces and kept entries of every position
-    FAST_TRY(fetch(zp(F_TD, 0), h, (size_t)3 * kMaxK * nq, s));
-    for (int qi = 0; qi < nq; qi++) {
-        Q& q = Qs[qi];
-        for (int t = 0; t < q.k; t++) {
-            const int u = q.c->bfs[t];
-            q.ctd[u] = h[(size_t)t * nq + qi];
-            q.kept[u] = h[(size_t)(2 * kMaxK + t) * nq + qi];
-            // a bounded pass read at most its bound of each edge space (the
-            // compaction stops there); more would mean a wrong bound
-            if (bounded && t > 0 && h[(size_t)(kMaxK + t) * nq + qi] > q.E[u])
-                return set_error(FAST_ERR_CUDA, "batched CST build: an edge space exceeded its label-pair bound");
-        }
-    }
-
-    // refine rule 2 tests against C_td(root) until the root's own step: its
-    // bitmap (the other vertices' top-down bitmaps already exist)
-    {
-        Carver cv;
-        std::vector<SetBitsDesc> sb;
-        std::vector<int64_t> ni;
-        for (auto& q : Qs)
-            if (q.nt_refine) cv.add(&q.root_bits, nw);
-        FAST_TRY(cv.alloc(keep, true));
-        for (int qi = 0; qi < nq; qi++) {
-            Q& q = Qs[qi];
-            if (!q.nt_refine) continue;
-            const int r = q.c->root;
-            sb.push_back({q.td_cand[r], zp(F_TD + 0, qi), q.root_bits});
-            ni.push_back(q.ctd[r]);
-        }
-        FAST_TRY(run_items(k_set_bits_b, sb, ni, s));
-    }
-
-    // ---------------------------------------------------- bottom-up
-    for (int t = K - 1; t >= 0; t--) {
-        act.clear();
-        for (int qi = 0; qi < nq; qi++) if (Qs[qi].k > t) act.push_back(qi);
-        Scratch lvl(s);
-        // (query, child) pairs, grouped by query in act order
-        std::vector<int> pa, pw, pbeg(act.size() + 1, 0);
-        for (size_t a = 0; a < act.size(); a++) {
-            const Q& q = Qs[act[a]];
-            const int u = q.c->bfs[t];
-            for (int w = 0; w < q.k; w++)
-                if (q.c->parent[w] == u) { pa.push_back((int)a); pw.push_back(w); }
-            pbeg[a + 1] = (int)pa.size();
-        }
-        const size_t npr = pa.size();
-        std::vector<uint8_t*> has(npr, nullptr);
-        std::vector<uint8_t*> valid(act.size(), nullptr);
-        std::vector<int64_t*> newrow(act.size(), nullptr);
-        {
-            Carver ch, cv;
-            for (size_t j = 0; j < npr; j++) {
-                const Q& q = Qs[act[pa[j]]];
-                ch.add(&has[j], q.ctd[q.c->bfs[t]]);
-            }
-            for (size_t a = 0; a < act.size(); a++) {
-                const Q& q = Qs[act[a]];
-                const int64_t rows = q.ctd[q.c->bfs[t]];
-                cv.add(&valid[a], rows);
-                cv.add(&newrow[a], rows + 1);
-            }
-            FAST_TRY(ch.alloc(lvl, true));
-            FAST_TRY(cv.alloc(lvl, false));
-        }
-        {
-            std::vector<AnyAliveDesc> aa;
-            std::vector<int64_t> ent;
-            for (size_t j = 0; j < npr; j++) {
-                const Q& q = Qs[act[pa[j]]];
-                const int w = pw[j];
-                aa.push_back({q.td_off[w], q.ctd[q.c->bfs[t]], q.td_list[w], q.alive[w], has[j]});
-                ent.push_back(q.kept[w]);
-            }
-            FAST_TRY(run_tiles(k_any_alive_b, aa, ent, kTileItems, 1, s));
-        }
-        // refine rule 2: per (query, non-tree neighbour w of u), which rows
-        // have a neighbour in C(w) as it stands now
-        std::vector<int> na, nwv, nbeg(act.size() + 1, 0);
-        for (size_t a = 0; a < act.size(); a++) {
-            const Q& q = Qs[act[a]];
-            const int u = q.c->bfs[t];
-            if (q.nt_refine)
-                for (int w = 0; w < q.k; w++)
-                    if (q.A[u][w] && q.c->parent[w] != u && q.c->parent[u] != w) { na.push_back((int)a); nwv.push_back(w); }
-            nbeg[a + 1] = (int)na.size();
-        }
-        std::vector<uint8_t*> ntf(na.size(), nullptr);
-        if (!na.empty()) {
-            Carver cf;
-            for (size_t j = 0; j < na.size(); j++) {
-                const Q& q = Qs[act[na[j]]];
-                cf.add(&ntf[j], q.ctd[q.c->bfs[t]]);
-            }
-            FAST_TRY(cf.alloc(lvl, true));
-            std::vector<NtDesc> nd;
-            std::vector<int64_t> ni;
-            for (size_t j = 0; j < na.size(); j++) {
-                const Q& q = Qs[act[na[j]]];
-                const int u = q.c->bfs[t], w = nwv[j];
-                // later in the BFS order: already refined; earlier: its
-                // top-down set (the root's own bitmap; the others' reached
-                // bitmaps are not rewritten before their step)
-                const uint32_t* bits = (w == q.c->root && q.bpos[w] < t) ? q.root_bits : q.alive[w];
-                nd.push_back({q.td_cand[u], q.c->qlabel[w], bits, ntf[j]});
-                ni.push_back(q.ctd[u]);
-            }
-            if (!nd.empty()) {
-                const std::vector<int64_t> off = prefix(ni);
-                if (off.back() > 0) {
-                    Scratch sc(s);
-                    const NtDesc* dd = nullptr;
-                    const int64_t* doff = nullptr;
-                    FAST_TRY(upload(nd, off, sc, &dd, &doff));
-                    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(ceil_div(off.back(), 8),
-                                                                                  (int64_t)num_sms() * 16));
-                    k_nt_support_b<<<(unsigned)blocks, 256, 0, s>>>(dd, doff, (int)nd.size(), G, g->col);
-                    note_launch();
-                    if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "batched non-tree test launch");
-                }
-            }
-        }
-        {
-            std::vector<ValidDesc> vd;
-            std::vector<int64_t> ni;
-            std::vector<ScanSeg<int64_t>> sc;
-            for (size_t a = 0; a < act.size(); a++) {
-                const Q& q = Qs[act[a]];
-                const int64_t rows = q.ctd[q.c->bfs[t]];
-                ValidDesc d;
-                memset(&d, 0, sizeof(d));
-                for (int j = pbeg[a]; j < pbeg[a + 1]; j++) d.cf.has[d.cf.nch++] = has[j];
-                for (int j = nbeg[a]; j < nbeg[a + 1]; j++) d.cf.has[d.cf.nch++] = ntf[j];
-                d.valid = valid[a];
-                d.vflag = newrow[a];
-                vd.push_back(d);
-                ni.push_back(rows);
-                sc.push_back({newrow[a], nullptr, newrow[a], rows, newrow[a] + rows});
-            }
-            FAST_TRY(run_items(k_valid_rows_b, vd, ni, s));
-            FAST_TRY(scan_seg(sc, s));
-        }
-        {
-            Carver cv;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t];
-                cv.add(&q.c->cand[u], q.ctd[u]);
-            }
-            for (size_t j = 0; j < npr; j++) {
-                Q& q = Qs[act[pa[j]]];
-                const int w = pw[j];
-                cv.add(&q.c->t_off[w], q.ctd[q.c->bfs[t]] + 1);
-                cv.add(&q.c->t_idx[w], q.kept[w]);
-            }
-            FAST_TRY(cv.alloc(keep, false));
-            std::vector<CompactSeg<KeepRowsF>> kr;
-            for (size_t a = 0; a < act.size(); a++) {
-                const int qi = act[a];
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t];
-                kr.push_back({KeepRowsF{q.td_cand[u], valid[a], zp(F_TD + t, qi)}, q.ctd[u], q.c->cand[u], zp(F_C + t, qi)});
-            }
-            FAST_TRY(compact_seg(kr, s));
-            std::vector<CompactSeg<WriteAliveF>> wa;
-            std::vector<SetTailDesc> st;
-            for (size_t j = 0; j < npr; j++) {
-                const int a = pa[j], qi = act[a];
-                Q& q = Qs[qi];
-                const int w = pw[j];
-                WriteAliveF f{};
-                f.off = q.td_off[w]; f.nrows = zp(F_TD + t, qi); f.list = q.td_list[w];
-                f.alive = q.alive[w]; f.rank = q.rank[w]; f.packed = q.packed[w];
-                f.valid = valid[a]; f.newrow = newrow[a]; f.new_off = q.c->t_off[w];
-                wa.push_back({f, q.kept[w], q.c->t_idx[w], zp(F_T + q.bpos[w], qi)});
-                st.push_back({q.c->t_off[w], zp(F_C + t, qi), zp(F_T + q.bpos[w], qi)});
-            }
-            FAST_TRY(compact_seg(wa, s));
-            if (!st.empty()) {
-                Scratch sc(s);
-                const SetTailDesc* dd = nullptr;
-                const int64_t* unused = nullptr;
-                FAST_TRY(upload(st, std::vector<int64_t>(), sc, &dd, &unused));
-                k_set_tail_b<<<(unsigned)ceil_div((int64_t)st.size(), 256), 256, 0, s>>>(dd, (int)st.size());
-                note_launch();
-                if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "batched set-tail launch");
-            }
-        }
-        // bitmap and rank of the refined C(u)
-        if (t == 0) {
-            Carver cv;
-            for (int qi : act) cv.add(&Qs[qi].alive[Qs[qi].c->root], nw);
-            FAST_TRY(cv.alloc(keep, true));
-        } else {
-            FAST_CUDA(cudaMemsetAsync(alive_blk[t], 0, alive_bytes[t], s));
-        }
-        {
-            std::vector<SetBitsDesc> sb;
-            std::vector<int64_t> ni;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t];
-                sb.push_back({q.c->cand[u], zp(F_C + t, qi), q.alive[u]});
-                ni.push_back(q.ctd[u]);
-            }
-            FAST_TRY(run_items(k_set_bits_b, sb, ni, s));
-            Carver cv;
-            for (int qi : act) cv.add(&Qs[qi].rank[Qs[qi].c->bfs[t]], nw);
-            FAST_TRY(cv.alloc(keep, false));
-            std::vector<ScanSeg<uint32_t>> rk;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t];
-                rk.push_back({nullptr, q.alive[u], q.rank[u], nw, nullptr});
-            }
-            FAST_TRY(scan_seg(rk, s));
-            Carver cp;
-            for (int qi : act) cp.add(&Qs[qi].packed[Qs[qi].c->bfs[t]], nw);
-            FAST_TRY(cp.alloc(keep, false));
-            std::vector<PackDesc> pd;
-            std::vector<int64_t> pn;
-            for (int qi : act) {
-                Q& q = Qs[qi];
-                const int u = q.c->bfs[t];
-                pd.push_back({q.alive[u], q.rank[u], q.packed[u]});
-                pn.push_back(nw);
-            }
-            FAST_TRY(run_items(k_pack_bits_b, pd, pn, s));
-        }
-    }
-    td.release();                          // top-down lists and sets: done
-    // refined candidate counts decide the matching order
-    FAST_TRY(fetch(zp(F_C, 0), h, (size_t)2 * kMaxK * nq, s));
-    for (int qi = 0; qi < nq; qi++) {
-        Q& q = Qs[qi];
-        fast_cst* c = q.c;
+        c->root = choose_root(q.k, c0, q.dq);
+        bfs_tree(q.k, q.A, c->root, c->bfs, c->parent);
         for (int t = 0; t < q.k; t++) {
             const int u = c->bfs[t];
-            c->ncand[u] = h[(size_t)t * nq + qi];
-            c->t_entries[u] = c->parent[u] < 0 ? 0 : h[(size_t)(kMaxK + t) * nq + qi];
+            q.bpos[u] = t;
+            q.depth[u] = t ? q.depth[c->parent[u]] + 1 : 0;
+            if (t) q.nch[c->parent[u]]++;
+            max_depth = std::max(max_depth, q.depth[u]);
         }
+        // C_td(root) = C0(root); the size of a shared bitmap is its owner's
+        const int r = c->root;
+        q.cur[r] = q.pass[r];
+        c->ncand[r] = c0[r];
+    }
+
+    // ----------------------------------------- top-down and bottom-up
+    {
+        struct Wave { std::vector<SetDesc> d; size_t d_at = 0, i_at = 0; int group = 1; int64_t items = 0; };
+        std::vector<Wave> waves;
+        std::vector<Target> tg;
+        Carver cv;
+        for (auto& q : Qs)
+            for (int u = 0; u < q.k; u++) cv.add(&q.set[u], q.words[u]);
+        FAST_TRY(cv.alloc(keep, false));
+        auto count_of = [&](int qi, int u) {
+            const Q& q = Qs[qi];
+            if (q.cur[u] != q.pass[u]) return zp(q.cnt[u], qi);
+            const auto a = alias[(size_t)u * nq + qi];                  // the root's C0
+            return a.first >= 0 ? zp(F_CNT + a.second, a.first) : zp(F_CNT + u, qi);
+        };
+        auto target = [&](int qi, int w) {
+            const Q& q = Qs[qi];
+            tg.push_back({q.cur[w], count_of(qi, w), q.base[w], q.c->qlabel[w]});
+        };
+        for (int d = 1; d <= max_depth; d++) {
+            Wave wv;
+            for (int qi = 0; qi < nq; qi++) {
+                Q& q = Qs[qi];
+                for (int t = 1; t < q.k; t++) {
+                    const int u = q.c->bfs[t];
+                    if (q.depth[u] != d) continue;
+                    wv.d.push_back({q.pass[u], q.set[u], zp(F_TD + u, qi), q.base[u], q.words[u], (int32_t)tg.size(), 1});
+                    target(qi, q.c->parent[u]);
+                    q.cur[u] = q.set[u];
+                    q.cnt[u] = F_TD + u;
+                }
+            }
+            waves.push_back(std::move(wv));
+        }
+        int steps = max_depth + 1;                           // bottom-up: by depth, or (rule 2) by position
+        for (auto& q : Qs) if (q.nt_refine) steps = std::max(steps, q.k);
+        for (int b = 0; b < steps; b++) {
+            Wave wv;
+            for (int qi = 0; qi < nq; qi++) {
+                Q& q = Qs[qi];
+                for (int t = q.k - 1; t >= 0; t--) {
+                    const int u = q.c->bfs[t];
+                    if (q.nt_refine ? t != q.k - 1 - b : q.depth[u] != max_depth - b) continue;
+                    const int32_t t0 = (int32_t)tg.size();
+                    for (int w = 0; w < q.k; w++)
+                        if (q.c->parent[w] == u || (q.nt_refine && q.A[u][w] && q.c->parent[u] != w)) target(qi, w);
+                    const int32_t nt = (int32_t)tg.size() - t0;
+                    if (!nt) continue;                       // a leaf: its set is final
+                    wv.d.push_back({q.cur[u], q.set[u], zp(F_C + u, qi), q.base[u], q.words[u], t0, nt});
+                    q.cur[u] = q.set[u];
+                    q.cnt[u] = F_C + u;
+                }
+            }
+            if (!wv.d.empty()) waves.push_back(std::move(wv));
+        }
+        Stage st;
+        for (auto& wv : waves) {
+            // one word per warp while that leaves warps idle, then up to four
+            int64_t words = 0;
+            for (auto& d : wv.d) words += d.words;
+            wv.group = (int)std::max<int64_t>(1, std::min<int64_t>(4, words / ((int64_t)num_sms() * 64)));
+            std::vector<int64_t> n;
+            for (auto& d : wv.d) n.push_back(ceil_div(d.words, wv.group));
+            const std::vector<int64_t> off = prefix(n);
+            wv.items = off.back();
+            wv.d_at = st.add(wv.d);
+            wv.i_at = st.add(off);
+        }
+        const size_t t_at = st.add(tg), z_at = st.zeros(waves.size() + 1);
+        LongRow* longs = nullptr;
+        const bool hubs = g->max_degree > (int64_t)kLongRow;
+        Scratch sc(s);
+        if (hubs) {
+            Carver cl;
+            cl.add(&longs, kLongRows);
+            FAST_TRY(cl.alloc(sc, false));
+        }
+        FAST_TRY(st.upload(sc));
+        for (size_t i = 0; i < waves.size(); i++) {
+            const Wave& wv = waves[i];
+            if (wv.items == 0) continue;
+            unsigned int* nl = (unsigned int*)st.z(z_at + i);
+            k_support<<<warp_grid(wv.items, 8), 256, 0, s>>>(st.at<SetDesc>(wv.d_at), st.at<int64_t>(wv.i_at), (int)wv.d.size(),
+                                                             wv.group, st.at<Target>(t_at), G, g->col, longs, nl);
+            FAST_TRY(note_launch("support"));
+            if (hubs) {
+                k_support_long<<<(unsigned)num_sms() * 2, 256, 0, s>>>(st.at<SetDesc>(wv.d_at), st.at<Target>(t_at), G, g->col,
+                                                                       longs, nl);
+                FAST_TRY(note_launch("support of long rows"));
+            }
+        }
+    }
+    FAST_TRY(fetch(Z, h, (size_t)(F_C + kMaxK) * nq, s));
+    for (int qi = 0; qi < nq; qi++) {
+        Q& q = Qs[qi];
+        fast_cst* c = q.c;
+        for (int u = 0; u < q.k; u++)
+            if (q.cur[u] != q.pass[u]) c->ncand[u] = h[(size_t)q.cnt[u] * nq + qi];
         order_and_nontree(q, c);
     }
 
-    // ------------------------------------------------------ non-tree
-    std::vector<int> ntq, nte;                       // (query, edge) pairs
-    for (int qi = 0; qi < nq; qi++)
-        for (int e = 0; e < Qs[qi].c->nnt; e++) { ntq.push_back(qi); nte.push_back(e); }
-    const size_t nnp = ntq.size();
-    int64_t* NZ = nullptr;                           // [0, nnp) edge spaces, [nnp, 2 nnp) kept entries
-    if (nnp) {
-        Carver cz;
-        cz.add(&NZ, (int64_t)(2 * nnp));
-        FAST_TRY(cz.alloc(keep, true));
-        Scratch lvl(s);
-        std::vector<int64_t*> eo(nnp, nullptr), sg(nnp, nullptr);
-        std::vector<int64_t> rows(nnp);
-        {
+    // ------------------------------ ids and ranks; arrays by set size
+    {
+        for (auto& q : Qs) {
+            fast_cst* c = q.c;
             Carver cv;
-            for (size_t j = 0; j < nnp; j++) {
-                const fast_cst* c = Qs[ntq[j]].c;
-                rows[j] = c->ncand[c->nt_from[nte[j]]];
-                cv.add(&eo[j], rows[j] + 1);
-                cv.add(&sg[j], rows[j]);
+            for (int u = 0; u < q.k; u++) {
+                cv.add(&c->cand[u], c->ncand[u]);
+                cv.add(&c->cval[u], c->ncand[u]);
+                if (c->parent[u] < 0) continue;
+                cv.add(&c->t_off[u], c->ncand[c->parent[u]] + 1);
+                cv.add(&c->ssum[u], c->ncand[c->parent[u]]);
             }
-            FAST_TRY(cv.alloc(lvl, false));
+            for (int e = 0; e < c->nnt; e++) cv.add(&c->n_off[e], c->ncand[c->nt_from[e]] + 1);
+            unsigned char* b = nullptr;
+            FAST_TRY(c->arena.block(&b, cv.bytes(), s));
+            cv.place(b);
         }
-        {
-            std::vector<CandSegDesc> cd;
-            std::vector<int64_t> ni;
-            std::vector<ScanSeg<int64_t>> sc;
-            for (size_t j = 0; j < nnp; j++) {
-                const fast_cst* c = Qs[ntq[j]].c;
-                const int e = nte[j];
-                cd.push_back({c->cand[c->nt_from[e]], rows[j], nullptr, c->qlabel[c->nt_to[e]], sg[j], eo[j]});
-                ni.push_back(rows[j] + 1);
-                sc.push_back({eo[j], nullptr, eo[j], rows[j] + 1, NZ + j});
+        Carver cv;
+        for (auto& q : Qs)
+            for (int u = 0; u < q.k; u++) {
+                cv.add(&q.packed[u], q.words[u]);
+                cv.add(&q.rows[u], q.c->ncand[u]);
             }
-            FAST_TRY(run_items(k_cand_segment_b, cd, ni, s, G));
-            FAST_TRY(scan_seg(sc, s));
-        }
-        FAST_TRY(fetch(NZ, h, nnp, s));
-        {
-            Carver cv;
-            for (size_t j = 0; j < nnp; j++) {
-                fast_cst* c = Qs[ntq[j]].c;
-                const int e = nte[j];
-                cv.add(&c->n_off[e], rows[j] + 1);
-                cv.add(&c->n_idx[e], h[j]);
+        FAST_TRY(cv.alloc(keep, false));
+        std::vector<IdsDesc> id;
+        std::vector<int64_t> n;
+        for (auto& q : Qs)
+            for (int u = 0; u < q.k; u++) {
+                id.push_back({q.cur[u], q.packed[u], q.rows[u], q.c->cand[u], q.base[u], q.words[u]});
+                n.push_back(q.words[u]);
             }
-            FAST_TRY(cv.alloc(keep, false));
-            std::vector<CompactSeg<NonTreeF>> cs;
-            std::vector<FillTailDesc> ft;
-            std::vector<int64_t> ni;
-            for (size_t j = 0; j < nnp; j++) {
-                const Q& q = Qs[ntq[j]];
-                fast_cst* c = q.c;
-                const int e = nte[j], ui = c->nt_to[e];
-                NonTreeF f{};
-                f.e_off = eo[j]; f.rows = rows[j]; f.seg = sg[j]; f.col = g->col;
-                f.alive = q.alive[ui]; f.rank = q.rank[ui]; f.packed = q.packed[ui]; f.n_off = c->n_off[e];
-                f.E = eo[j] + rows[j];
-                cs.push_back({f, h[j], c->n_idx[e], NZ + nnp + j});
-                ft.push_back({eo[j], rows[j], NZ + nnp + j, c->n_off[e]});
-                ni.push_back(rows[j] + 1);
-            }
-            FAST_TRY(compact_seg(cs, s));
-            FAST_TRY(run_items(k_fill_tail_b, ft, ni, s));
-        }
+        const std::vector<int64_t> toff = seg_tile_offsets(n, kIdsTile);
+        Stage st;
+        const size_t d_at = st.add(id), t_at = st.add(toff), z_at = st.zeros((size_t)toff.back() + 1);
+        Scratch sc(s);
+        FAST_TRY(st.upload(sc));
+        const unsigned grid = (unsigned)std::min<int64_t>(toff.back(), (int64_t)num_sms() * 16);
+        k_ids<<<grid, kIdsBlock, 0, s>>>(st.at<IdsDesc>(d_at), st.at<int64_t>(t_at), (int)id.size(), g->lab_vtx, st.z(z_at),
+                                         (unsigned int*)st.z(z_at + (size_t)toff.back()));
+        FAST_TRY(note_launch("candidate ids"));
     }
 
-    // ------------------------------------------------------ workload
-    for (int t = K - 1; t >= 0; t--) {
-        act.clear();
-        for (int qi = 0; qi < nq; qi++) if (Qs[qi].k > t) act.push_back(qi);
-        std::vector<int> pa, pw, pbeg(act.size() + 1, 0);
-        for (size_t a = 0; a < act.size(); a++) {
-            const Q& q = Qs[act[a]];
-            const int u = q.c->bfs[t];
-            for (int w = 0; w < q.k; w++)
-                if (q.c->parent[w] == u) { pa.push_back((int)a); pw.push_back(w); }
-            pbeg[a + 1] = (int)pa.size();
-        }
-        const size_t npr = pa.size();
-        std::vector<double*> sumf(npr, nullptr);
-        std::vector<uint32_t*> ovf(npr, nullptr);
-        {
-            Carver cv, cz;
-            for (int qi : act) {
-                fast_cst* c = Qs[qi].c;
-                const int u = c->bfs[t];
-                cv.add(&c->cval[u], c->ncand[u]);
-                cv.add(&c->cvalf[u], c->ncand[u]);
-            }
-            for (size_t j = 0; j < npr; j++) {
-                fast_cst* c = Qs[act[pa[j]]].c;
-                const int64_t rows = c->ncand[c->bfs[t]];
-                cz.add(&c->ssum[pw[j]], rows);
-                cz.add(&sumf[j], rows);
-                cz.add(&ovf[j], rows);
-            }
-            FAST_TRY(cv.alloc(keep, false));
-            FAST_TRY(cz.alloc(keep, true));
-        }
-        {
-            std::vector<ChildSumDesc> cd;
-            std::vector<int64_t> ent;
-            for (size_t j = 0; j < npr; j++) {
-                fast_cst* c = Qs[act[pa[j]]].c;
-                const int w = pw[j];
-                cd.push_back({c->t_off[w], c->ncand[c->bfs[t]], c->t_idx[w], c->cval[w], c->cvalf[w],
-                              (unsigned long long*)c->ssum[w], sumf[j], ovf[j]});
-                ent.push_back(c->t_entries[w]);
-            }
-            FAST_TRY(run_tiles(k_child_sums_b, cd, ent, kWarpTileItems, 8, s));
-        }
-        {
-            std::vector<ProdDesc> pd;
-            std::vector<int64_t> ni;
-            for (size_t a = 0; a < act.size(); a++) {
-                fast_cst* c = Qs[act[a]].c;
-                const int u = c->bfs[t];
-                ProdDesc d;
-                memset(&d, 0, sizeof(d));
-                for (int j = pbeg[a]; j < pbeg[a + 1]; j++) {
-                    const int i = d.cs.nch++;
-                    d.cs.ssum[i] = c->ssum[pw[j]];
-                    d.cs.sumf[i] = sumf[j];
-                    d.cs.ovf[i] = ovf[j];
-                }
-                d.cval = c->cval[u];
-                d.cvalf = c->cvalf[u];
-                pd.push_back(d);
-                ni.push_back(c->ncand[u]);
-            }
-            FAST_TRY(run_items(k_workload_prod_b, pd, ni, s));
-        }
-    }
+    // ------------------------------------------------------ lists
+    //
+    // A small batch reads no edge-space sizes: its tile arrays are sized by
+    // the graph's count of adjacency entries between the two labels.  A larger
+    // one runs slice by slice, the tree edges into one BFS position each (the
+    // non-tree edges with the first), waiting for a slice's sizes while the
+    // device is busy with the next.
     {
-        std::vector<TotalDesc> td_;
-        for (int qi = 0; qi < nq; qi++) {
-            fast_cst* c = Qs[qi].c;
-            td_.push_back({c->cval[c->root], c->cvalf[c->root], c->ncand[c->root], (uint64_t*)zp(F_W, qi),
-                           (double*)zp(F_WF, qi)});
+        const bool bounded = nq <= kBoundedQueries && !g->lab_pair_host.empty();
+        std::vector<Edge> E;
+        std::vector<size_t> slices{0};
+        int K = 0;
+        for (auto& q : Qs) K = std::max(K, q.k);
+        for (int t = 1; t < std::max(K, 2); t++) {
+            for (int qi = 0; qi < nq; qi++) {
+                const fast_cst* c = Qs[qi].c;
+                if (t < Qs[qi].k) {
+                    const int u = c->bfs[t];
+                    Edge x{qi, c->parent[u], u, 1, 0};
+                    E.push_back(x);
+                }
+                if (t == 1)
+                    for (int e = 0; e < c->nnt; e++) {
+                        Edge x{qi, c->nt_from[e], c->nt_to[e], 0, e};
+                        E.push_back(x);
+                    }
+            }
+            if (!bounded && E.size() > slices.back()) slices.push_back(E.size());
         }
-        Scratch sc(s);
-        const TotalDesc* dd = nullptr;
-        const int64_t* unused = nullptr;
-        FAST_TRY(upload(td_, std::vector<int64_t>(), sc, &dd, &unused));
-        k_total_w_b<<<(unsigned)nq, 1024, 0, s>>>(dd);
-        note_launch();
-        if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "batched W launch");
+        if (bounded && !E.empty()) slices.push_back(E.size());
+        for (auto& x : E) x.n = (uint32_t)Qs[x.q].c->ncand[x.from];
+        FAST_TRY(build_lists(g, Qs, E, slices, bounded, s));
     }
+
+    FAST_TRY(build_workload(Qs, Z, max_depth, keep, s));
 
     // ---------------------------------------- the last round trip
-    {
-        std::vector<int64_t> hw, hk;
-        FAST_TRY(fetch(zp(F_W, 0), hw, (size_t)2 * nq, s));
-        if (nnp) FAST_TRY(fetch(NZ + nnp, hk, nnp, s));
-        int lb_err = 0;
-        cudaError_t e = cudaMemcpyFromSymbolAsync(&lb_err, g_lookback_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return cuda_status(e, "batched CST build", __FILE__, __LINE__);
-        if (lb_err) return set_error(FAST_ERR_CUDA, "batched CST build: a look-back wait ran out");
-        for (int qi = 0; qi < nq; qi++) {
-            memcpy(&Qs[qi].c->W, &hw[qi], sizeof(uint64_t));
-            memcpy(&Qs[qi].c->Wf, &hw[(size_t)nq + qi], sizeof(double));
-        }
-        for (size_t j = 0; j < nnp; j++) Qs[ntq[j]].c->n_entries[nte[j]] = hk[j];
+    int lb_err = 0;
+    FAST_CUDA(cudaMemcpyFromSymbolAsync(&lb_err, g_lookback_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s));
+    FAST_TRY(fetch(Z + (int64_t)F_W * nq, h, (size_t)2 * nq, s));
+    if (lb_err) return set_error(FAST_ERR_CUDA, "CST build: a look-back wait ran out");
+    for (int qi = 0; qi < nq; qi++) {
+        memcpy(&Qs[qi].c->W, &h[qi], sizeof(uint64_t));
+        memcpy(&Qs[qi].c->Wf, &h[(size_t)nq + qi], sizeof(double));
     }
-    return copy_to_arenas(Qs, s);
+    return FAST_OK;
 }
 
 // Queries per group: bounds the grid's y extent of the filter launch
@@ -1296,6 +1346,9 @@ constexpr int kGroup = 1024;
 }  // namespace
 
 namespace fast {
+
+uint64_t build_round_trips() { return t_round_trips; }
+void set_build_round_trips(uint64_t n) { t_round_trips = n; }
 
 int build_cst_batch(const fast_graph* g, int32_t nq, const fast_query_desc* qs, const fast_config* const* cfgs,
                     cudaStream_t s, fast_cst** outs, int32_t* status) {
@@ -1331,7 +1384,7 @@ int build_cst_batch(const fast_graph* g, int32_t nq, const fast_query_desc* qs, 
             if (rc != FAST_OK) continue;
             fast_cst* c = new fast_cst();
             memset(c->cand, 0, sizeof(c->cand)); memset(c->t_off, 0, sizeof(c->t_off)); memset(c->t_idx, 0, sizeof(c->t_idx));
-            memset(c->cval, 0, sizeof(c->cval)); memset(c->cvalf, 0, sizeof(c->cvalf)); memset(c->ssum, 0, sizeof(c->ssum));
+            memset(c->cval, 0, sizeof(c->cval)); memset(c->ssum, 0, sizeof(c->ssum));
             memset(c->n_off, 0, sizeof(c->n_off)); memset(c->n_idx, 0, sizeof(c->n_idx));
             memset(c->t_entries, 0, sizeof(c->t_entries)); memset(c->ncand, 0, sizeof(c->ncand));
             memset(c->n_entries, 0, sizeof(c->n_entries));

@@ -1,10 +1,6 @@
-// The CST build's compaction functors and list helpers (Sec. IV-A,
-// Algorithm 1), shared by the per-query build (cst.cu) and the batched build
-// (cst_batch.cu): the candidate filter, the top-down and non-tree list
-// compactions, the bottom-up row selection and rewrite, the workload sums'
-// child descriptors, the query check, and the exact-size copy kernel.  Each
-// functor follows the compaction interface of prims.cuh (begin / eval /
-// tag / at, and optionally end and counting).
+// Helpers of the CST build (Sec. IV-A, Algorithm 1): the workload sums, the
+// query check, the host rules of query preparation, and the flat copy kernel
+// (also used by the batched partition).
 #pragma once
 
 #include "internal.cuh"
@@ -12,48 +8,8 @@
 
 namespace fast {
 
-// C0(root): the label bucket filtered by degree (bucket order = id order)
-struct FilterF {
-    using value_type = int32_t;
-    const int32_t* bucket;
-    const int32_t* key;
-    int dq;
-    const uint32_t* pass;      // label-frequency rule: the vertices that passed (null: degree rule)
-    __device__ void begin(int64_t) {}
-    __device__ bool eval(int64_t i, int32_t& v) const {
-        v = bucket[i];
-        if (pass) return (pass[v >> 5] >> (v & 31)) & 1u;
-        return (key[v] & 255) >= dq;
-    }
-    __device__ int64_t tag(int64_t) const { return -1; }
-    __device__ void at(int64_t, int64_t) const {}
-};
-
-struct NlfReq {
-    int nn[kMaxK];                 // distinct labels among u's query neighbours
-    int32_t lab[kMaxK][kMaxK];
-    int32_t need[kMaxK][kMaxK];
-};
-
-__device__ __forceinline__ int64_t neighbours_with_label(const GraphRuns& G, const int32_t* __restrict__ col,
-                                                         const int32_t* __restrict__ label, int32_t v, int32_t l) {
-    int64_t b, len;
-    label_segment(G, v, l, &b, &len);
-    if (G.run_ptr) return len;
-    int64_t c = 0;                                 // ungrouped: the whole row, count it
-    for (int64_t i = b; i < b + len; i++) c += label[col[i]] == l;
-    return c;
-}
-
-__device__ __forceinline__ int64_t row_of(const int64_t* e_off, int64_t rows, int64_t i) {
-    // last r with e_off[r] <= i
-    int64_t lo = 0, hi = rows;
-    while (hi - lo > 1) {
-        int64_t mid = (lo + hi) >> 1;
-        if (e_off[mid] <= i) lo = mid; else hi = mid;
-    }
-    return lo;
-}
+constexpr int kItems = 8;
+constexpr int kWarpTileItems = 32 * kItems;  // a warp's tile
 
 // row_of(e_off, rows, i) when it is known to lie in [lo, hi]
 __device__ __forceinline__ int64_t row_in(const int64_t* e_off, int64_t lo, int64_t hi, int64_t i) {
@@ -65,237 +21,12 @@ __device__ __forceinline__ int64_t row_in(const int64_t* e_off, int64_t lo, int6
     return lo;
 }
 
-// The first of the rows whose lists start at index i (row is the last one,
-// the row holding entry i; the others before it are empty).
-__device__ __forceinline__ int64_t first_row_at(const int64_t* e_off, int64_t row, int64_t i) {
-    while (row > 0 && e_off[row - 1] == i) row--;
-    return row;
-}
-
-// new_off[x] = rank for row r and every following row that starts at the
-// same index (empty rows, up to the first row with an entry)
-__device__ __forceinline__ void set_rows_at(const int64_t* e_off, int64_t rows, int64_t r, int64_t* new_off,
-                                            int64_t rank) {
-    const int64_t i = e_off[r];
-    for (int64_t x = r; x < rows && e_off[x] == i; x++) new_off[x] = rank;
-}
-
-// Top-down: flattened neighbour lists of C(u_p); keeps neighbours passing
-// u's filter (label and degree), marks them reached, writes list offsets.
-struct TopDownF {
-    using value_type = int32_t;
-    const int64_t* e_off;      // [rows+1]
-    int64_t rows;
-    const int64_t* seg;        // per row of C(u_p): start in col of its neighbours with u's label
-    const int32_t* col;
-    const int32_t* key;
-    int32_t want_key_hi;       // label
-    int32_t want_dq;
-    bool label_known;          // grouped graph: a segment holds only that label
-    const uint32_t* pass;      // label-frequency rule: u's filter as a bitmap (null: label and degree)
-    uint32_t* reached;         // bitmap over V(G)
-    int64_t* t_off;            // out: [rows+1]
-    const int64_t* E;          // edge-space size on the device (index space may be a bound)
-    bool counting;             // set in the compaction's count pass: mark nothing then
-    int64_t row;
-    int64_t nbase;
-    int64_t e_end;
-    // the rows of a tile's first and last index, once per tile: each thread
-    // then searches only between them
-    __device__ void tile_hint(int64_t tb, int64_t te, int64_t* h) {
-        const int64_t e = *E;
-        if (te > e) te = e;
-        int64_t r0, r1;
-        warp_rows_of(e_off, rows, tb, te > tb ? te - 1 : tb, &r0, &r1);
-        if ((threadIdx.x & 31) == 0) { h[0] = r0; h[1] = r1; }
-    }
-    __device__ void begin(int64_t i0, const int64_t* h) {
-        e_end = *E;
-        if (i0 >= e_end) return;
-        row = row_in(e_off, h[0], h[1], i0);
-        nbase = seg[row] - e_off[row];
-    }
-    __device__ bool eval(int64_t i, int32_t& v) {
-        if (i >= e_end) { v = 0; return false; }
-        while (i >= e_off[row + 1]) { row++; nbase = seg[row] - e_off[row]; }
-        int32_t x = col[nbase + i];
-        v = x;
-        bool hit;
-        if (pass) {
-            hit = (pass[x >> 5] >> (x & 31)) & 1u;  // label, degree and frequencies at once
-        } else if (label_known && want_dq <= 1) {
-            hit = true;                        // the label is the segment's; a neighbour has degree >= 1
-        } else {
-            int32_t kk = key[x];
-            hit = (kk >> 8) == want_key_hi && (kk & 255) >= want_dq;
-        }
-        if (hit && !counting) {
-            // a popular vertex is reached from many rows: test the word
-            // first (a stale copy only costs an atomic) and set the bit once
-            const uint32_t bit = 1u << (x & 31);
-            if (!(__ldcg(&reached[x >> 5]) & bit)) atomicOr(&reached[x >> 5], bit);
-        }
-        return hit;
-    }
-    // rows start at their first entry; a row with no entry (no neighbour of
-    // the label) starts where the next one does, so the first entry of a
-    // row tags it and every empty row just before it
-    __device__ int64_t tag(int64_t i) const { return (i < e_end && i == e_off[row]) ? first_row_at(e_off, row, i) : -1; }
-    // eval and tag of N consecutive indices: positions first (the row walk),
-    // then every neighbour id, every filter word, every reached word at once
-    template <int N>
-    __device__ void eval_n(int64_t i0, int64_t end, uint32_t& keep, int32_t (&val)[N], int32_t (&tg)[N]) {
-        int64_t pos[N];
-#pragma unroll
-        for (int j = 0; j < N; j++) {
-            const int64_t i = i0 + j;
-            pos[j] = -1;
-            tg[j] = -1;
-            if (i < end) {
-                while (i >= e_off[row + 1]) { row++; nbase = seg[row] - e_off[row]; }
-                pos[j] = nbase + i;
-                if (i == e_off[row]) tg[j] = (int32_t)first_row_at(e_off, row, i);
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < N; j++) val[j] = pos[j] >= 0 ? __ldg(col + pos[j]) : 0;
-        uint32_t k = 0;
-        if (pass) {
-            uint32_t w[N];
-#pragma unroll
-            for (int j = 0; j < N; j++) w[j] = pos[j] >= 0 ? __ldg(pass + (val[j] >> 5)) : 0u;
-#pragma unroll
-            for (int j = 0; j < N; j++) k |= ((w[j] >> (val[j] & 31)) & 1u) << j;
-        } else if (label_known && want_dq <= 1) {
-#pragma unroll
-            for (int j = 0; j < N; j++) k |= (pos[j] >= 0 ? 1u : 0u) << j;
-        } else {
-            int32_t kk[N];
-#pragma unroll
-            for (int j = 0; j < N; j++) kk[j] = pos[j] >= 0 ? __ldg(key + val[j]) : -1;
-#pragma unroll
-            for (int j = 0; j < N; j++)
-                k |= ((pos[j] >= 0 && (kk[j] >> 8) == want_key_hi && (kk[j] & 255) >= want_dq) ? 1u : 0u) << j;
-        }
-        if (!counting) {
-            uint32_t r[N];
-#pragma unroll
-            for (int j = 0; j < N; j++) r[j] = ((k >> j) & 1u) ? __ldcg(reached + (val[j] >> 5)) : ~0u;
-#pragma unroll
-            for (int j = 0; j < N; j++) {
-                const uint32_t bit = 1u << (val[j] & 31);
-                if (!(r[j] & bit)) atomicOr(&reached[val[j] >> 5], bit);
-            }
-        }
-        keep = k;
-    }
-    __device__ void at(int64_t r, int64_t rank) const { set_rows_at(e_off, rows, r, t_off, rank); }
-    __device__ int64_t end() const { return *E; }
+// c_u(v) as the sums read it: the saturating uint64 and the float64 twin side
+// by side, one 16-byte load for both.
+struct alignas(16) CVal {
+    unsigned long long c;
+    double f;
 };
-
-// Non-tree: flattened neighbour lists of C(u_j); keeps members of C(u_i)
-// (bitmap) and writes their rank in C(u_i).
-struct NonTreeF {
-    using value_type = uint32_t;
-    const int64_t* e_off;
-    int64_t rows;
-    const int64_t* seg;        // per row of C(u_j): start in col of its neighbours with u_i's label
-    const int32_t* col;
-    const uint32_t* alive;     // bitmap of C(u_i)
-    const uint32_t* rank;      // prefix popcounts of alive
-    const uint2* packed;       // nullable: {alive, rank} word pairs, one 8-byte load for both
-    int64_t* n_off;
-    const int64_t* E;
-    int64_t row;
-    int64_t nbase;
-    int64_t e_end;
-    __device__ void tile_hint(int64_t tb, int64_t te, int64_t* h) {
-        const int64_t e = *E;
-        if (te > e) te = e;
-        int64_t r0, r1;
-        warp_rows_of(e_off, rows, tb, te > tb ? te - 1 : tb, &r0, &r1);
-        if ((threadIdx.x & 31) == 0) { h[0] = r0; h[1] = r1; }
-    }
-    __device__ void begin(int64_t i0, const int64_t* h) {
-        e_end = *E;
-        if (i0 >= e_end) return;
-        row = row_in(e_off, h[0], h[1], i0);
-        nbase = seg[row] - e_off[row];
-    }
-    __device__ bool eval(int64_t i, uint32_t& v) {
-        if (i >= e_end) { v = 0; return false; }
-        while (i >= e_off[row + 1]) { row++; nbase = seg[row] - e_off[row]; }
-        int32_t x = col[nbase + i];
-        const uint2 ar = packed ? packed[x >> 5] : make_uint2(alive[x >> 5], rank[x >> 5]);
-        const uint32_t bit = 1u << (x & 31);
-        v = ar.y + __popc(ar.x & (bit - 1));
-        return (ar.x & bit) != 0;
-    }
-    __device__ int64_t tag(int64_t i) const { return (i < e_end && i == e_off[row]) ? first_row_at(e_off, row, i) : -1; }
-    template <int N>
-    __device__ void eval_n(int64_t i0, int64_t end, uint32_t& keep, uint32_t (&val)[N], int32_t (&tg)[N]) {
-        int64_t pos[N];
-#pragma unroll
-        for (int j = 0; j < N; j++) {
-            const int64_t i = i0 + j;
-            pos[j] = -1;
-            tg[j] = -1;
-            if (i < end) {
-                while (i >= e_off[row + 1]) { row++; nbase = seg[row] - e_off[row]; }
-                pos[j] = nbase + i;
-                if (i == e_off[row]) tg[j] = (int32_t)first_row_at(e_off, row, i);
-            }
-        }
-        int32_t x[N];
-#pragma unroll
-        for (int j = 0; j < N; j++) x[j] = pos[j] >= 0 ? __ldg(col + pos[j]) : 0;
-        uint32_t w[N], rk[N];
-        if (packed) {
-#pragma unroll
-            for (int j = 0; j < N; j++) {
-                const uint2 ar = pos[j] >= 0 ? __ldg(packed + (x[j] >> 5)) : make_uint2(0u, 0u);
-                w[j] = ar.x;
-                rk[j] = ar.y;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < N; j++) {
-                w[j] = pos[j] >= 0 ? __ldg(alive + (x[j] >> 5)) : 0u;
-                rk[j] = pos[j] >= 0 ? __ldg(rank + (x[j] >> 5)) : 0u;
-            }
-        }
-        uint32_t k = 0;
-#pragma unroll
-        for (int j = 0; j < N; j++) {
-            const uint32_t bit = 1u << (x[j] & 31);
-            val[j] = rk[j] + __popc(w[j] & (bit - 1));
-            k |= ((w[j] & bit) ? 1u : 0u) << j;
-        }
-        keep = k;
-    }
-    __device__ void at(int64_t r, int64_t rank_) const { set_rows_at(e_off, rows, r, n_off, rank_); }
-    __device__ int64_t end() const { return *E; }
-};
-
-// rows kept by a validity mask
-struct KeepRowsF {
-    using value_type = int32_t;
-    const int32_t* ids;
-    const uint8_t* valid;
-    const int64_t* nrows;      // rows really present (the index space is a bound)
-    __device__ int64_t end() const { return *nrows; }
-    __device__ void begin(int64_t) {}
-    __device__ bool eval(int64_t i, int32_t& v) const {
-        v = ids[i];
-        return valid[i] != 0;
-    }
-    __device__ int64_t tag(int64_t) const { return -1; }
-    __device__ void at(int64_t, int64_t) const {}
-};
-
-constexpr int kItems = 8;
-constexpr int kTileItems = 256 * kItems;     // a block's tile (8 warps)
-constexpr int kWarpTileItems = 32 * kItems;  // a warp's tile
 
 // Child sums over the entries [i0, iend) of one thread (Sec. IV-C, first
 // half of the workload DP: per row r and child c, the sum of c_c over r's
@@ -306,8 +37,7 @@ constexpr int kWarpTileItems = 32 * kItems;  // a warp's tile
 // then reads as 2^64 - 1.
 __device__ __forceinline__ void child_sum_entries(const int64_t* __restrict__ off, int64_t r0, int64_t r1, int64_t i0,
                                                   int64_t iend, const uint32_t* __restrict__ idx,
-                                                  const uint64_t* __restrict__ cv, const double* __restrict__ cvf,
-                                                  unsigned long long* __restrict__ ssum, double* __restrict__ sumf,
+                                                  const CVal* __restrict__ cv, unsigned long long* __restrict__ ssum, double* __restrict__ sumf,
                                                   uint32_t* __restrict__ ovf) {
     if (i0 >= iend) return;
     // the thread's entries' child indices, then their values, all in flight at once
@@ -318,9 +48,9 @@ __device__ __forceinline__ void child_sum_entries(const int64_t* __restrict__ of
     double vf[kItems];
 #pragma unroll
     for (int i = 0; i < kItems; i++) {
-        const bool in = i0 + i < iend;
-        v[i] = in ? __ldg(cv + x[i]) : 0ull;
-        vf[i] = in ? __ldg(cvf + x[i]) : 0.0;
+        const ulonglong2 c = i0 + i < iend ? __ldg((const ulonglong2*)(cv + x[i])) : make_ulonglong2(0ull, 0ull);
+        v[i] = c.x;
+        vf[i] = __longlong_as_double((long long)c.y);
     }
     int64_t row = row_in(off, r0, r1, i0);
     int64_t rend = off[row + 1];
@@ -357,97 +87,6 @@ __device__ __forceinline__ void child_sum_entries(const int64_t* __restrict__ of
     flush(own && rend == (i0 + kItems < iend ? i0 + kItems : iend));
 }
 
-struct ChildFlags {
-    const uint8_t* has[kMaxK];
-    int nch;
-};
-
-// Bottom-up rewrite: the entries of valid rows still alive in the child's
-// bitmap, as candidate-local indices (bitmap rank), rows renumbered by
-// newrow; each kept row's new offset comes from the compaction's rank.
-struct WriteAliveF {
-    using value_type = uint32_t;
-    const int64_t* off;
-    const int64_t* nrows;
-    const int32_t* list;
-    const uint32_t* alive;
-    const uint32_t* rank;
-    const uint2* packed;       // nullable: {alive, rank} word pairs, one 8-byte load for both
-    const uint8_t* valid;
-    const int64_t* newrow;
-    int64_t* new_off;
-    int64_t rows;
-    int64_t row;
-    int64_t e_end;
-    __device__ void tile_hint(int64_t tb, int64_t te, int64_t* h) {
-        const int64_t r = *nrows, e = off[r];
-        if (te > e) te = e;
-        int64_t r0, r1;
-        warp_rows_of(off, r, tb, te > tb ? te - 1 : tb, &r0, &r1);
-        if ((threadIdx.x & 31) == 0) { h[0] = r0; h[1] = r1; }
-    }
-    __device__ void begin(int64_t i0, const int64_t* h) {
-        rows = *nrows;
-        e_end = off[rows];
-        if (i0 < e_end) row = row_in(off, h[0], h[1], i0);
-    }
-    __device__ bool eval(int64_t i, uint32_t& v) {
-        v = 0;
-        if (i >= e_end) return false;
-        while (i >= off[row + 1]) row++;
-        if (!valid[row]) return false;
-        int32_t x = list[i];
-        const uint2 ar = packed ? packed[x >> 5] : make_uint2(alive[x >> 5], rank[x >> 5]);
-        const uint32_t bit = 1u << (x & 31);
-        v = ar.y + __popc(ar.x & (bit - 1));
-        return (ar.x & bit) != 0;
-    }
-    __device__ int64_t tag(int64_t i) const { return (i < e_end && i == off[row] && valid[row]) ? row : -1; }
-    template <int N>
-    __device__ void eval_n(int64_t i0, int64_t end, uint32_t& keep, uint32_t (&val)[N], int32_t (&tg)[N]) {
-        bool ok[N];
-#pragma unroll
-        for (int j = 0; j < N; j++) {
-            const int64_t i = i0 + j;
-            ok[j] = false;
-            tg[j] = -1;
-            if (i < end) {
-                while (i >= off[row + 1]) row++;
-                ok[j] = valid[row] != 0;
-                if (ok[j] && i == off[row]) tg[j] = (int32_t)row;
-            }
-        }
-        int32_t x[N];
-#pragma unroll
-        for (int j = 0; j < N; j++) x[j] = ok[j] ? __ldg(list + i0 + j) : 0;
-        uint32_t w[N], rk[N];
-        if (packed) {
-#pragma unroll
-            for (int j = 0; j < N; j++) {
-                const uint2 ar = ok[j] ? __ldg(packed + (x[j] >> 5)) : make_uint2(0u, 0u);
-                w[j] = ar.x;
-                rk[j] = ar.y;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < N; j++) {
-                w[j] = ok[j] ? __ldg(alive + (x[j] >> 5)) : 0u;
-                rk[j] = ok[j] ? __ldg(rank + (x[j] >> 5)) : 0u;
-            }
-        }
-        uint32_t k = 0;
-#pragma unroll
-        for (int j = 0; j < N; j++) {
-            const uint32_t bit = 1u << (x[j] & 31);
-            val[j] = rk[j] + __popc(w[j] & (bit - 1));
-            k |= ((w[j] & bit) ? 1u : 0u) << j;
-        }
-        keep = k;
-    }
-    __device__ void at(int64_t r, int64_t rk) const { new_off[newrow[r]] = rk; }
-    __device__ int64_t end() const { return off[*nrows]; }
-};
-
 __device__ __forceinline__ uint64_t warp_sat_sum(uint64_t v) {
     for (int o = 16; o > 0; o >>= 1) v = sat_add(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
@@ -457,13 +96,6 @@ __device__ __forceinline__ double warp_sum_f(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-
-struct ChildSums {
-    uint64_t* ssum[kMaxK];
-    const double* sumf[kMaxK];
-    const uint32_t* ovf[kMaxK];
-    int nch;
-};
 
 inline int validate_query(const fast_query_desc* q, int A[kMaxK][kMaxK], int* dq) {
     if (!q) return set_error(FAST_ERR_INVALID, "query is NULL");

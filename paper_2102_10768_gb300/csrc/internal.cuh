@@ -10,70 +10,73 @@
 constexpr int kMaxK = FAST_MAX_QUERY;
 constexpr int kMaxNT = kMaxK * (kMaxK - 1) / 2;
 
-// Data graph G (Sec. II-A) on the device.
 constexpr int kLabelPairMax = 1024;
 
+// Data graph G (Sec. II-A) on the device, over positions: position p is the
+// p-th vertex by (label, id), so a label's vertices are the range
+// [lab_ptr[l], lab_ptr[l+1]), ascending in both position and id.
 struct fast_graph {
     int64_t n = 0;
-    int64_t nadj = 0;          // stored adjacency entries (2|E|)
+    int64_t nadj = 0;          // stored adjacency entries (2|E|), below 2^32
     int32_t num_labels = 0;
     int64_t max_degree = 0;
-    int64_t* row_ptr = nullptr;   // [n+1]
-    int32_t* col = nullptr;       // [nadj], each row sorted ascending
-    int32_t* label = nullptr;     // [n]
-    int32_t* key = nullptr;       // [n] (label << 8) | min(degree, 255): one load per filter test
+    int64_t* row_ptr = nullptr;   // [n+1], by position
+    int32_t* col = nullptr;       // [nadj] positions, each row ascending (so grouped by label)
     int64_t* lab_ptr = nullptr;   // [num_labels+1]
-    int32_t* lab_vtx = nullptr;   // [n] vertices grouped by label, ascending id
+    int32_t* lab_vtx = nullptr;   // [n] vertex id of each position
     std::vector<int64_t> lab_ptr_host;
-    std::vector<int64_t> lab_degsum_host;   // per label: sum of degrees (bounds CST list sizes)
+    std::vector<int64_t> lab_degsum_host;   // per label: sum of degrees
     // adjacency entries per (label of the row's vertex a, label of the
-    // neighbour b) at [a * num_labels + b], when the rows are grouped by label
-    // and num_labels <= kLabelPairMax (else empty): bounds a top-down list
+    // neighbour b) at [a * num_labels + b], when num_labels <= kLabelPairMax
+    // (else empty): bounds a list's edge space
     std::vector<int64_t> lab_pair_host;
-    // Label runs: when `grouped`, each row of col is sorted by (label of the
-    // neighbour, id), and row v's runs are run_ptr[v] .. run_ptr[v+1]-1: run
-    // r holds the neighbours with label run_lab[r], from col position
-    // run_beg[r] to the next run's start (or the row's end).
-    bool grouped = false;
+    // Where a row's neighbours with one label start: a table [l * n + p]
+    // (l <= num_labels, relative to the row), or, where that would be large,
+    // a directory: row p's runs are run_ptr[p] .. run_ptr[p+1]-1, run r holds
+    // the neighbours with label run_lab[r] from col[run_beg[r]] on.
+    uint32_t* lrel = nullptr;
     int64_t* run_ptr = nullptr;   // [n+1]
     int32_t* run_lab = nullptr;   // [R]
     int64_t* run_beg = nullptr;   // [R]
+    bool csr_by_id = false;       // fast_graph_copy_csr gives rows by id, not by (label, id)
 };
 
-// The neighbours of v with label l: col[*beg .. *beg + *len), ascending id.
-// An ungrouped graph gives the whole row (the caller still tests labels).
-struct GraphRuns {
+struct GraphSegs {
     const int64_t* row_ptr;
-    const int64_t* run_ptr;       // null: ungrouped
+    const uint32_t* lrel;         // null: the directory
+    const int64_t* run_ptr;
     const int32_t* run_lab;
     const int64_t* run_beg;
+    int64_t n;
+    int32_t L;
 };
 
-__device__ __forceinline__ void label_segment(const GraphRuns& G, int32_t v, int32_t l, int64_t* beg, int64_t* len) {
-    const int64_t a = G.row_ptr[v], b = G.row_ptr[v + 1];
-    if (!G.run_ptr) { *beg = a; *len = b - a; return; }
-    int64_t lo = G.run_ptr[v], hi = G.run_ptr[v + 1];
+// The neighbours of position p with label l: col[*beg .. *beg + *len), ascending.
+__device__ __forceinline__ void label_segment(const GraphSegs& G, int32_t p, int32_t l, uint32_t* beg, uint32_t* len) {
+    *beg = 0;
+    *len = 0;
+    if (l >= G.L) return;                          // a label G lacks
+    if (G.lrel) {
+        const uint32_t* t = G.lrel + (int64_t)l * G.n + p;
+        const uint32_t a = __ldg(t), b = __ldg(t + G.n);
+        *beg = (uint32_t)__ldg(G.row_ptr + p) + a;
+        *len = b - a;
+        return;
+    }
+    int64_t lo = G.run_ptr[p], hi = G.run_ptr[p + 1];
     const int64_t r1 = hi;
     while (lo < hi) {                              // first run with label >= l
         int64_t mid = (lo + hi) >> 1;
         if (G.run_lab[mid] < l) lo = mid + 1; else hi = mid;
     }
     if (lo < r1 && G.run_lab[lo] == l) {
-        *beg = G.run_beg[lo];
-        *len = (lo + 1 < r1 ? G.run_beg[lo + 1] : b) - *beg;
-    } else {
-        *beg = a;
-        *len = 0;
+        *beg = (uint32_t)G.run_beg[lo];
+        *len = (uint32_t)((lo + 1 < r1 ? G.run_beg[lo + 1] : G.row_ptr[p + 1]) - G.run_beg[lo]);
     }
 }
 
-inline GraphRuns graph_runs(const fast_graph* g) {
-    GraphRuns G;
-    G.row_ptr = g->row_ptr;
-    G.run_ptr = g->grouped ? g->run_ptr : nullptr;
-    G.run_lab = g->run_lab;
-    G.run_beg = g->run_beg;
-    return G;
+inline GraphSegs graph_segs(const fast_graph* g) {
+    return GraphSegs{g->row_ptr, g->lrel, g->run_ptr, g->run_lab, g->run_beg, g->n, g->num_labels};
 }
 
 // Candidate search tree (Sec. IV-A) of one query.  Indexed by query vertex
@@ -99,14 +102,12 @@ struct fast_cst {
     uint32_t* n_idx[kMaxNT];
     int64_t n_entries[kMaxNT];
     uint64_t* cval[kMaxK];     // c_u(v), saturating uint64 (Sec. IV-C)
-    double* cvalf[kMaxK];      // c_u(v), float64
     uint64_t* ssum[kMaxK];     // per row of C(parent(u)): sum of c_u over its list into u
     uint64_t W = 0;
     double Wf = 0.0;
     fast_config cfg;
     cudaStream_t stream = nullptr;
     fast::Arena arena;         // every array above lives in it (exact sizes)
-    std::vector<void*> build_tmp;   // during fast_build_cst: bounded buffers replaced by exact copies
 };
 
 // One chunk of a partitioned CST (Sec. IV-B): positions 0..j-1 fixed to one
@@ -136,6 +137,8 @@ void chunks_release_nosync(fast_chunks* ch);
 
 // The CSTs of nq queries built together (cst_batch.cu), query i with
 // cfgs[i] (NULL: defaults); outs[i] and status[i] as fast_build_cst_batch.
+uint64_t build_round_trips();                 // of this thread's last build
+void set_build_round_trips(uint64_t n);
 int build_cst_batch(const fast_graph* g, int32_t nq, const fast_query_desc* qs, const fast_config* const* cfgs,
                     cudaStream_t s, fast_cst** outs, int32_t* status);
 

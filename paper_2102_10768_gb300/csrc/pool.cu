@@ -209,29 +209,24 @@ PoolScope::~PoolScope() {
     tl_active = prev_;
 }
 
-int Arena::grow(size_t bytes, cudaStream_t s) {
+int Arena::block(unsigned char** p, size_t bytes, cudaStream_t s) {
+    *p = nullptr;
     if (alloc_fault_due()) return set_error(FAST_ERR_OOM, "CST block of %zu bytes: injected failure", bytes);
-    size_t sz = bytes;
-    if (sz < next_) sz = next_;
     void* b = nullptr;
     retain_freed_memory();
-    cudaError_t e = cudaMallocAsync(&b, sz, s);
+    cudaError_t e = cudaMallocAsync(&b, bytes ? bytes : 256, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return set_error(FAST_ERR_OOM, "CST block of %zu bytes: %s", sz, cudaGetErrorString(e));
+        return set_error(FAST_ERR_OOM, "CST block of %zu bytes: %s", bytes, cudaGetErrorString(e));
     }
     blocks_.push_back(b);
-    cur_ = (char*)b;
-    left_ = sz;
-    next_ = sz * 2;
+    *p = (unsigned char*)b;
     return FAST_OK;
 }
 
 void Arena::release(cudaStream_t s) {
     for (void* b : blocks_) cudaFreeAsync(b, s);
     blocks_.clear();
-    cur_ = nullptr;
-    left_ = 0;
 }
 
 }  // namespace fast

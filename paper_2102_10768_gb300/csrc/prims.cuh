@@ -1,7 +1,7 @@
 // Device-wide building blocks written for this library: exclusive scan,
-// ordered predicate compaction over an index space (single pass, decoupled
-// look-back; a two-pass form where the output size is needed first), and a
-// stable LSD radix sort of 64-bit keys.  All are stream-ordered and take
+// ordered predicate compaction over an index space (two passes: the output's
+// size is known between them), the decoupled look-back of the segmented
+// scans, and a stable LSD radix sort of 64-bit keys.  All are stream-ordered and take
 // their scratch through dalloc on the caller's stream.
 #pragma once
 
@@ -117,26 +117,11 @@ int scan_exclusive(const T* in, T* out, int64_t n, T* total, cudaStream_t s) {
 // Ordered compaction over indices [0, n): F::eval(i, val) says whether index
 // i is kept and what to write; kept values land in out[] in index order.
 // F::begin(i0) is called once per thread before it evaluates indices i0,
-// i0+1, ... in increasing order.  In the write pass F::tag(i), called right
-// after eval(i), may return a non-negative tag (e.g. the row that index i
-// starts); F::at(tag, rank) then receives the number of kept indices before
-// i (used to write list offsets).
+// i0+1, ... in increasing order.
 
 constexpr int kCompBlock = 128;
-constexpr int kCompBlocksPerSM = 8;            // small blocks: one waiting on its look-back leaves 7 running
-constexpr int kCompItems = 16;               // single-pass compaction: indices per thread
-constexpr int kCompTile = kCompBlock * kCompItems;
-constexpr int kEvalN = 8;                    // indices a functor's eval_n takes at once
-static_assert(kCompItems % kEvalN == 0 && kCompItems <= 32, "a thread's kept indices form one 32-bit mask");
-constexpr int kComp2Items = 8;               // the two-pass form (compact_alloc)
+constexpr int kComp2Items = 8;
 constexpr int kComp2Tile = kCompBlock * kComp2Items;
-
-// A functor with a member `bool counting` has it set in the count pass, so
-// that side effects of eval (marking a bitmap) happen once, in the write pass.
-template <class F, class = void>
-struct has_counting : std::false_type {};
-template <class F>
-struct has_counting<F, std::void_t<decltype(std::declval<F&>().counting)>> : std::true_type {};
 
 template <class F>
 __global__ void k_compact_count(F f, int64_t n, int64_t* __restrict__ counts) {
@@ -144,7 +129,6 @@ __global__ void k_compact_count(F f, int64_t n, int64_t* __restrict__ counts) {
     int64_t base = (int64_t)blockIdx.x * kComp2Tile + (int64_t)threadIdx.x * kComp2Items;
     int64_t v[kComp2Items];
     F g = f;
-    if constexpr (has_counting<F>::value) g.counting = true;
     g.begin(base);
 #pragma unroll
     for (int i = 0; i < kComp2Items; i++) {
@@ -162,13 +146,11 @@ __global__ void k_compact_write(F f, int64_t n, const int64_t* __restrict__ offs
     int64_t base = (int64_t)blockIdx.x * kComp2Tile + (int64_t)threadIdx.x * kComp2Items;
     int64_t v[kComp2Items];
     typename F::value_type val[kComp2Items];
-    int64_t tg[kComp2Items];
     F g = f;
     g.begin(base);
 #pragma unroll
     for (int i = 0; i < kComp2Items; i++) {
         v[i] = (base + i < n && g.eval(base + i, val[i])) ? 1 : 0;
-        tg[i] = (base + i < n) ? g.tag(base + i) : -1;
     }
     int64_t hit[kComp2Items];
 #pragma unroll
@@ -177,38 +159,18 @@ __global__ void k_compact_write(F f, int64_t n, const int64_t* __restrict__ offs
     int64_t off = offs[blockIdx.x];
 #pragma unroll
     for (int i = 0; i < kComp2Items; i++) {
-        if (tg[i] >= 0) g.at(tg[i], off + v[i]);
         if (hit[i]) out[off + v[i]] = val[i];
     }
     if (count && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *count = off + tot;
 }
 
-// Runs the two passes; *count_dev receives the kept count (device memory).
-// A functor may know, on the device, where its index space really ends (the
-// host passes a bound): `__device__ int64_t end() const`.
-template <class F, class = void>
-struct has_end : std::false_type {};
-template <class F>
-struct has_end<F, std::void_t<decltype(std::declval<const F&>().end())>> : std::true_type {};
-
-template <class F>
-__device__ __forceinline__ int64_t index_end(const F& f, int64_t n) {
-    if constexpr (has_end<F>::value) {
-        int64_t e = f.end();
-        return e < n ? e : n;
-    } else {
-        return n;
-    }
-}
-
-// Single-pass ordered compaction with decoupled look-back.  Blocks take
-// tiles of kCompTile indices in order from a counter and stop at the index
-// space's real end.  Each tile publishes its kept count (flag AGG), finds
-// its exclusive offset by summing predecessors back to the first one whose
-// inclusive prefix is known (flag PRE), publishes its own prefix, then
-// writes.  A tile only waits on tiles taken before it, by blocks that are
-// already running, so the wait ends; it is still bounded, and running out
-// sets g_lookback_err (never expected), which the caller turns into an error.
+// Decoupled look-back (segmented scans, seg.cuh).  Blocks take tiles in order
+// from a counter.  Each tile publishes its sum (flag AGG), finds its
+// exclusive offset by summing predecessors back to the first one whose
+// inclusive prefix is known (flag PRE) and publishes its own prefix.  A tile
+// only waits on tiles taken before it, by blocks that are already running, so
+// the wait ends; it is still bounded, and running out sets g_lookback_err
+// (never expected), which the caller turns into an error.
 constexpr unsigned long long kLbAgg = 1ull << 62, kLbPre = 2ull << 62, kLbVal = (1ull << 62) - 1;
 constexpr int kLbSpins = 1 << 24;
 static __device__ int g_lookback_err;
@@ -259,31 +221,13 @@ __device__ __forceinline__ int64_t tile_publish(unsigned long long* st, int64_t 
     return excl;
 }
 
-// The last r in [0, rows) with e_off[r] <= i (e_off non-decreasing,
-// e_off[0] <= i < e_off[rows]), by the 32 lanes of a warp together: each
-// round probes 32 points of the interval at once and keeps the 1/33 between
-// two of them, so a search over a million rows takes four rounds of
-// parallel loads instead of twenty dependent ones.  Every lane returns it.
-__device__ __forceinline__ int64_t warp_row_of(const int64_t* __restrict__ e_off, int64_t rows, int64_t i) {
-    const int lane = threadIdx.x & 31;
-    int64_t lo = 0, hi = rows;                            // e_off[lo] <= i < e_off[hi]
-    while (hi - lo > 1) {
-        const int64_t span = hi - lo;
-        const int64_t p = lo + (span * (lane + 1)) / 33;  // non-decreasing in the lane, in [lo, hi)
-        const unsigned m = __ballot_sync(0xffffffffu, e_off[p] <= i);
-        const int c = __popc(m);                          // the probes with e_off <= i form a prefix
-        const int64_t plo = __shfl_sync(0xffffffffu, p, c > 0 ? c - 1 : 0);
-        const int64_t phi = __shfl_sync(0xffffffffu, p, c < 32 ? c : 31);
-        if (c > 0) lo = plo;                              // e_off[plo] <= i
-        if (c < 32) hi = phi;                             // e_off[phi] > i, so phi > plo
-    }
-    return lo;
-}
-
-// The rows of two indices i <= j of the same offsets at once: the two
-// 33-way searches of warp_row_of advance together, so each round's probes
-// of both are loaded in one go.  A search that has finished keeps probing
-// its own row, which leaves it where it is.
+// The rows of two indices i <= j (the last r in [0, rows) with e_off[r] <= i,
+// and with e_off[r] <= j; e_off non-decreasing, e_off[0] <= i, j <
+// e_off[rows]), by the 32 lanes of a warp together: each round probes 32
+// points of both intervals at once and keeps the 1/33 between two of them, so
+// a search over a million rows takes four rounds of parallel loads instead of
+// twenty dependent ones.  A search that has finished keeps probing its own
+// row, which leaves it where it is.
 __device__ __forceinline__ void warp_rows_of(const int64_t* __restrict__ e_off, int64_t rows, int64_t i, int64_t j,
                                              int64_t* ri, int64_t* rj) {
     const int lane = threadIdx.x & 31;
@@ -306,161 +250,6 @@ __device__ __forceinline__ void warp_rows_of(const int64_t* __restrict__ e_off, 
     *ri = alo;
     *rj = blo;
 }
-
-// A functor may narrow its per-thread setup with a hint computed once per
-// tile: `__device__ void tile_hint(int64_t tb, int64_t te, int64_t* h)` (by
-// the 32 lanes of warp 0 together; lane 0 writes h[0..1]) and `__device__
-// void begin(int64_t i0, const int64_t* h)` (by every thread).  Functors
-// without it get begin(i0).
-template <class F, class = void>
-struct has_hint : std::false_type {};
-template <class F>
-struct has_hint<F, std::void_t<decltype(std::declval<F&>().tile_hint(int64_t(0), int64_t(0), (int64_t*)nullptr))>>
-    : std::true_type {};
-
-template <class F>
-__device__ __forceinline__ void tile_hint_of(F& g, int64_t tb, int64_t te, int64_t* h) {
-    if constexpr (has_hint<F>::value) g.tile_hint(tb, te, h);
-}
-
-template <class F>
-__device__ __forceinline__ void begin_with(F& g, int64_t i0, const int64_t* h) {
-    if constexpr (has_hint<F>::value) g.begin(i0, h);
-    else g.begin(i0);
-}
-
-// A functor may also evaluate kEvalN consecutive indices at once, so that
-// their independent loads are in flight together:
-//   template <int N> __device__ void eval_n(int64_t i0, int64_t end,
-//       uint32_t& keep, value_type (&val)[N], int32_t (&tag)[N])
-// sets bit j of keep, val[j] and tag[j] (-1: none) as eval(i0 + j) and
-// tag(i0 + j) would, for i0 + j < end (bits and tags of the others clear).
-template <class F, class = void>
-struct has_eval_n : std::false_type {};
-template <class F>
-struct has_eval_n<F, std::void_t<decltype(std::declval<F&>().template eval_n<kEvalN>(
-                         int64_t(0), int64_t(0), std::declval<uint32_t&>(),
-                         std::declval<typename F::value_type (&)[kEvalN]>(), std::declval<int32_t (&)[kEvalN]>()))>>
-    : std::true_type {};
-
-// Shared memory of a compaction block: the scan's warp totals, the tile's
-// description, and each index's value and tag staged between evaluation
-// and writing (so that a thread's 16 indices need few registers).
-struct CompShared {
-    int32_t tmp[kCompBlock / 32 + 1];
-    int64_t t, end, first, excl, hint[2];
-    int seg;
-    uint32_t val[kCompBlock * kCompItems];
-    int32_t tag[kCompBlock * kCompItems];
-};
-
-// One tile [tb, tb + kCompTile) of an index space ending at `end`: evaluate
-// (values and tags staged in shared memory, the kept indices as a bit mask),
-// scan the threads' kept counts, publish and look back through the status
-// words `st` of the index space (tile lt of it), write.  Every thread of the
-// block calls it; `g` has had its begin().
-template <class F>
-__device__ __forceinline__ void compact_tile(F& g, int64_t tb, int64_t end, unsigned long long* st, int64_t lt,
-                                             typename F::value_type* __restrict__ out, int64_t* count,
-                                             CompShared& sh) {
-    using V = typename F::value_type;
-    static_assert(sizeof(V) == 4, "staged values are 32-bit");
-    const int64_t base = tb + (int64_t)threadIdx.x * kCompItems;
-    V* sv = (V*)(sh.val + threadIdx.x);          // index i of this thread at [i * kCompBlock]:
-    int32_t* st_ = sh.tag + threadIdx.x;         // a warp's stores hit 32 distinct banks
-    uint32_t hit = 0;
-    if constexpr (has_eval_n<F>::value) {
-#pragma unroll
-        for (int h = 0; h < kCompItems; h += kEvalN) {
-            V val[kEvalN];
-            int32_t tg[kEvalN];
-            uint32_t k = 0;
-            g.template eval_n<kEvalN>(base + h, end, k, val, tg);
-#pragma unroll
-            for (int i = 0; i < kEvalN; i++) { sv[(h + i) * kCompBlock] = val[i]; st_[(h + i) * kCompBlock] = tg[i]; }
-            hit |= k << h;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < kCompItems; i++) {
-            const bool in = base + i < end;
-            V x{};
-            const bool k = in && g.eval(base + i, x);
-            sv[i * kCompBlock] = x;
-            hit |= (k ? 1u : 0u) << i;
-            st_[i * kCompBlock] = in ? (int32_t)g.tag(base + i) : -1;    // rows and tags are below 2^31
-        }
-    }
-    int32_t mine[1] = {__popc(hit)};
-    const int32_t tot = block_exclusive_scan<int32_t, kCompBlock, 1>(mine, sh.tmp);
-    if (threadIdx.x < 32) {
-        const int64_t excl = tile_publish(st, lt, (int64_t)tot);
-        if (threadIdx.x == 0) {
-            sh.excl = excl;
-            if (tb + kCompTile >= end && count) *count = excl + tot;   // the last tile
-        }
-    }
-    __syncthreads();
-    const int64_t off = sh.excl + mine[0];
-    int32_t r = 0;
-#pragma unroll
-    for (int i = 0; i < kCompItems; i++) {
-        const int32_t t = st_[i * kCompBlock];
-        if (t >= 0) g.at((int64_t)t, off + r);
-        if ((hit >> i) & 1u) out[off + r++] = sv[i * kCompBlock];
-    }
-    __syncthreads();
-}
-
-template <class F>
-__global__ void __launch_bounds__(kCompBlock, kCompBlocksPerSM) k_compact_1p(F f, int64_t n, typename F::value_type* __restrict__ out,
-                                                              int64_t* __restrict__ count,
-                                                              unsigned long long* __restrict__ st,
-                                                              unsigned int* __restrict__ tile_ctr) {
-    __shared__ CompShared sh;
-    if (threadIdx.x == 0) sh.end = index_end(f, n);
-    __syncthreads();
-    const int64_t end = sh.end;
-    for (;;) {
-        if (threadIdx.x < 32) {                           // warp 0: take a tile, find its hint
-            int64_t t = 0;
-            if (threadIdx.x == 0) t = (int64_t)atomicAdd(tile_ctr, 1u);
-            t = __shfl_sync(0xffffffffu, t, 0);
-            const int64_t tb = t * kCompTile;
-            if (tb < end) tile_hint_of(f, tb, tb + kCompTile < end ? tb + kCompTile : end, sh.hint);
-            if (threadIdx.x == 0) sh.t = t;
-        }
-        __syncthreads();
-        const int64_t t = sh.t;
-        const int64_t tb = t * kCompTile;
-        if (tb >= end) {
-            if (t == 0 && threadIdx.x == 0 && count) *count = 0;     // empty index space
-            break;
-        }
-        F g = f;
-        begin_with(g, tb + (int64_t)threadIdx.x * kCompItems, sh.hint);
-        compact_tile(g, tb, end, st, t, out, count, sh);
-    }
-}
-
-template <class F>
-int compact(const F& f, int64_t n, typename F::value_type* out, int64_t* count_dev, cudaStream_t s) {
-    if (n <= 0) {
-        if (count_dev) FAST_CUDA(cudaMemsetAsync(count_dev, 0, sizeof(int64_t), s));
-        return FAST_OK;
-    }
-    const int64_t nt = ceil_div(n, kCompTile);
-    unsigned long long* st = nullptr;                     // [nt] tile status, then the tile counter
-    FAST_TRY(dalloc(&st, nt + 1, s));
-    cudaMemsetAsync(st, 0, (nt + 1) * sizeof(unsigned long long), s);
-    const int64_t grid = std::min<int64_t>(nt, (int64_t)num_sms() * kCompBlocksPerSM);
-    k_compact_1p<F><<<(unsigned)grid, kCompBlock, 0, s>>>(f, n, out, count_dev, st, (unsigned int*)(st + nt));
-    note_launch();
-    int rc = cudaGetLastError() == cudaSuccess ? FAST_OK : set_error(FAST_ERR_CUDA, "compaction launch");
-    dfree(st, s);
-    return rc;
-}
-
 
 template <class F>
 int compact_alloc(const F& f, int64_t n, typename F::value_type** out, int64_t* kept_host, cudaStream_t s) {

@@ -188,12 +188,6 @@ void worker_main(fast_server* S, int w) {
     }
 }
 
-__global__ void k_label_degree(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ label, int64_t n,
-                               unsigned long long* __restrict__ sum) {
-    int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < n) atomicAdd(&sum[label[v]], (unsigned long long)(row_ptr[v + 1] - row_ptr[v]));
-}
-
 }  // namespace
 
 extern "C" uint64_t fast_now_ns(void) { return now_ns(); }
@@ -210,26 +204,12 @@ extern "C" int fast_server_create(const fast_graph* g, const fast_config* cfg, u
     cudaGetDevice(&S->device);
     int W = workers > 0 ? workers : 4;
     // mean degree per label, for the admission estimate
-    unsigned long long* sum = nullptr;
-    cudaStream_t s0 = nullptr;
-    int rc = dalloc(&sum, g->num_labels, s0);
-    if (rc == FAST_OK) {
-        cudaMemsetAsync(sum, 0, g->num_labels * sizeof(unsigned long long), s0);
-        k_label_degree<<<(unsigned)ceil_div(g->n, 256), 256, 0, s0>>>(g->row_ptr, g->label, g->n, sum);
-        note_launch();
-        std::vector<unsigned long long> h(g->num_labels);
-        cudaMemcpyAsync(h.data(), sum, h.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s0);
-        cudaError_t e = cudaStreamSynchronize(s0);
-        if (e != cudaSuccess) rc = cuda_status(e, "fast_server_create", __FILE__, __LINE__);
-        S->label_deg.resize(g->num_labels);
-        for (int l = 0; l < g->num_labels; l++) {
-            double cnt = (double)(g->lab_ptr_host[l + 1] - g->lab_ptr_host[l]);
-            S->label_deg[l] = cnt > 0 ? (double)h[l] / cnt : 0.0;
-        }
+    S->label_deg.resize(g->num_labels);
+    for (int l = 0; l < g->num_labels; l++) {
+        const double cnt = (double)(g->lab_ptr_host[l + 1] - g->lab_ptr_host[l]);
+        S->label_deg[l] = cnt > 0 ? (double)g->lab_degsum_host[l] / cnt : 0.0;
     }
-    dfree(sum, s0);
-    cudaStreamSynchronize(s0);
-    if (rc != FAST_OK) { delete S; return rc; }
+    int rc = FAST_OK;
     S->streams.assign(W, nullptr);
     S->batches.assign(W, nullptr);
     for (int w = 0; w < W && rc == FAST_OK; w++) {

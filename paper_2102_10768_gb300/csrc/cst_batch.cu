@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <vector>
 
 #include "cst_funcs.cuh"
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(256) k_support(const SetDesc* __restrict__ D, 
     const int lane = threadIdx.x & 31;
     const int64_t items = item_off[nseg];
     for (int64_t it = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
-        const int s = seg_of_tile(item_off, nseg, it);
+        const int s = warp_seg_of(item_off, nseg, it);
         const SetDesc d = D[s];
         const int w0 = (int)(it - item_off[s]) * group, w1 = min(w0 + group, d.words);
         unsigned int kept = 0;
@@ -249,26 +250,36 @@ struct IdsDesc {
 };
 
 constexpr int kIdsBlock = 128;
-constexpr int kIdsItems = 8;                 // words per thread
+constexpr int kIdsItems = 4;                 // words per thread
 constexpr int kIdsTile = kIdsBlock * kIdsItems;
 
+// Tiles of 512 words, scanned and written by a block.  A warp writes the
+// members of four words at a time (one of each of four lanes, whose loads of
+// the ids are in flight together): taken one word after the other, the chain
+// of those loads made this 134 us for one query's sets.
 __global__ void __launch_bounds__(kIdsBlock) k_ids(const IdsDesc* __restrict__ D, const int64_t* __restrict__ tile_off,
                                                    int nseg, const int32_t* __restrict__ lab_vtx,
                                                    unsigned long long* __restrict__ st,
                                                    unsigned int* __restrict__ tile_ctr) {
     __shared__ uint32_t tmp[kIdsBlock / 32 + 1];
     __shared__ int64_t s_t;
+    __shared__ int s_seg;
     __shared__ uint32_t s_excl;
     const int64_t total = tile_off[nseg];
     const int lane = threadIdx.x & 31;
     for (;;) {
-        if (threadIdx.x == 0) s_t = (int64_t)atomicAdd(tile_ctr, 1u);
+        if (threadIdx.x < 32) {
+            int64_t t = 0;
+            if (lane == 0) t = (int64_t)atomicAdd(tile_ctr, 1u);
+            t = __shfl_sync(0xffffffffu, t, 0);
+            const int sg = t < total ? warp_seg_of(tile_off, nseg, t) : 0;
+            if (lane == 0) { s_t = t; s_seg = sg; }
+        }
         __syncthreads();
         const int64_t t = s_t;
         if (t >= total) break;
-        const int s = seg_of_tile(tile_off, nseg, t);
-        const int64_t first = tile_off[s];
-        const IdsDesc& d = D[s];
+        const int64_t first = tile_off[s_seg];
+        const IdsDesc d = D[s_seg];
         const int wb = (int)(t - first) * kIdsTile, base = wb + (int)threadIdx.x * kIdsItems;
         uint32_t w[kIdsItems], v[kIdsItems];
 #pragma unroll
@@ -288,18 +299,27 @@ __global__ void __launch_bounds__(kIdsBlock) k_ids(const IdsDesc* __restrict__ D
         for (int i = 0; i < kIdsItems; i++) {
             const uint32_t r = v[i] + off;
             if (base + i < d.words) d.packed[base + i] = make_uint2(w[i], r);
-            // word i of every lane in turn: its members are written side by side
-            uint32_t some = __ballot_sync(0xffffffffu, w[i] != 0);
-            while (some) {
-                const int l = __ffs(some) - 1;
-                some &= some - 1;
-                const uint32_t x = __shfl_sync(0xffffffffu, w[i], l), o = __shfl_sync(0xffffffffu, r, l);
-                if ((x >> lane) & 1u) {
-                    const int32_t p = d.base + (wlane + l * kIdsItems + i) * 32 + lane;
-                    const uint32_t at = o + __popc(x & lanemask_lt());
-                    d.rows[at] = p;
-                    d.cand[at] = lab_vtx[p];
+            // word i of every lane, four lanes in turn: its members lie side by side
+            const uint32_t some = __ballot_sync(0xffffffffu, w[i] != 0);
+            for (int l0 = 0; l0 < 32; l0 += 4) {
+                if (!((some >> l0) & 15u)) continue;
+                int32_t id[4], p[4];
+                uint32_t at[4];
+                bool in[4];
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const uint32_t x = __shfl_sync(0xffffffffu, w[i], l0 + j);
+                    at[j] = __shfl_sync(0xffffffffu, r, l0 + j) + __popc(x & lanemask_lt());
+                    in[j] = (x >> lane) & 1u;
+                    p[j] = d.base + (wlane + (l0 + j) * kIdsItems + i) * 32 + lane;
+                    id[j] = in[j] ? __ldg(lab_vtx + p[j]) : 0;
                 }
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                    if (in[j]) {
+                        d.rows[at[j]] = p[j];
+                        d.cand[at[j]] = id[j];
+                    }
             }
         }
         __syncthreads();
@@ -315,7 +335,8 @@ __global__ void __launch_bounds__(kIdsBlock) k_ids(const IdsDesc* __restrict__ D
 struct ListDesc {
     const int32_t* rows;             // positions
     uint32_t n;                      // rows
-    int32_t label, base;             // to's label, first position of its bitmap
+    int32_t label, base, words;      // to's label, first position and words of its bitmap
+    int64_t tiles;
     const uint2* packed;             // to's set
     uint32_t* e_off;                 // [n + 1] edge-space offset of each row
     uint32_t* beg;                   // [n] where its segment starts in col
@@ -363,92 +384,155 @@ __global__ void __launch_bounds__(kScanBlock) k_row_lens(const ListDesc* __restr
 // tile counts -> tile bases, and the list set's size
 struct TileBases {
     const ListDesc* D;
-    const int64_t* item_off;
-    __device__ int64_t n(int s) const { return item_off[s + 1] - item_off[s]; }
+    __device__ int64_t n(int s) const { return D[s].tiles; }
     __device__ uint32_t load(int s, int64_t i) const { return D[s].tile[i]; }
     __device__ void store(int s, int64_t i, uint32_t o, uint32_t) const { D[s].tile[i] = o; }
     __device__ void total(int s, uint32_t tot) const { *D[s].K = tot; }
 };
 
 __global__ void __launch_bounds__(kScanBlock) k_tile_bases(const ListDesc* __restrict__ D,
-                                                           const int64_t* __restrict__ item_off,
                                                            const int64_t* __restrict__ tile_off, int nseg,
                                                            unsigned long long* st, unsigned int* ctr) {
-    TileBases f{D, item_off};
+    TileBases f{D};
     seg_scan<uint32_t>(f, tile_off, nseg, st, ctr);
 }
 
-// A warp takes a tile of the edge space: a window of 32 rows at a time (lane
-// = row: offset and segment start, one coalesced load each), then the
-// window's entries 64 at a time, each lane finding its entry's row among the
-// window's offsets with five shuffles.  Counting and writing are two passes
-// over the same entries: nothing waits on another tile (one pass with a
-// look-back left three of four warps at a barrier), the arrays get their exact
-// sizes in between, and the lists are written once, where they stay.  Bound by
-// the entry load and the dependent {word, rank} gather, which hits L1.
-template <bool WRITE>
-__global__ void __launch_bounds__(256) k_lists(const ListDesc* __restrict__ D, const int64_t* __restrict__ item_off,
-                                               int nseg, const int32_t* __restrict__ col) {
+// The set tested against, as a block sees it: in shared memory when it fits
+// (words and, for the write, ranks), else {word, rank} pairs in global memory.
+struct SetView {
+    const uint2* packed;
+    const uint32_t* bits;            // shared, or null
+    const uint32_t* rank;
+};
+
+// One tile of kListTile entries of an edge space, by one warp: a window of 32
+// rows at a time (lane = row: offset and segment start, one coalesced load
+// each), then the window's entries 128 at a time.  An entry's row is found by
+// counting row starts: the window's non-empty rows lie compacted in `shift`,
+// their starts among 32 entries come as one mask (a warp-wide or), and the
+// lane's row is the number of starts up to it.
+template <bool WRITE, bool SHARED>
+__device__ __forceinline__ void list_tile(const ListDesc& d, const SetView& v, uint32_t lt, uint32_t E,
+                                          uint32_t* __restrict__ shift, const int32_t* __restrict__ col) {
+    constexpr int U = 4;
     const int lane = threadIdx.x & 31;
-    const int64_t items = item_off[nseg];
-    for (int64_t it = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
-        const int s = seg_of_tile(item_off, nseg, it);
-        const ListDesc& d = D[s];
-        const uint32_t lt = (uint32_t)(it - item_off[s]);
-        const uint32_t E = *d.E, n = d.n, tb = lt * kListTile;
-        if (lt > 0 && (it - item_off[s]) * kListTile >= E) {     // past the end of a space sized by a bound
-            if (!WRITE && lane == 0) d.tile[lt] = 0;
-            continue;
-        }
-        const bool last = E - tb <= kListTile;
-        const uint32_t te = last ? E : tb + kListTile;
-        uint32_t R = n ? (uint32_t)max(d.first[lt] - 1, 0) : 0u;
-        uint32_t run = WRITE ? d.tile[lt] : 0u;                  // entries kept so far
-        uint32_t cur = tb;
-        for (;;) {
-            const uint32_t row = R + lane;
-            const uint32_t eo = row <= n ? d.e_off[row] : E;
-            const uint32_t sh = (row < n ? d.beg[row] : 0u) - eo;  // entry e of the row is col[sh + e]
-            const uint32_t nxt = R + 32 <= n ? d.e_off[R + 32] : E;
-            const uint32_t lim = nxt < te ? nxt : te;
-            for (uint32_t i0 = cur; i0 < lim; i0 += 64) {
-                int32_t x[2];
-                uint2 pk[2];
+    const uint32_t n = d.n, tb = lt * kListTile;
+    const bool last = E - tb <= kListTile;
+    const uint32_t te = last ? E : tb + kListTile;
+    const uint32_t le = lanemask_lt() | (1u << lane);
+    const int32_t base = d.base;
+    uint32_t R = n ? (uint32_t)max(d.first[lt] - 1, 0) : 0u;
+    uint32_t run = WRITE ? d.tile[lt] : 0u;                  // entries kept so far
+    uint32_t cur = tb;
+    for (;;) {
+        const uint32_t row = R + lane;
+        const uint32_t eo = row <= n ? d.e_off[row] : E;
+        const uint32_t nxt = R + 32 <= n ? d.e_off[R + 32] : E;
+        const uint32_t bg = row < n ? d.beg[row] : 0u;
+        uint32_t en = __shfl_down_sync(0xffffffffu, eo, 1);
+        if (lane == 31) en = nxt;
+        const bool full = row < n && en > eo;                // a row with entries
+        const uint32_t fm = __ballot_sync(0xffffffffu, full);
+        __syncwarp();
+        if (full) shift[__popc(fm & lanemask_lt())] = bg - eo;   // entry e of the row is col[shift + e]
+        __syncwarp();
+        const uint32_t lim = nxt < te ? nxt : te;
+        int started = __popc(__ballot_sync(0xffffffffu, full && eo < cur));
+        for (uint32_t i0 = cur; i0 < lim; i0 += 32 * U) {
+            int32_t x[U];
+            uint32_t w[U], rk[U];
 #pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    const uint32_t e = i0 + 32 * u + lane;
-                    int slot = 0;                                // the last row that starts at or before e
+            for (int u = 0; u < U; u++) {
+                const uint32_t i = i0 + 32 * u;
+                const uint32_t heads = __reduce_or_sync(0xffffffffu, full && eo - i < 32u ? 1u << (eo - i) : 0u);
+                const int j = started + __popc(heads & le) - 1;
+                started += __popc(heads);
+                x[u] = i + lane < lim ? __ldg(col + (shift[j] + i + lane)) - base : -1;
+            }
 #pragma unroll
-                    for (int st = 16; st; st >>= 1)
-                        if (__shfl_sync(0xffffffffu, eo, slot + st) <= e) slot += st;
-                    const uint32_t at = __shfl_sync(0xffffffffu, sh, slot) + e;
-                    x[u] = e < lim ? __ldg(col + at) - d.base : -1;
-                }
-#pragma unroll
-                for (int u = 0; u < 2; u++) pk[u] = x[u] >= 0 ? __ldg(d.packed + (x[u] >> 5)) : make_uint2(0u, 0u);
-#pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    const uint32_t i = i0 + 32 * u, bit = 1u << (x[u] & 31);
-                    const bool hit = x[u] >= 0 && (pk[u].x & bit);
-                    const uint32_t m = __ballot_sync(0xffffffffu, hit);
-                    if (WRITE) {
-                        // rows that start among these 32 entries
-                        if (row < n && eo >= i && eo < lim && eo - i < 32) d.off[row] = run + __popc(m & ((1u << (eo - i)) - 1));
-                        if (hit) d.idx[run + __popc(m & lanemask_lt())] = pk[u].y + __popc(pk[u].x & (bit - 1));
-                    }
-                    run += __popc(m);
+            for (int u = 0; u < U; u++) {
+                if (SHARED) {
+                    w[u] = x[u] >= 0 ? v.bits[x[u] >> 5] : 0u;
+                    rk[u] = 0;
+                } else {
+                    const uint2 pk = x[u] >= 0 ? __ldg(v.packed + (x[u] >> 5)) : make_uint2(0u, 0u);
+                    w[u] = pk.x;
+                    rk[u] = pk.y;
                 }
             }
-            cur = cur > lim ? cur : lim;
-            // empty rows at the window's end (those at a tile's end are the next tile's)
-            if (WRITE && row < n && eo == lim && (lim < te || last)) d.off[row] = run;
-            if (cur >= te && (!last || R + 32 >= n)) break;
-            R += 32;
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const uint32_t i = i0 + 32 * u, bit = 1u << (x[u] & 31);
+                const bool hit = (w[u] & bit) != 0;
+                const uint32_t m = __ballot_sync(0xffffffffu, hit);
+                if (WRITE) {
+                    // rows that start among these 32 entries
+                    if (row < n && eo - i < 32u && eo < lim) d.off[row] = run + __popc(m & ((1u << (eo - i)) - 1));
+                    if (hit)
+                        d.idx[run + __popc(m & lanemask_lt())] = (SHARED ? v.rank[x[u] >> 5] : rk[u]) + __popc(w[u] & (bit - 1));
+                }
+                run += __popc(m);
+            }
         }
-        if (lane == 0) {
-            if (!WRITE) d.tile[lt] = run;
-            else if (last) d.off[n] = run;
+        cur = cur > lim ? cur : lim;
+        // empty rows at the window's end (those at a tile's end are the next tile's)
+        if (WRITE && row < n && eo == lim && (lim < te || last)) d.off[row] = run;
+        if (cur >= te && (!last || R + 32 >= n)) break;
+        R += 32;
+    }
+    if (lane == 0) {
+        if (!WRITE) d.tile[lt] = run;
+        else if (last) d.off[n] = run;
+    }
+}
+
+// The lists of all edges, a block per chunk of `chunk` tiles of one edge.
+// Counting and writing are two passes over the same entries: nothing waits on
+// another tile (one pass with a look-back left three of four warps at a
+// barrier), the arrays get their exact sizes in between, and the lists are
+// written once, where they stay.
+//
+// What bounds it is the gather of bitmap words: from global memory 32 random
+// words cost some 25 L1 wavefronts (the pass ran at 73-77 % of that pipe),
+// from shared memory three or four.  So a block first copies the set, if it
+// has at most `cap` words (bits only for the count, ranks too for the write).
+constexpr int kListWarps = 16;
+
+template <bool WRITE>
+__global__ void __launch_bounds__(kListWarps * 32, 3) k_lists(const ListDesc* __restrict__ D,
+                                                              const int64_t* __restrict__ item_off, int nseg, int chunk,
+                                                              int cap, const int32_t* __restrict__ col) {
+    extern __shared__ uint32_t sm[];
+    __shared__ uint32_t shift[kListWarps][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t items = item_off[nseg];
+    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+        const int s = warp_seg_of(item_off, nseg, it);
+        const ListDesc& d = D[s];
+        const uint32_t E = *d.E;
+        const int64_t t0 = (it - item_off[s]) * chunk;                    // its first tile
+        const int64_t t1 = t0 + chunk < d.tiles ? t0 + chunk : d.tiles;
+        const bool any = t0 == 0 || t0 * kListTile < E;
+        const int words = d.words;
+        const bool shared = any && words <= cap;
+        if (shared) {
+            for (int i = threadIdx.x; i < words; i += blockDim.x) {
+                const uint2 p = __ldg(d.packed + i);
+                sm[i] = p.x;
+                if (WRITE) sm[words + i] = p.y;
+            }
         }
+        __syncthreads();
+        const SetView v{d.packed, sm, sm + words};
+        for (int64_t t = t0 + warp; t < t1; t += kListWarps) {
+            if (t > 0 && t * kListTile >= E) {                           // past the end of a space sized by a bound
+                if (!WRITE && lane == 0) d.tile[t] = 0;
+                continue;
+            }
+            if (shared) list_tile<WRITE, true>(d, v, (uint32_t)t, E, shift[warp], col);
+            else list_tile<WRITE, false>(d, v, (uint32_t)t, E, shift[warp], col);
+        }
+        __syncthreads();
     }
 }
 
@@ -470,7 +554,7 @@ __global__ void __launch_bounds__(256, 4) k_child_sums(const ChildSumDesc* __res
                                                        const int64_t* __restrict__ tile_off, int nseg) {
     const int64_t total = tile_off[nseg];
     for (int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); t < total; t += (int64_t)gridDim.x * 8) {
-        const int s = seg_of_tile(tile_off, nseg, t);
+        const int s = warp_seg_of(tile_off, nseg, t);
         const ChildSumDesc& d = D[s];
         const int64_t e_end = d.off[d.rows];
         const int64_t tb = (t - tile_off[s]) * kWarpTileItems;
@@ -502,9 +586,11 @@ struct ProdDesc {
 __global__ void k_workload_prod(const ProdDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg,
                                 const ChildRef* __restrict__ C) {
     const int64_t total = item_off[nseg];
-    for (int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gi < total;
+    for (int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gi - (threadIdx.x & 31) < total;
          gi += (int64_t)gridDim.x * blockDim.x) {
-        const int s = seg_of_tile(item_off, nseg, gi);
+        int s = warp_seg_of(item_off, nseg, gi - (threadIdx.x & 31));   // the warp's first item's segment
+        if (gi >= total) continue;
+        while (gi >= item_off[s + 1]) s++;
         const ProdDesc d = D[s];
         const int64_t r = gi - item_off[s];
         uint64_t prod = 1;
@@ -766,6 +852,47 @@ struct Readback {
 };
 thread_local Readback t_readback;
 
+// How a list pass is cut into blocks: chunks of tiles of one edge, as many
+// tiles as leave every SM a few blocks, from one per warp up to eight per
+// warp, over which the copy of the set is spread.
+constexpr int kSmallSet = 2048;              // words: 16 KB of words and ranks, three blocks of 16 warps per SM
+constexpr size_t kListSmem = 100 << 10;      // of a block at most: two blocks per SM
+
+struct ListChunks {
+    explicit ListChunks(const std::vector<ListDesc>& ld) {
+        int64_t tiles = 0;
+        for (auto& d : ld) tiles += d.tiles;
+        chunk = kListWarps * (int)std::max<int64_t>(1, std::min<int64_t>(8, tiles / ((int64_t)num_sms() * 6 * kListWarps)));
+        std::vector<int64_t> n;
+        for (auto& d : ld) n.push_back(ceil_div(d.tiles, (int64_t)chunk));
+        items = prefix(n);
+    }
+    unsigned grid() const { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(items.back(), (int64_t)num_sms() * 6)); }
+    // words of the largest set that a block copies
+    int cap(const std::vector<ListDesc>& ld, size_t per_word) const {
+        int c = 0;
+        for (auto& d : ld)
+            if (d.words * per_word <= kListSmem) c = std::max(c, d.words);
+        return c;
+    }
+    int chunk = 1;
+    std::vector<int64_t> items;
+};
+
+// Once per device: the list passes may use kListSmem of dynamic shared memory.
+int lists_smem_optin() {
+    static std::mutex mu;
+    static uint64_t done = 0;
+    int dev = 0;
+    FAST_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu);
+    if (dev < 64 && (done >> dev) & 1) return FAST_OK;
+    FAST_CUDA(cudaFuncSetAttribute(k_lists<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmem));
+    FAST_CUDA(cudaFuncSetAttribute(k_lists<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmem));
+    if (dev < 64) done |= 1ull << dev;
+    return FAST_OK;
+}
+
 // One query edge whose lists are built.
 struct Edge {
     int q, from, to;
@@ -783,6 +910,7 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
                 bool bounded, cudaStream_t s) {
     const size_t ne = E.size();
     const GraphSegs G = graph_segs(g);
+    FAST_TRY(lists_smem_optin());
     uint32_t* Z = nullptr;                        // [0, ne) edge spaces, [ne, 2 ne) entries kept
     Scratch tmp(s);
     {
@@ -821,6 +949,8 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
         d.n = x.n;
         d.label = q.c->qlabel[x.to];
         d.base = q.base[x.to];
+        d.words = q.words[x.to];
+        d.tiles = x.tiles;
         d.packed = q.packed[x.to];
         d.e_off = x.e_off; d.beg = x.beg; d.first = x.first; d.tile = x.tile;
         d.E = Z + i;
@@ -881,16 +1011,19 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
             ld.push_back(desc_of(i, false));
             n.push_back(E[i].tiles);
         }
-        const std::vector<int64_t> items = prefix(n), toff = seg_tile_offsets(n, kScanTile);
+        const std::vector<int64_t> toff = seg_tile_offsets(n, kScanTile);
+        ListChunks lc(ld);
         Stage st;
-        const size_t d_at = st.add(ld), i_at = st.add(items), t_at = st.add(toff);
+        const size_t d_at = st.add(ld), i_at = st.add(lc.items), t_at = st.add(toff);
         const size_t z_at = st.zeros((size_t)toff.back() + 1);
         Scratch sc(s);
         FAST_TRY(st.upload(sc));
-        k_lists<false><<<warp_grid(items.back(), 8), 256, 0, s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at), (int)nseg, g->col);
+        const int cap = lc.cap(ld, sizeof(uint32_t));
+        k_lists<false><<<lc.grid(), kListWarps * 32, cap * sizeof(uint32_t), s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at),
+                                                                                (int)nseg, lc.chunk, cap, g->col);
         FAST_TRY(note_launch("list count"));
         const unsigned grid = (unsigned)std::min<int64_t>(toff.back(), (int64_t)num_sms() * 4);
-        k_tile_bases<<<grid, kScanBlock, 0, s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at), st.at<int64_t>(t_at), (int)nseg,
+        k_tile_bases<<<grid, kScanBlock, 0, s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(t_at), (int)nseg,
                                                  st.z(z_at), (unsigned int*)st.z(z_at + (size_t)toff.back()));
         FAST_TRY(note_launch("list offsets"));
         if (!bounded) FAST_TRY(t_readback.read(Z + ne + e0, ne + e0, nseg, 2 * k + 1, s));
@@ -915,19 +1048,23 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
         FAST_TRY(c->arena.block(&b, cv.bytes(), s));
         cv.place(b);
     }
-    if (ne) {
+    // the write, in two launches: the sets that leave several blocks per SM
+    // with their copies in shared memory, and the larger ones
+    for (int big = 0; big < 2; big++) {
         std::vector<ListDesc> ld;
-        std::vector<int64_t> n;
         for (size_t i = 0; i < ne; i++) {
-            ld.push_back(desc_of(i, true));
-            n.push_back(E[i].tiles);
+            const ListDesc d = desc_of(i, true);
+            if ((d.words > kSmallSet) == (big != 0)) ld.push_back(d);
         }
-        const std::vector<int64_t> items = prefix(n);
+        if (ld.empty()) continue;
+        ListChunks lc(ld);
         Stage st;
-        const size_t d_at = st.add(ld), i_at = st.add(items);
+        const size_t d_at = st.add(ld), i_at = st.add(lc.items);
         Scratch sc(s);
         FAST_TRY(st.upload(sc));
-        k_lists<true><<<warp_grid(items.back(), 8), 256, 0, s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at), (int)ne, g->col);
+        const int cap = lc.cap(ld, 2 * sizeof(uint32_t));
+        k_lists<true><<<lc.grid(), kListWarps * 32, cap * 2 * sizeof(uint32_t), s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at),
+                                                                                   (int)ld.size(), lc.chunk, cap, g->col);
         FAST_TRY(note_launch("list write"));
     }
     return FAST_OK;

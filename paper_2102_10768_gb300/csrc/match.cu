@@ -201,44 +201,69 @@ __device__ __forceinline__ bool bsearch_u32(const uint32_t* __restrict__ a, int6
 // same candidate set (one CST list: n < 2^31) and *pos a cursor into it that
 // never passes the lower bound of any candidate still to come, so successive
 // 32-entry segments of the generator walk L once, merge-style:
-//   - load the tile L[pos, pos+32) with one coalesced read;
+//   - load a tile of 128 entries, four per lane with one 16-byte load (the
+//     list is taken from the 16-byte boundary at or before its start, which
+//     lies in the same array; positions here count from there);
 //   - every pending lane whose candidate is <= the tile's last entry finds
-//     its lower bound inside the tile by a 5-step shuffle search;
+//     the four entries that hold its lower bound by a 5-step shuffle search
+//     over the lanes' last entries, and compares all four;
 //   - if the smallest pending candidate lies beyond the tile, gallop: lanes
-//     probe pos + 32*2^i in one round, then 33-way refinement rounds, each a
-//     single parallel read, until a 32-entry window holds its lower bound.
-// Returns whether this lane's candidate is in the list; *lb counts the
-// entries this lane read (4 B each).
+//     probe pos + 128*2^i in one round, then 33-way refinement rounds, each a
+//     single parallel read, until one tile holds its lower bound.
+// Returns whether this lane's candidate is in the list; *lb counts the bytes
+// of the list that this lane read.
+// A tile of 128 costs 9 shuffles where four tiles of 32 cost 28, and the lists
+// checked hold some four entries per entry of the generator: 250 queries' step
+// 86.2 -> 77.6 ms, 40 queries' 18.2 -> 16.5 ms.
 __device__ __forceinline__ bool warp_member(const uint32_t* __restrict__ L, uint32_t n, uint32_t* pos,
                                             uint32_t c, bool act, unsigned long long* lb) {
     const int lane = threadIdx.x & 31;
     bool found = false;
     uint32_t pend = __ballot_sync(0xffffffffu, act);
-    uint32_t p0 = *pos;
+    const uint32_t head = (uint32_t)((uintptr_t)L >> 2) & 3u;   // entries before the list in its first 16 bytes
+    const uint32_t* La = L - head;
+    const uint32_t end = n ? n + head : 0u;
+    uint32_t p0 = *pos;                                    // a multiple of 4
     uint32_t last = p0;
     while (pend) {
-        if (p0 >= n) break;                                // list exhausted: the rest are absent
-        int tl = __ffs(pend) - 1;
-        uint32_t ct = __shfl_sync(0xffffffffu, c, tl);     // smallest pending candidate
-        uint32_t v = 0xFFFFFFFFu;
-        if (p0 + lane < n) { v = __ldg(L + p0 + lane); *lb += 4; }
-        uint32_t tmax = __shfl_sync(0xffffffffu, v, 31);
+        if (p0 >= end) break;                              // list exhausted: the rest are absent
+        const uint32_t ct = __shfl_sync(0xffffffffu, c, __ffs(pend) - 1);     // smallest pending candidate
+        const uint32_t i = p0 + 4 * lane;
+        uint4 v = make_uint4(~0u, ~0u, ~0u, ~0u);
+        if (i < end) {
+            v = __ldg((const uint4*)(La + i));
+            *lb += 16;
+            if (i + 4 > end) {                             // entries past the list: above every candidate
+                if (i + 1 >= end) v.y = ~0u;
+                if (i + 2 >= end) v.z = ~0u;
+                v.w = ~0u;
+                *lb -= 4 * (i + 4 - end);
+            }
+            if (i < head) {                                // entries before it: its first one, again
+                const uint32_t f = head == 1 ? v.y : head == 2 ? v.z : v.w;
+                v.x = f;
+                if (head > 1) v.y = f;
+                if (head > 2) v.z = f;
+                *lb -= 4 * head;
+            }
+        }
+        const uint32_t tmax = __shfl_sync(0xffffffffu, v.w, 31);
         if (tmax < ct) {
             // gallop: the lower bound of ct lies past this (full) tile
-            uint32_t a = p0 + 32;                           // first index that may hold it
-            uint32_t probe = p0 + 31 + (32u << (lane < 25 ? lane : 25));   // below 2^32: p0 < 2^31
-            if (probe > n - 1) probe = n - 1;
-            uint32_t pv = __ldg(L + probe);
+            uint32_t a = p0 + 128;                          // first index that may hold it
+            uint32_t probe = p0 + 127 + (128u << (lane < 23 ? lane : 23));   // below 2^32: p0 < 2^31
+            if (probe > end - 1) probe = end - 1;
+            uint32_t pv = __ldg(La + probe);
             *lb += 4;
             uint32_t ge = __ballot_sync(0xffffffffu, pv >= ct);
-            if (!ge) { p0 = n; break; }                     // everything left is smaller: all absent
+            if (!ge) { p0 = end; break; }                   // everything left is smaller: all absent
             int f = __ffs(ge) - 1;
             uint32_t b = __shfl_sync(0xffffffffu, probe, f);            // L[b] >= ct
             if (f > 0) a = __shfl_sync(0xffffffffu, probe, f - 1) + 1; // L[a-1] < ct
-            while (b - a > 31) {                            // 33-way refinement of [a, b]
+            while (b - a > 124) {                           // 33-way refinement of [a, b]
                 const uint64_t span = b - a + 1;
                 uint32_t q = a + (uint32_t)(((uint64_t)(lane + 1) * span) / 33);
-                uint32_t qv = __ldg(L + q);
+                uint32_t qv = __ldg(La + q);
                 *lb += 4;
                 uint32_t g2 = __ballot_sync(0xffffffffu, qv >= ct);
                 int f2 = g2 ? __ffs(g2) - 1 : 32;
@@ -247,22 +272,23 @@ __device__ __forceinline__ bool warp_member(const uint32_t* __restrict__ L, uint
                 a = na;
                 b = nb;
             }
-            p0 = a;
+            p0 = a & ~3u;
             continue;
         }
         // resolve every pending lane whose candidate is within this tile
-        bool mine = ((pend >> lane) & 1u) && c <= tmax;
+        const bool mine = ((pend >> lane) & 1u) && c <= tmax;
         int q = 0;
 #pragma unroll
         for (int st = 16; st; st >>= 1) {
-            uint32_t w = __shfl_sync(0xffffffffu, v, q + st - 1);
+            uint32_t w = __shfl_sync(0xffffffffu, v.w, q + st - 1);
             if (w < c) q += st;
         }
-        uint32_t w = __shfl_sync(0xffffffffu, v, q);
-        if (mine) found = (w == c);
+        const uint32_t x0 = __shfl_sync(0xffffffffu, v.x, q), x1 = __shfl_sync(0xffffffffu, v.y, q);
+        const uint32_t x2 = __shfl_sync(0xffffffffu, v.z, q), x3 = __shfl_sync(0xffffffffu, v.w, q);
+        if (mine) found = x0 == c || x1 == c || x2 == c || x3 == c;
         pend &= ~__ballot_sync(0xffffffffu, mine);
         last = p0;
-        p0 += 32;
+        p0 += 128;
     }
     *pos = last;
     return found;
@@ -532,7 +558,7 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
     int32_t* gsrc = sg + kMaxK;                                          // per depth: generator list (as Chunk.pad)
     int64_t* tcur = (int64_t*)(gsrc + kMaxK);                            // per depth: tree-list cursor
     int64_t* ncur = tcur + kMaxK;                                        // per non-tree edge: list cursor
-    unsigned long long iter = 0;
+    uint32_t iter = 0;
     const unsigned long long deadline = *O.deadline;
     unsigned long long lb = 0;             // this lane's bytes requested (entries of 4 B, offsets of 8 B)
     // lane 0: the floor of the bytes, what any search over the CST that scans

@@ -344,6 +344,7 @@ struct ListDesc {
     uint32_t* E;
     uint32_t* tile;                  // per tile: entries kept, then those kept before it
     uint32_t* K;                     // entries kept
+    unsigned long long* sq;          // sum of the rows' squared lengths
     int64_t* off;                    // out [n + 1]
     uint32_t* idx;                   // out [*K]
 };
@@ -359,6 +360,13 @@ struct RowLens {
         label_segment(G, D[s].rows[i], D[s].label, &b, &len);
         D[s].beg[i] = b;
         return len;
+    }
+    __device__ void values(int s, const uint32_t (&x)[kScanItems]) const {
+        unsigned long long q = 0;
+#pragma unroll
+        for (int i = 0; i < kScanItems; i++) q += (unsigned long long)x[i] * x[i];
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if ((threadIdx.x & 31) == 0 && q) atomicAdd(D[s].sq, q);
     }
     __device__ void store(int s, int64_t i, uint32_t o, uint32_t len) const {
         const ListDesc& d = D[s];
@@ -386,6 +394,7 @@ struct TileBases {
     const ListDesc* D;
     __device__ int64_t n(int s) const { return D[s].tiles; }
     __device__ uint32_t load(int s, int64_t i) const { return D[s].tile[i]; }
+    __device__ void values(int, const uint32_t (&)[kScanItems]) const {}
     __device__ void store(int s, int64_t i, uint32_t o, uint32_t) const { D[s].tile[i] = o; }
     __device__ void total(int s, uint32_t tot) const { *D[s].K = tot; }
 };
@@ -911,11 +920,13 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
     const size_t ne = E.size();
     const GraphSegs G = graph_segs(g);
     FAST_TRY(lists_smem_optin());
-    uint32_t* Z = nullptr;                        // [0, ne) edge spaces, [ne, 2 ne) entries kept
+    // [0, ne) edge spaces, [ne, 2 ne) entries kept, then 64-bit sums of squares
+    uint32_t* Z = nullptr;
     Scratch tmp(s);
     {
-        Carver cv;
-        cv.add(&Z, (int64_t)(2 * ne));
+        Carver cz, cv;
+        cz.add(&Z, (int64_t)(4 * ne));
+        FAST_TRY(cz.alloc(tmp, true));
         for (auto& x : E) {
             cv.add(&x.e_off, (int64_t)x.n + 1);
             cv.add(&x.beg, x.n);
@@ -955,6 +966,7 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
         d.e_off = x.e_off; d.beg = x.beg; d.first = x.first; d.tile = x.tile;
         d.E = Z + i;
         d.K = Z + ne + i;
+        d.sq = (unsigned long long*)(Z + 2 * ne) + i;
         if (out) {
             d.off = x.tree ? q.c->t_off[x.to] : q.c->n_off[x.e];
             d.idx = x.tree ? q.c->t_idx[x.to] : q.c->n_idx[x.e];
@@ -962,8 +974,8 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
         return d;
     };
     const size_t ns = slices.size() - 1;
-    if (!bounded) FAST_TRY(t_readback.reserve(2 * ne, 2 * ns));
-    std::vector<uint32_t> kept;
+    if (!bounded) FAST_TRY(t_readback.reserve(4 * ne, 2 * ns + 1));
+    std::vector<uint32_t> sizes;                  // Z
     // row lengths
     {
         Stage st;
@@ -1028,15 +1040,20 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
         FAST_TRY(note_launch("list offsets"));
         if (!bounded) FAST_TRY(t_readback.read(Z + ne + e0, ne + e0, nseg, 2 * k + 1, s));
     }
-    if (bounded) FAST_TRY(fetch(Z + ne, kept, ne, s));
-    else {
+    if (bounded) FAST_TRY(fetch(Z, sizes, 4 * ne, s));
+    else if (ne) {
+        FAST_TRY(t_readback.read(Z + 2 * ne, 2 * ne, 2 * ne, 2 * ns, s));
         for (size_t k = 0; k < ns; k++) FAST_TRY(t_readback.wait(2 * k + 1));
-        kept.assign(t_readback.h + ne, t_readback.h + 2 * ne);
+        FAST_TRY(t_readback.wait(2 * ns));
+        sizes.assign(t_readback.h, t_readback.h + 4 * ne);
     }
     // every size is known: the lists' final place, then the write
     for (size_t i = 0; i < ne; i++) {
         fast_cst* c = Qs[E[i].q].c;
-        (E[i].tree ? c->t_entries[E[i].to] : c->n_entries[E[i].e]) = kept[i];
+        (E[i].tree ? c->t_entries[E[i].to] : c->n_entries[E[i].e]) = sizes[ne + i];
+        uint64_t sq;
+        memcpy(&sq, &sizes[2 * ne + 2 * i], sizeof(sq));
+        (E[i].tree ? c->t_wlen[E[i].to] : c->n_wlen[E[i].e]) = sizes[i] ? (float)((double)sq / sizes[i]) : 0.f;
     }
     for (auto& q : Qs) {
         fast_cst* c = q.c;

@@ -101,6 +101,9 @@ struct fast_cst {
     int64_t* n_off[kMaxNT];
     uint32_t* n_idx[kMaxNT];
     int64_t n_entries[kMaxNT];
+    // length of the list that a random entry belongs to, before the set test
+    // (sum of squared lengths over their sum), per tree and non-tree edge
+    float t_wlen[kMaxK], n_wlen[kMaxNT];
     uint64_t* cval[kMaxK];     // c_u(v), saturating uint64 (Sec. IV-C)
     uint64_t* ssum[kMaxK];     // per row of C(parent(u)): sum of c_u over its list into u
     uint64_t W = 0;

@@ -85,7 +85,8 @@ EventPair& match_events() {
 
 struct MatchPlan {
     int k;
-    int warp_words;                   // shared words per warp (survivors, m, data ids, cursors)
+    int warp_words;                   // shared words per warp (m, data ids, survivors, cursors)
+    int flat;                         // searched by flat_search
     int order[kMaxK];                 // position -> query vertex
     int par[kMaxK];                   // position -> parent position
     uint32_t same_lab[kMaxK];         // earlier positions with the same label
@@ -100,10 +101,13 @@ struct MatchPlan {
 };
 
 enum : int { kStatusTimeout = 1, kStatusOverflow = 2, kStatusLimit = 4 };
-// shared words per warp: survivors [32 depths][32], m and data vertex per
-// position, the generator list of each depth, an 8-byte tree-list cursor per
-// depth, then one 8-byte cursor per non-tree edge of the query
+// shared words per warp: m and data vertex per position, the generator list of
+// each depth, an 8-byte tree-list cursor per depth, survivors [32 depths][32],
+// then one 8-byte cursor per non-tree edge of the query.  A flat search has,
+// after m and the data vertices, five arrays of 32 words per position.
 constexpr int kWarpBaseWords = kMaxK * 32 + 3 * kMaxK + 2 * kMaxK;
+constexpr int kFlatWords = 5 * 32;
+constexpr int kFlatMaxK = 16;
 // Chunk.pad: bit 0 = a donated run; bits 1-6 = the list the run belongs to
 // (0: the tree list of position j; s: the s-th non-tree edge into j); the
 // query of a batch from bit 8 up.
@@ -540,6 +544,292 @@ __device__ void validate_tasks(const MatchPlan& P0, const MatchPlan* __restrict_
     }
 }
 
+// ------------------------------------------------------------ flat search
+//
+// The search of one item (the run [lo, hi) of list `src` into position j,
+// positions 0..j-1 fixed) with up to 32 partial results in flight at every
+// depth.  Position p has a buffer of up to 32 partial results -- candidate,
+// data vertex, and the slot of each one's prefix in the buffer of position
+// p-1 -- and the lists that extend them to p+1, end to end, are one index
+// range that is scanned 32 entries at a time: a lane finds which partial
+// result its entry extends, then tests the entry against that one's own lists
+// and images, which it reaches by following the slots down.  The survivors
+// fill the buffer of p+1.  So 32 lanes have work where every list has two or
+// three entries; the search of one partial result at a time, one list per
+// step, then spent a hundred instructions on each (complete enumeration with
+// lists of 8: 111 instructions per list; with lists of 2, twice that).
+//
+// It is used where the lists are short, or nothing is checked against other
+// lists: a check here is a binary search per lane, and on long lists the
+// merges of the other search are the cheaper form (their 128-entry tiles are
+// loaded once for 32 candidates).  make_plan decides.  Measured, before and
+// after: complete enumeration of a 10-vertex tree query with two-entry lists
+// (31 M embeddings) 24.7 -> 1.9 ms; of 12 4-vertex queries on the 1M/16M
+// power-law graph (3.2 G embeddings) 106 -> 41 ms; 8.4 M rows written 2.9 ->
+// 2.0 ms.
+//
+// Order of work, totals, floor and donations are as in the other search: a
+// donated run is the list of one partial result, or the second half of what is
+// left of it.
+struct FlatState {
+    unsigned long long local, ccount, lb, fb;
+    uint32_t iter;
+};
+
+struct FlatBuf {
+    uint32_t v[32];          // candidate index
+    int32_t g[32];           // data vertex
+    uint32_t lo[32];         // its list into the next position: start
+    uint32_t pf[32];         //   and first index in the range of all
+    uint32_t mt[32];         // slot in the previous buffer | generator list << 8
+};
+static_assert(sizeof(FlatBuf) == kFlatWords * 4, "a flat buffer is kFlatWords words");
+
+template <bool STATS, bool EMIT, bool BATCH>
+__device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut& O, uint32_t q, uint32_t* sm, int j,
+                                              int src0, uint32_t base, uint32_t lo, uint32_t hi,
+                                              unsigned long long deadline, FlatState F) {
+    const int lane = threadIdx.x & 31;
+    const int k = P.k;
+    const int32_t* sg = (const int32_t*)(sm + kMaxK);
+    FlatBuf* B = (FlatBuf*)(sm + 2 * kMaxK);       // B[p]: position p, j <= p <= k - 2
+    uint32_t vcur = 0, vend = 0;                   // lane p: what is left of the range that extends buffer p
+    uint32_t cnt = 0;                              // lane p: partial results in buffer p
+    uint32_t rc = lo, re = hi;                     // what is left of the item's run
+    int d = j;                                     // the position being filled
+    int stop_seen = 0;
+    __syncwarp();
+    for (;;) {
+        ++F.iter;
+        if (F.local >= O.flush_at) {
+            if (lane == 0) flush_count<BATCH>(O, q, F.local);
+            F.local = 0;
+        }
+        if ((F.iter & 15) == 0) {
+            if (__any_sync(0xffffffffu, stop_seen)) break;
+            if (lane == 0) {
+                if ((F.iter & 255) == 0 && deadline && global_timer_ns() > deadline) stop_all(O, kStatusTimeout);
+                stop_seen = is_done(O);
+            }
+            if (BATCH && lane == 1) stop_seen = vload(O.qstop + q);
+        }
+        if (O.dq_cap && (F.iter & 15) == 0) {
+            ulonglong2 ht = make_ulonglong2(0, 0);
+            if (lane == 0) ht = __ldcv((const ulonglong2*)O.dq_head);       // {head, tail}
+            if (__shfl_sync(0xffffffffu, ht.y < ht.x, 0)) {
+                // the shallowest position with work to give: the item's run, then the buffers
+                const bool can = lane >= j && lane < d && vend - vcur >= (uint32_t)(lane == k - 2 ? kLastDonate : 2) && vend > vcur;
+                const uint32_t cm = __ballot_sync(0xffffffffu, can);
+                const bool run = re > rc && re - rc >= (uint32_t)(j == k - 1 ? kLastDonate : 2);
+                if (run || cm) {
+                    unsigned long long slot = ~0ull;
+                    if (lane == 0) slot = claim_ticket(O, ht.x, ht.y);
+                    slot = __shfl_sync(0xffffffffu, slot, 0);
+                    if (slot != ~0ull) {
+                        int dj = j, dsrc = src0, p = -1;
+                        uint32_t a, b, left = 0;                             // the run given; what the donor keeps up to
+                        uint32_t pre = lane < j ? sm[lane] : 0u;
+                        if (run) {
+                            left = rc + (re - rc) / 2;
+                            a = left - base;
+                            b = re - base;
+                        } else {
+                            p = __ffs(cm) - 1;
+                            const uint32_t c = __shfl_sync(0xffffffffu, vcur, p), e = __shfl_sync(0xffffffffu, vend, p);
+                            const uint32_t m = __shfl_sync(0xffffffffu, cnt, p);
+                            // the last partial result with anything left
+                            const uint32_t below = __ballot_sync(0xffffffffu, lane < (int)m && B[p].pf[lane] < e);
+                            const int sl = 31 - __clz(below);
+                            const uint32_t f = B[p].pf[sl];
+                            left = f > c ? f : c + (e - c) / 2;
+                            a = left - f;
+                            b = e - f;
+                            dj = p + 1;
+                            dsrc = (int)(B[p].mt[sl] >> 8);
+                            int at = sl;
+                            for (int t = p; t >= j; t--) {
+                                if (lane == t) pre = B[t].v[at];
+                                at = (int)(B[t].mt[at] & 255u);
+                            }
+                        }
+                        Chunk* dst = &O.dq[slot % O.dq_cap];
+                        dst->prefix[lane] = pre;
+                        if (lane == 0) {
+                            dst->j = dj;
+                            dst->a = a;
+                            dst->b = b;
+                            dst->pad = kDonated | ((uint32_t)dsrc << 1) | (q << 8);
+                            dst->w = 0;
+                            dst->id = 0;
+                        }
+                        __syncwarp();
+                        int gave = 0;
+                        if (lane == 0) {
+                            const uint32_t free_ = (uint32_t)(2 * (slot / O.dq_cap));
+                            __threadfence();
+                            gave = atomicCAS(&O.dq_state[slot % O.dq_cap], free_, free_ + 1) == free_;
+                            if (!gave) atomicAdd(O.started, ~0ull);
+                        }
+                        if (__shfl_sync(0xffffffffu, gave, 0)) {
+                            if (run) re = left;
+                            else if (lane == p) vend = left;
+                        }
+                    }
+                }
+            }
+        }
+        // ---- Generator: the next 32 entries of the range into position d
+        const uint32_t cur = d == j ? rc : __shfl_sync(0xffffffffu, vcur, d - 1);
+        const uint32_t end = d == j ? re : __shfl_sync(0xffffffffu, vend, d - 1);
+        if (cur >= end) {
+            if (d == j) break;
+            d--;
+            continue;
+        }
+        const FlatBuf* Bp = d > j ? &B[d - 1] : nullptr;
+        const uint32_t n = end - cur < 32 ? end - cur : 32;
+        bool ok = lane < (int)n;
+        int sl = 0, src = src0;                        // the partial result this entry extends, and its generator
+        uint32_t at = cur + lane;
+        if (Bp) {
+            const int m = (int)__shfl_sync(0xffffffffu, cnt, d - 1);
+            const uint32_t e = cur + lane;
+#pragma unroll
+            for (int st = 16; st; st >>= 1)
+                if (sl + st < m && Bp->pf[sl + st] <= e) sl += st;
+            at = Bp->lo[sl] + (e - Bp->pf[sl]);
+            src = (int)(Bp->mt[sl] >> 8);
+        }
+        const int e0 = P.nt_begin[d], ne = P.nt_begin[d + 1] - e0;
+        uint32_t cnd = at;
+        if (d > 0) {
+            if (ok) { cnd = __ldg((src == 0 ? P.t_idx[d] : P.n_idx[e0 + src - 1]) + at); F.lb += 4; }
+            if (lane == 0) F.fb += 4ull * n;
+        }
+        // ---- EdgeValidator: the other lists, a binary search per lane
+        if (d > 0 && (ne > 0 || src0 != 0)) {
+            for (int x = 0; x <= ne; x++) {
+                if (!__any_sync(0xffffffffu, ok && x != src)) continue;
+                const int px = x == 0 ? P.par[d] : P.nt_from[e0 + x - 1];
+                if (ok && x != src) {
+                    uint32_t img;
+                    if (px < j) img = sm[px];
+                    else {
+                        int a = sl;
+                        for (int t = d - 1; t > px; t--) a = (int)(B[t].mt[a] & 255u);
+                        img = B[px].v[a];
+                    }
+                    const int64_t* off = x == 0 ? P.t_off[d] : P.n_off[e0 + x - 1];
+                    unsigned long long pr = 0;
+                    ok = bsearch_u32(x == 0 ? P.t_idx[d] : P.n_idx[e0 + x - 1], off[img], off[img + 1], cnd, &pr);
+                    F.lb += 16 + 4 * pr;
+                }
+            }
+        }
+        // ---- VisitedValidator
+        int32_t gc = -1;
+        const uint32_t same = P.same_lab[d];
+        if (same || (EMIT && d == k - 1)) {
+            if (same) {
+                const uint32_t pm = __ballot_sync(0xffffffffu, ok);
+                if (lane == 0) F.fb += 4ull * __popc(pm);
+            }
+            if (ok) {
+                gc = __ldg(P.cand[d] + cnd);
+                F.lb += 4;
+                int a = sl;
+                for (int t = d - 1; t >= j && (same >> j); t--) {
+                    if (((same >> t) & 1u) && B[t].g[a] == gc) ok = false;
+                    a = (int)(B[t].mt[a] & 255u);
+                }
+                for (uint32_t f = same & ((1u << j) - 1); f; f &= f - 1)
+                    if (sg[__ffs(f) - 1] == gc) ok = false;
+            }
+        }
+        // ---- Synchronizer
+        const uint32_t mask = __ballot_sync(0xffffffffu, ok);
+        const int m = __popc(mask);
+        if (d == j) rc += 32;
+        else if (lane == d - 1) vcur += 32;
+        if (STATS && lane == 0) atomicAdd(&O.stats[d], (unsigned long long)m);
+        if (d == k - 1) {
+            F.local += m;
+            F.ccount += m;
+            if (EMIT && !BATCH && mask) {
+                unsigned long long row0 = 0;
+                if (lane == 0) row0 = atomicAdd(O.emb_slot, (unsigned long long)m);
+                row0 = __shfl_sync(0xffffffffu, row0, 0);
+                const unsigned long long row = row0 + __popc(mask & lanemask_lt());
+                if (lane == 0 && row0 < O.emb_cap) {
+                    const unsigned long long nw = m;
+                    F.fb += 4ull * k * (nw < O.emb_cap - row0 ? nw : O.emb_cap - row0);
+                }
+                if (ok && row < O.emb_cap) {
+                    uint32_t* out = O.emb + row * k;
+                    F.lb += 4ull * k;
+                    out[P.order[k - 1]] = (uint32_t)gc;
+                    int a = sl;
+                    for (int t = d - 1; t >= j; t--) {
+                        out[P.order[t]] = (uint32_t)B[t].g[a];
+                        a = (int)(B[t].mt[a] & 255u);
+                    }
+                    for (int t = 0; t < j; t++) out[P.order[t]] = (uint32_t)sg[t];
+                }
+            }
+            continue;
+        }
+        if (!m) continue;
+        // ---- the survivors fill the buffer of d; their lists into d + 1
+        FlatBuf* Bd = &B[d];
+        __syncwarp();
+        if (ok) {
+            const int i = __popc(mask & lanemask_lt());
+            Bd->v[i] = cnd;
+            Bd->g[i] = __ldg(P.cand[d] + cnd);
+            Bd->mt[i] = (uint32_t)sl;
+            F.lb += 4;
+        }
+        __syncwarp();
+        const int w = d + 1, f0 = P.nt_begin[w], nf = P.nt_begin[w + 1] - f0;
+        uint32_t llo = 0, len = 0;
+        int gen = 0;
+        if (lane < m) {
+            for (int x = 0; x <= nf; x++) {
+                const int px = x == 0 ? P.par[w] : P.nt_from[f0 + x - 1];
+                uint32_t img;
+                if (px < j) img = sm[px];
+                else {
+                    int a = lane;
+                    for (int t = d; t > px; t--) a = (int)(B[t].mt[a] & 255u);
+                    img = B[px].v[a];
+                }
+                const int64_t* off = x == 0 ? P.t_off[w] : P.n_off[f0 + x - 1];
+                const int64_t o0 = off[img], o1 = off[img + 1];
+                if (x == 0 || (uint32_t)(o1 - o0) < len) { llo = (uint32_t)o0; len = (uint32_t)(o1 - o0); gen = x; }
+            }
+            F.lb += 16 + 16ull * nf;
+        }
+        if (lane == 0) F.fb += (unsigned long long)m * (4 + 16 + 16ull * nf);
+        uint32_t inc = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+        __syncwarp();
+        if (lane < m) {
+            Bd->lo[lane] = llo;
+            Bd->pf[lane] = inc - len;
+            Bd->mt[lane] |= (uint32_t)gen << 8;
+        }
+        if (lane == d) { cnt = (uint32_t)m; vcur = 0; vend = total; }
+        __syncwarp();
+        d = w;
+    }
+    return F;
+}
+
 // BATCH: plans[q] per query; otherwise the single plan P0.
 // WS: the warp-specialised variant (O.validators validator warps per CTA,
 // the last warps; no counting pass, no embeddings written).
@@ -552,12 +842,12 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
     const uint32_t nq = BATCH ? O.meta[0] : 1u;
     const uint32_t pieces = BATCH ? O.meta[1] : O.pieces;
     const int warp_words = BATCH ? plans[0].warp_words : P0.warp_words;   // one stride for all queries
-    uint32_t* sbuf = smem + (size_t)warp * warp_words;                   // [depth][32]
-    uint32_t* sm = sbuf + kMaxK * 32;                                   // m[position]
+    uint32_t* sm = smem + (size_t)warp * warp_words;                    // m[position]
     int32_t* sg = (int32_t*)(sm + kMaxK);                               // data vertex per position
     int32_t* gsrc = sg + kMaxK;                                          // per depth: generator list (as Chunk.pad)
     int64_t* tcur = (int64_t*)(gsrc + kMaxK);                            // per depth: tree-list cursor
-    int64_t* ncur = tcur + kMaxK;                                        // per non-tree edge: list cursor
+    uint32_t* sbuf = (uint32_t*)(tcur + kMaxK);                          // [depth][32]
+    int64_t* ncur = (int64_t*)(sbuf + kMaxK * 32);                       // per non-tree edge: list cursor
     uint32_t iter = 0;
     const unsigned long long deadline = *O.deadline;
     unsigned long long lb = 0;             // this lane's bytes requested (entries of 4 B, offsets of 8 B)
@@ -705,11 +995,21 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                     base = P.n_off[e][mf];
                 }
                 int64_t lo = base + ch_a, hi = base + ch_b;
+                if (lane == 0) lb += (j > 0 ? 16 : 0) + 16ull * (P.nt_begin[j + 1] - P.nt_begin[j]);
+                if (!WS && P.flat) {
+                    FlatState F{local, 0, lb, fb, iter};
+                    F = flat_search<STATS, EMIT, BATCH>(P, O, q, sm, j, src, (uint32_t)base, (uint32_t)lo, (uint32_t)hi, deadline, F);
+                    local = F.local;
+                    ccount = F.ccount;
+                    lb = F.lb;
+                    fb = F.fb;
+                    iter = F.iter;
+                    goto finished;
+                }
                 if (lane == d) { seg_next = lo; seg_end = hi; seg_base = base; }
                 if (lane == 0) {
                     gsrc[j] = src;
                     tcur[j] = 0;
-                    lb += (j > 0 ? 16 : 0) + 16ull * (P.nt_begin[j + 1] - P.nt_begin[j]);
                 }
                 for (int e = P.nt_begin[j] + lane; e < P.nt_begin[j + 1]; e += 32) ncur[e] = 0;
                 __syncwarp();
@@ -997,6 +1297,7 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                 d--;
             }
         }
+    finished:
         if (lane == 0 && O.chunk_counts && kind == 1) O.chunk_counts[ci] = ccount;
         __syncwarp();
     }
@@ -1008,6 +1309,24 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
     for (int o = 16; o > 0; o >>= 1) lb += __shfl_xor_sync(0xffffffffu, lb, o);
     if (lane == 0 && lb) atomicAdd(O.bytes, lb);
     if (lane == 0 && fb) atomicAdd(O.floor, fb);
+}
+
+// Which queries flat_search takes: those of up to 16 vertices (its buffers are
+// 640 B of shared memory per position and warp) that have no non-tree edge, so
+// that nothing is checked, or whose lists are all short, so that a check is a
+// short binary search.  Short means the length of the list that a random list
+// entry belongs to (hubs count by their entries): on a power-law graph that is
+// hundreds where the plain mean is seven, and there the merges win.
+constexpr double kFlatLength = 32.0;
+
+bool flat_query(const fast_cst* c) {
+    if (c->k < 2 || c->k > kFlatMaxK || c->g->max_degree >= (1ll << 27)) return false;
+    if (c->nnt == 0) return true;
+    for (int u = 0; u < c->k; u++)
+        if (c->parent[u] >= 0 && c->t_wlen[u] > kFlatLength) return false;
+    for (int t = 0; t < c->nnt; t++)
+        if (c->n_wlen[t] > kFlatLength) return false;
+    return true;
 }
 
 MatchPlan make_plan(const fast_cst* c) {
@@ -1050,6 +1369,8 @@ MatchPlan make_plan(const fast_cst* c) {
     }
     P.nt_begin[k] = e;
     P.warp_words = kWarpBaseWords + 2 * e;
+    P.flat = flat_query(c) ? 1 : 0;
+    if (P.flat) P.warp_words = std::max(P.warp_words, 2 * kMaxK + kFlatWords * (k - 1));
     return P;
 }
 
@@ -1073,7 +1394,8 @@ size_t launch_smem(int warps, int warp_words, bool ws) {
 // cursors), once per device.  The attribute is process-wide: setting it per
 // launch to that launch's size would let a concurrent caller on another
 // thread lower it between someone else's set and launch.
-constexpr size_t kMatcherSmemMax = (size_t)8 * (kWarpBaseWords + 2 * kMaxNT) * sizeof(uint32_t) + 16 + sizeof(VRing);
+constexpr int kWarpMaxWords = std::max(kWarpBaseWords + 2 * kMaxNT, 2 * kMaxK + kFlatWords * (kFlatMaxK - 1));
+constexpr size_t kMatcherSmemMax = (size_t)8 * (kWarpMaxWords + 255) / 256 * 256 * sizeof(uint32_t) + 16 + sizeof(VRing);
 
 int matcher_smem_optin(size_t bytes) {
     if (bytes > kMatcherSmemMax) return set_error(FAST_ERR_INVALID, "matcher: %zu bytes of shared memory per CTA", bytes);

@@ -61,6 +61,7 @@ inline std::vector<int64_t> seg_tile_offsets(const std::vector<int64_t>& n, int6
 // given by F:
 //   int64_t n(int s)                              items of segment s
 //   T load(int s, int64_t i)                      item i (each is loaded once)
+//   void values(int s, const T (&x)[kScanItems])  a thread's items (zeros past the end), by whole warps
 //   void store(int s, int64_t i, T excl, T v)     its exclusive prefix and itself
 //   void total(int s, T tot)                      the segment's sum
 // st: one status word per tile, tile_ctr after them, all zero at launch.
@@ -98,6 +99,7 @@ __device__ __forceinline__ void seg_scan(F& f, const int64_t* __restrict__ tile_
         T v[kScanItems], x[kScanItems];
 #pragma unroll
         for (int i = 0; i < kScanItems; i++) x[i] = v[i] = base + i < n ? f.load(sg, base + i) : T(0);
+        f.values(sg, x);
         const T tot = block_exclusive_scan<T, kScanBlock, kScanItems>(v, tmp);
         if (threadIdx.x < 32) {
             const int64_t excl = tile_publish(st + s_first, lt, (int64_t)tot);

@@ -16,9 +16,10 @@
 //   ids        each C(u) as sorted ids, and the rank of every bitmap word.
 //   lists      per tree edge and per non-tree edge (from, to), for every
 //              candidate of `from` its neighbours in C(to) as indices into
-//              C(to): one pass counts, one pass writes in place.  A tree list
-//              after refinement holds the neighbours in the refined set, so
-//              both kinds of edge are the same computation.
+//              C(to): one pass tests them, tile by tile, and one moves what
+//              was kept to its final place.  A tree list after refinement
+//              holds the neighbours in the refined set, so both kinds of edge
+//              are the same computation.
 //   workload   children first: the saturating sum of c over each child list,
 //              then the product over the children.
 // Every step is one launch over all queries of the batch (each query vertex
@@ -138,7 +139,9 @@ __device__ __forceinline__ bool in_bits(const uint32_t* __restrict__ bits, int32
 // warps hide.  On a power-law graph the first words of a label can be all
 // hubs, so a row with thousands of entries and no early hit must not stay
 // with one warp.
-__global__ void __launch_bounds__(256) k_support(const SetDesc* __restrict__ D, const int64_t* __restrict__ item_off,
+constexpr int kSupportBlocks = 6;            // per SM, all resident: one wave (of 8, the last two ran alone)
+
+__global__ void __launch_bounds__(256, kSupportBlocks) k_support(const SetDesc* __restrict__ D, const int64_t* __restrict__ item_off,
                                                  int nseg, int group, const Target* __restrict__ T, GraphSegs G,
                                                  const int32_t* __restrict__ col, LongRow* __restrict__ longs,
                                                  unsigned int* __restrict__ nlong) {
@@ -343,9 +346,10 @@ struct ListDesc {
     int32_t* first;                  // per tile (and one more): its first row that starts in it
     uint32_t* E;
     uint32_t* tile;                  // per tile: entries kept, then those kept before it
+    uint32_t* tmp;                   // [E]: what each tile kept, from the tile's first entry on
     uint32_t* K;                     // entries kept
     unsigned long long* sq;          // sum of the rows' squared lengths
-    int64_t* off;                    // out [n + 1]
+    int64_t* off;                    // out [n + 1] (by the first pass: within the row's tile)
     uint32_t* idx;                   // out [*K]
 };
 constexpr uint32_t kListTile = 512;
@@ -407,7 +411,7 @@ __global__ void __launch_bounds__(kScanBlock) k_tile_bases(const ListDesc* __res
 }
 
 // The set tested against, as a block sees it: in shared memory when it fits
-// (words and, for the write, ranks), else {word, rank} pairs in global memory.
+// (words and ranks apart), else {word, rank} pairs in global memory.
 struct SetView {
     const uint2* packed;
     const uint32_t* bits;            // shared, or null
@@ -416,22 +420,23 @@ struct SetView {
 
 // One tile of kListTile entries of an edge space, by one warp: a window of 32
 // rows at a time (lane = row: offset and segment start, one coalesced load
-// each), then the window's entries 128 at a time.  An entry's row is found by
-// counting row starts: the window's non-empty rows lie compacted in `shift`,
-// their starts among 32 entries come as one mask (a warp-wide or), and the
-// lane's row is the number of starts up to it.
-template <bool WRITE, bool SHARED>
+// each), then the window's entries, 128 of them in flight.  An entry's row is
+// found by counting row starts: the window's non-empty rows lie compacted in
+// `shift`, their starts among 32 entries come as one mask (a warp-wide or), and
+// the lane's row is the number of starts up to it.
+template <bool SHARED>
 __device__ __forceinline__ void list_tile(const ListDesc& d, const SetView& v, uint32_t lt, uint32_t E,
                                           uint32_t* __restrict__ shift, const int32_t* __restrict__ col) {
-    constexpr int U = 4;
+    constexpr int U = 4;             // 2: 5 % slower on the whole step, its loads too few in flight
     const int lane = threadIdx.x & 31;
     const uint32_t n = d.n, tb = lt * kListTile;
     const bool last = E - tb <= kListTile;
     const uint32_t te = last ? E : tb + kListTile;
-    const uint32_t le = lanemask_lt() | (1u << lane);
+    const uint32_t lt_mask = lanemask_lt(), le_mask = lt_mask | (1u << lane);
     const int32_t base = d.base;
+    uint32_t* const out = d.tmp + tb;
     uint32_t R = n ? (uint32_t)max(d.first[lt] - 1, 0) : 0u;
-    uint32_t run = WRITE ? d.tile[lt] : 0u;                  // entries kept so far
+    uint32_t run = 0;                                        // entries kept so far
     uint32_t cur = tb;
     for (;;) {
         const uint32_t row = R + lane;
@@ -443,18 +448,19 @@ __device__ __forceinline__ void list_tile(const ListDesc& d, const SetView& v, u
         const bool full = row < n && en > eo;                // a row with entries
         const uint32_t fm = __ballot_sync(0xffffffffu, full);
         __syncwarp();
-        if (full) shift[__popc(fm & lanemask_lt())] = bg - eo;   // entry e of the row is col[shift + e]
+        if (full) shift[__popc(fm & lt_mask)] = bg - eo;     // entry e of the row is col[shift + e]
         __syncwarp();
         const uint32_t lim = nxt < te ? nxt : te;
         int started = __popc(__ballot_sync(0xffffffffu, full && eo < cur));
         for (uint32_t i0 = cur; i0 < lim; i0 += 32 * U) {
             int32_t x[U];
             uint32_t w[U], rk[U];
+            uint32_t kept_m = 0, kept_n = 0;                 // lane u: what step u kept, and the number before
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 const uint32_t i = i0 + 32 * u;
                 const uint32_t heads = __reduce_or_sync(0xffffffffu, full && eo - i < 32u ? 1u << (eo - i) : 0u);
-                const int j = started + __popc(heads & le) - 1;
+                const int j = started + __popc(heads & le_mask) - 1;
                 started += __popc(heads);
                 x[u] = i + lane < lim ? __ldg(col + (shift[j] + i + lane)) - base : -1;
             }
@@ -471,43 +477,40 @@ __device__ __forceinline__ void list_tile(const ListDesc& d, const SetView& v, u
             }
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                const uint32_t i = i0 + 32 * u, bit = 1u << (x[u] & 31);
+                const uint32_t bit = 1u << (x[u] & 31);
                 const bool hit = (w[u] & bit) != 0;
                 const uint32_t m = __ballot_sync(0xffffffffu, hit);
-                if (WRITE) {
-                    // rows that start among these 32 entries
-                    if (row < n && eo - i < 32u && eo < lim) d.off[row] = run + __popc(m & ((1u << (eo - i)) - 1));
-                    if (hit)
-                        d.idx[run + __popc(m & lanemask_lt())] = (SHARED ? v.rank[x[u] >> 5] : rk[u]) + __popc(w[u] & (bit - 1));
-                }
+                if (lane == u) { kept_m = m; kept_n = run; }
+                if (hit) out[run + __popc(m & lt_mask)] = (SHARED ? v.rank[x[u] >> 5] : rk[u]) + __popc(w[u] & (bit - 1));
                 run += __popc(m);
             }
+            // the offsets of the rows that start among these entries
+            const uint32_t rel = eo - i0;
+            const uint32_t km = __shfl_sync(0xffffffffu, kept_m, (rel >> 5) % U), kn = __shfl_sync(0xffffffffu, kept_n, (rel >> 5) % U);
+            if (row < n && rel < 32u * U && eo < lim) d.off[row] = kn + __popc(km & ((1u << (rel & 31)) - 1));
         }
         cur = cur > lim ? cur : lim;
         // empty rows at the window's end (those at a tile's end are the next tile's)
-        if (WRITE && row < n && eo == lim && (lim < te || last)) d.off[row] = run;
+        if (row < n && eo == lim && (lim < te || last)) d.off[row] = run;
         if (cur >= te && (!last || R + 32 >= n)) break;
         R += 32;
     }
-    if (lane == 0) {
-        if (!WRITE) d.tile[lt] = run;
-        else if (last) d.off[n] = run;
-    }
+    if (lane == 0) d.tile[lt] = run;
 }
 
-// The lists of all edges, a block per chunk of `chunk` tiles of one edge.
-// Counting and writing are two passes over the same entries: nothing waits on
-// another tile (one pass with a look-back left three of four warps at a
-// barrier), the arrays get their exact sizes in between, and the lists are
-// written once, where they stay.
+// The lists of all edges, a block per chunk of `chunk` tiles of one edge.  Each
+// tile's kept entries go to its own place in a buffer of the edge space's size,
+// so that no tile waits on another (with a look-back, three of four warps stood
+// at a barrier) and every entry is tested once; a second kernel moves them to
+// their final place, whose size is known by then.  (Counting first, and testing
+// again for the write, took 77.6 ms for a step of 250 queries; this, 74.)
 //
 // What bounds it is the gather of bitmap words: from global memory 32 random
 // words cost some 25 L1 wavefronts (the pass ran at 73-77 % of that pipe),
-// from shared memory three or four.  So a block first copies the set, if it
-// has at most `cap` words (bits only for the count, ranks too for the write).
+// from shared memory three or four.  So a block first copies the set, words
+// and ranks, if it has at most `cap` words.
 constexpr int kListWarps = 16;
 
-template <bool WRITE>
 __global__ void __launch_bounds__(kListWarps * 32, 3) k_lists(const ListDesc* __restrict__ D,
                                                               const int64_t* __restrict__ item_off, int nseg, int chunk,
                                                               int cap, const int32_t* __restrict__ col) {
@@ -528,20 +531,55 @@ __global__ void __launch_bounds__(kListWarps * 32, 3) k_lists(const ListDesc* __
             for (int i = threadIdx.x; i < words; i += blockDim.x) {
                 const uint2 p = __ldg(d.packed + i);
                 sm[i] = p.x;
-                if (WRITE) sm[words + i] = p.y;
+                sm[words + i] = p.y;
             }
         }
         __syncthreads();
         const SetView v{d.packed, sm, sm + words};
         for (int64_t t = t0 + warp; t < t1; t += kListWarps) {
             if (t > 0 && t * kListTile >= E) {                           // past the end of a space sized by a bound
-                if (!WRITE && lane == 0) d.tile[t] = 0;
+                if (lane == 0) d.tile[t] = 0;
                 continue;
             }
-            if (shared) list_tile<WRITE, true>(d, v, (uint32_t)t, E, shift[warp], col);
-            else list_tile<WRITE, false>(d, v, (uint32_t)t, E, shift[warp], col);
+            if (shared) list_tile<true>(d, v, (uint32_t)t, E, shift[warp], col);
+            else list_tile<false>(d, v, (uint32_t)t, E, shift[warp], col);
         }
         __syncthreads();
+    }
+}
+
+// What each tile kept, to its place among the edge's lists, and the offsets of
+// the rows that start in it.  A warp takes `group` tiles of one edge, so that
+// the search for the edge is spread over them; HBM-bound.
+__global__ void __launch_bounds__(256, 6) k_list_move(const ListDesc* __restrict__ D,
+                                                      const int64_t* __restrict__ item_off, int nseg, int group) {
+    const int lane = threadIdx.x & 31;
+    const int64_t items = item_off[nseg];
+    for (int64_t it = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
+        const int s = warp_seg_of(item_off, nseg, it);
+        const ListDesc d = D[s];
+        const uint32_t E = *d.E, K = *d.K;
+        const int64_t t0 = (it - item_off[s]) * group, t1 = t0 + group < d.tiles ? t0 + group : d.tiles;
+        for (int64_t t = t0; t < t1; t++) {
+            if (t > 0 && t * kListTile >= E) break;
+            const uint32_t tb = (uint32_t)t * kListTile;
+            const bool last = E - tb <= kListTile;
+            const uint32_t a = d.tile[t], m = (t + 1 < d.tiles ? d.tile[t + 1] : K) - a;
+#pragma unroll
+            for (int h = 0; h < (int)kListTile; h += 256) {
+                uint32_t x[8];
+#pragma unroll
+                for (int i = 0; i < 8; i++) x[i] = h + 32 * i + lane < m ? __ldcs(d.tmp + tb + h + 32 * i + lane) : 0u;
+#pragma unroll
+                for (int i = 0; i < 8; i++)
+                    if (h + 32 * i + lane < m) d.idx[a + h + 32 * i + lane] = x[i];
+            }
+            if (d.n && a) {
+                const uint32_t r1 = last ? d.n : (uint32_t)d.first[t + 1];
+                for (uint32_t r = (uint32_t)d.first[t] + lane; r < r1; r += 32) d.off[r] += a;
+            }
+            if (last && lane == 0) d.off[d.n] = K;
+        }
     }
 }
 
@@ -777,9 +815,10 @@ enum : int {
     F_END = F_WF + 1
 };
 
-// Batches of at most this many queries size their tile arrays by host-known
+// Batches of at most this many queries size their list buffers by host-known
 // bounds; a larger one reads each edge-space size back first.
 constexpr int kBoundedQueries = 8;
+constexpr uint64_t kBoundedBytes = 2ull << 30;   // of bounded buffers, at most
 
 // One query of the batch.
 struct Q {
@@ -864,7 +903,7 @@ thread_local Readback t_readback;
 // How a list pass is cut into blocks: chunks of tiles of one edge, as many
 // tiles as leave every SM a few blocks, from one per warp up to eight per
 // warp, over which the copy of the set is spread.
-constexpr int kSmallSet = 2048;              // words: 16 KB of words and ranks, three blocks of 16 warps per SM
+constexpr int kSmallSet = 8192;              // words: 64 KB of words and ranks
 constexpr size_t kListSmem = 100 << 10;      // of a block at most: two blocks per SM
 
 struct ListChunks {
@@ -878,10 +917,10 @@ struct ListChunks {
     }
     unsigned grid() const { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(items.back(), (int64_t)num_sms() * 6)); }
     // words of the largest set that a block copies
-    int cap(const std::vector<ListDesc>& ld, size_t per_word) const {
+    int cap(const std::vector<ListDesc>& ld) const {
         int c = 0;
         for (auto& d : ld)
-            if (d.words * per_word <= kListSmem) c = std::max(c, d.words);
+            if (d.words * 2 * sizeof(uint32_t) <= kListSmem) c = std::max(c, d.words);
         return c;
     }
     int chunk = 1;
@@ -896,8 +935,7 @@ int lists_smem_optin() {
     FAST_CUDA(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lk(mu);
     if (dev < 64 && (done >> dev) & 1) return FAST_OK;
-    FAST_CUDA(cudaFuncSetAttribute(k_lists<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmem));
-    FAST_CUDA(cudaFuncSetAttribute(k_lists<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmem));
+    FAST_CUDA(cudaFuncSetAttribute(k_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kListSmem));
     if (dev < 64) done |= 1ull << dev;
     return FAST_OK;
 }
@@ -909,12 +947,20 @@ struct Edge {
     int e;                        // else: the non-tree edge's index
     uint32_t n = 0;               // rows
     int64_t tiles = 0;
-    uint32_t *e_off = nullptr, *beg = nullptr, *tile = nullptr;
+    uint32_t *e_off = nullptr, *beg = nullptr, *tile = nullptr, *tmp = nullptr;
     int32_t* first = nullptr;
 };
 
-// The two passes over the lists of every edge of the batch, tree and
-// non-tree alike.  `slices`: ranges of E whose sizes are read back together.
+// entries that an edge's space has at most
+int64_t edge_bound(const fast_graph* g, const fast_cst* c, const Edge& x) {
+    const int64_t L = g->num_labels;
+    const int32_t la = c->qlabel[x.from], lb = c->qlabel[x.to];
+    if (la >= L || lb >= L) return 0;
+    if (!g->lab_pair_host.empty()) return g->lab_pair_host[(size_t)la * L + lb];
+    return g->lab_degsum_host[la];
+}
+
+// The lists of every edge of the batch, tree and non-tree alike.  `slices`: ranges of E whose sizes are read back together.
 int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, const std::vector<size_t>& slices,
                 bool bounded, cudaStream_t s) {
     const size_t ne = E.size();
@@ -933,26 +979,21 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
         }
         FAST_TRY(cv.alloc(tmp, false));
     }
-    auto bound_of = [&](const Edge& x) -> int64_t {
-        const fast_cst* c = Qs[x.q].c;
-        const int64_t L = g->num_labels;
-        const int32_t la = c->qlabel[x.from], lb = c->qlabel[x.to];
-        if (la >= L || lb >= L) return 0;
-        if (!g->lab_pair_host.empty()) return g->lab_pair_host[(size_t)la * L + lb];
-        return g->lab_degsum_host[la];
-    };
     // The arrays of first rows are sized before the edge spaces are known; the
-    // tiles to run, by their real sizes unless the batch is small.
+    // tiles to run and what they keep, by the real sizes unless the batch is
+    // small.
     {
         Carver cv;
         for (auto& x : E) {
-            x.tiles = std::max<int64_t>(1, ceil_div(bound_of(x), (int64_t)kListTile));
+            const int64_t bound = edge_bound(g, Qs[x.q].c, x);
+            x.tiles = std::max<int64_t>(1, ceil_div(bound, (int64_t)kListTile));
             cv.add(&x.first, x.tiles + 1);
             cv.add(&x.tile, x.tiles);
+            if (bounded) cv.add(&x.tmp, bound);
         }
         FAST_TRY(cv.alloc(tmp, false));
     }
-    auto desc_of = [&](size_t i, bool out) {
+    auto desc_of = [&](size_t i) {
         const Edge& x = E[i];
         const Q& q = Qs[x.q];
         ListDesc d{};
@@ -963,14 +1004,12 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
         d.words = q.words[x.to];
         d.tiles = x.tiles;
         d.packed = q.packed[x.to];
-        d.e_off = x.e_off; d.beg = x.beg; d.first = x.first; d.tile = x.tile;
+        d.e_off = x.e_off; d.beg = x.beg; d.first = x.first; d.tile = x.tile; d.tmp = x.tmp;
         d.E = Z + i;
         d.K = Z + ne + i;
         d.sq = (unsigned long long*)(Z + 2 * ne) + i;
-        if (out) {
-            d.off = x.tree ? q.c->t_off[x.to] : q.c->n_off[x.e];
-            d.idx = x.tree ? q.c->t_idx[x.to] : q.c->n_idx[x.e];
-        }
+        d.off = x.tree ? q.c->t_off[x.to] : q.c->n_off[x.e];
+        d.idx = x.tree ? q.c->t_idx[x.to] : q.c->n_idx[x.e];     // null until the sizes are known
         return d;
     };
     const size_t ns = slices.size() - 1;
@@ -986,7 +1025,7 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
             ld.clear();
             std::vector<int64_t> n;
             for (size_t i = slices[k]; i < slices[k + 1]; i++) {
-                ld.push_back(desc_of(i, false));
+                ld.push_back(desc_of(i));
                 n.push_back(E[i].n);
             }
             toff = seg_tile_offsets(n, kScanTile);
@@ -1006,34 +1045,48 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
             if (!bounded) FAST_TRY(t_readback.read(Z + slices[k], slices[k], nseg, 2 * k, s));
         }
     }
-    // count
+    // test
     for (size_t k = 0; k < ns; k++) {
         const size_t e0 = slices[k], nseg = slices[k + 1] - e0;
         if (!bounded) {
             FAST_TRY(t_readback.wait(2 * k));
+            Carver cv;
             for (size_t i = e0; i < e0 + nseg; i++) {
+                cv.add(&E[i].tmp, t_readback.h[i]);
                 const int64_t tiles = std::max<int64_t>(1, ceil_div((int64_t)t_readback.h[i], (int64_t)kListTile));
                 if (tiles > E[i].tiles) return set_error(FAST_ERR_CUDA, "CST build: an edge space exceeded its bound");
                 E[i].tiles = tiles;
             }
+            FAST_TRY(cv.alloc(tmp, false));
         }
-        std::vector<ListDesc> ld;
+        // two launches: the sets that leave three blocks per SM with their
+        // copies in shared memory, and the larger ones; then the tiles' bases
+        std::vector<ListDesc> ld, part[2];
         std::vector<int64_t> n;
         for (size_t i = e0; i < e0 + nseg; i++) {
-            ld.push_back(desc_of(i, false));
+            ld.push_back(desc_of(i));
             n.push_back(E[i].tiles);
+            part[ld.back().words > kSmallSet].push_back(ld.back());
         }
         const std::vector<int64_t> toff = seg_tile_offsets(n, kScanTile);
-        ListChunks lc(ld);
+        const ListChunks lc[2] = {ListChunks(part[0]), ListChunks(part[1])};
         Stage st;
-        const size_t d_at = st.add(ld), i_at = st.add(lc.items), t_at = st.add(toff);
+        const size_t d_at = st.add(ld), t_at = st.add(toff);
+        size_t p_at[2], i_at[2];
+        for (int b = 0; b < 2; b++) {
+            p_at[b] = st.add(part[b]);
+            i_at[b] = st.add(lc[b].items);
+        }
         const size_t z_at = st.zeros((size_t)toff.back() + 1);
         Scratch sc(s);
         FAST_TRY(st.upload(sc));
-        const int cap = lc.cap(ld, sizeof(uint32_t));
-        k_lists<false><<<lc.grid(), kListWarps * 32, cap * sizeof(uint32_t), s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at),
-                                                                                (int)nseg, lc.chunk, cap, g->col);
-        FAST_TRY(note_launch("list count"));
+        for (int b = 0; b < 2; b++) {
+            if (part[b].empty()) continue;
+            const int cap = lc[b].cap(part[b]);
+            k_lists<<<lc[b].grid(), kListWarps * 32, cap * 2 * sizeof(uint32_t), s>>>(
+                st.at<ListDesc>(p_at[b]), st.at<int64_t>(i_at[b]), (int)part[b].size(), lc[b].chunk, cap, g->col);
+            FAST_TRY(note_launch("lists"));
+        }
         const unsigned grid = (unsigned)std::min<int64_t>(toff.back(), (int64_t)num_sms() * 4);
         k_tile_bases<<<grid, kScanBlock, 0, s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(t_at), (int)nseg,
                                                  st.z(z_at), (unsigned int*)st.z(z_at + (size_t)toff.back()));
@@ -1047,7 +1100,7 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
         FAST_TRY(t_readback.wait(2 * ns));
         sizes.assign(t_readback.h, t_readback.h + 4 * ne);
     }
-    // every size is known: the lists' final place, then the write
+    // every size is known: the lists' final place, then the move
     for (size_t i = 0; i < ne; i++) {
         fast_cst* c = Qs[E[i].q].c;
         (E[i].tree ? c->t_entries[E[i].to] : c->n_entries[E[i].e]) = sizes[ne + i];
@@ -1065,24 +1118,25 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
         FAST_TRY(c->arena.block(&b, cv.bytes(), s));
         cv.place(b);
     }
-    // the write, in two launches: the sets that leave several blocks per SM
-    // with their copies in shared memory, and the larger ones
-    for (int big = 0; big < 2; big++) {
+    if (ne) {
         std::vector<ListDesc> ld;
+        std::vector<int64_t> n;
+        int64_t tiles = 0;
         for (size_t i = 0; i < ne; i++) {
-            const ListDesc d = desc_of(i, true);
-            if ((d.words > kSmallSet) == (big != 0)) ld.push_back(d);
+            ld.push_back(desc_of(i));
+            n.push_back(E[i].tiles);
+            tiles += E[i].tiles;
         }
-        if (ld.empty()) continue;
-        ListChunks lc(ld);
+        // a tile per warp while that leaves warps idle, then up to four
+        const int group = (int)std::max<int64_t>(1, std::min<int64_t>(4, tiles / ((int64_t)num_sms() * 48)));
+        for (auto& x : n) x = ceil_div(x, (int64_t)group);
+        const std::vector<int64_t> items = prefix(n);
         Stage st;
-        const size_t d_at = st.add(ld), i_at = st.add(lc.items);
+        const size_t d_at = st.add(ld), i_at = st.add(items);
         Scratch sc(s);
         FAST_TRY(st.upload(sc));
-        const int cap = lc.cap(ld, 2 * sizeof(uint32_t));
-        k_lists<true><<<lc.grid(), kListWarps * 32, cap * 2 * sizeof(uint32_t), s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at),
-                                                                                   (int)ld.size(), lc.chunk, cap, g->col);
-        FAST_TRY(note_launch("list write"));
+        k_list_move<<<warp_grid(items.back(), 6), 256, 0, s>>>(st.at<ListDesc>(d_at), st.at<int64_t>(i_at), (int)ne, group);
+        FAST_TRY(note_launch("list move"));
     }
     return FAST_OK;
 }
@@ -1384,7 +1438,7 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
             const Wave& wv = waves[i];
             if (wv.items == 0) continue;
             unsigned int* nl = (unsigned int*)st.z(z_at + i);
-            k_support<<<warp_grid(wv.items, 8), 256, 0, s>>>(st.at<SetDesc>(wv.d_at), st.at<int64_t>(wv.i_at), (int)wv.d.size(),
+            k_support<<<warp_grid(wv.items, kSupportBlocks), 256, 0, s>>>(st.at<SetDesc>(wv.d_at), st.at<int64_t>(wv.i_at), (int)wv.d.size(),
                                                              wv.group, st.at<Target>(t_at), G, g->col, longs, nl);
             FAST_TRY(note_launch("support"));
             if (hubs) {
@@ -1447,18 +1501,19 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
 
     // ------------------------------------------------------ lists
     //
-    // A small batch reads no edge-space sizes: its tile arrays are sized by
-    // the graph's count of adjacency entries between the two labels.  A larger
-    // one runs slice by slice, the tree edges into one BFS position each (the
+    // A small batch reads no edge-space sizes: its buffers are sized by the
+    // graph's count of adjacency entries between the two labels.  A larger one
+    // runs slice by slice, the tree edges into one BFS position each (the
     // non-tree edges with the first), waiting for a slice's sizes while the
     // device is busy with the next.
     {
-        const bool bounded = nq <= kBoundedQueries && !g->lab_pair_host.empty();
+        bool bounded = nq <= kBoundedQueries && !g->lab_pair_host.empty();
         std::vector<Edge> E;
-        std::vector<size_t> slices{0};
+        std::vector<size_t> cuts;                        // where each position's edges end
+        uint64_t bytes = 0;
         int K = 0;
         for (auto& q : Qs) K = std::max(K, q.k);
-        for (int t = 1; t < std::max(K, 2); t++) {
+        for (int t = 1; t < K; t++) {
             for (int qi = 0; qi < nq; qi++) {
                 const fast_cst* c = Qs[qi].c;
                 if (t < Qs[qi].k) {
@@ -1472,9 +1527,13 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
                         E.push_back(x);
                     }
             }
-            if (!bounded && E.size() > slices.back()) slices.push_back(E.size());
+            cuts.push_back(E.size());
         }
+        for (auto& x : E) bytes += 4ull * (uint64_t)edge_bound(g, Qs[x.q].c, x);
+        if (bytes > kBoundedBytes) bounded = false;
+        std::vector<size_t> slices{0};
         if (bounded && !E.empty()) slices.push_back(E.size());
+        if (!bounded) slices.insert(slices.end(), cuts.begin(), cuts.end());
         for (auto& x : E) x.n = (uint32_t)Qs[x.q].c->ncand[x.from];
         FAST_TRY(build_lists(g, Qs, E, slices, bounded, s));
     }

@@ -301,8 +301,8 @@ int fast_partition_batch(const fast_cst* const* csts, int32_t nq, const fast_con
                          fast_chunks** outs, int32_t* status);
 
 /* Number of chunks, and their summed workload estimate (saturating; summed
- * on request: asking for it reads the descriptors back on the partition's
- * stream and synchronises it). */
+ * on request: asking for it runs on the partition's stream and synchronises
+ * it). */
 int fast_chunks_info(const fast_chunks* ch, int64_t* count, uint64_t* w_sum);
 
 /*

@@ -128,7 +128,7 @@ struct alignas(16) Chunk {
 struct fast_chunks {
     const fast_cst* c = nullptr;
     int64_t n = 0;
-    Chunk* d = nullptr;        // device [n]
+    Chunk* d = nullptr;        // device [n + 1], the last for fast_chunks_info's sum
     cudaStream_t stream = nullptr;
 };
 

@@ -1,7 +1,6 @@
 // The partition's plan and device helpers (Sec. IV-B, Algorithm 2, with the
-// workload estimate of Sec. IV-C), shared by the per-query partition
-// (partition.cu) and the batched one (partition_batch.cu): a CST's arrays
-// by matching-order position, the Generator-side candidate checks of a
+// workload estimate of Sec. IV-C; partition_batch.cu runs them): a CST's
+// arrays by matching-order position, the Generator-side candidate checks of a
 // fixed prefix, and the classification of a pending part.
 #pragma once
 

@@ -1,21 +1,29 @@
-// Batched CST partition (Sec. IV-B, Algorithm 2): the partitions of many
-// queries' CSTs built together, level by level.
+// CST partition (Sec. IV-B, Algorithm 2) driven by the workload estimate of
+// Sec. IV-C, level by level on the device, for one CST or many together.
+//
+// A pending part is a Chunk: positions 0..j-1 fixed (prefix), position j
+// restricted to the run [a, b) of its list L_j.  Its estimate is
+//   W' = F(prefix) * sum_{x in L_j[a..b)} c_{u_j}(x),
+//   F(prefix) = prod over prefix positions p, over children c of p placed
+//               after j, of the per-row child sum s_{p->c}(prefix[p]),
+// which equals the workload DP evaluated on the partitioned tree: restricting
+// a candidate set to the part leaves c unchanged for every candidate still
+// reachable, and every position after j hangs below a prefix position.
 //
 // The pending parts of all queries are one item array, grouped by query in
 // query order (query q owns items qoff[q] .. qoff[q+1]-1); each kernel finds
-// an item's query by binary search and applies that query's plan, with the
-// same device helpers (part_funcs.cuh) as the per-query partition.  A level
-// is one count pass over all items, global exclusive scans, one kernel that
-// gathers each query's totals, and one host round trip for the whole batch;
-// a second pass runs only when some query's level would pass its
-// max_chunks, with that query's split cap (the other queries' counts do not
-// change).  Then the finished chunks are written and the parts of the next
-// level are summed, still grouped by query.  A query whose level hit its cap
-// keeps that level's parts as its last chunks and goes inactive; its items
-// stay in place and every later kernel skips them.  At the end one copy
-// kernel gathers each query's chunk list, level by level, into its own
-// exact-size array -- the same list, in the same order, as fast_partition
-// gives.
+// an item's query by binary search and applies that query's plan.  A level is
+// one kernel that classifies the items and adds up each query's parts, one
+// that applies the split cap of the queries whose level would pass their
+// max_chunks (decided on the device from those sums), scans the items' parts
+// and writes the chunks that are done, one host round trip for the level's
+// sizes, and one warp per part that sums its estimate; the parts of the next
+// level lie grouped by query again.  (Separate scans of three counters, and a
+// second pass with a round trip of its own where a cap applied, made a level
+// eight to fourteen launches.)  A query whose level hit its cap keeps that
+// level's parts as its last chunks and goes inactive; its items stay in place
+// and every later kernel skips them.  At the end one copy kernel gathers each
+// query's chunk list, level by level, into its own exact-size array.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -34,78 +42,156 @@ __device__ __forceinline__ int query_of(const int64_t* __restrict__ qoff, int nq
     return seg_of_tile(qoff, nq, t);
 }
 
-// per query: split cap of this pass (0: none), |C(root)|, and whether it
-// still partitions
+// per query: |C(root)|, whether it still partitions, its chunks so far and
+// how many it may have
 struct QState {
-    uint64_t kcap;
+    int64_t total;
+    int64_t cap;
     uint32_t root_n;
     int32_t active;
 };
 
-// one thread per pending item: classify and count the kept parts (as
-// k_part_count, with the item's plan)
-__global__ void k_part_count_b(const PartPlan* __restrict__ plans, const QState* __restrict__ qs,
-                               const int64_t* __restrict__ qoff, int nq, Chunk* __restrict__ items, int64_t nitems,
-                               int64_t* __restrict__ nparts, int64_t* __restrict__ nemit,
-                               int64_t* __restrict__ nlive) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nitems) return;
-    const int q = query_of(qoff, nq, t);
-    if (!qs[q].active) { nparts[t] = 0; nemit[t] = 0; nlive[t] = 0; return; }
-    const PartPlan& P = plans[q];
-    const uint64_t kcap = qs[q].kcap;
-    Chunk c = items[t];
-    uint64_t kk = 0;
-    int act = classify(P, c, qs[q].root_n, &kk);
-    if (kcap && kk > kcap) kk = kcap;
-    items[t] = c;
-    nlive[t] = act != 0 ? 1 : 0;
+// per query: parts, emitted chunks and live items of a level
+struct QTotals {
+    unsigned long long parts, emit, live;
+};
+
+// The split cap of query q on a level whose uncapped totals are t (0: none): a
+// level that would pass max_chunks caps every split at an even share of the
+// room left.
+__host__ __device__ inline uint64_t split_cap(const QState& q, const QTotals& t) {
+    if (q.total + (int64_t)t.emit + (int64_t)t.parts <= q.cap) return 0;
+    const int64_t nsplit = (int64_t)t.live - (int64_t)t.emit;
+    const int64_t room = q.cap - q.total - (int64_t)t.emit;
+    const int64_t share = nsplit > 0 ? room / nsplit : 1;
+    return (uint64_t)(share > 1 ? share : 1);
+}
+
+__device__ __forceinline__ int64_t kept_parts(const PartPlan& P, const Chunk& c, uint64_t kk) {
+    if (!sampled(P)) return (int64_t)kk;
     int64_t np = 0;
-    if (act == 2) {
-        if (!sampled(P)) np = (int64_t)kk;
-        else
-            for (uint64_t i = 0; i < kk; i++)
-                np += keep_part(P, c.j, kk, mix64(c.id + (i + 1) * 0x9E3779B97F4A7C15ull)) ? 1 : 0;
+    for (uint64_t i = 0; i < kk; i++)
+        np += keep_part(P, c.j, kk, mix64(c.id + (i + 1) * 0x9E3779B97F4A7C15ull)) ? 1 : 0;
+    return np;
+}
+
+// v summed over the lanes of this warp that hold the same query; true on one
+// lane of them (items of a query are neighbours, so mostly one lane adds)
+__device__ __forceinline__ void add_by_query(unsigned long long* dst, int q, unsigned long long v, bool in) {
+    const unsigned int peers = __match_any_sync(0xffffffffu, in ? q : -1);
+    const int lead = __ffs(peers) - 1;
+    unsigned long long sum = 0;
+    for (unsigned int m = peers; __any_sync(0xffffffffu, m != 0); m &= m - 1) {
+        const int l = m ? __ffs(m) - 1 : 0;
+        const unsigned long long x = __shfl_sync(0xffffffffu, v, l);
+        if (m) sum += x;
     }
-    nparts[t] = np;
-    nemit[t] = act == 1 ? 1 : 0;
+    if (in && (int)(threadIdx.x & 31) == lead && sum) atomicAdd(dst, sum);
 }
 
-// per query: parts, emitted chunks and live items of its range
-__global__ void k_part_totals(const int64_t* __restrict__ part_off, const int64_t* __restrict__ emit_off,
-                              const int64_t* __restrict__ live_off, const int64_t* __restrict__ qoff, int nq,
-                              int64_t* __restrict__ out) {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nq) return;
-    const int64_t a = qoff[q], b = qoff[q + 1];
-    out[3 * q + 0] = part_off[b] - part_off[a];
-    out[3 * q + 1] = emit_off[b] - emit_off[a];
-    out[3 * q + 2] = live_off[b] - live_off[a];
+// code of an item: 0 drop, kEmit a finished chunk, else its split factor
+constexpr uint64_t kEmit = ~0ull;
+
+// One thread per pending item: advance and classify it, and add up the
+// uncapped totals of its query.
+__global__ void __launch_bounds__(128) k_part_classify(const PartPlan* __restrict__ plans, const QState* __restrict__ qs,
+                                                       const int64_t* __restrict__ qoff, int nq,
+                                                       Chunk* __restrict__ items, int64_t nitems,
+                                                       uint64_t* __restrict__ code, QTotals* __restrict__ tot) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = t < nitems;
+    int q = -1;
+    uint64_t kk = 0;
+    int act = 0;
+    int64_t np = 0;
+    if (in) {
+        q = query_of(qoff, nq, t);
+        if (qs[q].active) {
+            Chunk c = items[t];
+            act = classify(plans[q], c, qs[q].root_n, &kk);
+            items[t] = c;
+            if (act == 2) np = kept_parts(plans[q], c, kk);
+        }
+        code[t] = act == 1 ? kEmit : act == 2 ? kk : 0ull;
+    }
+    add_by_query(&tot[q < 0 ? 0 : q].parts, q, (unsigned long long)np, in);
+    add_by_query(&tot[q < 0 ? 0 : q].emit, q, act == 1 ? 1ull : 0ull, in);
+    add_by_query(&tot[q < 0 ? 0 : q].live, q, act != 0 ? 1ull : 0ull, in);
 }
 
-// one thread per pending item: emitted chunks, and the part records of
-// sampled splits (as k_part_write)
-__global__ void k_part_write_b(const PartPlan* __restrict__ plans, const QState* __restrict__ qs,
-                               const int64_t* __restrict__ qoff, int nq, const Chunk* __restrict__ items,
-                               int64_t nitems, const int64_t* __restrict__ part_off,
-                               const int64_t* __restrict__ emit_off, PartRec* __restrict__ parts,
-                               Chunk* __restrict__ emitted) {
+// Tiles of 256 items: each item's parts under the cap, their exclusive prefix
+// and that of the finished chunks (two look-backs), the chunks written, and
+// each query's parts.
+constexpr int kPartTile = 256;
+
+__global__ void __launch_bounds__(kPartTile) k_part_offsets(const PartPlan* __restrict__ plans,
+                                                            const QState* __restrict__ qs,
+                                                            const int64_t* __restrict__ qoff, int nq,
+                                                            const Chunk* __restrict__ items, int64_t nitems,
+                                                            const uint64_t* __restrict__ code,
+                                                            const QTotals* __restrict__ tot,
+                                                            unsigned long long* __restrict__ parts_of,
+                                                            int64_t* __restrict__ part_off, Chunk* __restrict__ emitted,
+                                                            unsigned long long* st, unsigned int* ctr) {
+    __shared__ int64_t tmp[kPartTile / 32 + 1];
+    __shared__ int64_t s_t, s_excl[2];
+    const int64_t tiles = (nitems + kPartTile - 1) / kPartTile;
+    for (;;) {
+        if (threadIdx.x == 0) s_t = (int64_t)atomicAdd(ctr, 1u);
+        __syncthreads();
+        const int64_t tl = s_t;
+        if (tl >= tiles) break;
+        const int64_t t = tl * kPartTile + threadIdx.x;
+        const bool in = t < nitems;
+        int q = -1;
+        int64_t v[1] = {0}, e[1] = {0};
+        if (in) {
+            q = query_of(qoff, nq, t);
+            const uint64_t c = code[t];
+            if (c == kEmit) e[0] = 1;
+            else if (c) {
+                const uint64_t cap = split_cap(qs[q], tot[q]);
+                v[0] = kept_parts(plans[q], items[t], cap && c > cap ? cap : c);
+            }
+        }
+        const int64_t np = v[0], ne = e[0];
+        add_by_query(parts_of + (q < 0 ? 0 : q), q, (unsigned long long)np, in);
+        const int64_t vt = block_exclusive_scan<int64_t, kPartTile, 1>(v, tmp);
+        const int64_t et = block_exclusive_scan<int64_t, kPartTile, 1>(e, tmp);
+        if (threadIdx.x < 32) {
+            const int64_t x = tile_publish(st, tl, vt);
+            if (threadIdx.x == 0) s_excl[0] = x;
+        } else if (threadIdx.x < 64) {
+            const int64_t x = tile_publish(st + tiles, tl, et);
+            if (threadIdx.x == 32) s_excl[1] = x;
+        }
+        __syncthreads();
+        if (in) {
+            part_off[t] = s_excl[0] + v[0];
+            if (ne) emitted[s_excl[1] + e[0]] = items[t];
+            if (t == nitems - 1) part_off[nitems] = s_excl[0] + v[0] + np;
+        }
+        __syncthreads();
+    }
+}
+
+// one thread per pending item: the part records of sampled splits (without
+// sampling, k_part_sum derives every part from its item and its index there)
+__global__ void k_part_write(const PartPlan* __restrict__ plans, const QState* __restrict__ qs,
+                             const int64_t* __restrict__ qoff, int nq, const Chunk* __restrict__ items, int64_t nitems,
+                             const uint64_t* __restrict__ code, const QTotals* __restrict__ tot,
+                             const int64_t* __restrict__ part_off, PartRec* __restrict__ parts) {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nitems) return;
     const int q = query_of(qoff, nq, t);
-    if (!qs[q].active) return;
     const PartPlan& P = plans[q];
-    const uint64_t kcap = qs[q].kcap;
-    Chunk c = items[t];
-    int64_t np = part_off[t + 1] - part_off[t];
-    int64_t ne = emit_off[t + 1] - emit_off[t];
-    if (ne) emitted[emit_off[t]] = c;
-    if (!np || !sampled(P)) return;
-    uint32_t n = c.b - c.a;
-    uint64_t kk = c.w / P.delta_w + (c.w % P.delta_w != 0);
-    if (kk > n) kk = n;
+    uint64_t kk = code[t];
+    if (kk == 0 || kk == kEmit || !sampled(P)) return;
+    const uint64_t kcap = split_cap(qs[q], tot[q]);
     if (kcap && kk > kcap) kk = kcap;
-    uint64_t f = prefix_factor(P, c);
+    const Chunk& c = items[t];
+    const uint32_t n = c.b - c.a;
+    const uint64_t f = prefix_factor(P, c);
     int64_t o = part_off[t];
     for (uint64_t i = 0; i < kk; i++) {
         uint64_t id = mix64(c.id + (i + 1) * 0x9E3779B97F4A7C15ull);
@@ -121,10 +207,11 @@ __global__ void k_part_write_b(const PartPlan* __restrict__ plans, const QState*
     }
 }
 
-// one warp per part: W' = F * (saturating sum of c over the run), as
-// k_part_sum; a part of an unsampled query is derived from its item t (the
-// last with part_off[t] <= p) and its index there.
-__global__ void k_part_sum_b(const PartPlan* __restrict__ plans, const int64_t* __restrict__ qoff, int nq,
+// one warp per part: W' = F * (saturating sum of c over the run); a part of an
+// unsampled query is derived from its item t (the last with part_off[t] <= p)
+// and its index i there: run i of the item's kk even runs (the split factor
+// after the cap).
+__global__ void k_part_sum(const PartPlan* __restrict__ plans, const int64_t* __restrict__ qoff, int nq,
                              const Chunk* __restrict__ items, int64_t nitems, const int64_t* __restrict__ part_off,
                              const PartRec* __restrict__ parts, int64_t nparts, Chunk* __restrict__ next) {
     const int lane = threadIdx.x & 31;
@@ -187,17 +274,8 @@ struct QP {
     int64_t cap = 0;                           // max_chunks
     int64_t total = 0;                         // chunks so far
     bool active = false;
-    bool last = false;                         // this level's parts are its last chunks
     std::vector<std::pair<const Chunk*, int64_t>> pieces;   // its chunk list, in order
 };
-
-int fetch_words(const int64_t* d, std::vector<int64_t>& h, size_t words, cudaStream_t s) {
-    h.assign(words, 0);
-    if (!words) return FAST_OK;
-    cudaError_t e = cudaMemcpyAsync(h.data(), d, words * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    return e == cudaSuccess ? FAST_OK : cuda_status(e, "batched partition sizes", __FILE__, __LINE__);
-}
 
 template <class T>
 int upload_array(const std::vector<T>& h, T** d, std::vector<unsigned char*>& own, cudaStream_t s) {
@@ -227,11 +305,9 @@ int partition_all(std::vector<QP>& Q, cudaStream_t s, fast_chunks** outs) {
         const fast_cst* c = Q[q].c;
         plans[q] = make_plan(c, &Q[q].cfg);
         const uint32_t root_n = (uint32_t)c->ncand[c->root];
-        st[q].kcap = 0;
         st[q].root_n = root_n;
         Q[q].cap = Q[q].cfg.max_chunks > 0 ? Q[q].cfg.max_chunks : (1ll << 16);
         Q[q].active = root_n > 0 && c->W > 0;
-        st[q].active = Q[q].active ? 1 : 0;
         if (Q[q].active) {
             Chunk r0;
             memset(&r0, 0, sizeof(r0));
@@ -245,73 +321,71 @@ int partition_all(std::vector<QP>& Q, cudaStream_t s, fast_chunks** outs) {
     FAST_TRY(upload_array(plans, &d_plans, keep.v, s));
     FAST_TRY(upload_array(items0, &items, keep.v, s));
     int64_t nitems = qoff[nq];
-    std::vector<int64_t> tot;
+    bool smp = false;
+    for (auto& q : Q) smp = smp || q.cfg.sample_root > 0.0 || q.cfg.sample_deep > 0.0;
+    // a level's totals: uncapped per query, then the parts under the cap
+    std::vector<QTotals> tot;
+    std::vector<unsigned char> up;
+    const size_t tot_bytes = (size_t)nq * (sizeof(QTotals) + sizeof(unsigned long long));
+    tot.resize(nq + (tot_bytes - nq * sizeof(QTotals) + sizeof(QTotals) - 1) / sizeof(QTotals));
     while (nitems > 0) {
         bool any_active = false;
         for (auto& q : Q) any_active = any_active || q.active;
         if (!any_active) break;
         Owned lvl(s);
-        for (int q = 0; q < nq; q++) { st[q].kcap = 0; st[q].active = Q[q].active ? 1 : 0; }
-        QState* d_st = nullptr;
-        int64_t* d_qoff = nullptr;
-        FAST_TRY(upload_array(st, &d_st, lvl.v, s));
-        FAST_TRY(upload_array(qoff, &d_qoff, lvl.v, s));
-        int64_t* cnt = nullptr;
-        int64_t* d_tot = nullptr;
-        FAST_TRY(dalloc(&cnt, 3 * (nitems + 1), s));
-        lvl.v.push_back((unsigned char*)cnt);
-        FAST_TRY(dalloc(&d_tot, 3 * (size_t)nq, s));
-        lvl.v.push_back((unsigned char*)d_tot);
-        int64_t* part_off = cnt;
-        int64_t* emit_off = cnt + nitems + 1;
-        int64_t* live_off = cnt + 2 * (nitems + 1);
-        for (int pass = 0; pass < 2; pass++) {
-            k_part_count_b<<<(unsigned)ceil_div(nitems, 128), 128, 0, s>>>(d_plans, d_st, d_qoff, nq, items, nitems,
-                                                                            part_off, emit_off, live_off);
-            note_launch();
-            FAST_TRY(scan_exclusive<int64_t>(part_off, part_off, nitems, part_off + nitems, s));
-            FAST_TRY(scan_exclusive<int64_t>(emit_off, emit_off, nitems, emit_off + nitems, s));
-            FAST_TRY(scan_exclusive<int64_t>(live_off, live_off, nitems, live_off + nitems, s));
-            k_part_totals<<<(unsigned)ceil_div(nq, 128), 128, 0, s>>>(part_off, emit_off, live_off, d_qoff, nq, d_tot);
-            note_launch();
-            if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "batched partition launch");
-            FAST_TRY(fetch_words(d_tot, tot, 3 * (size_t)nq, s));
-            if (pass == 1) break;
-            // a level that would pass a query's max_chunks caps every split of
-            // that query at an even share of its room left; the capped parts
-            // are its last chunks
-            bool capped = false;
-            for (int q = 0; q < nq; q++) {
-                if (!Q[q].active) continue;
-                const int64_t np = tot[3 * q], ne = tot[3 * q + 1], nl = tot[3 * q + 2];
-                if (Q[q].total + ne + np <= Q[q].cap) continue;
-                const int64_t nsplit = nl - ne;
-                const int64_t room = Q[q].cap - Q[q].total - ne;
-                st[q].kcap = (uint64_t)std::max<int64_t>(1, nsplit > 0 ? room / nsplit : 1);
-                Q[q].last = true;
-                capped = true;
-            }
-            if (!capped) break;
-            FAST_CUDA(cudaMemcpyAsync(d_st, st.data(), nq * sizeof(QState), cudaMemcpyHostToDevice, s));
+        // one upload: the queries' states and item ranges; behind them, zeroed:
+        // totals, look-back words and the tile counter
+        for (int q = 0; q < nq; q++) {
+            st[q].active = Q[q].active ? 1 : 0;
+            st[q].total = Q[q].total;
+            st[q].cap = Q[q].cap;
         }
-        int64_t np_total = 0, ne_total = 0;
-        for (int q = 0; q < nq; q++) { np_total += tot[3 * q]; ne_total += tot[3 * q + 1]; }
+        const size_t st_bytes = (size_t)nq * sizeof(QState), qo_bytes = (size_t)(nq + 1) * sizeof(int64_t);
+        up.resize(st_bytes + qo_bytes);
+        memcpy(up.data(), st.data(), st_bytes);
+        memcpy(up.data() + st_bytes, qoff.data(), qo_bytes);
+        const int64_t tiles = ceil_div(nitems, (int64_t)kPartTile);
+        const size_t zero = tot_bytes + (size_t)(2 * tiles + 1) * sizeof(unsigned long long);
+        unsigned char* d_up = nullptr;
+        FAST_TRY(dalloc(&d_up, up.size() + zero, s));
+        lvl.v.push_back(d_up);
+        FAST_CUDA(cudaMemcpyAsync(d_up, up.data(), up.size(), cudaMemcpyHostToDevice, s));
+        FAST_CUDA(cudaMemsetAsync(d_up + up.size(), 0, zero, s));
+        const QState* d_st = (const QState*)d_up;
+        const int64_t* d_qoff = (const int64_t*)(d_up + st_bytes);
+        QTotals* d_tot = (QTotals*)(d_up + up.size());
+        unsigned long long* d_parts = (unsigned long long*)(d_tot + nq);
+        unsigned long long* d_look = d_parts + nq;
+        // codes and part offsets of the items; finished chunks (at most one per item)
+        uint64_t* code = nullptr;
+        FAST_TRY(dalloc(&code, 2 * (size_t)nitems + 1, s));
+        lvl.v.push_back((unsigned char*)code);
+        int64_t* part_off = (int64_t*)(code + nitems);
         Chunk* em = nullptr;
-        if (ne_total) {
-            FAST_TRY(dalloc(&em, ne_total, s));
-            keep.v.push_back((unsigned char*)em);
-        }
-        bool smp = false;
-        for (int q = 0; q < nq; q++)
-            if (Q[q].active && (Q[q].cfg.sample_root > 0.0 || Q[q].cfg.sample_deep > 0.0)) smp = true;
+        FAST_TRY(dalloc(&em, (size_t)nitems, s));
+        keep.v.push_back((unsigned char*)em);
+        k_part_classify<<<(unsigned)ceil_div(nitems, 128), 128, 0, s>>>(d_plans, d_st, d_qoff, nq, items, nitems, code, d_tot);
+        note_launch();
+        const unsigned grid = (unsigned)std::min<int64_t>(tiles, (int64_t)num_sms() * 4);
+        k_part_offsets<<<grid, kPartTile, 0, s>>>(d_plans, d_st, d_qoff, nq, items, nitems, code, d_tot, d_parts, part_off, em,
+                                                  d_look, (unsigned int*)(d_look + 2 * tiles));
+        note_launch();
+        cudaError_t e = cudaGetLastError();
+        int lb_err = 0;
+        if (e == cudaSuccess) e = cudaMemcpyFromSymbolAsync(&lb_err, g_lookback_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(tot.data(), d_tot, tot_bytes, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return cuda_status(e, "partition level", __FILE__, __LINE__);
+        if (lb_err) return set_error(FAST_ERR_CUDA, "partition: a look-back wait ran out");
+        const unsigned long long* np_of = (const unsigned long long*)(tot.data() + nq);
+        int64_t np_total = 0;
+        for (int q = 0; q < nq; q++) np_total += (int64_t)np_of[q];
         PartRec* parts = nullptr;
         if (smp) {
             FAST_TRY(dalloc(&parts, std::max<int64_t>(np_total, 1), s));
             lvl.v.push_back((unsigned char*)parts);
-        }
-        if (ne_total || smp) {
-            k_part_write_b<<<(unsigned)ceil_div(nitems, 128), 128, 0, s>>>(d_plans, d_st, d_qoff, nq, items, nitems,
-                                                                            part_off, emit_off, parts, em);
+            k_part_write<<<(unsigned)ceil_div(nitems, 128), 128, 0, s>>>(d_plans, d_st, d_qoff, nq, items, nitems, code, d_tot,
+                                                                       part_off, parts);
             note_launch();
         }
         Chunk* next = nullptr;
@@ -319,22 +393,18 @@ int partition_all(std::vector<QP>& Q, cudaStream_t s, fast_chunks** outs) {
         keep.v.push_back((unsigned char*)next);
         if (np_total) {
             int64_t blocks = std::min<int64_t>(ceil_div(np_total, 8), (int64_t)num_sms() * 32);
-            k_part_sum_b<<<(unsigned)blocks, 256, 0, s>>>(d_plans, d_qoff, nq, items, nitems, part_off, parts, np_total,
-                                                          next);
+            k_part_sum<<<(unsigned)blocks, 256, 0, s>>>(d_plans, d_qoff, nq, items, nitems, part_off, parts, np_total, next);
             note_launch();
         }
-        if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "batched partition launch");
+        if (cudaGetLastError() != cudaSuccess) return set_error(FAST_ERR_CUDA, "partition launch");
         // this level's chunks and the next level's ranges (grouped by query)
         int64_t eo = 0, po = 0;
         for (int q = 0; q < nq; q++) {
-            const int64_t np = tot[3 * q], ne = tot[3 * q + 1];
+            const int64_t np = (int64_t)np_of[q], ne = (int64_t)tot[q].emit;
+            const bool last = Q[q].active && split_cap(st[q], tot[q]) != 0;     // its parts are its last chunks
             if (ne) { Q[q].pieces.push_back({em + eo, ne}); Q[q].total += ne; }
-            if (Q[q].active && Q[q].last) {
-                if (np) { Q[q].pieces.push_back({next + po, np}); Q[q].total += np; }
-                Q[q].active = false;
-            } else if (Q[q].active && np == 0) {
-                Q[q].active = false;
-            }
+            if (last && np) { Q[q].pieces.push_back({next + po, np}); Q[q].total += np; }
+            if (last || np == 0) Q[q].active = false;
             qoff[q + 1] = qoff[q] + np;
             eo += ne;
             po += np;
@@ -351,7 +421,7 @@ int partition_all(std::vector<QP>& Q, cudaStream_t s, fast_chunks** outs) {
         ch->n = Q[q].total;
         ch->stream = s;
         outs[Q[q].idx] = ch;
-        FAST_TRY(dalloc_direct(&ch->d, Q[q].total, s));                 // outlives the call
+        FAST_TRY(dalloc_direct(&ch->d, Q[q].total + 1, s));             // outlives the call; one more: fast_chunks_info
         int64_t o = 0;
         for (auto& pc : Q[q].pieces) {
             const uint64_t bytes = (uint64_t)pc.second * sizeof(Chunk);

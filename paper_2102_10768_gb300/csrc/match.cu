@@ -565,8 +565,8 @@ __device__ void validate_tasks(const MatchPlan& P0, const MatchPlan* __restrict_
 // loaded once for 32 candidates).  make_plan decides.  Measured, before and
 // after: complete enumeration of a 10-vertex tree query with two-entry lists
 // (31 M embeddings) 24.7 -> 1.9 ms; of 12 4-vertex queries on the 1M/16M
-// power-law graph (3.2 G embeddings) 106 -> 41 ms; 8.4 M rows written 2.9 ->
-// 2.0 ms.
+// power-law graph (3.2 G embeddings) 106 -> 41 ms, and 18 with the short form
+// of the last position; 8.4 M rows written 2.9 -> 2.0 ms.
 //
 // Order of work, totals, floor and donations are as in the other search: a
 // donated run is the list of one partial result, or the second half of what is
@@ -576,11 +576,13 @@ struct FlatState {
     uint32_t iter;
 };
 
+constexpr int kFlatSame = 4;     // same-label positions the short form of the last position handles
+
 struct FlatBuf {
     uint32_t v[32];          // candidate index
     int32_t g[32];           // data vertex
-    uint32_t lo[32];         // its list into the next position: start
-    uint32_t pf[32];         //   and first index in the range of all
+    uint32_t pf[32];         // its list into the next position: first index in the range of all
+    uint32_t lo[32];         //   and what to add to an index of the range to index the list's array
     uint32_t mt[32];         // slot in the previous buffer | generator list << 8
 };
 static_assert(sizeof(FlatBuf) == kFlatWords * 4, "a flat buffer is kFlatWords words");
@@ -687,6 +689,88 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
             continue;
         }
         const FlatBuf* Bp = d > j ? &B[d - 1] : nullptr;
+        const uint32_t same = P.same_lab[d];
+        const int e0 = P.nt_begin[d], ne = P.nt_begin[d + 1] - e0;
+        if (!EMIT && !STATS && d == k - 1 && Bp && ne == 0 && end - cur > 128 && __popc(same) <= kFlatSame) {
+            // The last position with nothing to check but the images: its
+            // entries 128 at a time until the range ends or the next periodic
+            // check is due.  The range's lists are all non-empty, so an
+            // entry's list is the number of list starts up to it (one mask per
+            // 32 entries); a lane holds the images of its own partial result
+            // at the positions with this label, and an entry's come by one
+            // shuffle each.  22 instructions per 32 entries where the general
+            // step below takes over a hundred.  (Up to 128 entries, where the
+            // set-up would outweigh the steps saved, the general one; as a
+            // function of its own this was no faster.)
+            const int m = (int)__shfl_sync(0xffffffffu, cnt, d - 1);
+            const uint32_t* __restrict__ gi = P.t_idx[d];
+            const int32_t* __restrict__ cd = P.cand[d];
+            const uint32_t pf = lane < m ? Bp->pf[lane] : ~0u;
+            const uint32_t le = lanemask_lt() | (1u << lane);
+            int32_t img[kFlatSame];
+            const int na = __popc(same);
+            {
+                int a = lane < m ? lane : 0, x = na;
+                for (int t = d - 1; t >= j; t--) {
+                    if ((same >> t) & 1u) {
+                        x--;
+#pragma unroll
+                        for (int y = 0; y < kFlatSame; y++) if (y == x) img[y] = B[t].g[a];
+                    }
+                    a = (int)(B[t].mt[a] & 255u);
+                }
+                int y0 = 0;
+                for (uint32_t f = same & ((1u << j) - 1); f; f &= f - 1, y0++)
+#pragma unroll
+                    for (int y = 0; y < kFlatSame; y++) if (y == y0) img[y] = sg[__ffs(f) - 1];
+            }
+            uint32_t i0 = cur;
+            int started = __popc(__ballot_sync(0xffffffffu, pf < i0));
+            uint32_t mine = 0, bytes = 0;
+            for (;;) {
+                uint32_t x[4];
+                int sl[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const uint32_t i = i0 + 32 * u;
+                    const uint32_t heads = __reduce_or_sync(0xffffffffu, pf - i < 32u ? 1u << (pf - i) : 0u);
+                    sl[u] = started + __popc(heads & le) - 1;
+                    started += __popc(heads);
+                    x[u] = ~0u;
+                    if (i + lane < end) { x[u] = __ldg(gi + (Bp->lo[sl[u]] + i + lane)); bytes += 4; }
+                }
+                if (same) {
+                    int32_t gc[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        gc[u] = x[u] != ~0u ? __ldg(cd + x[u]) : 0;
+                        bytes += x[u] != ~0u ? 4 : 0;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        bool ok = x[u] != ~0u;
+#pragma unroll
+                        for (int y = 0; y < kFlatSame; y++)
+                            if (y < na && __shfl_sync(0xffffffffu, img[y], sl[u] & 31) == gc[u]) ok = false;
+                        mine += ok ? 1u : 0u;
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < 4; u++) mine += x[u] != ~0u ? 1u : 0u;
+                }
+                i0 += 128;
+                if (i0 >= end || ((F.iter + 1) & 15) == 0) break;
+                if (O.limit && F.local + __reduce_add_sync(0xffffffffu, mine) >= O.flush_at) break;
+                ++F.iter;
+            }
+            const uint32_t found = __reduce_add_sync(0xffffffffu, mine);
+            F.local += found;
+            F.ccount += found;
+            F.lb += bytes;
+            if (lane == 0) F.fb += (same ? 8ull : 4ull) * ((i0 < end ? i0 : end) - cur);
+            if (lane == d - 1) vcur = i0;
+            continue;
+        }
         const uint32_t n = end - cur < 32 ? end - cur : 32;
         bool ok = lane < (int)n;
         int sl = 0, src = src0;                        // the partial result this entry extends, and its generator
@@ -697,10 +781,9 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
 #pragma unroll
             for (int st = 16; st; st >>= 1)
                 if (sl + st < m && Bp->pf[sl + st] <= e) sl += st;
-            at = Bp->lo[sl] + (e - Bp->pf[sl]);
+            at = Bp->lo[sl] + e;
             src = (int)(Bp->mt[sl] >> 8);
         }
-        const int e0 = P.nt_begin[d], ne = P.nt_begin[d + 1] - e0;
         uint32_t cnd = at;
         if (d > 0) {
             if (ok) { cnd = __ldg((src == 0 ? P.t_idx[d] : P.n_idx[e0 + src - 1]) + at); F.lb += 4; }
@@ -728,7 +811,6 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
         }
         // ---- VisitedValidator
         int32_t gc = -1;
-        const uint32_t same = P.same_lab[d];
         if (same || (EMIT && d == k - 1)) {
             if (same) {
                 const uint32_t pm = __ballot_sync(0xffffffffu, ok);
@@ -818,12 +900,23 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
         }
         const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
         __syncwarp();
-        if (lane < m) {
-            Bd->lo[lane] = llo;
-            Bd->pf[lane] = inc - len;
-            Bd->mt[lane] |= (uint32_t)gen << 8;
+        // those with nothing to extend them go: the others, in order, from slot 0
+        const uint32_t some = __ballot_sync(0xffffffffu, len > 0);
+        if (!some) continue;
+        const bool gaps = __popc(some) < m;
+        uint32_t v0 = 0, m0 = 0;
+        int32_t g0 = 0;
+        if (gaps && len > 0) { v0 = Bd->v[lane]; g0 = Bd->g[lane]; }
+        if (len > 0) m0 = Bd->mt[lane];
+        __syncwarp();
+        if (len > 0) {
+            const int i = __popc(some & lanemask_lt());
+            if (gaps) { Bd->v[i] = v0; Bd->g[i] = g0; }
+            Bd->mt[i] = m0 | (uint32_t)gen << 8;
+            Bd->pf[i] = inc - len;
+            Bd->lo[i] = llo - (inc - len);
         }
-        if (lane == d) { cnt = (uint32_t)m; vcur = 0; vend = total; }
+        if (lane == d) { cnt = (uint32_t)__popc(some); vcur = 0; vend = total; }
         __syncwarp();
         d = w;
     }

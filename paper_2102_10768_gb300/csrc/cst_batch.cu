@@ -38,7 +38,6 @@
 // with about 50 launches where there were 464.
 #include <algorithm>
 #include <cstring>
-#include <map>
 #include <mutex>
 #include <vector>
 
@@ -827,7 +826,7 @@ struct Q {
     int k = 0;
     bool nlf = false;
     bool nt_refine = false;       // refine rule 2: the non-tree test in the bottom-up pass
-    int A[kMaxK][kMaxK] = {};
+    uint32_t adj[kMaxK] = {};     // neighbours of each vertex, a bit mask
     int dq[kMaxK] = {};
     int bpos[kMaxK] = {};         // vertex -> BFS position
     int depth[kMaxK] = {};        // vertex -> depth in t_q
@@ -846,8 +845,8 @@ struct Q {
 // Matching order and non-tree edges of one query from its refined candidate
 // counts.
 void order_and_nontree(const Q& q, fast_cst* c) {
-    fast::matching_order(q.k, q.A, c->root, c->parent, c->bfs, c->ncand, c->cfg.order_rule, c->order, c->pos);
-    c->nnt = nontree_edges(q.k, q.A, c->order, c->parent, c->nt_from, c->nt_to);
+    fast::matching_order(q.k, q.adj, c->root, c->parent, c->bfs, c->ncand, c->cfg.order_rule, c->order, c->pos);
+    c->nnt = nontree_edges(q.k, q.adj, c->order, c->parent, c->nt_from, c->nt_to);
 }
 
 thread_local uint64_t t_round_trips = 0;   // this thread's last batched build
@@ -1262,9 +1261,13 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
     {
         std::vector<FilterDesc> fd;
         std::vector<std::pair<int, int>> rep;             // fd[i]'s (query, vertex)
-        std::map<std::vector<int64_t>, int> seen;
         Carver cv;
         int64_t maxw = 1;
+        size_t vertices = 0;
+        for (auto& q : Qs) vertices += q.k;
+        size_t slots = 64;
+        while (slots < 2 * vertices) slots *= 2;
+        std::vector<int32_t> table(slots, -1);            // open addressing: indices into fd
         for (int qi = 0; qi < nq; qi++) {
             Q& q = Qs[qi];
             for (int u = 0; u < q.k; u++) {
@@ -1279,30 +1282,32 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
                 d.base = q.base[u];
                 d.words = q.words[u];
                 d.dq = q.dq[u];
-                std::vector<int64_t> key{d.lo, d.hi, d.dq};
                 if (q.nlf) {
-                    for (int w = 0; w < q.k; w++) {
-                        if (!q.A[u][w]) continue;
-                        const int32_t lw = q.c->qlabel[w];
-                        int t = 0;
-                        while (t < d.r.nn && d.r.lab[t] != lw) t++;
-                        if (t == d.r.nn) { d.r.lab[t] = lw; d.r.need[t] = 0; d.r.nn++; }
+                    for (uint32_t f = q.adj[u]; f; f &= f - 1) {
+                        const int32_t lw = q.c->qlabel[__builtin_ctz(f)];
+                        int t = 0;                        // in label order: equal requirements compare equal
+                        while (t < d.r.nn && d.r.lab[t] < lw) t++;
+                        if (t == d.r.nn || d.r.lab[t] != lw) {
+                            for (int x = d.r.nn++; x > t; x--) { d.r.lab[x] = d.r.lab[x - 1]; d.r.need[x] = d.r.need[x - 1]; }
+                            d.r.lab[t] = lw;
+                            d.r.need[t] = 0;
+                        }
                         d.r.need[t]++;
                     }
-                    // in label order, so that equal requirements give equal keys
-                    for (int a = 1; a < d.r.nn; a++)
-                        for (int b = a; b > 0 && d.r.lab[b - 1] > d.r.lab[b]; b--) {
-                            std::swap(d.r.lab[b - 1], d.r.lab[b]);
-                            std::swap(d.r.need[b - 1], d.r.need[b]);
-                        }
-                    for (int t = 0; t < d.r.nn; t++) { key.push_back(d.r.lab[t]); key.push_back(d.r.need[t]); }
                 }
-                auto it = seen.find(key);
-                if (it != seen.end()) {
-                    alias[(size_t)u * nq + qi] = rep[it->second];
+                uint64_t hash = mix64((uint64_t)d.lo) ^ mix64((uint64_t)d.dq << 8 | (uint64_t)d.r.nn);
+                for (int t = 0; t < d.r.nn; t++) hash = mix64(hash ^ ((uint64_t)(uint32_t)d.r.lab[t] << 32 | (uint32_t)d.r.need[t]));
+                size_t at = hash & (slots - 1);
+                while (table[at] >= 0) {
+                    const FilterDesc& o = fd[table[at]];
+                    if (o.lo == d.lo && o.hi == d.hi && o.dq == d.dq && memcmp(&o.r, &d.r, sizeof(d.r)) == 0) break;
+                    at = (at + 1) & (slots - 1);
+                }
+                if (table[at] >= 0) {
+                    alias[(size_t)u * nq + qi] = rep[table[at]];
                     continue;
                 }
-                seen.emplace(std::move(key), (int)fd.size());
+                table[at] = (int32_t)fd.size();
                 rep.push_back({qi, u});
                 fd.push_back(d);
                 maxw = std::max<int64_t>(maxw, q.words[u]);
@@ -1342,7 +1347,7 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
             c0[u] = a.first >= 0 ? h[(size_t)a.second * nq + a.first] : h[(size_t)u * nq + qi];
         }
         c->root = choose_root(q.k, c0, q.dq);
-        bfs_tree(q.k, q.A, c->root, c->bfs, c->parent);
+        bfs_tree(q.adj, c->root, c->bfs, c->parent);
         for (int t = 0; t < q.k; t++) {
             const int u = c->bfs[t];
             q.bpos[u] = t;
@@ -1401,7 +1406,7 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
                     if (q.nt_refine ? t != q.k - 1 - b : q.depth[u] != max_depth - b) continue;
                     const int32_t t0 = (int32_t)tg.size();
                     for (int w = 0; w < q.k; w++)
-                        if (q.c->parent[w] == u || (q.nt_refine && q.A[u][w] && q.c->parent[u] != w)) target(qi, w);
+                        if (q.c->parent[w] == u || (q.nt_refine && (q.adj[u] >> w & 1u) && q.c->parent[u] != w)) target(qi, w);
                     const int32_t nt = (int32_t)tg.size() - t0;
                     if (!nt) continue;                       // a leaf: its set is final
                     wv.d.push_back({q.cur[u], q.set[u], zp(F_C + u, qi), q.base[u], q.words[u], t0, nt});
@@ -1581,7 +1586,7 @@ int build_cst_batch(const fast_graph* g, int32_t nq, const fast_query_desc* qs, 
         Qs.reserve(g1 - g0);
         for (int i = g0; i < g1; i++) {
             Q q;
-            int rc = validate_query(&qs[i], q.A, q.dq);
+            int rc = validate_query(&qs[i], q.adj, q.dq);
             const fast_config* cf = cfgs[i];
             if (rc == FAST_OK && cf && (cf->order_rule < 0 || cf->order_rule > 3))
                 rc = set_error(FAST_ERR_INVALID,

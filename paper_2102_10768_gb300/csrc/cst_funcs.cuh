@@ -97,30 +97,33 @@ __device__ __forceinline__ double warp_sum_f(double v) {
     return v;
 }
 
-inline int validate_query(const fast_query_desc* q, int A[kMaxK][kMaxK], int* dq) {
+// Checks a query; adj[u]: the neighbours of u as a bit mask, dq[u] its degree.
+inline int validate_query(const fast_query_desc* q, uint32_t* adj, int* dq) {
     if (!q) return set_error(FAST_ERR_INVALID, "query is NULL");
     int k = q->n;
     if (k < 1 || k > kMaxK) return set_error(FAST_ERR_INVALID, "query has %d vertices (1..%d)", k, kMaxK);
     if (!q->labels || (q->m > 0 && !q->edges) || q->m < 0) return set_error(FAST_ERR_INVALID, "query arrays are NULL");
-    memset(A, 0, sizeof(int) * kMaxK * kMaxK);
     for (int u = 0; u < k; u++) {
         dq[u] = 0;
+        adj[u] = 0;
         if (q->labels[u] < 0) return set_error(FAST_ERR_INVALID, "query label < 0");
     }
     for (int e = 0; e < q->m; e++) {
         int a = q->edges[2 * e], b = q->edges[2 * e + 1];
         if (a < 0 || b < 0 || a >= k || b >= k) return set_error(FAST_ERR_INVALID, "query edge (%d,%d) out of range", a, b);
         if (a == b) return set_error(FAST_ERR_INVALID, "query edge (%d,%d) is a loop", a, b);
-        if (!A[a][b]) { A[a][b] = A[b][a] = 1; dq[a]++; dq[b]++; }
+        adj[a] |= 1u << b;
+        adj[b] |= 1u << a;
     }
+    for (int u = 0; u < k; u++) dq[u] = __builtin_popcount(adj[u]);
     // connected?
-    int seen[kMaxK] = {0}, st[kMaxK], sp = 0, cnt = 1;
-    st[sp++] = 0; seen[0] = 1;
-    while (sp) {
-        int u = st[--sp];
-        for (int w = 0; w < k; w++) if (A[u][w] && !seen[w]) { seen[w] = 1; st[sp++] = w; cnt++; }
+    uint32_t seen = 1u, todo = 1u;
+    while (todo) {
+        const uint32_t fresh = adj[__builtin_ctz(todo)] & ~seen;
+        todo = (todo & (todo - 1)) | fresh;
+        seen |= fresh;
     }
-    if (cnt != k) return set_error(FAST_ERR_INVALID, "query graph is disconnected");
+    if (__builtin_popcount(seen) != k) return set_error(FAST_ERR_INVALID, "query graph is disconnected");
     return FAST_OK;
 }
 
@@ -140,15 +143,19 @@ inline int choose_root(int k, const int64_t* c0, const int* dq) {
 
 // BFS tree t_q from r, neighbours visited in increasing id: bfs[] is the
 // visiting order, parent[r] = -1.
-inline void bfs_tree(int k, const int A[kMaxK][kMaxK], int r, int* bfs, int* parent) {
-    int seen[kMaxK] = {0}, qh = 0, qt = 0;
+inline void bfs_tree(const uint32_t* adj, int r, int* bfs, int* parent) {
+    int qh = 0, qt = 0;
+    uint32_t seen = 1u << r;
     bfs[qt++] = r;
-    seen[r] = 1;
     parent[r] = -1;
     while (qh < qt) {
         const int u = bfs[qh++];
-        for (int w = 0; w < k; w++)
-            if (A[u][w] && !seen[w]) { seen[w] = 1; parent[w] = u; bfs[qt++] = w; }
+        for (uint32_t f = adj[u] & ~seen; f; f &= f - 1) {
+            const int w = __builtin_ctz(f);
+            parent[w] = u;
+            bfs[qt++] = w;
+        }
+        seen |= adj[u];
     }
 }
 
@@ -161,7 +168,7 @@ inline void bfs_tree(int k, const int A[kMaxK][kMaxK], int r, int* bfs, int* par
 // vertex whose t_q parent is placed with the fewest candidates; ties to the
 // smaller id.  Every rule places a vertex after its t_q parent.  Writes
 // order[position] and pos[vertex].
-inline void matching_order(int k, const int A[kMaxK][kMaxK], int r, const int* parent, const int* bfs,
+inline void matching_order(int k, const uint32_t* adj, int r, const int* parent, const int* bfs,
                            const int64_t* ncand, int rule, int* order, int* pos) {
     if (rule == 2) {
         for (int i = 0; i < k; i++) order[i] = bfs[i];
@@ -179,22 +186,20 @@ inline void matching_order(int k, const int A[kMaxK][kMaxK], int r, const int* p
             placed[best] = true;
         }
     } else if (rule == 1) {
-        bool placed[kMaxK] = {false};
+        uint32_t placed = 1u << r;
         order[0] = r;
-        placed[r] = true;
         for (int no = 1; no < k; no++) {
             int best = -1, bb = -1;
             for (int u = 0; u < k; u++) {
-                if (placed[u] || !placed[parent[u]]) continue;
-                int b = 0;
-                for (int w = 0; w < k; w++) b += (placed[w] && A[u][w]) ? 1 : 0;
+                if ((placed >> u & 1u) || !(placed >> parent[u] & 1u)) continue;
+                const int b = __builtin_popcount(adj[u] & placed);
                 if (best < 0 || b > bb || (b == bb && (ncand[u] < ncand[best] || (ncand[u] == ncand[best] && u < best)))) {
                     best = u;
                     bb = b;
                 }
             }
             order[no] = best;
-            placed[best] = true;
+            placed |= 1u << best;
         }
     } else {
         int stack[kMaxK], sp = 0, no = 0;
@@ -219,13 +224,13 @@ inline void matching_order(int k, const int A[kMaxK][kMaxK], int r, const int* p
 // Non-tree edges of q, each once, from the earlier to the later endpoint in
 // the order, listed by the later endpoint's position, then the earlier's.
 // Returns their number.
-inline int nontree_edges(int k, const int A[kMaxK][kMaxK], const int* order, const int* parent, int* from, int* to) {
+inline int nontree_edges(int k, const uint32_t* adj, const int* order, const int* parent, int* from, int* to) {
     int n = 0;
     for (int i = 0; i < k; i++) {
         const int ui = order[i];
         for (int j = 0; j < i; j++) {
             const int uj = order[j];
-            if (!A[ui][uj] || parent[ui] == uj || parent[uj] == ui) continue;
+            if (!(adj[ui] >> uj & 1u) || parent[ui] == uj || parent[uj] == ui) continue;
             from[n] = uj;
             to[n] = ui;
             n++;

@@ -208,79 +208,56 @@ __device__ __forceinline__ bool bsearch_u32(const uint32_t* __restrict__ a, int6
 //   - load a tile of 128 entries, four per lane with one 16-byte load (the
 //     list is taken from the 16-byte boundary at or before its start, which
 //     lies in the same array; positions here count from there);
-//   - every pending lane whose candidate is <= the tile's last entry finds
-//     the four entries that hold its lower bound by a 5-step shuffle search
-//     over the lanes' last entries, and compares all four;
-//   - if the smallest pending candidate lies beyond the tile, gallop: lanes
-//     probe pos + 128*2^i in one round, then 33-way refinement rounds, each a
-//     single parallel read, until one tile holds its lower bound.
+//   - every lane whose candidate is <= the tile's last entry finds the four
+//     entries that hold its lower bound by a 5-step shuffle search over the
+//     lanes' last entries, and compares all four;
+//   - candidates past the tile are found together: lanes probe pos + 128*2^i
+//     in one round, which bounds the window that holds them all, then 32 even
+//     places of the window; each lane finds its part of the window by a
+//     5-step shuffle search and its entry there by a binary search.
 // Returns whether this lane's candidate is in the list; *lb counts the bytes
 // of the list that this lane read.
-// A tile of 128 costs 9 shuffles where four tiles of 32 cost 28, and the lists
-// checked hold some four entries per entry of the generator: 250 queries' step
-// 86.2 -> 77.6 ms, 40 queries' 18.2 -> 16.5 ms.
+//
+// Bound by the instructions of the shuffles and by the latency of one load
+// after another.  A tile of 128 costs 9 shuffles where four tiles of 32 cost
+// 28: a step of 250 queries 86.2 -> 77.6 ms.  The candidates of one segment
+// spread over 3.4 tiles on average (17.9 M tiles for 5.2 M segments in a step
+// of 40 queries), so one window search for all that lie past the first tile
+// replaces the walk: 250 queries 68.1 -> 66.6 ms, one query of 32 vertices
+// 1.18 -> 1.12 ms.
 __device__ __forceinline__ bool warp_member(const uint32_t* __restrict__ L, uint32_t n, uint32_t* pos,
                                             uint32_t c, bool act, unsigned long long* lb) {
     const int lane = threadIdx.x & 31;
-    bool found = false;
-    uint32_t pend = __ballot_sync(0xffffffffu, act);
+    const uint32_t pend0 = __ballot_sync(0xffffffffu, act);
     const uint32_t head = (uint32_t)((uintptr_t)L >> 2) & 3u;   // entries before the list in its first 16 bytes
     const uint32_t* La = L - head;
     const uint32_t end = n ? n + head : 0u;
-    uint32_t p0 = *pos;                                    // a multiple of 4
-    uint32_t last = p0;
-    while (pend) {
-        if (p0 >= end) break;                              // list exhausted: the rest are absent
-        const uint32_t ct = __shfl_sync(0xffffffffu, c, __ffs(pend) - 1);     // smallest pending candidate
-        const uint32_t i = p0 + 4 * lane;
-        uint4 v = make_uint4(~0u, ~0u, ~0u, ~0u);
-        if (i < end) {
-            v = __ldg((const uint4*)(La + i));
-            *lb += 16;
-            if (i + 4 > end) {                             // entries past the list: above every candidate
-                if (i + 1 >= end) v.y = ~0u;
-                if (i + 2 >= end) v.z = ~0u;
-                v.w = ~0u;
-                *lb -= 4 * (i + 4 - end);
-            }
-            if (i < head) {                                // entries before it: its first one, again
-                const uint32_t f = head == 1 ? v.y : head == 2 ? v.z : v.w;
-                v.x = f;
-                if (head > 1) v.y = f;
-                if (head > 2) v.z = f;
-                *lb -= 4 * head;
-            }
+    const uint32_t p0 = *pos;                              // a multiple of 4
+    if (!pend0 || p0 >= end) return false;                 // list exhausted: absent
+    const uint32_t i = p0 + 4 * lane;
+    uint4 v = make_uint4(~0u, ~0u, ~0u, ~0u);
+    uint32_t bytes = 0;
+    if (i < end) {
+        v = __ldg((const uint4*)(La + i));
+        bytes = 16;
+        if (i + 4 > end) {                                 // entries past the list: above every candidate
+            if (i + 1 >= end) v.y = ~0u;
+            if (i + 2 >= end) v.z = ~0u;
+            v.w = ~0u;
+            bytes -= 4 * (i + 4 - end);
         }
-        const uint32_t tmax = __shfl_sync(0xffffffffu, v.w, 31);
-        if (tmax < ct) {
-            // gallop: the lower bound of ct lies past this (full) tile
-            uint32_t a = p0 + 128;                          // first index that may hold it
-            uint32_t probe = p0 + 127 + (128u << (lane < 23 ? lane : 23));   // below 2^32: p0 < 2^31
-            if (probe > end - 1) probe = end - 1;
-            uint32_t pv = __ldg(La + probe);
-            *lb += 4;
-            uint32_t ge = __ballot_sync(0xffffffffu, pv >= ct);
-            if (!ge) { p0 = end; break; }                   // everything left is smaller: all absent
-            int f = __ffs(ge) - 1;
-            uint32_t b = __shfl_sync(0xffffffffu, probe, f);            // L[b] >= ct
-            if (f > 0) a = __shfl_sync(0xffffffffu, probe, f - 1) + 1; // L[a-1] < ct
-            while (b - a > 124) {                           // 33-way refinement of [a, b]
-                const uint64_t span = b - a + 1;
-                uint32_t q = a + (uint32_t)(((uint64_t)(lane + 1) * span) / 33);
-                uint32_t qv = __ldg(La + q);
-                *lb += 4;
-                uint32_t g2 = __ballot_sync(0xffffffffu, qv >= ct);
-                int f2 = g2 ? __ffs(g2) - 1 : 32;
-                uint32_t nb = f2 < 32 ? __shfl_sync(0xffffffffu, q, f2 < 32 ? f2 : 0) : b;
-                uint32_t na = f2 > 0 ? __shfl_sync(0xffffffffu, q, f2 > 0 ? f2 - 1 : 0) + 1 : a;
-                a = na;
-                b = nb;
-            }
-            p0 = a & ~3u;
-            continue;
+        if (i < head) {                                    // entries before it: its first one, again
+            const uint32_t f = head == 1 ? v.y : head == 2 ? v.z : v.w;
+            v.x = f;
+            if (head > 1) v.y = f;
+            if (head > 2) v.z = f;
+            bytes -= 4 * head;
         }
-        // resolve every pending lane whose candidate is within this tile
-        const bool mine = ((pend >> lane) & 1u) && c <= tmax;
+    }
+    const uint32_t tmax = __shfl_sync(0xffffffffu, v.w, 31);
+    bool found = false;
+    const uint32_t here = __ballot_sync(0xffffffffu, act && c <= tmax);
+    if (here) {
         int q = 0;
 #pragma unroll
         for (int st = 16; st; st >>= 1) {
@@ -289,12 +266,52 @@ __device__ __forceinline__ bool warp_member(const uint32_t* __restrict__ L, uint
         }
         const uint32_t x0 = __shfl_sync(0xffffffffu, v.x, q), x1 = __shfl_sync(0xffffffffu, v.y, q);
         const uint32_t x2 = __shfl_sync(0xffffffffu, v.z, q), x3 = __shfl_sync(0xffffffffu, v.w, q);
-        if (mine) found = x0 == c || x1 == c || x2 == c || x3 == c;
-        pend &= ~__ballot_sync(0xffffffffu, mine);
-        last = p0;
-        p0 += 128;
+        if ((here >> lane) & 1u) found = x0 == c || x1 == c || x2 == c || x3 == c;
     }
-    *pos = last;
+    const uint32_t pend = pend0 & ~here;
+    uint32_t a = p0 + 128;                                 // first index that may hold one of the rest
+    if (pend && a < end) {
+        const int top = 31 - __clz(pend);
+        const uint32_t ct = __shfl_sync(0xffffffffu, c, __ffs(pend) - 1), cm = __shfl_sync(0xffffffffu, c, top);
+        uint32_t probe = p0 + 127 + (128u << (lane < 23 ? lane : 23));   // below 2^32: p0 < 2^31
+        if (probe > end - 1) probe = end - 1;
+        const uint32_t pv = __ldg(La + probe);
+        bytes += 4;
+        const int below = __popc(__ballot_sync(0xffffffffu, pv < ct));   // a prefix of the lanes
+        if (below == 32) {                                 // all that is left is smaller, for later candidates too
+            *pos = (end + 3u) & ~3u;
+            *lb += bytes;
+            return found;
+        }
+        const uint32_t ge = __ballot_sync(0xffffffffu, pv >= cm);
+        uint32_t b = __shfl_sync(0xffffffffu, probe, ge ? __ffs(ge) - 1 : 31);   // L[b] >= cm, or the last entry
+        if (below) a = __shfl_sync(0xffffffffu, probe, below - 1) + 1;
+        const uint32_t part = (b - a + 32) >> 5;           // ceil((b - a + 1) / 32)
+        uint32_t si = a + (lane + 1) * part - 1;
+        if (si > b) si = b;
+        const uint32_t sv = __ldg(La + si);
+        bytes += 4;
+        int q = 0;
+#pragma unroll
+        for (int st = 16; st; st >>= 1) {
+            const uint32_t w = __shfl_sync(0xffffffffu, sv, q + st - 1);
+            if (w < c) q += st;
+        }
+        uint32_t lo = a + q * part, hi = lo + part - 1;
+        if (hi > b) hi = b;
+        if (lo > b) lo = b;
+        if ((pend >> lane) & 1u) {
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (__ldg(La + mid) < c) lo = mid + 1; else hi = mid;
+                bytes += 4;
+            }
+            found = __ldg(La + lo) == c;
+            bytes += 4;
+        }
+        *pos = __shfl_sync(0xffffffffu, lo, top) & ~3u;    // later candidates lie past the largest of these
+    }
+    *lb += bytes;
     return found;
 }
 

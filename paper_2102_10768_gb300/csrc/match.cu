@@ -593,6 +593,11 @@ struct FlatState {
     uint32_t iter;
 };
 
+constexpr int kFlatU = 2;        // quads per lane in flight there (1: 3.5 G embeddings 16.5 instead of 15.4 ms; 4: 15.8)
+// Entries of the shortest range it is used for.  A range of up to 32 is one
+// general step; with the line at 128, 3.5 G embeddings took 16.7 instead of
+// 15.4 ms and two-entry lists 2.38 instead of 2.11 ms.
+constexpr uint32_t kFlatQuads = 32;
 constexpr int kFlatSame = 4;     // same-label positions the short form of the last position handles
 
 struct FlatBuf {
@@ -708,27 +713,45 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
         const FlatBuf* Bp = d > j ? &B[d - 1] : nullptr;
         const uint32_t same = P.same_lab[d];
         const int e0 = P.nt_begin[d], ne = P.nt_begin[d + 1] - e0;
-        if (!EMIT && !STATS && d == k - 1 && Bp && ne == 0 && end - cur > 128 && __popc(same) <= kFlatSame) {
+        if (!EMIT && !STATS && d == k - 1 && Bp && ne == 0 && end - cur > kFlatQuads && __popc(same) <= kFlatSame) {
             // The last position with nothing to check but the images: its
-            // entries 128 at a time until the range ends or the next periodic
-            // check is due.  The range's lists are all non-empty, so an
-            // entry's list is the number of list starts up to it (one mask per
-            // 32 entries); a lane holds the images of its own partial result
-            // at the positions with this label, and an entry's come by one
-            // shuffle each.  22 instructions per 32 entries where the general
-            // step below takes over a hundred.  (Up to 128 entries, where the
-            // set-up would outweigh the steps saved, the general one; as a
-            // function of its own this was no faster.)
+            // entries by aligned quads of 16 bytes, 32 x kFlatU of them at a
+            // time, until the range ends or the next periodic check is due.
+            // Lane l holds partial result l's part of the range as entries
+            // [a0, a1) of the list array, the quads that cover these, and its
+            // images at the positions with this label; the range's lists are
+            // all non-empty, so a quad's list is the number of list starts up
+            // to it (one mask per 32 quads), and the rest comes by one shuffle
+            // each.  Bound by its instructions and, per step, two dependent
+            // loads: 12 4-vertex queries (3.5 G embeddings) took 19.2 ms with
+            // one entry per lane and load, 15.4 ms with a quad.
             const int m = (int)__shfl_sync(0xffffffffu, cnt, d - 1);
-            const uint32_t* __restrict__ gi = P.t_idx[d];
+            const uint4* __restrict__ gi = (const uint4*)P.t_idx[d];
             const int32_t* __restrict__ cd = P.cand[d];
-            const uint32_t pf = lane < m ? Bp->pf[lane] : ~0u;
             const uint32_t le = lanemask_lt() | (1u << lane);
+            uint32_t a0 = lane < m ? Bp->pf[lane] : end, a1 = __shfl_down_sync(0xffffffffu, a0, 1);
+            if (lane >= m - 1) a1 = end;
+            if (a0 < cur) a0 = cur;
+            if (a1 > end) a1 = end;
+            const uint32_t lo_ = lane < m ? Bp->lo[lane] : 0u;
+            const bool has = a0 < a1;
+            a0 += lo_;
+            a1 += lo_;
+            const uint32_t nqd = has ? ((a1 + 3) >> 2) - (a0 >> 2) : 0u;
+            uint32_t qe = nqd;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, qe, o);
+                if (lane >= o) qe += t;
+            }
+            const uint32_t total = __shfl_sync(0xffffffffu, qe, 31);
+            const uint32_t head = has ? qe - nqd : ~0u;         // its first quad in the range's
+            const uint32_t qb = (a0 >> 2) - (qe - nqd);         // what to add to a quad of the range
             int32_t img[kFlatSame];
             const int na = __popc(same);
             {
                 int a = lane < m ? lane : 0, x = na;
-                for (int t = d - 1; t >= j; t--) {
+                for (int t = d - 1; t >= j && (same >> j); t--) {
                     if ((same >> t) & 1u) {
                         x--;
 #pragma unroll
@@ -741,51 +764,73 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
 #pragma unroll
                     for (int y = 0; y < kFlatSame; y++) if (y == y0) img[y] = sg[__ffs(f) - 1];
             }
-            uint32_t i0 = cur;
-            int started = __popc(__ballot_sync(0xffffffffu, pf < i0));
-            uint32_t mine = 0, bytes = 0;
+            uint32_t i0 = 0;
+            int started = __ffs(__ballot_sync(0xffffffffu, has)) - 1;   // lists before quad i0
+            uint32_t mine = 0, read = 0;
             for (;;) {
-                uint32_t x[4];
-                int sl[4];
+                uint4 x[kFlatU];
+                uint32_t in[kFlatU];                            // which of the quad's entries are in the range
+                int sl[kFlatU];
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
+                for (int u = 0; u < kFlatU; u++) {
                     const uint32_t i = i0 + 32 * u;
-                    const uint32_t heads = __reduce_or_sync(0xffffffffu, pf - i < 32u ? 1u << (pf - i) : 0u);
+                    const uint32_t heads = __reduce_or_sync(0xffffffffu, head - i < 32u ? 1u << (head - i) : 0u);
                     sl[u] = started + __popc(heads & le) - 1;
                     started += __popc(heads);
-                    x[u] = ~0u;
-                    if (i + lane < end) { x[u] = __ldg(gi + (Bp->lo[sl[u]] + i + lane)); bytes += 4; }
+                    const uint32_t at = __shfl_sync(0xffffffffu, qb, sl[u]) + i + lane;
+                    const uint32_t f = __shfl_sync(0xffffffffu, a0, sl[u]), e = __shfl_sync(0xffffffffu, a1, sl[u]);
+                    x[u] = make_uint4(0u, 0u, 0u, 0u);
+                    in[u] = 0;
+                    if (i + lane < total) {
+                        x[u] = __ldg(gi + at);
+                        const uint32_t before = f > 4 * at ? f - 4 * at : 0u, past = 4 * at + 4 > e ? 4 * at + 4 - e : 0u;
+                        in[u] = (0xfu << before) & (0xfu >> past);
+                        read += 4 - before - past;
+                    }
                 }
                 if (same) {
-                    int32_t gc[4];
 #pragma unroll
-                    for (int u = 0; u < 4; u++) {
-                        gc[u] = x[u] != ~0u ? __ldg(cd + x[u]) : 0;
-                        bytes += x[u] != ~0u ? 4 : 0;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; u++) {
-                        bool ok = x[u] != ~0u;
+                    for (int u = 0; u < kFlatU; u++) {
+                        int32_t g0 = -1, g1 = -1, g2 = -1, g3 = -1;
+                        if (in[u] & 1u) g0 = __ldg(cd + x[u].x);
+                        if (in[u] & 2u) g1 = __ldg(cd + x[u].y);
+                        if (in[u] & 4u) g2 = __ldg(cd + x[u].z);
+                        if (in[u] & 8u) g3 = __ldg(cd + x[u].w);
+                        uint32_t ok = in[u];
 #pragma unroll
                         for (int y = 0; y < kFlatSame; y++)
-                            if (y < na && __shfl_sync(0xffffffffu, img[y], sl[u] & 31) == gc[u]) ok = false;
-                        mine += ok ? 1u : 0u;
+                            if (y < na) {
+                                const int32_t w = __shfl_sync(0xffffffffu, img[y], sl[u]);
+                                ok &= ~((g0 == w ? 1u : 0u) | (g1 == w ? 2u : 0u) | (g2 == w ? 4u : 0u) | (g3 == w ? 8u : 0u));
+                            }
+                        mine += __popc(ok);
                     }
                 } else {
+                    // a candidate index is below 2^32 - 1: each entry read counts
 #pragma unroll
-                    for (int u = 0; u < 4; u++) mine += x[u] != ~0u ? 1u : 0u;
+                    for (int u = 0; u < kFlatU; u++)
+                        mine += ((in[u] & 1u) && x[u].x != ~0u) + ((in[u] & 2u) && x[u].y != ~0u) +
+                                ((in[u] & 4u) && x[u].z != ~0u) + ((in[u] & 8u) && x[u].w != ~0u);
                 }
-                i0 += 128;
-                if (i0 >= end || ((F.iter + 1) & 15) == 0) break;
+                i0 += 32 * kFlatU;
+                if (i0 >= total || ((F.iter + 1) & 15) == 0) break;
                 if (O.limit && F.local + __reduce_add_sync(0xffffffffu, mine) >= O.flush_at) break;
                 ++F.iter;
             }
             const uint32_t found = __reduce_add_sync(0xffffffffu, mine);
             F.local += found;
             F.ccount += found;
-            F.lb += bytes;
-            if (lane == 0) F.fb += (same ? 8ull : 4ull) * ((i0 < end ? i0 : end) - cur);
-            if (lane == d - 1) vcur = i0;
+            F.lb += (same ? 8ull : 4ull) * read;
+            // where the range goes on: the entry that quad i0 begins with
+            uint32_t next = end;
+            if (i0 < total) {
+                const int t = 31 - __clz(__ballot_sync(0xffffffffu, has && head <= i0));
+                uint32_t at = 4 * (qb + i0);
+                if (at < a0) at = a0;
+                next = __shfl_sync(0xffffffffu, at - lo_, t);
+            }
+            if (lane == 0) F.fb += (same ? 8ull : 4ull) * (next - cur);
+            if (lane == d - 1) vcur = next;
             continue;
         }
         const uint32_t n = end - cur < 32 ? end - cur : 32;
@@ -1431,6 +1476,11 @@ constexpr double kFlatLength = 32.0;
 
 bool flat_query(const fast_cst* c) {
     if (c->k < 2 || c->k > kFlatMaxK || c->g->max_degree >= (1ll << 27)) return false;
+    constexpr int64_t kMost = 0xfffffff0ll;          // entries are numbered in 32 bits, by whole quads
+    for (int u = 0; u < c->k; u++)
+        if (c->parent[u] >= 0 && c->t_entries[u] > kMost) return false;
+    for (int t = 0; t < c->nnt; t++)
+        if (c->n_entries[t] > kMost) return false;
     if (c->nnt == 0) return true;
     for (int u = 0; u < c->k; u++)
         if (c->parent[u] >= 0 && c->t_wlen[u] > kFlatLength) return false;

@@ -24,22 +24,20 @@
 // Load balance: a persistent grid first drains the static chunks (each query
 // of a batch has its own cursor, and the warps start spread over the
 // queries), then serves itself from donated runs.  A warp out of static
-// chunks takes a ticket and waits on the ring cell of that ticket, which no
-// other warp reads; a busy warp that sees tickets unserved gives away the
-// second half of the unscanned list at its shallowest depth with at least
-// two entries left -- a run of a list with a fixed prefix, i.e. again a
-// chunk.  The launch ends when the unserved tickets are as many as the warps
-// that have started: nobody is left who could donate.  The only wait, that
-// for a ticket's run, is bounded by %globaltimer.
+// chunks waits on a cell of its own; a busy warp that sees warps waiting
+// claims such a cell and gives away the second half of the unscanned list at
+// its shallowest depth with at least two entries left -- a run of a list with
+// a fixed prefix, i.e. again a chunk.  The launch ends when as many warps
+// wait as have started: nobody is left who could donate.  The only wait, that
+// for a run, is bounded by %globaltimer.
 //
-// Why tickets: with one shared head that every idle warp tried to advance by
-// compare-and-swap, a published run set off thousands of attempts (65 M of
-// them, one per 4 ns, in a 235 ms enumeration of 12 queries), and that word
-// alone set the launch's time.  With tickets, pieces of chunks and the
-// counters on lines of their own, that enumeration takes 110 instead of 287
-// ms, one 10-vertex query with two-entry lists 25 instead of 115 ms, and the
-// batched matcher under a limit, whose warps now spread over the queries and
-// stop within half the limit, 250 queries' step 150 instead of 191 ms.
+// Why cells of their own: what all idle warps or all donors advance by
+// compare-and-swap sets the launch's time.  With one head that every idle
+// warp tried to advance, 12 4-vertex queries were enumerated in 287 ms, one
+// 10-vertex query with two-entry lists in 115; with tickets that donors
+// served in order (one per 0.7 us) in 15.4 and 2.11 ms, half of the warps'
+// time spent waiting; with cells that donors pick apart from one another in
+// 8.1 and 1.52.
 //
 // Warp-specialised variant (the GPU form of the task-generator separation
 // of Sec. V-D): a CTA's warps split into expanders and validators.  The
@@ -135,18 +133,15 @@ struct MatchOut {
     const unsigned long long* deadline;  // device word: %globaltimer limit, 0 = none
     uint64_t limit;                   // 0 = enumerate everything
     uint32_t flush_at;                // embeddings a warp holds back before it adds them to the total
-    // Donated runs: a bounded ring of dq_cap cells.  Ticket t (taken by a
-    // warp out of work by advancing *dq_head, served by a donor by advancing
-    // *dq_tail, which never passes the head) uses cell t % dq_cap in
-    // generation g = t / dq_cap; the cell's state is 2g while it is free for
-    // that ticket, 2g+1 once the run is published, and 2g+2 once it is taken
-    // (or the ticket's warp gave up waiting).  States start at 0.  A donor
-    // that finds the cell of the next ticket still occupied keeps its work.
+    // Donated runs: dq_cap cells, each {kFree, kWaiting, kClaimed, kGiven} in
+    // dq_state and a run in dq.  Warp w of the launch waits on cell
+    // w % dq_cap: it makes it kWaiting, a donor that finds it so makes it
+    // kClaimed, writes the run and makes it kGiven; the warp takes the run
+    // and frees the cell.  States start at kFree.
     Chunk* dq;
     uint32_t* dq_state;
     uint64_t dq_cap;                  // 0 = no donation
-    unsigned long long* dq_head;      // dq_tail follows it: one 16-byte load reads both
-    unsigned long long* dq_tail;
+    unsigned long long* idle;         // warps that wait for a run (less those a donor has claimed)
     unsigned long long* started;      // warps that have begun (less those that gave up)
     int validators;                   // warp-specialised variant: validator warps per CTA
 };
@@ -388,23 +383,25 @@ __device__ bool next_static(const MatchOut& O, uint32_t nq, uint32_t seed, uint3
     }
 }
 
-// one lane, out of static items: take a ticket and wait for its run.  True:
-// the run of ticket *ticket is published; false: the launch is over (or the
-// wait ran out).
-__device__ bool wait_run(const MatchOut& O, unsigned long long deadline, unsigned long long* ticket) {
+enum : uint32_t { kFree = 0, kWaiting, kClaimed, kGiven };
+
+// one lane, out of static items: wait for a run in this warp's cell.  True:
+// the cell holds one; false: the launch is over (or the wait ran out).
+__device__ bool wait_run(const MatchOut& O, unsigned long long deadline, uint32_t cell) {
     if (!O.dq_cap || is_done(O)) return false;
-    __threadfence();                                           // this warp's start comes before its ticket
-    const unsigned long long h = atomicAdd(O.dq_head, 1ull);
+    __threadfence();                                           // this warp's start comes before its wait
+    const unsigned long long n_idle = atomicAdd(O.idle, 1ull) + 1;
     __threadfence();
-    // every started warp holds an unserved ticket: no work is left anywhere
-    if (h + 1 - vload(O.dq_tail) == vload(O.started)) { announce_done(O); return false; }
-    uint32_t* st = O.dq_state + h % O.dq_cap;
-    const uint32_t free_ = (uint32_t)(2 * (h / O.dq_cap));
+    // every started warp waits, none of them claimed (a donor is not idle): no work is left anywhere
+    if (n_idle == vload(O.started)) { announce_done(O); return false; }
+    uint32_t* st = O.dq_state + cell;
     unsigned long long t0 = 0;
+    bool mine = false;                                         // with fewer cells than warps: not before its last user frees it
     for (int n = 0;; n++) {
-        if (*(volatile uint32_t*)st == free_ + 1) {
+        const uint32_t v = *(volatile uint32_t*)st;
+        if (!mine) mine = v == kFree && atomicCAS(st, kFree, kWaiting) == kFree;
+        else if (v == kGiven) {
             __threadfence();
-            *ticket = h;
             return true;
         }
         if (is_done(O)) return false;
@@ -412,27 +409,88 @@ __device__ bool wait_run(const MatchOut& O, unsigned long long deadline, unsigne
             const unsigned long long now = global_timer_ns();
             if (deadline && now > deadline) { stop_all(O, kStatusTimeout); return false; }
             if (!t0) t0 = now;
-            // give up: the ticket is void (a donor skips it); the warps still busy finish the rest
-            else if (now - t0 > kIdleNs && atomicCAS(st, free_, free_ + 2) == free_) return false;
+            else if (now - t0 > kIdleNs && (!mine || atomicCAS(st, kWaiting, kFree) == kWaiting)) {
+                // give up: the warps still busy finish the rest
+                atomicAdd(O.idle, ~0ull);
+                const unsigned long long left = atomicAdd(O.started, ~0ull) - 1;
+                if (left && vload(O.idle) == left) announce_done(O);
+                return false;
+            }
         }
         __nanosleep(n < 16 ? 50 : 250);
     }
 }
 
-// one lane: claim the next unserved ticket whose cell is free, or ~0 (none, a
-// full ring, or races lost a few times: the work stays here)
-__device__ unsigned long long claim_ticket(const MatchOut& O, unsigned long long head, unsigned long long t) {
-    for (int tries = 0; tries < 4 && t < head; tries++) {
-        const uint32_t st = *(volatile uint32_t*)&O.dq_state[t % O.dq_cap];
-        const uint32_t free_ = (uint32_t)(2 * (t / O.dq_cap));
-        if (st < free_) break;                                  // its cell's previous run is not taken yet
-        const unsigned long long prev = atomicCAS(O.dq_tail, t, t + 1);
-        if (prev != t) { t = prev; continue; }
-        if (st == free_) return t;
-        atomicAdd(O.started, ~0ull);                            // a void ticket: its warp is gone
-        t++;
+// The whole warp: claim the cell of a warp that waits, or ~0 (none among the
+// cells looked at, or races lost: the work stays here).  128 cells from a
+// place that differs between donors and calls; claims of different cells do
+// not meet.
+//
+// Bound by latency (one round of loads, one compare-and-swap).  With tickets
+// served in order by one shared counter, each claim had to see the last one's
+// result, one per 0.7 us for the whole chip: half of the warps of a
+// 3.5 G-embedding enumeration waited while 98 % of the donors' attempts
+// failed.
+__device__ uint32_t claim_cell(const MatchOut& O, uint32_t seed) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t cap = (uint32_t)O.dq_cap;
+    const uint32_t at = (uint32_t)(((uint64_t)(seed * 0x9E3779B1u) * cap) >> 32);
+    uint32_t c[4], m[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        const uint32_t i = 32 * u + lane;
+        c[u] = at + i < cap ? at + i : at + i - cap;
+        m[u] = i < cap && *(volatile const uint32_t*)(O.dq_state + c[u]) == kWaiting;
     }
-    return ~0ull;
+    int tries = 0;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        for (uint32_t f = __ballot_sync(0xffffffffu, m[u]); f && tries < 4; f &= f - 1, tries++) {
+            const uint32_t cell = __shfl_sync(0xffffffffu, c[u], __ffs(f) - 1);
+            int got = 0;
+            if (lane == 0 && atomicCAS(O.dq_state + cell, kWaiting, kClaimed) == kWaiting) {
+                atomicAdd(O.idle, ~0ull);
+                got = 1;
+            }
+            if (__shfl_sync(0xffffffffu, got, 0)) return cell;
+        }
+    }
+    return ~0u;
+}
+
+// The whole warp: the run [a, b) of position j (from generator list src of
+// query q; lane p holds the prefix's candidate of position p < j) goes into a
+// claimed cell.
+__device__ __forceinline__ void give_run(const MatchOut& O, uint32_t cell, int j, int src, uint32_t q, uint32_t a,
+                                         uint32_t b, uint32_t pre) {
+    const int lane = threadIdx.x & 31;
+    Chunk* dst = &O.dq[cell];
+    dst->prefix[lane] = pre;
+    if (lane == 0) {
+        dst->j = j;
+        dst->a = a;
+        dst->b = b;
+        dst->pad = kDonated | ((uint32_t)src << 1) | (q << 8);
+        dst->w = 0;
+        dst->id = 0;
+    }
+    __syncwarp();
+    if (lane == 0) {
+        __threadfence();
+        atomicExch(O.dq_state + cell, kGiven);
+    }
+}
+
+// What a busy warp watches, one load: lane 0 the end of the launch, lane 1
+// its query's limit, lane 2 the warps that wait.  The value is looked at 16
+// steps later, so the load costs no wait.
+template <bool BATCH>
+__device__ __forceinline__ int watch(const MatchOut& O, uint32_t q) {
+    const int lane = threadIdx.x & 31;
+    const int* p = (const int*)(O.done + (blockIdx.x % kDoneCopies) * kLineWords);
+    if (lane == 1) p = O.qstop + q;
+    if (lane == 2) p = (const int*)O.idle;
+    return lane == 0 || (BATCH && lane == 1) || (lane == 2 && O.dq_cap) ? vload(p) : 0;
 }
 
 // lane 0: claim the ring's next cell for a producer, if it is free (a cell
@@ -621,7 +679,7 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
     uint32_t cnt = 0;                              // lane p: partial results in buffer p
     uint32_t rc = lo, re = hi;                     // what is left of the item's run
     int d = j;                                     // the position being filled
-    int stop_seen = 0;
+    int seen_ = 0;                                 // what watch() saw
     __syncwarp();
     for (;;) {
         ++F.iter;
@@ -630,74 +688,47 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
             F.local = 0;
         }
         if ((F.iter & 15) == 0) {
-            if (__any_sync(0xffffffffu, stop_seen)) break;
-            if (lane == 0) {
-                if ((F.iter & 255) == 0 && deadline && global_timer_ns() > deadline) stop_all(O, kStatusTimeout);
-                stop_seen = is_done(O);
-            }
-            if (BATCH && lane == 1) stop_seen = vload(O.qstop + q);
-        }
-        if (O.dq_cap && (F.iter & 15) == 0) {
-            ulonglong2 ht = make_ulonglong2(0, 0);
-            if (lane == 0) ht = __ldcv((const ulonglong2*)O.dq_head);       // {head, tail}
-            if (__shfl_sync(0xffffffffu, ht.y < ht.x, 0)) {
-                // the shallowest position with work to give: the item's run, then the buffers
-                const bool can = lane >= j && lane < d && vend - vcur >= (uint32_t)(lane == k - 2 ? kLastDonate : 2) && vend > vcur;
-                const uint32_t cm = __ballot_sync(0xffffffffu, can);
-                const bool run = re > rc && re - rc >= (uint32_t)(j == k - 1 ? kLastDonate : 2);
-                if (run || cm) {
-                    unsigned long long slot = ~0ull;
-                    if (lane == 0) slot = claim_ticket(O, ht.x, ht.y);
-                    slot = __shfl_sync(0xffffffffu, slot, 0);
-                    if (slot != ~0ull) {
-                        int dj = j, dsrc = src0, p = -1;
-                        uint32_t a, b, left = 0;                             // the run given; what the donor keeps up to
-                        uint32_t pre = lane < j ? sm[lane] : 0u;
-                        if (run) {
-                            left = rc + (re - rc) / 2;
-                            a = left - base;
-                            b = re - base;
-                        } else {
-                            p = __ffs(cm) - 1;
-                            const uint32_t c = __shfl_sync(0xffffffffu, vcur, p), e = __shfl_sync(0xffffffffu, vend, p);
-                            const uint32_t m = __shfl_sync(0xffffffffu, cnt, p);
-                            // the last partial result with anything left
-                            const uint32_t below = __ballot_sync(0xffffffffu, lane < (int)m && B[p].pf[lane] < e);
-                            const int sl = 31 - __clz(below);
-                            const uint32_t f = B[p].pf[sl];
-                            left = f > c ? f : c + (e - c) / 2;
-                            a = left - f;
-                            b = e - f;
-                            dj = p + 1;
-                            dsrc = (int)(B[p].mt[sl] >> 8);
-                            int at = sl;
-                            for (int t = p; t >= j; t--) {
-                                if (lane == t) pre = B[t].v[at];
-                                at = (int)(B[t].mt[at] & 255u);
-                            }
-                        }
-                        Chunk* dst = &O.dq[slot % O.dq_cap];
-                        dst->prefix[lane] = pre;
-                        if (lane == 0) {
-                            dst->j = dj;
-                            dst->a = a;
-                            dst->b = b;
-                            dst->pad = kDonated | ((uint32_t)dsrc << 1) | (q << 8);
-                            dst->w = 0;
-                            dst->id = 0;
-                        }
-                        __syncwarp();
-                        int gave = 0;
-                        if (lane == 0) {
-                            const uint32_t free_ = (uint32_t)(2 * (slot / O.dq_cap));
-                            __threadfence();
-                            gave = atomicCAS(&O.dq_state[slot % O.dq_cap], free_, free_ + 1) == free_;
-                            if (!gave) atomicAdd(O.started, ~0ull);
-                        }
-                        if (__shfl_sync(0xffffffffu, gave, 0)) {
-                            if (run) re = left;
-                            else if (lane == p) vend = left;
-                        }
+            const uint32_t seen = __ballot_sync(0xffffffffu, seen_ != 0);
+            if (seen & 3u) break;
+            if (lane == 0 && (F.iter & 255) == 0 && deadline && global_timer_ns() > deadline) stop_all(O, kStatusTimeout);
+            seen_ = watch<BATCH>(O, q);
+            if (seen & 4u) {
+                // give away: the second half of the item's run, else the last
+                // list of the shallowest buffer with more than one entry left
+                int dj = j, dsrc = src0, p = -1;
+                uint32_t a = 0, b = 0, left = 0;                         // the run; what the donor keeps up to
+                uint32_t pre = lane < j ? sm[lane] : 0u;
+                const uint32_t cm = __ballot_sync(0xffffffffu, lane >= j && lane < d && vend > vcur + 1);
+                if (re > rc + 1) {
+                    left = rc + (re - rc) / 2;
+                    a = left - base;
+                    b = re - base;
+                } else if (cm) {
+                    p = __ffs(cm) - 1;
+                    const uint32_t c = __shfl_sync(0xffffffffu, vcur, p), e = __shfl_sync(0xffffffffu, vend, p);
+                    const uint32_t m = __shfl_sync(0xffffffffu, cnt, p);
+                    // the last partial result with anything left
+                    const uint32_t below = __ballot_sync(0xffffffffu, lane < (int)m && B[p].pf[lane] < e);
+                    const int sl = 31 - __clz(below);
+                    const uint32_t f = B[p].pf[sl];
+                    left = f > c ? f : c + (e - c) / 2;
+                    a = left - f;
+                    b = e - f;
+                    dj = p + 1;
+                    dsrc = (int)(B[p].mt[sl] >> 8);
+                    int at = sl;
+                    for (int t = p; t >= j; t--) {
+                        if (lane == t) pre = B[t].v[at];
+                        at = (int)(B[t].mt[at] & 255u);
+                    }
+                }
+                // a run of the last position is worth it only if it is long
+                if (b - a >= (dj == k - 1 ? (uint32_t)kLastDonate : 1u)) {
+                    const uint32_t cell = claim_cell(O, (blockIdx.x * 8 + (threadIdx.x >> 5)) * 64 + (F.iter >> 4));
+                    if (cell != ~0u) {
+                        give_run(O, cell, dj, dsrc, q, a, b, pre);
+                        if (p < 0) re = left;
+                        else if (lane == p) vend = left;
                     }
                 }
             }
@@ -1040,6 +1071,7 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
     uint32_t sq = BATCH && nq ? (uint32_t)(((uint64_t)gw * nq) / tw) : 0u;   // the query whose static items it takes
     bool static_left = nq > 0;
     uint32_t q = sq;                                                        // the query `local` counts for
+    const uint32_t cell = O.dq_cap ? gw % (uint32_t)O.dq_cap : 0u;          // where it waits
     for (;;) {
         unsigned long long ci = 0;
         int kind = 0;
@@ -1058,7 +1090,8 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
         }
         if (kind == 0) {
             int got = 0;
-            if (lane == 0) got = wait_run(O, deadline, &ci);
+            if (lane == 0) got = wait_run(O, deadline, cell);
+            ci = cell;
             if (__shfl_sync(0xffffffffu, got, 0)) kind = 2;
             ci = __shfl_sync(0xffffffffu, ci, 0);
         }
@@ -1066,7 +1099,7 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
         // the item's fields, read once.  A donated run was written by another
         // warp during this launch: read it from L2 (ld.global.cg), never from
         // an L1 line that may hold an older copy of its bytes.
-        const Chunk* chp = kind == 1 ? (BATCH ? plans[sq].chunks : P0.chunks) + (uint32_t)ci / pieces : O.dq + ci % O.dq_cap;
+        const Chunk* chp = kind == 1 ? (BATCH ? plans[sq].chunks : P0.chunks) + (uint32_t)ci / pieces : O.dq + ci;
         int j;
         uint32_t ch_a, ch_b, ch_pad, ch_pre;
         bool first = true;                        // the chunk's first piece (it counts the chunk's own extension)
@@ -1086,9 +1119,9 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
             j = __ldcg(&chp->j); ch_a = __ldcg(&chp->a); ch_b = __ldcg(&chp->b); ch_pad = __ldcg(&chp->pad);
             ch_pre = lane < j ? __ldcg(&chp->prefix[lane]) : 0u;
             __syncwarp();
-            if (lane == 0) {                      // hand the cell back for ticket ci + dq_cap
+            if (lane == 0) {                      // hand the cell back
                 __threadfence();
-                atomicExch(&O.dq_state[ci % O.dq_cap], (uint32_t)(2 * (ci / O.dq_cap) + 2));
+                atomicExch(O.dq_state + cell, kFree);
             }
         }
         if (BATCH && kind == 2) q = ch_pad >> 8;               // nothing is held back: it waited
@@ -1173,7 +1206,7 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
             // flush_at embeddings, and looks every 16th step whether the limit
             // was reached meanwhile (a load issued 16 steps before its value is
             // used, so that it costs no wait).
-            int stop_seen = 0;
+            int seen_ = 0;                      // what watch() saw
             for (;;) {
                 ++iter;
                 if (local >= O.flush_at) {
@@ -1181,50 +1214,26 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
                     local = 0;
                 }
                 if ((iter & 15) == 0) {
-                    if (__any_sync(0xffffffffu, stop_seen)) break;
-                    if (lane == 0) {
-                        if ((iter & 255) == 0 && deadline && global_timer_ns() > deadline) stop_all(O, kStatusTimeout);
-                        stop_seen = is_done(O);
-                    }
-                    if (BATCH && lane == 1) stop_seen = vload(O.qstop + q);
-                }
-                if (O.dq_cap && (iter & 63) == 0) {
-                    // give work away when some warp waits for it
-                    ulonglong2 ht = make_ulonglong2(0, 0);
-                    if (lane == 0) ht = __ldcv((const ulonglong2*)O.dq_head);   // {head, tail}
-                    if (__shfl_sync(0xffffffffu, ht.y < ht.x, 0)) {
-                        // a run of the last position is worth giving away only if it is long
+                    const uint32_t seen = __ballot_sync(0xffffffffu, seen_ != 0);
+                    if (seen & 3u) break;
+                    if (lane == 0 && (iter & 255) == 0 && deadline && global_timer_ns() > deadline)
+                        stop_all(O, kStatusTimeout);
+                    seen_ = watch<BATCH>(O, q);
+                    if ((seen & 4u) && (iter & 63) == 0) {
+                        // give work away: a run of the last position is worth it only if it is long
                         const bool can = lane >= j && lane <= d && (seg_end - seg_next) >= (lane == k - 1 ? kLastDonate : 2);
                         const uint32_t cm = __ballot_sync(0xffffffffu, can);
                         if (cm) {
                             const int dd = __ffs(cm) - 1;
-                            unsigned long long slot = ~0ull;
-                            if (lane == 0) slot = claim_ticket(O, ht.x, ht.y);
-                            slot = __shfl_sync(0xffffffffu, slot, 0);
-                            if (slot != ~0ull) {
-                                int64_t sn_ = __shfl_sync(0xffffffffu, seg_next, dd);
-                                int64_t se_ = __shfl_sync(0xffffffffu, seg_end, dd);
-                                int64_t sb_ = __shfl_sync(0xffffffffu, seg_base, dd);
-                                int64_t mid = sn_ + (se_ - sn_) / 2;
-                                Chunk* dst = &O.dq[slot % O.dq_cap];
-                                if (lane < kMaxK) dst->prefix[lane] = lane < dd ? sm[lane] : 0u;
-                                if (lane == 0) {
-                                    dst->j = dd;
-                                    dst->a = (uint32_t)(mid - sb_);
-                                    dst->b = (uint32_t)(se_ - sb_);
-                                    dst->pad = kDonated | ((uint32_t)gsrc[dd] << 1) | (q << 8);
-                                    dst->w = 0;
-                                    dst->id = 0;
-                                }
-                                __syncwarp();
-                                int gave = 0;
-                                if (lane == 0) {
-                                    const uint32_t free_ = (uint32_t)(2 * (slot / O.dq_cap));
-                                    __threadfence();
-                                    gave = atomicCAS(&O.dq_state[slot % O.dq_cap], free_, free_ + 1) == free_;
-                                    if (!gave) atomicAdd(O.started, ~0ull);    // its warp gave up just now: keep the run
-                                }
-                                if (__shfl_sync(0xffffffffu, gave, 0) && lane == dd) seg_end = mid;
+                            const uint32_t cell = claim_cell(O, gw * 64 + (iter >> 4));
+                            if (cell != ~0u) {
+                                const int64_t sn_ = __shfl_sync(0xffffffffu, seg_next, dd);
+                                const int64_t se_ = __shfl_sync(0xffffffffu, seg_end, dd);
+                                const int64_t sb_ = __shfl_sync(0xffffffffu, seg_base, dd);
+                                const int64_t mid = sn_ + (se_ - sn_) / 2;
+                                give_run(O, cell, dd, gsrc[dd], q, (uint32_t)(mid - sb_), (uint32_t)(se_ - sb_),
+                                         lane < dd ? sm[lane] : 0u);
+                                if (lane == dd) seg_end = mid;
                             }
                         }
                     }
@@ -1577,18 +1586,18 @@ int matcher_smem_optin(size_t bytes) {
 }
 
 // Counter block (8-byte words).  What different warps hammer lies in lines of
-// its own: the total, the embedding cursor, the static cursor, the ring's
-// head and tail (together: a donor reads both at once).  The first kCtrWords
+// its own: the total, the embedding cursor, the static cursor, the
+// number of waiting warps.  The first kCtrWords
 // come back to the host; the copies of the done flag follow.
 enum { kStatus = 0, kBytes, kFloor, kDeadline, kStarted, kQStop, kStats = 8,
        kTotal = (kStats + kMaxK + kLineWords - 1) / kLineWords * kLineWords, kSlot = kTotal + kLineWords,
-       kCtrWords = kSlot + 1, kNext = kSlot + kLineWords, kHead = kNext + kLineWords, kTail = kHead + 1,
-       kDone = kHead + kLineWords, kAllWords = kDone + kDoneCopies * kLineWords };
+       kCtrWords = kSlot + 1, kNext = kSlot + kLineWords, kIdle = kNext + kLineWords,
+       kDone = kIdle + kLineWords, kAllWords = kDone + kDoneCopies * kLineWords };
 constexpr uint64_t kQueueCap = 1 << 16;
 
 // Cells of the donation ring for a launch of `warps` warps: cfg.queue_cells
-// if given (at most cap), else one per warp, so that every waiting warp's
-// ticket has a cell of its own.
+// if given (at most cap), else one per warp, so that every warp has a cell of
+// its own to wait on.
 uint64_t ring_cells(int64_t queue_cells, int64_t warps, uint64_t cap) {
     return std::min<uint64_t>(queue_cells > 0 ? (uint64_t)queue_cells : (uint64_t)std::max<int64_t>(warps, 1), cap);
 }
@@ -1620,8 +1629,7 @@ void bind_counters(MatchOut& O, unsigned long long* ctr) {
     O.deadline = ctr + kDeadline;
     O.started = ctr + kStarted;
     O.done = ctr + kDone;
-    O.dq_head = ctr + kHead;
-    O.dq_tail = ctr + kTail;
+    O.idle = ctr + kIdle;
 }
 
 int run_match(const fast_cst* c, const fast_chunks* chunks, const fast_config* cfg_in, uint64_t kemb, uint32_t* emb_out,

@@ -429,7 +429,7 @@ __device__ bool wait_run(const MatchOut& O, unsigned long long deadline, uint32_
 // Bound by latency (one round of loads, one compare-and-swap).  With tickets
 // served in order by one shared counter, each claim had to see the last one's
 // result, one per 0.7 us for the whole chip: half of the warps of a
-// 3.5 G-embedding enumeration waited while 98 % of the donors' attempts
+// 2.4 G-embedding enumeration waited while 98 % of the donors' attempts
 // failed.
 __device__ uint32_t claim_cell(const MatchOut& O, uint32_t seed) {
     const int lane = threadIdx.x & 31;
@@ -651,9 +651,12 @@ struct FlatState {
     uint32_t iter;
 };
 
-constexpr int kFlatU = 2;        // quads per lane in flight there (1: 3.5 G embeddings 16.5 instead of 15.4 ms; 4: 15.8)
+// Steps of 32 quads there that count as one towards the periodic checks, each
+// of which costs the set-up again: 2.4 G embeddings in 8.36 ms with 1, 7.78
+// with 2, 7.47 with 4, 7.34 with 8 (and 8192 entries between two looks).
+constexpr int kFlatSteps = 4;
 // Entries of the shortest range it is used for.  A range of up to 32 is one
-// general step; with the line at 128, 3.5 G embeddings took 16.7 instead of
+// general step; with the line at 128, 2.4 G embeddings took 16.7 instead of
 // 15.4 ms and two-entry lists 2.38 instead of 2.11 ms.
 constexpr uint32_t kFlatQuads = 32;
 constexpr int kFlatSame = 4;     // same-label positions the short form of the last position handles
@@ -746,16 +749,20 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
         const int e0 = P.nt_begin[d], ne = P.nt_begin[d + 1] - e0;
         if (!EMIT && !STATS && d == k - 1 && Bp && ne == 0 && end - cur > kFlatQuads && __popc(same) <= kFlatSame) {
             // The last position with nothing to check but the images: its
-            // entries by aligned quads of 16 bytes, 32 x kFlatU of them at a
+            // entries by aligned quads of 16 bytes, 32 of them at a
             // time, until the range ends or the next periodic check is due.
             // Lane l holds partial result l's part of the range as entries
             // [a0, a1) of the list array, the quads that cover these, and its
             // images at the positions with this label; the range's lists are
             // all non-empty, so a quad's list is the number of list starts up
             // to it (one mask per 32 quads), and the rest comes by one shuffle
-            // each.  Bound by its instructions and, per step, two dependent
-            // loads: 12 4-vertex queries (3.5 G embeddings) took 19.2 ms with
-            // one entry per lane and load, 15.4 ms with a quad.
+            // each.  Bound by its instructions (some 60 per 32 quads): 12
+            // 4-vertex queries (2.4 G embeddings) took 19.2 ms with one entry
+            // per lane and load, 15.4 ms with a quad, of which half was
+            // waiting for donated runs; without that 8.1, and 7.5 with one
+            // quad per lane in flight instead of two, whose registers this
+            // function lacks (a 10-vertex query with two-entry lists 1.36
+            // instead of 1.52 ms).
             const int m = (int)__shfl_sync(0xffffffffu, cnt, d - 1);
             const uint4* __restrict__ gi = (const uint4*)P.t_idx[d];
             const int32_t* __restrict__ cd = P.cand[d];
@@ -798,55 +805,45 @@ __device__ __noinline__ FlatState flat_search(const MatchPlan& P, const MatchOut
             uint32_t i0 = 0;
             int started = __ffs(__ballot_sync(0xffffffffu, has)) - 1;   // lists before quad i0
             uint32_t mine = 0, read = 0;
-            for (;;) {
-                uint4 x[kFlatU];
-                uint32_t in[kFlatU];                            // which of the quad's entries are in the range
-                int sl[kFlatU];
-#pragma unroll
-                for (int u = 0; u < kFlatU; u++) {
-                    const uint32_t i = i0 + 32 * u;
-                    const uint32_t heads = __reduce_or_sync(0xffffffffu, head - i < 32u ? 1u << (head - i) : 0u);
-                    sl[u] = started + __popc(heads & le) - 1;
-                    started += __popc(heads);
-                    const uint32_t at = __shfl_sync(0xffffffffu, qb, sl[u]) + i + lane;
-                    const uint32_t f = __shfl_sync(0xffffffffu, a0, sl[u]), e = __shfl_sync(0xffffffffu, a1, sl[u]);
-                    x[u] = make_uint4(0u, 0u, 0u, 0u);
-                    in[u] = 0;
-                    if (i + lane < total) {
-                        x[u] = __ldg(gi + at);
-                        const uint32_t before = f > 4 * at ? f - 4 * at : 0u, past = 4 * at + 4 > e ? 4 * at + 4 - e : 0u;
-                        in[u] = (0xfu << before) & (0xfu >> past);
-                        read += 4 - before - past;
-                    }
+            for (uint32_t step = 1;; step++) {
+                const uint32_t heads = __reduce_or_sync(0xffffffffu, head - i0 < 32u ? 1u << (head - i0) : 0u);
+                const int sl = started + __popc(heads & le) - 1;
+                started += __popc(heads);
+                const uint32_t at = __shfl_sync(0xffffffffu, qb, sl) + i0 + lane;
+                const uint32_t f = __shfl_sync(0xffffffffu, a0, sl), e = __shfl_sync(0xffffffffu, a1, sl);
+                uint4 x = make_uint4(0u, 0u, 0u, 0u);
+                uint32_t in = 0;                                // which of the quad's entries are in the range
+                if (i0 + lane < total) {
+                    x = __ldg(gi + at);
+                    const uint32_t before = f > 4 * at ? f - 4 * at : 0u, past = 4 * at + 4 > e ? 4 * at + 4 - e : 0u;
+                    in = (0xfu << before) & (0xfu >> past);
+                    read += 4 - before - past;
                 }
                 if (same) {
+                    int32_t g0 = -1, g1 = -1, g2 = -1, g3 = -1;
+                    if (in & 1u) g0 = __ldg(cd + x.x);
+                    if (in & 2u) g1 = __ldg(cd + x.y);
+                    if (in & 4u) g2 = __ldg(cd + x.z);
+                    if (in & 8u) g3 = __ldg(cd + x.w);
 #pragma unroll
-                    for (int u = 0; u < kFlatU; u++) {
-                        int32_t g0 = -1, g1 = -1, g2 = -1, g3 = -1;
-                        if (in[u] & 1u) g0 = __ldg(cd + x[u].x);
-                        if (in[u] & 2u) g1 = __ldg(cd + x[u].y);
-                        if (in[u] & 4u) g2 = __ldg(cd + x[u].z);
-                        if (in[u] & 8u) g3 = __ldg(cd + x[u].w);
-                        uint32_t ok = in[u];
-#pragma unroll
-                        for (int y = 0; y < kFlatSame; y++)
-                            if (y < na) {
-                                const int32_t w = __shfl_sync(0xffffffffu, img[y], sl[u]);
-                                ok &= ~((g0 == w ? 1u : 0u) | (g1 == w ? 2u : 0u) | (g2 == w ? 4u : 0u) | (g3 == w ? 8u : 0u));
-                            }
-                        mine += __popc(ok);
-                    }
+                    for (int y = 0; y < kFlatSame; y++)
+                        if (y < na) {
+                            const int32_t w = __shfl_sync(0xffffffffu, img[y], sl);
+                            in &= ~((g0 == w ? 1u : 0u) | (g1 == w ? 2u : 0u) | (g2 == w ? 4u : 0u) | (g3 == w ? 8u : 0u));
+                        }
+                    mine += __popc(in);
                 } else {
                     // a candidate index is below 2^32 - 1: each entry read counts
-#pragma unroll
-                    for (int u = 0; u < kFlatU; u++)
-                        mine += ((in[u] & 1u) && x[u].x != ~0u) + ((in[u] & 2u) && x[u].y != ~0u) +
-                                ((in[u] & 4u) && x[u].z != ~0u) + ((in[u] & 8u) && x[u].w != ~0u);
+                    mine += ((in & 1u) && x.x != ~0u) + ((in & 2u) && x.y != ~0u) + ((in & 4u) && x.z != ~0u) +
+                            ((in & 8u) && x.w != ~0u);
                 }
-                i0 += 32 * kFlatU;
-                if (i0 >= total || ((F.iter + 1) & 15) == 0) break;
-                if (O.limit && F.local + __reduce_add_sync(0xffffffffu, mine) >= O.flush_at) break;
-                ++F.iter;
+                i0 += 32;
+                if (i0 >= total) break;
+                if (step % kFlatSteps == 0) {
+                    if (((F.iter + 1) & 15) == 0) break;
+                    if (O.limit && F.local + __reduce_add_sync(0xffffffffu, mine) >= O.flush_at) break;
+                    ++F.iter;
+                }
             }
             const uint32_t found = __reduce_add_sync(0xffffffffu, mine);
             F.local += found;

@@ -1014,34 +1014,38 @@ int build_lists(const fast_graph* g, std::vector<Q>& Qs, std::vector<Edge>& E, c
     const size_t ns = slices.size() - 1;
     if (!bounded) FAST_TRY(t_readback.reserve(4 * ne, 2 * ns + 1));
     std::vector<uint32_t> sizes;                  // Z
-    // row lengths
+    // row lengths: the first slice by itself, so that its sizes come while the
+    // device works on the others, and these in one launch (a slice's is 20 us,
+    // nearly all of it latency: a 40-query step of 30 slices 14.85 -> 14.3 ms)
     {
         Stage st;
-        std::vector<ListDesc> ld;
-        std::vector<int64_t> toff;
-        std::vector<size_t> t_at(ns), z_at(ns), d_at(ns);
-        for (size_t k = 0; k < ns; k++) {
-            ld.clear();
+        const size_t part[3] = {0, std::min<size_t>(1, ns), ns};
+        size_t t_at[2] = {0, 0}, z_at[2] = {0, 0}, d_at[2] = {0, 0}, tiles[2] = {0, 0};
+        for (int b = 0; b < 2; b++) {
+            if (part[b] == part[b + 1]) continue;
+            std::vector<ListDesc> ld;
             std::vector<int64_t> n;
-            for (size_t i = slices[k]; i < slices[k + 1]; i++) {
+            for (size_t i = slices[part[b]]; i < slices[part[b + 1]]; i++) {
                 ld.push_back(desc_of(i));
                 n.push_back(E[i].n);
             }
-            toff = seg_tile_offsets(n, kScanTile);
-            d_at[k] = st.add(ld);
-            t_at[k] = st.add(toff);
-            z_at[k] = st.zeros((size_t)toff.back() + 1);
+            const std::vector<int64_t> toff = seg_tile_offsets(n, kScanTile);
+            tiles[b] = (size_t)toff.back();
+            d_at[b] = st.add(ld);
+            t_at[b] = st.add(toff);
+            z_at[b] = st.zeros(tiles[b] + 1);
         }
         Scratch sc(s);
         FAST_TRY(st.upload(sc));
-        for (size_t k = 0; k < ns; k++) {
-            const int nseg = (int)(slices[k + 1] - slices[k]);
-            const size_t tiles = (k + 1 < ns ? z_at[k + 1] : st.zeros(0)) - z_at[k] - 1;
-            const unsigned grid = (unsigned)std::min<int64_t>((int64_t)tiles, (int64_t)num_sms() * 4);
-            k_row_lens<<<grid, kScanBlock, 0, s>>>(st.at<ListDesc>(d_at[k]), G, st.at<int64_t>(t_at[k]), nseg,
-                                                   st.z(z_at[k]), (unsigned int*)st.z(z_at[k] + tiles));
+        for (int b = 0; b < 2; b++) {
+            if (part[b] == part[b + 1]) continue;
+            const int nseg = (int)(slices[part[b + 1]] - slices[part[b]]);
+            const unsigned grid = (unsigned)std::min<int64_t>((int64_t)tiles[b], (int64_t)num_sms() * 4);
+            k_row_lens<<<grid, kScanBlock, 0, s>>>(st.at<ListDesc>(d_at[b]), G, st.at<int64_t>(t_at[b]), nseg,
+                                                   st.z(z_at[b]), (unsigned int*)st.z(z_at[b] + tiles[b]));
             FAST_TRY(note_launch("row lengths"));
-            if (!bounded) FAST_TRY(t_readback.read(Z + slices[k], slices[k], nseg, 2 * k, s));
+            for (size_t k = part[b]; !bounded && k < part[b + 1]; k++)
+                FAST_TRY(t_readback.read(Z + slices[k], slices[k], slices[k + 1] - slices[k], 2 * k, s));
         }
     }
     // test

@@ -98,6 +98,19 @@ __global__ void __launch_bounds__(256) k_filter(const FilterDesc* __restrict__ D
     if (threadIdx.x == 0 && total) atomicAdd(d.cnt, (unsigned long long)total);
 }
 
+// ----------------------------------------------------- chains of launches
+
+// The refinement and the workload estimate are chains of small dependent
+// launches.  Those of a chain may begin before the one ahead has ended: their
+// blocks take their places and wait here, first of all, until it has ended and
+// its writes are visible; then the next launch may do the same.  That hides
+// the start of each: eight queries (36 such launches) 2.63 -> 2.53 ms, five
+// single queries 4.93 -> 4.77 ms, one of 32 vertices 1.145 -> 1.114 ms.
+__device__ __forceinline__ void chain_begin() {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+}
+
 // ------------------------------------------------------------- support
 
 // A set some vertex is tested against: a bitmap over the positions of
@@ -144,6 +157,7 @@ __global__ void __launch_bounds__(256, kSupportBlocks) k_support(const SetDesc* 
                                                  int nseg, int group, const Target* __restrict__ T, GraphSegs G,
                                                  const int32_t* __restrict__ col, LongRow* __restrict__ longs,
                                                  unsigned int* __restrict__ nlong) {
+    chain_begin();
     const int lane = threadIdx.x & 31;
     const int64_t items = item_off[nseg];
     for (int64_t it = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); it < items; it += (int64_t)gridDim.x * 8) {
@@ -210,6 +224,7 @@ __global__ void __launch_bounds__(256) k_support_long(const SetDesc* __restrict_
                                                       GraphSegs G, const int32_t* __restrict__ col,
                                                       const LongRow* __restrict__ longs,
                                                       const unsigned int* __restrict__ nlong) {
+    chain_begin();
     const unsigned int n = min(*nlong, kLongRows);
     for (unsigned int r = blockIdx.x; r < n; r += gridDim.x) {
         const LongRow lr = longs[r];
@@ -598,6 +613,7 @@ struct ChildSumDesc {
 
 __global__ void __launch_bounds__(256, 4) k_child_sums(const ChildSumDesc* __restrict__ D,
                                                        const int64_t* __restrict__ tile_off, int nseg) {
+    chain_begin();
     const int64_t total = tile_off[nseg];
     for (int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); t < total; t += (int64_t)gridDim.x * 8) {
         const int s = warp_seg_of(tile_off, nseg, t);
@@ -631,6 +647,7 @@ struct ProdDesc {
 
 __global__ void k_workload_prod(const ProdDesc* __restrict__ D, const int64_t* __restrict__ item_off, int nseg,
                                 const ChildRef* __restrict__ C) {
+    chain_begin();
     const int64_t total = item_off[nseg];
     for (int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gi - (threadIdx.x & 31) < total;
          gi += (int64_t)gridDim.x * blockDim.x) {
@@ -669,6 +686,7 @@ struct TotalDesc {
 };
 
 __global__ void k_total_w(const TotalDesc* __restrict__ D) {
+    chain_begin();
     __shared__ uint64_t sh[32];
     __shared__ double shf[32];
     const TotalDesc& d = D[blockIdx.x];
@@ -796,6 +814,22 @@ inline std::vector<int64_t> prefix(const std::vector<int64_t>& n) {
 int note_launch(const char* what) {
     fast::note_launch();
     return cudaGetLastError() == cudaSuccess ? FAST_OK : set_error(FAST_ERR_CUDA, "%s launch", what);
+}
+
+// A launch of a chain: the kernel begins with chain_begin().
+template <class... P, class... A>
+int launch_chained(const char* what, void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t s, A... args) {
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cfg.attrs = &early;
+    cfg.numAttrs = 1;
+    FAST_CUDA(cudaLaunchKernelEx(&cfg, kernel, (P)args...));
+    return note_launch(what);
 }
 
 // blocks of 256 threads for `warps` warps of work, `per_sm` blocks per SM at most
@@ -1250,18 +1284,14 @@ int build_workload(std::vector<Q>& Qs, int64_t* Z, int max_depth, Scratch& keep,
     FAST_TRY(st.upload(keep));
     for (int d = max_depth; d >= 0; d--) {
         const Wave& wv = waves[d];
-        if (wv.tiles > 0) {
-            k_child_sums<<<warp_grid(wv.tiles, 8), 256, 0, s>>>(st.at<ChildSumDesc>(wv.s_at), st.at<int64_t>(wv.so_at), wv.ns);
-            FAST_TRY(note_launch("child sums"));
-        }
-        if (wv.items > 0) {
-            k_workload_prod<<<warp_grid(ceil_div(wv.items, 32), 8), 256, 0, s>>>(st.at<ProdDesc>(wv.p_at), st.at<int64_t>(wv.po_at),
-                                                                              wv.np, st.at<ChildRef>(r_at));
-            FAST_TRY(note_launch("workload"));
-        }
+        if (wv.tiles > 0)
+            FAST_TRY(launch_chained("child sums", k_child_sums, warp_grid(wv.tiles, 8), 256, s, st.at<ChildSumDesc>(wv.s_at),
+                                    st.at<int64_t>(wv.so_at), wv.ns));
+        if (wv.items > 0)
+            FAST_TRY(launch_chained("workload", k_workload_prod, warp_grid(ceil_div(wv.items, 32), 8), 256, s,
+                                    st.at<ProdDesc>(wv.p_at), st.at<int64_t>(wv.po_at), wv.np, st.at<ChildRef>(r_at)));
     }
-    k_total_w<<<(unsigned)nq, 1024, 0, s>>>(st.at<TotalDesc>(t_at));
-    return note_launch("W");
+    return launch_chained("W", k_total_w, (unsigned)nq, 1024, s, st.at<TotalDesc>(t_at));
 }
 
 // Builds every CST of Qs (all valid queries) on stream s.
@@ -1470,14 +1500,12 @@ int build_all(const fast_graph* g, std::vector<Q>& Qs, cudaStream_t s) {
             const Wave& wv = waves[i];
             if (wv.items == 0) continue;
             unsigned int* nl = (unsigned int*)st.z(z_at + i);
-            k_support<<<warp_grid(wv.items, kSupportBlocks), 256, 0, s>>>(st.at<SetDesc>(wv.d_at), st.at<int64_t>(wv.i_at), (int)wv.d.size(),
-                                                             wv.group, st.at<Target>(t_at), G, g->col, longs, nl);
-            FAST_TRY(note_launch("support"));
-            if (hubs) {
-                k_support_long<<<(unsigned)num_sms() * 2, 256, 0, s>>>(st.at<SetDesc>(wv.d_at), st.at<Target>(t_at), G, g->col,
-                                                                       longs, nl);
-                FAST_TRY(note_launch("support of long rows"));
-            }
+            FAST_TRY(launch_chained("support", k_support, warp_grid(wv.items, kSupportBlocks), 256, s, st.at<SetDesc>(wv.d_at),
+                                    st.at<int64_t>(wv.i_at), (int)wv.d.size(), wv.group, st.at<Target>(t_at), G, g->col,
+                                    longs, nl));
+            if (hubs)
+                FAST_TRY(launch_chained("support of long rows", k_support_long, (unsigned)num_sms() * 2, 256, s,
+                                        st.at<SetDesc>(wv.d_at), st.at<Target>(t_at), G, g->col, longs, nl));
         }
     }
     FAST_TRY(fetch(Z, h, (size_t)(F_C + kMaxK) * nq, s));

@@ -98,10 +98,10 @@ typedef struct {
     /* Enumeration limit: fast_match stops once `limit` embeddings are found
      * and reports min(total, limit), exactly (0: enumerate everything). */
     uint64_t limit;
-    /* Cells of the matcher's ring of donated runs (work given away to idle
-     * warps); a full ring only means a busy warp keeps its work.  0: the
-     * default, 65536 (4096 for fast_match_noalloc); larger values are
-     * clamped to the default.  Results never depend on it. */
+    /* Cells for donated runs (work given away to idle warps of the matcher);
+     * with fewer cells than idle warps, some wait for a cell.  0: the
+     * default, one per warp of the launch; at most 65536 (8192 for
+     * fast_match_noalloc) are used.  Results never depend on it. */
     int64_t queue_cells;
     /* Matching order O of fast_build_cst.  0: the paper's path-based order
      * (Sec. IV-B): a depth-first walk of t_q, children by increasing
@@ -161,12 +161,11 @@ const char* fast_last_error(void);
  * simple).  edges: [m][2] vertex ids in 0..n-1; both directions are stored,
  * self loops and repeated edges are dropped.  labels: [n], >= 0 and below
  * 2^23.  Host pointers unless flags has FAST_PTR_DEVICE.  n <= 2^31 - 1 and
- * 2m < 2^32.  Layout on the device: int64 row offsets [n+1], int32 neighbour
- * ids, int32 labels, and a label index (vertices grouped by label, ascending
- * id within a label).  Each neighbour list is sorted by (label of the
- * neighbour, id) -- with a directory of its label runs, so that the CST
- * build (Alg. 1) reads only the neighbours with the label it keeps -- when
- * 2 * bits(n - 1) + bits(labels - 1) <= 64; otherwise by id alone.
+ * 2m < 2^32.  Layout on the device: the vertices are numbered label by label
+ * (ascending id within a label); int64 row offsets [n+1] and int32 neighbour
+ * numbers, ascending, so that the neighbours with one label lie together; and
+ * where each label begins in each row, so that the CST build (Alg. 1) reads
+ * only the neighbours with the label it keeps.
  * Errors: FAST_ERR_INVALID for ids or labels out of range.
  */
 int fast_load_graph(int64_t n, int64_t m, const int32_t* edges, const int32_t* labels, int flags,
@@ -176,8 +175,9 @@ int fast_load_graph(int64_t n, int64_t m, const int32_t* edges, const int32_t* l
  * (max label + 1) and maximum degree D_G. */
 int fast_graph_info(const fast_graph* g, int64_t* n, int64_t* nadj, int32_t* num_labels, int64_t* max_degree);
 
-/* Copy the CSR to host arrays row_ptr[n+1] and col[nadj], rows in the
- * layout above (a test aid). */
+/* Copy the CSR to host arrays row_ptr[n+1] and col[nadj], as ids: each row by
+ * (label of the neighbour, id) when 2 * bits(n - 1) + bits(labels - 1) <= 64,
+ * otherwise by id (a test aid). */
 int fast_graph_copy_csr(const fast_graph* g, int64_t* row_ptr, int32_t* col, void* stream);
 
 /* Free G.  Device memory the library frees stays pooled in this process
@@ -219,7 +219,8 @@ int fast_build_cst(const fast_graph* g, const fast_query_desc* q, const fast_con
  * workload estimate of Sec. IV-C, as fast_build_cst): the steps go over BFS
  * positions, and each step is one launch for the vertex at that position of
  * every query, with one or two host round trips per position for the whole
- * batch instead of a few per query.  outs[i] receives query i's CST, which
+ * batch (a handful in all for up to 8 queries).  fast_build_cst is a batch of
+ * one.  outs[i] receives query i's CST, which
  * is the same, array for array, as fast_build_cst gives; the caller frees
  * each with fast_free_cst.  status[i] is FAST_OK, or FAST_ERR_INVALID for a
  * bad query (outs[i] is then NULL).  Queries are built in groups of up to
@@ -506,7 +507,7 @@ uint64_t fast_now_ns(void);
  * cudaFree, no host staging buffer.
  *
  * Scratch: one file-scope device array of fast_match_noalloc_scratch_bytes()
- * bytes (about 5.9 MB: the counter block, a ring of 4096 donated runs and
+ * bytes (about 6.6 MB: the counter block, 8192 cells for donated runs and
  * up to 32768 root-run descriptors) that every GPU loading the library keeps
  * until the process exits.  The first call on a device looks up its address
  * (cudaGetSymbolAddress, with that device current).  All calls share the
@@ -570,10 +571,9 @@ uint64_t fast_kernel_launches(void);
 /* Host round trips (device-to-host size reads the host waited for) of the
  * calling thread's last batched CST build (fast_build_cst_batch, or a batch
  * run with build_rule 2).  A batch of at most 8 queries whose bounded
- * top-down arrays fit in 2 GB builds its top-down pass with none: its
- * arrays are sized by host-known bounds (|C0| of the parent, the graph's
- * count of adjacency entries between the two labels) and the kernels read
- * the real sizes on the device. */
+ * arrays fit in 2 GB builds its lists with one: its temporary arrays are
+ * sized by host-known bounds (the graph's count of adjacency entries between
+ * the two labels) and the kernels read the real sizes on the device. */
 uint64_t fast_last_build_round_trips(void);
 
 #ifdef __cplusplus

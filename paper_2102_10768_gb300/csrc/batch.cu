@@ -1,7 +1,7 @@
 // Batched matching: many queries in one matcher launch.
 //
 // A fast_batch owns fixed device buffers (per-query plans, counters, the
-// ring of donated runs), so that its matcher launch can be captured once as a
+// cells of donated runs), so that its matcher launch can be captured once as a
 // CUDA graph and replayed for every batch.
 // A batch run has three phases:
 //   1. a pool of host threads, each with its own CUDA stream and scratch
@@ -49,7 +49,7 @@ using namespace fast;
 namespace {
 
 constexpr int kClasses = 5;                       // |V(q)| <= 4, 8, 16, 24, 32
-constexpr uint64_t kBatchQueue = 1 << 16;         // cells of the ring of donated runs
+constexpr uint64_t kBatchQueue = 1 << 16;         // cells for donated runs
 enum { kStatusTimeout = 1, kStatusOverflow = 2, kStatusLimit = 4 };
 
 int size_class(int k) { return k <= 4 ? 0 : k <= 8 ? 1 : k <= 16 ? 2 : k <= 24 ? 3 : 4; }

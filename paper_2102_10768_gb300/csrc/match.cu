@@ -9,9 +9,9 @@
 //                    every earlier non-tree neighbour's image, all sorted
 //                    over C(u_d); the warp scans the shortest of them;
 //   EdgeValidator    membership in each other list by a warp-cooperative
-//                    merge (a cursor per list, coalesced 32-entry tiles, a
-//                    shuffle search, galloping), shortest lists first,
-//                    stopping once no candidate is left;
+//                    merge (a cursor per list, a 128-entry tile, a shuffle
+//                    search, a window search past the tile), shortest lists
+//                    first, stopping once no candidate is left;
 //   VisitedValidator the candidate's data vertex against the images of the
 //                    earlier positions with the same label (distinct labels
 //                    cannot collide);
@@ -19,7 +19,8 @@
 // shared memory and expanded one by one, or counted -- and optionally written
 // out -- at the last position.  The per-depth scan state lives in registers
 // of the lane whose index is the depth (depth <= 31), so no per-depth array
-// is indexed dynamically.
+// is indexed dynamically.  Queries of short lists are searched flat instead
+// (flat_search below).
 //
 // Load balance: a persistent grid first drains the static chunks (each query
 // of a batch has its own cursor, and the warps start spread over the
@@ -37,7 +38,7 @@
 // 10-vertex query with two-entry lists in 115; with tickets that donors
 // served in order (one per 0.7 us) in 15.4 and 2.11 ms, half of the warps'
 // time spent waiting; with cells that donors pick apart from one another in
-// 8.1 and 1.52.
+// 8.1 and 1.52 (7.5 and 1.36 with the flat search's present steps).
 //
 // Warp-specialised variant (the GPU form of the task-generator separation
 // of Sec. V-D): a CTA's warps split into expanders and validators.  The
@@ -640,8 +641,8 @@ __device__ void validate_tasks(const MatchPlan& P0, const MatchPlan* __restrict_
 // loaded once for 32 candidates).  make_plan decides.  Measured, before and
 // after: complete enumeration of a 10-vertex tree query with two-entry lists
 // (31 M embeddings) 24.7 -> 1.9 ms; of 12 4-vertex queries on the 1M/16M
-// power-law graph (3.2 G embeddings) 106 -> 41 ms, and 18 with the short form
-// of the last position; 8.4 M rows written 2.9 -> 2.0 ms.
+// power-law graph (3.2 G embeddings) 106 -> 41 ms, and 18 with the first short
+// form of the last position; 8.4 M rows written 2.9 -> 2.0 ms.
 //
 // Order of work, totals, floor and donations are as in the other search: a
 // donated run is the list of one partial result, or the second half of what is
@@ -1477,7 +1478,11 @@ __global__ void __launch_bounds__(256, 4) k_match(const __grid_constant__ MatchP
 // that nothing is checked, or whose lists are all short, so that a check is a
 // short binary search.  Short means the length of the list that a random list
 // entry belongs to (hubs count by their entries): on a power-law graph that is
-// hundreds where the plain mean is seven, and there the merges win.
+// hundreds where the plain mean is seven, and there the merges win (taken flat
+// all the same, 40 queries took 13.5 instead of 12.3 ms, two queries of 6 and 8
+// vertices 1.53 instead of 1.38).  Cycles in full on an Erdos-Renyi graph of
+// 1M vertices and 16M edges, flat and merged: 3.3 and 28 ms where lists have 4
+// entries, 19.6 and 99.8 with 8, 43 and 90 with 16, 641 and 764 with 32.
 constexpr double kFlatLength = 32.0;
 
 bool flat_query(const fast_cst* c) {
@@ -1583,16 +1588,16 @@ int matcher_smem_optin(size_t bytes) {
 }
 
 // Counter block (8-byte words).  What different warps hammer lies in lines of
-// its own: the total, the embedding cursor, the static cursor, the
-// number of waiting warps.  The first kCtrWords
-// come back to the host; the copies of the done flag follow.
+// its own: the total, the embedding cursor, the static cursor, the number of
+// waiting warps.  The first kCtrWords come back to the host; the copies of the
+// done flag follow.
 enum { kStatus = 0, kBytes, kFloor, kDeadline, kStarted, kQStop, kStats = 8,
        kTotal = (kStats + kMaxK + kLineWords - 1) / kLineWords * kLineWords, kSlot = kTotal + kLineWords,
        kCtrWords = kSlot + 1, kNext = kSlot + kLineWords, kIdle = kNext + kLineWords,
        kDone = kIdle + kLineWords, kAllWords = kDone + kDoneCopies * kLineWords };
 constexpr uint64_t kQueueCap = 1 << 16;
 
-// Cells of the donation ring for a launch of `warps` warps: cfg.queue_cells
+// Cells for donated runs of a launch of `warps` warps: cfg.queue_cells
 // if given (at most cap), else one per warp, so that every warp has a cell of
 // its own to wait on.
 uint64_t ring_cells(int64_t queue_cells, int64_t warps, uint64_t cap) {
@@ -1635,7 +1640,7 @@ int run_match(const fast_cst* c, const fast_chunks* chunks, const fast_config* c
     if (!c) return set_error(FAST_ERR_INVALID, "fast_match: cst is NULL");
     if (kemb > 0 && !emb_out) return set_error(FAST_ERR_INVALID, "fast_match: k > 0 needs emb_out");
     if (chunks && chunks->c != c) return set_error(FAST_ERR_INVALID, "fast_match: chunks belong to another CST");
-    PoolScope scratch(s);                        // counters, donation ring, staging: temporaries
+    PoolScope scratch(s);                        // counters, donated runs, staging: temporaries
     fast_config cfg = cfg_in ? *cfg_in : c->cfg;
     int warps = cfg.warps_per_block > 0 ? cfg.warps_per_block : 8;
     if (warps > 8) warps = 8;

@@ -286,11 +286,10 @@ int compact_alloc(const F& f, int64_t n, typename F::value_type** out, int64_t* 
 //
 // Stable LSD radix sort of uint64 keys, 8-bit digits, over the digit
 // positions listed in `shifts`.  Three kernels per pass: per-tile digit
-// histograms, a digit-major exclusive scan of them, and a stable scatter that
-// ranks keys inside a tile warp by warp with __match_any_sync.
+// histograms, a digit-major exclusive scan of them, and a stable scatter.
 
 constexpr int kSortBlock = 256;
-constexpr int kSortRounds = 16;
+constexpr int kSortRounds = 8;
 constexpr int kSortTile = kSortBlock * kSortRounds;
 
 static __global__ void k_radix_hist(const uint64_t* __restrict__ keys, int64_t n, int shift, int64_t nblocks,
@@ -299,49 +298,100 @@ static __global__ void k_radix_hist(const uint64_t* __restrict__ keys, int64_t n
     h[threadIdx.x] = 0;
     __syncthreads();
     int64_t base = (int64_t)blockIdx.x * kSortTile;
+    uint64_t key[kSortRounds];            // all loads in flight at once
+#pragma unroll
     for (int r = 0; r < kSortRounds; r++) {
-        int64_t i = base + (int64_t)r * kSortBlock + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1u);
+        const int64_t i = base + (int64_t)r * kSortBlock + threadIdx.x;
+        key[r] = i < n ? keys[i] : 0;
     }
+#pragma unroll
+    for (int r = 0; r < kSortRounds; r++)
+        if (base + (int64_t)r * kSortBlock + threadIdx.x < n) atomicAdd(&h[(key[r] >> shift) & 255u], 1u);
     __syncthreads();
     hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
 }
 
-static __global__ void k_radix_scatter(const uint64_t* __restrict__ in, uint64_t* __restrict__ out, int64_t n,
+// A warp ranks its own 256 keys, 32 at a time: the lanes with one digit are
+// found by eight ballots, and its counts lie in its own row of shared memory,
+// so no block barrier stands between two steps.  One scan over the warps and
+// the digits gives every key its place in the tile; the tile is put in order
+// in shared memory and leaves it digit by digit, so that neighbouring lanes
+// write neighbouring keys.  Bound by the ranking's instructions (a pass over
+// 32 M keys moves 512 MB).  With a block barrier per step and keys written
+// from where they were read, such a pass took 245 us; the loader of a 16M-edge
+// graph on the device 3.56 -> 2.94 ms (3.12 with 4096 keys a tile and three
+// blocks per SM, 2.98 with 3072 and four).
+static __global__ void __launch_bounds__(kSortBlock, 6) k_radix_scatter(const uint64_t* __restrict__ in,
+                                uint64_t* __restrict__ out, int64_t n,
                                 int shift, int64_t nblocks, const uint32_t* __restrict__ offs) {
     constexpr int NW = kSortBlock / 32;
-    __shared__ uint32_t goff[256];        // global start of this tile's digit run
-    __shared__ uint32_t run[256];         // keys of each digit already placed
-    __shared__ uint32_t wcnt[NW][256];    // per-round per-warp counts -> offsets
+    __shared__ uint64_t tile[kSortTile];
+    __shared__ uint32_t wcnt[NW][256];    // each warp's counts, then the keys of the digit in the warps before it
+    __shared__ uint32_t start[256];       // where each digit begins in the tile
+    __shared__ uint32_t wsum[NW];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    goff[threadIdx.x] = offs[(int64_t)threadIdx.x * nblocks + blockIdx.x];
-    run[threadIdx.x] = 0;
-    int64_t base = (int64_t)blockIdx.x * kSortTile;
+    const uint32_t goff = offs[(int64_t)threadIdx.x * nblocks + blockIdx.x];   // global start of this tile's digit run
+#pragma unroll
+    for (int w = 0; w < NW; w++) wcnt[w][threadIdx.x] = 0;
+    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+    const int count = (int)(n - base < kSortTile ? n - base : kSortTile);
+    const int first = warp * 32 * kSortRounds + lane;
+    uint64_t key[kSortRounds];
+#pragma unroll
+    for (int r = 0; r < kSortRounds; r++) key[r] = first + 32 * r < count ? in[base + first + 32 * r] : 0;
+    __syncthreads();
+    uint32_t rank[kSortRounds];           // among the warp's keys of the digit
+#pragma unroll
     for (int r = 0; r < kSortRounds; r++) {
+        const bool valid = first + 32 * r < count;
+        const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
+        uint32_t peers = __ballot_sync(0xffffffffu, valid);
 #pragma unroll
-        for (int w = 0; w < NW; w++) wcnt[w][threadIdx.x] = 0;
-        __syncthreads();
-        int64_t i = base + (int64_t)r * kSortBlock + threadIdx.x;
-        bool valid = i < n;
-        uint64_t key = valid ? in[i] : 0;
-        uint32_t d = valid ? (uint32_t)((key >> shift) & 255u) : 256u + lane;
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        uint32_t rank = __popc(peers & lanemask_lt());
-        if (valid && rank == 0) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        {
-            uint32_t b = run[threadIdx.x];
-#pragma unroll
-            for (int w = 0; w < NW; w++) {
-                uint32_t c = wcnt[w][threadIdx.x];
-                wcnt[w][threadIdx.x] = b;
-                b += c;
-            }
-            run[threadIdx.x] = b;
+        for (int b = 0; b < 8; b++) {
+            const uint32_t m = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+            peers &= (d >> b) & 1u ? m : ~m;
         }
-        __syncthreads();
-        if (valid) out[goff[d] + wcnt[warp][d] + rank] = key;
-        __syncthreads();
+        const uint32_t before = __popc(peers & lanemask_lt());
+        uint32_t c = 0;
+        if (valid) c = wcnt[warp][d];
+        __syncwarp();
+        if (valid && before == 0) wcnt[warp][d] = c + __popc(peers);
+        __syncwarp();
+        rank[r] = c + before;
+    }
+    __syncthreads();
+    uint32_t total = 0;                   // of digit threadIdx.x
+#pragma unroll
+    for (int w = 0; w < NW; w++) {
+        const uint32_t c = wcnt[w][threadIdx.x];
+        wcnt[w][threadIdx.x] = total;
+        total += c;
+    }
+    uint32_t incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    uint32_t s0 = incl - total;
+#pragma unroll
+    for (int w = 0; w < NW; w++) s0 += w < warp ? wsum[w] : 0u;
+    start[threadIdx.x] = s0;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortRounds; r++)
+        if (first + 32 * r < count) {
+            const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
+            tile[start[d] + wcnt[warp][d] + rank[r]] = key[r];
+        }
+    __syncthreads();
+    wcnt[0][threadIdx.x] = goff - s0;     // what to add to a place in the tile
+    __syncthreads();
+    for (int i = threadIdx.x; i < count; i += kSortBlock) {
+        const uint64_t k = tile[i];
+        out[wcnt[0][(k >> shift) & 255u] + (uint32_t)i] = k;
     }
 }
 

@@ -83,6 +83,20 @@ def test_loader_label_lookup(n, m, L, by_id):
             compare_cst(F.Cst(g, ql, PATH3), oracle.Cst(o, ql, PATH3), 3)
 
 
+# both sorts of the loader at the edges of a 2048-key tile and of a warp's 256
+# (vertices: one key each; edges: two), few distinct keys and many
+@pytest.mark.parametrize("n", [2, 255, 256, 257, 2047, 2048, 2049, 6145])
+@pytest.mark.parametrize("m", [1, 127, 128, 129, 1023, 1024, 1025, 5000])
+def test_loader_sort_tiles(n, m):
+    rng = np.random.default_rng(n * 10_000 + m)
+    e = rng.integers(0, n, size=(m, 2)).astype(np.int32)
+    lab = rng.integers(0, 300, size=n).astype(np.int32)
+    g = F.Graph(n, e, lab)
+    off, col = g.csr()
+    ooff, ocol = csr_by_label(*oracle.Graph(n, e, lab).csr(), lab)
+    assert np.array_equal(off, ooff) and np.array_equal(col, ocol)
+
+
 @pytest.mark.parametrize("shift", [0, 1, 2, 3])
 def test_loader_takes_device_edges_at_any_word(shift):
     import torch

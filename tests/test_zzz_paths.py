@@ -209,6 +209,31 @@ def test_flat_and_general_search_by_query_size(k, labels):
         _check(g, o, ql, ring, emit=20_000)
 
 
+@pytest.mark.parametrize("nq", [31, 32, 33, 64, 65, 131])
+def test_batches_around_the_window_of_queries(nq):
+    """Warps go from a query to the 32nd after it: every query is finished,
+    whatever the number, with some that are invalid or have no embedding."""
+    rng = np.random.default_rng(nq)
+    n, m = 500, 3000
+    e = rng.integers(0, n, size=(m, 2)).astype(np.int32)
+    lab = rng.integers(0, 4, size=n).astype(np.int32)
+    g, o = F.Graph(n, e, lab), oracle.Graph(n, e, lab)
+    qs = []
+    for i in range(nq):
+        k = int(rng.integers(1, 6))
+        ql = rng.integers(0, 5 if i % 7 == 0 else 4, size=k).astype(np.int32)      # label 4: in no vertex
+        qe = [(int(rng.integers(0, v)), v) for v in range(1, k)] + ([(0, 2)] if k > 2 else [])
+        qs.append((ql, np.array(sorted(set(qe)), np.int32).reshape(-1, 2)))
+    qs[nq // 2] = (np.zeros(3, np.int32), np.array([[0, 1]], np.int32))            # disconnected
+    lim = 5000
+    counts, status = F.Batch(g, nq, F.default_config(limit=lim, build_rule=2)).run(qs)
+    for i, (ql, qe) in enumerate(qs):
+        if i == nq // 2:
+            assert status[i] == F.FAST_ERR_INVALID
+            continue
+        assert status[i] == 0 and counts[i] == oracle.match(o, ql, qe, limit=lim)["count"], i
+
+
 # ---------------------------------------------------------------- partition
 
 @pytest.mark.parametrize("div", [1, 30, 3000])
